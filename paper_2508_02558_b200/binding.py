@@ -1,4 +1,5 @@
-"""ctypes binding of libsdllm.so: same names as the C ABI (include/sdllm.h), argument marshalling only.
+"""Binding of libsdllm.so: same names as the C ABI (include/sdllm.h), argument marshalling only - ctypes for the host
+helpers, native builtins (csrc/marshal.cpp) for the device calls, which a decoding loop issues every few microseconds.
 
 Every step of the path runs inside the CUDA library; nothing here computes. Tensors are passed as
 torch tensors (their data_ptr() is taken), raw integer addresses, or None for nullable arguments.
@@ -12,6 +13,7 @@ from typing import Optional, Sequence
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libsdllm.so")
+MARSHAL_PATH = os.path.join(_PKG, "_marshal.so")
 
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT = range(6)
 F32, BF16 = 0, 1
@@ -72,6 +74,7 @@ def lib() -> ctypes.CDLL:
         L.sdllm_cache_state.argtypes = [ctypes.c_int32, ctypes.c_int32]
         L.sdllm_read_status.restype = ctypes.c_int
         L.sdllm_read_status.argtypes = [vp, vp, ctypes.POINTER(ctypes.c_int32)]
+        # (the device calls are issued by the builtins of csrc/marshal.cpp; these declarations serve direct users of lib())
         L.sdllm_refresh_scores.restype = ctypes.c_int
         L.sdllm_refresh_scores.argtypes = [dp, vp, vp, vp, i32p, i32p, vp, vp, vp, vp, ctypes.c_size_t, vp]
         L.sdllm_sparse_block_attn_static.restype = ctypes.c_int
@@ -95,6 +98,28 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+_native = None
+
+# Entry points of the device calls, in the order csrc/marshal.cpp numbers them.
+_DEVICE_CALLS = ("sdllm_refresh_scores", "sdllm_select_topk", "sdllm_compact_kv", "sdllm_select_compact", "sdllm_sparse_block_attn",
+                 "sdllm_sparse_block_attn_static", "sdllm_dense_attn")
+
+
+def native():
+    """The builtins that marshal the device calls (csrc/marshal.cpp), bound to the library; raises if they are missing."""
+    global _native
+    if _native is None:
+        import torch
+        L = lib()
+        if not os.path.exists(MARSHAL_PATH):
+            raise RuntimeError(f"{MARSHAL_PATH} is missing: run `python -m paper_2508_02558_b200.build` "
+                               "(there is no fallback path)")
+        from . import _marshal
+        _marshal.bind(torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice, *(ctypes.cast(getattr(L, f), ctypes.c_void_p).value for f in _DEVICE_CALLS))
+        _native = _marshal
+    return _native
+
+
 def _ptr(x) -> Optional[int]:
     if x is None:
         return None
@@ -103,14 +128,6 @@ def _ptr(x) -> Optional[int]:
     if isinstance(x, tuple):          # (address, bytes) pair for a workspace
         return x[0]
     return x.data_ptr()
-
-
-def _nbytes(x) -> int:
-    if x is None or isinstance(x, int):
-        return 0
-    if isinstance(x, tuple):
-        return int(x[1])
-    return x.numel() * x.element_size()
 
 
 def _stream(stream) -> Optional[int]:
@@ -195,48 +212,41 @@ def read_status(workspace, stream=None) -> int:
 
 
 def refresh_scores(desc: Desc, q_blk, k, v, seq_len, block_off, out, lse, pooled_scores, workspace, stream=None):
-    _check(lib().sdllm_refresh_scores(ctypes.byref(desc), _ptr(q_blk), _ptr(k), _ptr(v), _ptr(seq_len), _ptr(block_off),
-                                      _ptr(out), _ptr(lse), _ptr(pooled_scores), _ptr(workspace), _nbytes(workspace),
-                                      _stream(stream)), "sdllm_refresh_scores")
+    _check((_native or native()).refresh_scores(desc, q_blk, k, v, seq_len, block_off, out, lse, pooled_scores, workspace, stream),
+           "sdllm_refresh_scores")
 
 
 def select_topk(desc: Desc, pooled_scores, seq_len, block_off, kept_idx, kept_cnt, workspace=None, stream=None):
-    _check(lib().sdllm_select_topk(ctypes.byref(desc), _ptr(pooled_scores), _ptr(seq_len), _ptr(block_off), _ptr(kept_idx),
-                                   _ptr(kept_cnt), _ptr(workspace), _nbytes(workspace), _stream(stream)),
+    _check((_native or native()).select_topk(desc, pooled_scores, seq_len, block_off, kept_idx, kept_cnt, workspace, stream),
            "sdllm_select_topk")
 
 
 def compact_kv(desc: Desc, k, v, kept_idx, kept_cnt, k_c, v_c, stream=None):
-    _check(lib().sdllm_compact_kv(ctypes.byref(desc), _ptr(k), _ptr(v), _ptr(kept_idx), _ptr(kept_cnt), _ptr(k_c),
-                                  _ptr(v_c), _stream(stream)), "sdllm_compact_kv")
+    _check((_native or native()).compact_kv(desc, k, v, kept_idx, kept_cnt, k_c, v_c, stream), "sdllm_compact_kv")
 
 
 def select_compact(desc: Desc, pooled_scores, seq_len, block_off, k, v, kept_idx, kept_cnt, k_c, v_c, stream=None):
     """sdllm_select_topk and sdllm_compact_kv in one call (one launch while a head's candidates fit a CTA)."""
-    _check(lib().sdllm_select_compact(ctypes.byref(desc), _ptr(pooled_scores), _ptr(seq_len), _ptr(block_off), _ptr(k), _ptr(v),
-                                      _ptr(kept_idx), _ptr(kept_cnt), _ptr(k_c), _ptr(v_c), _stream(stream)),
+    _check((_native or native()).select_compact(desc, pooled_scores, seq_len, block_off, k, v, kept_idx, kept_cnt, k_c, v_c, stream),
            "sdllm_select_compact")
 
 
 def sparse_block_attn(desc: Desc, q_blk, k_c, v_c, kept_cnt, k_blk, v_blk, out, workspace, stream=None):
-    _check(lib().sdllm_sparse_block_attn(ctypes.byref(desc), _ptr(q_blk), _ptr(k_c), _ptr(v_c), _ptr(kept_cnt),
-                                         _ptr(k_blk), _ptr(v_blk), _ptr(out), _ptr(workspace), _nbytes(workspace),
-                                         _stream(stream)), "sdllm_sparse_block_attn")
+    _check((_native or native()).sparse_block_attn(desc, q_blk, k_c, v_c, kept_cnt, k_blk, v_blk, out, workspace, stream),
+           "sdllm_sparse_block_attn")
 
 
 def sparse_block_attn_static(desc: Desc, q_blk, k_c, v_c, kept_cnt, k_blk, v_blk, out, stream=None):
     """The reuse step without a caller workspace (scratch built into the library; shapes above its 8 MiB are refused)."""
-    _check(lib().sdllm_sparse_block_attn_static(ctypes.byref(desc), _ptr(q_blk), _ptr(k_c), _ptr(v_c), _ptr(kept_cnt),
-                                                _ptr(k_blk), _ptr(v_blk), _ptr(out), _stream(stream)),
+    _check((_native or native()).sparse_block_attn_static(desc, q_blk, k_c, v_c, kept_cnt, k_blk, v_blk, out, stream),
            "sdllm_sparse_block_attn_static")
 
 
 def dense_attn(desc: Desc, q, k, v, seq_len, out, lse, workspace, stream=None):
     """Full-sequence bidirectional attention; q and out are [B, Hq, seq_len_max, D] tensors whose strides are passed on."""
-    qs = (ctypes.c_int64 * 3)(*(q.stride()[:3] if q is not None else (0, 0, 0)))
-    os_ = (ctypes.c_int64 * 3)(*(out.stride()[:3] if out is not None else (0, 0, 0)))
-    _check(lib().sdllm_dense_attn(ctypes.byref(desc), _ptr(q), qs, _ptr(k), _ptr(v), _ptr(seq_len), _ptr(out), os_, _ptr(lse),
-                                  _ptr(workspace), _nbytes(workspace), _stream(stream)), "sdllm_dense_attn")
+    strides = (ctypes.c_int64 * 6)(*(q.stride()[:3] if q is not None else (0, 0, 0)), *(out.stride()[:3] if out is not None else (0, 0, 0)))
+    at = ctypes.addressof(strides)
+    _check((_native or native()).dense_attn(desc, q, at, k, v, seq_len, out, at + 24, lse, workspace, stream), "sdllm_dense_attn")
 
 
 def tuning_set(name: str, value: int):

@@ -1,9 +1,11 @@
-"""Builds libsdllm.so in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Builds libsdllm.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and beside it the native part of the
+Python binding (`_marshal.so`, host C++ only)."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -12,6 +14,8 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OBJ_DIR = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libsdllm.so")
+MARSHAL = os.path.join(PKG, "_marshal.so")
+MARSHAL_SRC = os.path.join(CSRC, "marshal.cpp")
 
 NVCC_FLAGS = ["-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
               "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
@@ -32,8 +36,16 @@ def _deps_mtime() -> float:
     return max(os.path.getmtime(f) for f in files)
 
 
+def _build_marshal() -> None:
+    subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-I", sysconfig.get_paths()["include"],
+                    "-I", INCLUDE, "-o", MARSHAL, MARSHAL_SRC], check=True)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu under csrc/ and link libsdllm.so; a no-op when the library is newer than its sources."""
+    """Compile every .cu under csrc/ and link libsdllm.so, and compile _marshal.so; a no-op when both are newer than their
+    sources."""
+    if force or not os.path.exists(MARSHAL) or os.path.getmtime(MARSHAL) < max(os.path.getmtime(MARSHAL_SRC), _deps_mtime()):
+        _build_marshal()
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _deps_mtime():
         return LIB
     os.makedirs(OBJ_DIR, exist_ok=True)

@@ -1,0 +1,170 @@
+// Native argument marshalling of the Python binding: one builtin per device call of the C ABI.
+//
+// A reuse step keeps the GPU busy for 7 us, and a step through a model is a chain of such calls from one Python thread, so
+// what the host spends per call decides whether the GPU ever waits. Marshalled through ctypes and torch.cuda.current_stream()
+// a call took 9.5 us of host time (3.1 us for the stream object, 2.3 us of argument conversion); through these builtins it
+// takes the library's own time plus about 0.7 us.
+//
+// Arguments: the description (any object with the buffer interface, a ctypes Structure here), then device pointers given as
+// tensors (their data_ptr()), integers or None, then - where the call takes one - the workspace (tensor, (address, bytes) or
+// None) and the stream (None: torch's current stream of the current device, an integer, or a stream object). Each returns the
+// call's status as an integer; the GIL is released while the library runs.
+#define PY_SSIZE_T_CLEAN
+#include <Python.h>
+
+#include <stdint.h>
+
+#include <utility>
+
+#include "sdllm.h"
+
+namespace {
+
+PyObject *s_data_ptr, *s_nbytes, *s_cuda_stream;      // interned attribute names
+PyObject *g_raw_stream, *g_device;                    // torch's current-stream and current-device getters
+void* g_fn[8];                                        // the library's entry points, in the order of `Entry`
+enum Entry { kRefresh, kSelect, kCompact, kSelectCompact, kSparse, kSparseStatic, kDense, kEntries };
+
+bool to_address(PyObject* v, uintptr_t* out) {
+  const unsigned long long x = PyLong_AsUnsignedLongLong(v);
+  if (x == (unsigned long long)-1 && PyErr_Occurred()) return false;
+  *out = (uintptr_t)x;
+  return true;
+}
+
+bool pointer_of(PyObject* x, uintptr_t* out) {
+  if (x == Py_None) { *out = 0; return true; }
+  if (PyLong_Check(x)) return to_address(x, out);
+  if (PyTuple_Check(x) && PyTuple_GET_SIZE(x) == 2) return to_address(PyTuple_GET_ITEM(x, 0), out);
+  PyObject* v = PyObject_CallMethodNoArgs(x, s_data_ptr);
+  if (!v) return false;
+  const bool ok = to_address(v, out);
+  Py_DECREF(v);
+  return ok;
+}
+
+// A bare address carries no size, as in the ctypes path.
+bool bytes_of(PyObject* x, size_t* out) {
+  uintptr_t n = 0;
+  bool ok = true;
+  if (PyTuple_Check(x) && PyTuple_GET_SIZE(x) == 2) {
+    ok = to_address(PyTuple_GET_ITEM(x, 1), &n);
+  } else if (x != Py_None && !PyLong_Check(x)) {
+    PyObject* v = PyObject_GetAttr(x, s_nbytes);
+    ok = v && to_address(v, &n);
+    Py_XDECREF(v);
+  }
+  *out = n;
+  return ok;
+}
+
+bool stream_of(PyObject* x, uintptr_t* out) {
+  if (PyLong_Check(x)) return to_address(x, out);
+  PyObject* v;
+  if (x == Py_None) {
+    PyObject* dev = PyObject_CallNoArgs(g_device);
+    if (!dev) return false;
+    v = PyObject_CallOneArg(g_raw_stream, dev);
+    Py_DECREF(dev);
+  } else {
+    v = PyObject_GetAttr(x, s_cuda_stream);
+  }
+  if (!v) return false;
+  const bool ok = to_address(v, out);
+  Py_DECREF(v);
+  return ok;
+}
+
+struct Buffer {                                       // the bytes of a buffer object while the call runs
+  Py_buffer view{};
+  bool held = false;
+  ~Buffer() { if (held) PyBuffer_Release(&view); }
+  bool get(PyObject* x) { return held = PyObject_GetBuffer(x, &view, PyBUF_SIMPLE) == 0; }
+};
+
+template <size_t>
+using Ptr = void*;
+
+// N device pointers, then (WS) the workspace and its size, then the stream.
+template <int ENTRY, bool WS, size_t... I>
+PyObject* call_impl(PyObject* const* args, Py_ssize_t n, std::index_sequence<I...>) {
+  constexpr size_t N = sizeof...(I);
+  if (n != (Py_ssize_t)(1 + N + (WS ? 1 : 0) + 1)) {
+    PyErr_SetString(PyExc_TypeError, "wrong number of arguments");
+    return nullptr;
+  }
+  if (!g_fn[ENTRY]) {
+    PyErr_SetString(PyExc_RuntimeError, "the library's entry points are not bound");
+    return nullptr;
+  }
+  Buffer desc;
+  uintptr_t p[N], ws = 0, stream = 0;
+  size_t ws_bytes = 0;
+  if (!desc.get(args[0])) return nullptr;
+  if ((size_t)desc.view.len < sizeof(sdllm_desc)) {
+    PyErr_SetString(PyExc_ValueError, "the description is too short");
+    return nullptr;
+  }
+  for (size_t i = 0; i < N; ++i)
+    if (!pointer_of(args[1 + i], &p[i])) return nullptr;
+  if (WS && (!pointer_of(args[1 + N], &ws) || !bytes_of(args[1 + N], &ws_bytes))) return nullptr;
+  if (!stream_of(args[n - 1], &stream)) return nullptr;
+  int st;
+  Py_BEGIN_ALLOW_THREADS
+  if constexpr (WS)
+    st = reinterpret_cast<int (*)(const void*, Ptr<I>..., void*, size_t, void*)>(g_fn[ENTRY])(
+        desc.view.buf, reinterpret_cast<void*>(p[I])..., reinterpret_cast<void*>(ws), ws_bytes, reinterpret_cast<void*>(stream));
+  else
+    st = reinterpret_cast<int (*)(const void*, Ptr<I>..., void*)>(g_fn[ENTRY])(desc.view.buf, reinterpret_cast<void*>(p[I])...,
+                                                                             reinterpret_cast<void*>(stream));
+  Py_END_ALLOW_THREADS
+  return PyLong_FromLong(st);
+}
+
+template <int ENTRY, int N, bool WS>
+PyObject* call(PyObject*, PyObject* const* args, Py_ssize_t n) {
+  return call_impl<ENTRY, WS>(args, n, std::make_index_sequence<N>());
+}
+
+// bind(raw_stream, device, address...): torch's getters and the addresses of the entry points, in the order of `Entry`.
+PyObject* bind(PyObject*, PyObject* const* args, Py_ssize_t n) {
+  if (n != 2 + kEntries) {
+    PyErr_SetString(PyExc_TypeError, "wrong number of arguments");
+    return nullptr;
+  }
+  for (int i = 0; i < kEntries; ++i) {
+    uintptr_t a;
+    if (!to_address(args[2 + i], &a)) return nullptr;
+    g_fn[i] = reinterpret_cast<void*>(a);
+  }
+  Py_XSETREF(g_raw_stream, Py_NewRef(args[0]));
+  Py_XSETREF(g_device, Py_NewRef(args[1]));
+  Py_RETURN_NONE;
+}
+
+template <typename F>
+constexpr PyCFunction fast(F f) { return reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(f)); }
+
+// (the strides of the dense call are host arrays, passed like pointers: their addresses)
+PyMethodDef methods[] = {
+    {"bind", fast(bind), METH_FASTCALL, nullptr},
+    {"refresh_scores", fast(call<kRefresh, 8, true>), METH_FASTCALL, nullptr},
+    {"select_topk", fast(call<kSelect, 5, true>), METH_FASTCALL, nullptr},
+    {"compact_kv", fast(call<kCompact, 6, false>), METH_FASTCALL, nullptr},
+    {"select_compact", fast(call<kSelectCompact, 9, false>), METH_FASTCALL, nullptr},
+    {"sparse_block_attn", fast(call<kSparse, 7, true>), METH_FASTCALL, nullptr},
+    {"sparse_block_attn_static", fast(call<kSparseStatic, 7, false>), METH_FASTCALL, nullptr},
+    {"dense_attn", fast(call<kDense, 8, true>), METH_FASTCALL, nullptr},
+    {nullptr, nullptr, 0, nullptr}};
+
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__marshal(void) {
+  s_data_ptr = PyUnicode_InternFromString("data_ptr");
+  s_nbytes = PyUnicode_InternFromString("nbytes");
+  s_cuda_stream = PyUnicode_InternFromString("cuda_stream");
+  if (!s_data_ptr || !s_nbytes || !s_cuda_stream) return nullptr;
+  return PyModule_Create(&module);
+}
