@@ -166,9 +166,10 @@ sdllm_status sdllm_compact_kv(const sdllm_desc* desc, const void* k, const void*
 
 /* Refresh step, parts 2 and 3 in one call (Algorithm 1 from "n <- floor(|I| r)" to the cache store): exactly the results of
  * sdllm_select_topk followed by sdllm_compact_kv - the same kept_idx, kept_cnt, k_c and v_c, bit for bit - but, while the
- * candidates of a head fit the shared memory of a CTA (seq_len_max - block_len <= 8192), in ONE launch: the CTAs that
- * select a head's entries copy its rows themselves, so the index list makes no round trip through memory. Longer
- * sequences run the two kernels one after the other inside this call (sdllm_launch_count tells which). The launch may
+ * candidates of a head fit the registers of a CTA (seq_len_max - block_len <= 8192) and there are no more (sequence, KV head)
+ * pairs than SMs, in ONE launch: the CTAs that select a head's entries copy its rows themselves, so the index list makes no
+ * round trip through memory. Longer sequences and larger batches run two kernels inside this call, the second of which
+ * starts while the first finishes (sdllm_launch_count tells which). The launch may
  * start while the kernel in front of it in the stream is finishing and reads pooled_scores only once that kernel has
  * completed; it holds its own dependents back until it has completed, so the reuse step that follows may read the
  * compacted cache early (see sdllm_sparse_block_attn). seq_len and block_off are older than the scores (the refresh

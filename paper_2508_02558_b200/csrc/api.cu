@@ -215,7 +215,7 @@ int32_t sdllm_launch_count(const sdllm_desc* d, int op) {
   if (op == SDLLM_OP_SELECT_TOPK) return 1;
   if (op == SDLLM_OP_COMPACT_KV) return d->n_keep_max > 0 ? 1 : 0;
   if (op == SDLLM_OP_SELECT_COMPACT)
-    return select_compact_is_fused(d->seq_len_max, d->block_len, d->n_keep_max) ? 1 : 1 + (d->n_keep_max > 0 ? 1 : 0);
+    return select_compact_is_fused(d->batch, d->n_kv_heads, d->seq_len_max, d->block_len, d->n_keep_max) ? 1 : 1 + (d->n_keep_max > 0 ? 1 : 0);
   if (op == SDLLM_OP_DENSE_ATTN) return dense_supported(d) ? 1 : -1;
   if (op != SDLLM_OP_REFRESH_SCORES && op != SDLLM_OP_SPARSE_BLOCK_ATTN) return -1;
   const bool refresh = op == SDLLM_OP_REFRESH_SCORES;
@@ -316,8 +316,6 @@ sdllm_status sdllm_select_topk(const sdllm_desc* d, const float* pooled_scores, 
   p.pooled = pooled_scores; p.seq_len = seq_len; p.block_off = block_off; p.kept_idx = kept_idx; p.kept_cnt = kept_cnt;
   p.B = d->batch; p.Hkv = d->n_kv_heads; p.Lmax = d->seq_len_max; p.b = d->block_len; p.n_keep_max = d->n_keep_max;
   p.mode = d->select; p.retention = d->retention;
-  const int cand = d->seq_len_max - d->block_len;
-  p.smem_keys = cand <= 45056 ? cand : 0;
   if (cuda_failed(launch_select_topk(p, reinterpret_cast<cudaStream_t>(cuda_stream)), "select launch")) return SDLLM_ERR_CUDA;
   return SDLLM_OK;
 }
@@ -353,8 +351,6 @@ sdllm_status sdllm_select_compact(const sdllm_desc* d, const float* pooled_score
   p.pooled = pooled_scores; p.seq_len = seq_len; p.block_off = block_off; p.kept_idx = kept_idx; p.kept_cnt = kept_cnt;
   p.B = d->batch; p.Hkv = d->n_kv_heads; p.Lmax = d->seq_len_max; p.b = d->block_len; p.n_keep_max = d->n_keep_max;
   p.mode = d->select; p.retention = d->retention;
-  const int cand = d->seq_len_max - d->block_len;
-  p.smem_keys = cand <= 45056 ? cand : 0;
   p.early_inputs = (tuning().pdl != 0 && tuning().early_loads != 0) ? 1 : 0;
   CompactParams c{};
   c.k = k; c.v = v; c.kept_idx = kept_idx; c.kept_cnt = kept_cnt; c.k_c = k_c; c.v_c = v_c;

@@ -88,7 +88,7 @@ struct SelectParams {
   int32_t* kept_idx; int32_t* kept_cnt;
   int B, Hkv, Lmax, b, n_keep_max, mode;
   double retention;
-  int smem_keys;               // candidates cached in shared memory (0 = read global every pass)
+  int gather_follows;          // selection alone: the next kernel in the stream is the gather, which waits for this one before it reads
   int early_inputs;            // fused kernel: seq_len and block_off are read ahead of the grid dependency
 };
 
@@ -112,7 +112,7 @@ cudaError_t launch_merge_pool(const MergeParams& p, cudaStream_t st);
 cudaError_t launch_select_topk(const SelectParams& p, cudaStream_t st);
 cudaError_t launch_compact(const CompactParams& p, cudaStream_t st);
 cudaError_t launch_select_compact(const SelectParams& p, const CompactParams& cp, cudaStream_t st);
-bool select_compact_is_fused(int Lmax, int b, int n_keep_max);
+bool select_compact_is_fused(int B, int Hkv, int Lmax, int b, int n_keep_max);
 
 __host__ __device__ inline int keep_count_total(int pre, int suf, double r, int mode, int* n_pre, int* n_suf) {
   // Algorithm 1: n = floor(|I| * r) in double; the other policies are described in sdllm.h.
