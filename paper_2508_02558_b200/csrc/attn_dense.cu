@@ -3,12 +3,21 @@
 // A dense contraction, bound by the tensor pipe and, in front of it, by the softmax. One CTA owns TWO 128-row query
 // tiles of one query head and streams the head's K/V once for both:
 //   warp 0      TMA producer: the two Q tiles, then K and V tiles (128 keys, 128-byte swizzle) into a two-slot ring
-//   warp 1      one thread issues tcgen05.mma. Per key tile j:  S0 = Q0 K_j^T,  O1 += P1(j-1) V_(j-1),  S1 = Q1 K_j^T,
+//   warp 1      tcgen05.mma issuer. Per key tile j:  S0 = Q0 K_j^T,  O1 += P1(j-1) V_(j-1),  S1 = Q1 K_j^T,
 //               O0 += P0(j) V_j  -  while the softmax warps of one query tile work, the tensor pipe serves the other
-//   warps 2-5   softmax of query tile 0, warps 6-9 of query tile 1: a thread owns one accumulator row (TMEM lane),
+//   warps 4-7   softmax of query tile 0, warps 8-11 of query tile 1: a thread owns one accumulator row (TMEM lane),
 //               reads its S row, keeps the running max / sum and writes P (bf16) over S in TMEM; O accumulates in
 //               TMEM and is rescaled in place only when the row's maximum grows by more than 2^8
 // Tensor memory (512 columns): S0 | S1 | O0 | O1, 128 columns each (D = 64 uses half of an O region).
+// The chain of one query tile is S -> softmax -> P V -> next S (P lies over S), so a key tile of a pair costs
+// softmax + hand-overs + 1024 tensor cycles, with the other query tile's 1024 inside the softmax. What was taken off it
+// (4540 -> 3000 cycles per pair of 128 x 128 tiles at D = 128):
+//   - the MMA warp runs its loop warp-uniformly: an MMA no longer costs more to issue than to execute;
+//   - P is handed over in two parts (96 keys, then 32), so that the first MMAs of P V run under the last exponentials;
+//   - three-operand maxima, two-lane fp32 arithmetic, a quarter of the exponentials on the FMA pipe (poly_exp2), one
+//     warp-uniform branch for the rare rescale, registers moved to the softmax warps (208 instead of 168).
+// 32 heads x 1280 rows: 56.3 -> 46.2 us; 32 (8 KV) heads x 32768 rows: 17.1 -> 14.6 ms, 1206 TFLOP/s. The long case is
+// bound by power (1.6 GHz under the 1000 W cap, where a library GEMM sustains 1408); a burst at full clock runs at 1368.
 // The finished rows go from TMEM through registers straight to global memory (bf16), normalised by the row sum.
 // Every wait on an mbarrier is bounded; on expiry the CTA sets an abort flag, records a code in the status word and
 // runs to its end (freeing its TMEM); the outputs of that call are then invalid.
@@ -23,8 +32,9 @@ namespace sdllm {
 using namespace dev;
 namespace {
 
-constexpr int DN_THREADS = 320;
+constexpr int DN_THREADS = 384;        // three warpgroups: producer and MMA issuer (and two idle warps), softmax, softmax
 constexpr int DN_STAGES = 2;
+constexpr int DN_POLY = 4;             // one pair of exponentials in DN_POLY is a polynomial (3 and 8 measured 1 to 2 % slower)
 
 struct DenseMaps {
   CUtensorMap q, k, v;
@@ -69,7 +79,7 @@ __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __
   const uint32_t bars = smem_u32(smem);
   auto BAR = [&](int i) { return bars + 8u * (uint32_t)i; };
   const int Q_FULL = 0, FULL_K = 1, FULL_V = 1 + NS, EMPTY_K = 1 + 2 * NS, EMPTY_V = 1 + 3 * NS;
-  const int S_FULL = 1 + 4 * NS, P_FULL = S_FULL + 2, PV_DONE = S_FULL + 4, DRAIN = S_FULL + 6;
+  const int S_FULL = 1 + 4 * NS, P_FULL = S_FULL + 2, PV_DONE = S_FULL + 6, DRAIN = S_FULL + 8;   // P_FULL: two parts per query tile
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + 256);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + 260);
   unsigned char* q_s = smem + 1024;
@@ -84,7 +94,8 @@ __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(BAR(S_FULL + i), 1);
-      mbar_init(BAR(P_FULL + i), 4);       // the four softmax warps of a query tile
+      mbar_init(BAR(P_FULL + 2 * i), 4);   // the four softmax warps of a query tile
+      mbar_init(BAR(P_FULL + 2 * i + 1), 4);
       mbar_init(BAR(PV_DONE + i), 1);
     }
     mbar_init(BAR(DRAIN), 1);
@@ -103,93 +114,115 @@ __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __
 
   auto tile_nv = [&](int j) { return min(n - j * KT, KT); };     // valid keys of tile j (> 0 for j < nt)
 
-  if (warp == 0) {
-    // ======================================= TMA producer =======================================
-    if (lane == 0) {
-      mbar_expect_tx(BAR(Q_FULL), (uint32_t)((act1 ? 2 : 1) * TILE));
-      for (int t = 0; t < (act1 ? 2 : 1); ++t)
-        for (int hh = 0; hh < H; ++hh)
-          tma_load_4d(smem_u32(q_s + t * TILE + hh * HALF), &tm.q, BAR(Q_FULL), hh * 64, row00 + t * 128, h, bi);
-      int issued = 0;
-      bool ok = true;
-      for (int j = 0; j < nt && ok; ++j) {
-        const int s = j % NS;
-        const uint32_t ph = ((j / NS) - 1) & 1;
-        const uint32_t kdst = smem_u32(stage0 + (size_t)s * 2 * TILE), vdst = kdst + TILE;
-        if (j >= NS && !wait_bar(BAR(EMPTY_K + s), ph, abort_flag, p.status, 21, p.wait_cycles)) { ok = false; break; }
-        mbar_expect_tx(BAR(FULL_K + s), (uint32_t)TILE);
-        for (int hh = 0; hh < H; ++hh) tma_load_4d(kdst + hh * HALF, &tm.k, BAR(FULL_K + s), hh * 64, j * KT, g, bi);
-        if (j >= NS && !wait_bar(BAR(EMPTY_V + s), ph, abort_flag, p.status, 22, p.wait_cycles)) {
-          drain_bar(BAR(FULL_K + s), (j / NS) & 1);                 // the K half of this slot is already on its way
-          ok = false; break;
+  // Registers move from the first warpgroup to the softmax warps: 128 * (72 + 2 * 208) of the 384 * 168 at launch.
+  if (warp < 4) {
+    regs_dec_72();
+    if (warp == 0) {
+      // ======================================= TMA producer =======================================
+      if (lane == 0) {
+        mbar_expect_tx(BAR(Q_FULL), (uint32_t)((act1 ? 2 : 1) * TILE));
+        for (int t = 0; t < (act1 ? 2 : 1); ++t)
+          for (int hh = 0; hh < H; ++hh)
+            tma_load_4d(smem_u32(q_s + t * TILE + hh * HALF), &tm.q, BAR(Q_FULL), hh * 64, row00 + t * 128, h, bi);
+        int issued = 0;
+        bool ok = true;
+        for (int j = 0; j < nt && ok; ++j) {
+          const int s = j % NS;
+          const uint32_t ph = ((j / NS) - 1) & 1;
+          const uint32_t kdst = smem_u32(stage0 + (size_t)s * 2 * TILE), vdst = kdst + TILE;
+          if (j >= NS && !wait_bar(BAR(EMPTY_K + s), ph, abort_flag, p.status, 21, p.wait_cycles)) { ok = false; break; }
+          mbar_expect_tx(BAR(FULL_K + s), (uint32_t)TILE);
+          for (int hh = 0; hh < H; ++hh) tma_load_4d(kdst + hh * HALF, &tm.k, BAR(FULL_K + s), hh * 64, j * KT, g, bi);
+          if (j >= NS && !wait_bar(BAR(EMPTY_V + s), ph, abort_flag, p.status, 22, p.wait_cycles)) {
+            drain_bar(BAR(FULL_K + s), (j / NS) & 1);                 // the K half of this slot is already on its way
+            ok = false; break;
+          }
+          mbar_expect_tx(BAR(FULL_V + s), (uint32_t)TILE);
+          for (int hh = 0; hh < H; ++hh) tma_load_4d(vdst + hh * HALF, &tm.v, BAR(FULL_V + s), hh * 64, j * KT, g, bi);
+          issued = j + 1;
         }
-        mbar_expect_tx(BAR(FULL_V + s), (uint32_t)TILE);
-        for (int hh = 0; hh < H; ++hh) tma_load_4d(vdst + hh * HALF, &tm.v, BAR(FULL_V + s), hh * 64, j * KT, g, bi);
-        issued = j + 1;
-      }
-      if (*abort_flag) {                    // let the copies that were issued land before the CTA retires
-        for (int j = max(issued - NS, 0); j < issued; ++j) {
-          drain_bar(BAR(FULL_K + j % NS), (j / NS) & 1);
-          drain_bar(BAR(FULL_V + j % NS), (j / NS) & 1);
+        if (*abort_flag) {                    // let the copies that were issued land before the CTA retires
+          for (int j = max(issued - NS, 0); j < issued; ++j) {
+            drain_bar(BAR(FULL_K + j % NS), (j / NS) & 1);
+            drain_bar(BAR(FULL_V + j % NS), (j / NS) & 1);
+          }
+          drain_bar(BAR(Q_FULL), 0);
         }
-        drain_bar(BAR(Q_FULL), 0);
       }
-    }
-  } else if (warp == 1) {
-    // ======================================= MMA issuer =======================================
-    if (lane == 0) {
+    } else if (warp == 1) {
+      // ======================================= MMA issuer =======================================
+      // The whole warp walks the tiles and one elected lane issues: with everything around the MMAs warp-uniform their
+      // descriptors live in uniform registers and an MMA costs a few instructions. (A loop run by one lane alone took about
+      // 600 cycles to issue eight MMAs, more than their 512 cycles of execution.)
+      const bool leader = elect_one();
       const uint32_t idesc_pv = instr_desc(D, true);
-      const uint32_t qsm = smem_u32(q_s);
-      bool ok = wait_bar(BAR(Q_FULL), 0, abort_flag, p.status, 23, p.wait_cycles);
+      const uint64_t q_desc = smem_desc(smem_u32(q_s), 16u, 1024u), k_desc = smem_desc(smem_u32(stage0), 16u, 1024u);
+      const uint64_t v_desc = smem_desc(smem_u32(stage0) + TILE, (uint32_t)HALF, 1024u);
+      bool ok = wait_bar_warp(BAR(Q_FULL), 0, abort_flag, p.status, 23, p.wait_cycles);
       // S_t = Q_t K_j^T into the S region of query tile t
       auto issue_s = [&](int t, int j) {
-        const uint32_t ksm = smem_u32(stage0 + (size_t)(j % NS) * 2 * TILE);
         const uint32_t idesc_s = instr_desc((tile_nv(j) + 15) & ~15, false);
         const uint32_t d_t = tmem_base + S_COL0 + (uint32_t)t * T_STRIDE;
+        const uint64_t qd = q_desc + (uint64_t)(t * (TILE >> 4)), kd = k_desc + (uint64_t)((j % NS) * (2 * TILE >> 4));
+        if (leader) {
 #pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) {
-          const uint32_t off = (ks >> 2) * HALF + (ks & 3) * 32;
-          mma_ss(d_t, smem_desc(qsm + t * TILE + off, 16u, 1024u), smem_desc(ksm + off, 16u, 1024u), idesc_s, ks > 0 ? 1u : 0u);
+          for (int ks = 0; ks < D / 16; ++ks) {
+            const uint64_t off = (uint64_t)(((ks >> 2) * HALF + (ks & 3) * 32) >> 4);
+            mma_ss(d_t, qd + off, kd + off, idesc_s, ks > 0 ? 1u : 0u);
+          }
+          tc_commit(BAR(S_FULL + t));
         }
-        tc_commit(BAR(S_FULL + t));
+        __syncwarp();
       };
-      // O_t += P_t V_j once the softmax warps of query tile t have written P_t; `release` frees the V slot afterwards
+      // O_t += P_t V_j as the softmax warps of query tile t hand P_t over; `release` frees the V slot afterwards
       auto issue_pv = [&](int t, int j, bool release) -> bool {
         const int s = j % NS;
-        if (!wait_bar(BAR(P_FULL + t), j & 1, abort_flag, p.status, 24, p.wait_cycles)) return false;
-        if (!wait_bar(BAR(FULL_V + s), (j / NS) & 1, abort_flag, p.status, 25, p.wait_cycles)) return false;
-        tc_fence_after();
-        const uint32_t vsm = smem_u32(stage0 + (size_t)s * 2 * TILE) + TILE;
-        const uint32_t a_t = tmem_base + S_COL0 + (uint32_t)t * T_STRIDE;
-        const int n_mma = (tile_nv(j) + 15) & ~15;
-        for (int ks = 0; ks < n_mma / 16; ++ks)
-          mma_ts(tmem_base + O_COL0 + (uint32_t)t * T_STRIDE, a_t + ks * 8, smem_desc(vsm + ks * 2048, (uint32_t)HALF, 1024u), idesc_pv,
-                 (j > 0 || ks > 0) ? 1u : 0u);
-        tc_commit(BAR(PV_DONE + t));
-        if (release) tc_commit(BAR(EMPTY_V + s));
+        if (!wait_bar_warp(BAR(FULL_V + s), (j / NS) & 1, abort_flag, p.status, 25, p.wait_cycles)) return false;
+        const uint64_t vd = v_desc + (uint64_t)(s * (2 * TILE >> 4));
+        const uint32_t a_t = tmem_base + S_COL0 + (uint32_t)t * T_STRIDE, o_t = tmem_base + O_COL0 + (uint32_t)t * T_STRIDE;
+        const int n_ks = (tile_nv(j) + 15) >> 4;
+#pragma unroll
+        for (int part = 0; part < 2; ++part) {          // the first 96 keys start while P of the other 32 is still being made
+          if (!wait_bar_warp(BAR(P_FULL + 2 * t + part), j & 1, abort_flag, p.status, 24, p.wait_cycles)) return false;
+          tc_fence_after();
+          if (leader) {
+#pragma unroll
+            for (int ks = part * 6; ks < 6 + 2 * part; ++ks)
+              if (ks < n_ks) mma_ts(o_t, a_t + ks * 8, vd + ks * (2048 >> 4), idesc_pv, (j > 0 || ks > 0) ? 1u : 0u);
+          }
+        }
+        if (leader) {
+          tc_commit(BAR(PV_DONE + t));
+          if (release) tc_commit(BAR(EMPTY_V + s));
+        }
+        __syncwarp();
         return true;
       };
+      ok = ok && wait_bar_warp(BAR(FULL_K), 0, abort_flag, p.status, 26, p.wait_cycles);
       for (int j = 0; j < nt && ok; ++j) {
         const int s = j % NS;
-        if (!wait_bar(BAR(FULL_K + s), (j / NS) & 1, abort_flag, p.status, 26, p.wait_cycles)) { ok = false; break; }
         tc_fence_after();
         issue_s(0, j);
         if (act1) {
           if (j > 0 && !issue_pv(1, j - 1, true)) { ok = false; break; }
           issue_s(1, j);
         }
-        tc_commit(BAR(EMPTY_K + s));
+        if (leader) tc_commit(BAR(EMPTY_K + s));
+        // (the next K tile is waited for here, ahead of P: nothing then stands between this P V and the next S)
+        if (j + 1 < nt && !wait_bar_warp(BAR(FULL_K + (j + 1) % NS), ((j + 1) / NS) & 1, abort_flag, p.status, 26, p.wait_cycles)) { ok = false; break; }
         if (!issue_pv(0, j, !act1)) { ok = false; break; }
       }
       if (ok && act1) ok = issue_pv(1, nt - 1, true);
-      if (*abort_flag) {                    // wait for the tensor pipe to finish what was issued before TMEM is freed
+      if (*abort_flag && leader) {            // wait for the tensor pipe to finish what was issued before TMEM is freed
         tc_commit(BAR(DRAIN));
         drain_bar(BAR(DRAIN), 0);
       }
+      __syncwarp();
     }
   } else {
     // ======================================= softmax warps =======================================
-    const int t = (warp - 2) >> 2;                     // query tile of this warp
+    regs_inc_208();
+    const int t = (warp - 4) >> 2;                     // query tile of this warp
     const int q4 = warp & 3;                           // TMEM lane quadrant this warp may access
     const int row = q4 * 32 + lane;
     if (t == 0 || act1) {
@@ -213,55 +246,38 @@ __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __
             for (int i = 0; i < 32; ++i)
               if (c * 32 + i >= nv) sv[c][i] = __float_as_uint(-INFINITY);
         }
-        float mx = -INFINITY;
+        float m8[8];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+        for (int c = 0; c < 4; ++c)
 #pragma unroll
-          for (int i = 0; i < 32; ++i) m4[i & 3] = fmaxf(m4[i & 3], __uint_as_float(sv[c][i]));
-          mx = fmaxf(mx, fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])));
-        }
+          for (int i = 0; i < 16; ++i) {
+            const float a = __uint_as_float(sv[c][2 * i]), b = __uint_as_float(sv[c][2 * i + 1]);
+            m8[i & 7] = c == 0 && i < 8 ? fmaxf(a, b) : max3(m8[i & 7], a, b);
+          }
+        const float mx = max3(max3(m8[0], m8[1], m8[2]), max3(m8[3], m8[4], m8[5]), fmaxf(m8[6], m8[7]));
         // running maximum: O (in TMEM) and l are rescaled only when the maximum grows by more than 2^8
         const float m_new = fmaxf(m_run, mx * p.scale_log2);
         const bool grow = m_new > m_run + 8.f;          // also true on the first finite maximum
-        float alpha = 1.f;
-        if (grow) {
-          alpha = fast_exp2(m_run - m_new);             // 0 when m_run is -inf
-          m_run = m_new;
+        if (__any_sync(0xffffffffu, grow)) {
+          const float alpha = grow ? fast_exp2(m_run - m_new) : 1.f;      // 0 when m_run is -inf
+          if (grow) m_run = m_new;
           l_run *= alpha;
-        }
-        if (j > 0 && __any_sync(0xffffffffu, grow)) {
-          // every PV of this query tile issued so far must have landed before its rows are rewritten
-          if (!wait_bar_warp(BAR(PV_DONE + t), (j - 1) & 1, abort_flag, p.status, 28, p.wait_cycles)) { ok = false; break; }
-          tc_fence_after();
+          if (j > 0) {
+            // every PV of this query tile issued so far must have landed before its rows are rewritten
+            if (!wait_bar_warp(BAR(PV_DONE + t), (j - 1) & 1, abort_flag, p.status, 28, p.wait_cycles)) { ok = false; break; }
+            tc_fence_after();
 #pragma unroll 1
-          for (int c = 0; c < D / 16; ++c) {
-            uint32_t ov[16];
-            tmem_ld16(o_addr + c * 16, ov);
-            tc_wait_ld();
+            for (int c = 0; c < D / 16; ++c) {
+              uint32_t ov[16];
+              tmem_ld16(o_addr + c * 16, ov);
+              tc_wait_ld();
 #pragma unroll
-            for (int i = 0; i < 16; ++i) ov[i] = __float_as_uint(__uint_as_float(ov[i]) * alpha);
-            tmem_st16(o_addr + c * 16, ov);
+              for (int i = 0; i < 16; ++i) ov[i] = __float_as_uint(__uint_as_float(ov[i]) * alpha);
+              tmem_st16(o_addr + c * 16, ov);
+            }
           }
         }
         const float mu = (m_run == -INFINITY) ? 0.f : m_run;
-        // P = exp2(S * scale_log2 - mu) as bf16 over the first 64 columns of the S region
-        float psum = 0.f;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          uint32_t pk[16];
-          float ps4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const float e0 = fast_exp2(fmaf(__uint_as_float(sv[c][2 * i]), p.scale_log2, -mu));
-            const float e1 = fast_exp2(fmaf(__uint_as_float(sv[c][2 * i + 1]), p.scale_log2, -mu));
-            ps4[i & 3] += e0 + e1;
-            pk[i] = pack_bf16(e0, e1);
-          }
-          psum += (ps4[0] + ps4[1]) + (ps4[2] + ps4[3]);
-          tmem_st16(s_addr + c * 16, pk);
-        }
-        l_run += psum;
         // V rows past the sequence's end may hold anything: query tile 0 zeroes them so that 0 * V stays 0
         const int n_mma = (nv + 15) & ~15;
         if (t == 0 && nv < n_mma) {
@@ -269,16 +285,44 @@ __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __
           if (!wait_bar_warp(BAR(FULL_V + s), (j / NS) & 1, abort_flag, p.status, 29, p.wait_cycles)) { ok = false; break; }
           unsigned char* vs = stage0 + (size_t)s * 2 * TILE + TILE;
           const int nz = (n_mma - nv) * H * 8;           // 16-byte chunks to clear
-          for (int i = (warp - 2) * 32 + lane; i < nz; i += 128) {
+          for (int i = q4 * 32 + lane; i < nz; i += 128) {
             const int rr = nv + i / (H * 8), c = i % (H * 8);
             *reinterpret_cast<uint4*>(vs + (c >> 3) * HALF + rr * 128 + (((c & 7) ^ (rr & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
           }
           fence_proxy_async();
         }
-        tc_wait_st();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(BAR(P_FULL + t));
+        // P = exp2(S * scale_log2 - mu) as bf16 over the first 64 columns of the S region, handed over in two parts
+        const uint64_t scale2 = pack_f2(p.scale_log2, p.scale_log2), mu2 = pack_f2(-mu, -mu);
+        uint64_t ps[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          uint32_t pk[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            float x0, x1, e0, e1;
+            unpack_f2(fma_f2(pack_f2(__uint_as_float(sv[c][2 * i]), __uint_as_float(sv[c][2 * i + 1])), scale2, mu2), x0, x1);
+            if (i % DN_POLY == DN_POLY - 1) {
+              poly_exp2(x0, x1, e0, e1);
+            } else {
+              e0 = fast_exp2(x0);
+              e1 = fast_exp2(x1);
+            }
+            ps[i & 3] = add_f2(ps[i & 3], pack_f2(e0, e1));
+            pk[i] = pack_bf16(e0, e1);
+          }
+          tmem_st16(s_addr + c * 16, pk);
+          if (c >= 2) {
+            tc_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(BAR(P_FULL + 2 * t + (c - 2)));
+          }
+        }
+        {
+          float a, b;
+          unpack_f2(add_f2(add_f2(ps[0], ps[1]), add_f2(ps[2], ps[3])), a, b);
+          l_run += a + b;
+        }
       }
       // ---- the finished row: TMEM -> registers -> normalise -> bf16 -> global memory ----
       if (ok) ok = wait_bar_warp(BAR(PV_DONE + t), (nt - 1) & 1, abort_flag, p.status, 30, p.wait_cycles);

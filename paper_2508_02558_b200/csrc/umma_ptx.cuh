@@ -65,6 +65,12 @@ __device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_
       " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n"
       ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
+// One lane of a converged warp: the code around it stays warp-uniform, so descriptors are computed in uniform registers.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(ok));
+  return ok != 0;
+}
 // 32 lanes x 32 consecutive 32-bit columns: thread i of the warp receives lane (base lane + i)
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
@@ -94,6 +100,51 @@ __device__ __forceinline__ float fast_exp2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;\n" : "=f"(y) : "f"(x));
   return y;
 }
+
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;\n" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+// Two fp32 operations per instruction (same rounding as the scalar forms).
+__device__ __forceinline__ uint64_t pack_f2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};\n" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack_f2(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;\n" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ uint64_t fma_f2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;\n" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t add_f2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;\n" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+// 2^x for two values on the FMA pipe, beside the exponential unit (16 results per clock and SM, the bottleneck of a softmax
+// that feeds tcgen05): x = n + f with n the nearest integer (round by adding 1.5 * 2^23), 2^f by the degree-5 polynomial of
+// least relative error on [-1/2, 1/2] (Remez exchange; 7.5e-8, 2.1e-7 evaluated in fp32 - ex2.approx is within 2.4e-7), n added
+// to the exponent. Values below 2^-126 come out as about 2^-126 instead of 0.
+__device__ __forceinline__ void poly_exp2(float x0, float x1, float& e0, float& e1) {
+  const uint64_t x = pack_f2(fmaxf(x0, -126.f), fmaxf(x1, -126.f));
+  const uint64_t magic = pack_f2(12582912.f, 12582912.f), minus_one = pack_f2(-1.f, -1.f);
+  const uint64_t t = add_f2(x, magic);
+  const uint64_t f = add_f2(x, fma_f2(t, minus_one, magic));
+  uint64_t y = fma_f2(pack_f2(1.3276472454890609e-3f, 1.3276472454890609e-3f), f, pack_f2(9.675540961325169e-3f, 9.675540961325169e-3f));
+  y = fma_f2(y, f, pack_f2(5.550713092088699e-2f, 5.550713092088699e-2f));
+  y = fma_f2(y, f, pack_f2(2.4022120237350464e-1f, 2.4022120237350464e-1f));
+  y = fma_f2(y, f, pack_f2(6.931469440460205e-1f, 6.931469440460205e-1f));
+  y = fma_f2(y, f, pack_f2(1.0000001192092896f, 1.0000001192092896f));
+  float y0, y1, t0, t1;
+  unpack_f2(y, y0, y1);
+  unpack_f2(t, t0, t1);
+  e0 = __uint_as_float(__float_as_uint(y0) + (__float_as_uint(t0) << 23));
+  e1 = __uint_as_float(__float_as_uint(y1) + (__float_as_uint(t1) << 23));
+}
+__device__ __forceinline__ void regs_dec_72() { asm volatile("setmaxnreg.dec.sync.aligned.u32 72;\n"); }
+__device__ __forceinline__ void regs_inc_208() { asm volatile("setmaxnreg.inc.sync.aligned.u32 208;\n"); }
 
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
