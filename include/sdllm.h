@@ -232,7 +232,8 @@ sdllm_status sdllm_sparse_block_attn_static(const sdllm_desc* desc, const void* 
  * them. Host-only, thread-safe; takes effect for calls made afterwards. `name` is a NUL-terminated host string:
  *   "splits"      > 0: key splits per (sequence, KV head) of the attention calls
  *   "kernel"      attention kernel family: 0 automatic, 1 cp.async, 2 tcgen05 with the queries on the accumulator rows,
- *                 3 tcgen05 with the keys on the accumulator rows (only where that kernel covers the shape)
+ *                 (one softmax warpgroup), 3 tcgen05 with the keys on the accumulator rows, 4 as 2 with two softmax
+ *                 warpgroups (each only where that kernel covers the shape)
  *   "pdl"         0: no programmatic dependent launch     "early_loads" 0: no loads ahead of the grid dependency
  *   "cluster", "fused_tail", "dual", "key_tile", "lpt", "stages", "trigger", "persist"   plan details of the tcgen05 kernels
  *   "select"      top-k kernel: 1 one CTA per head, 2 one cluster per head

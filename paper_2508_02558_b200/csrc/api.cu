@@ -200,7 +200,7 @@ sdllm_status sdllm_plan_describe(const sdllm_desc* d, int op, char* buf, size_t 
   if (check_desc(d) != SDLLM_OK || (op != SDLLM_OP_REFRESH_SCORES && op != SDLLM_OP_SPARSE_BLOCK_ATTN)) return SDLLM_ERR_INVALID_ARG;
   const AttnPlan pl = plan_for(d, op);
   const char* name = pl.kind == 3 ? (pl.persistent ? "attn_kt_stream_kernel" : "attn_kt_kernel")
-                                  : (pl.kind == 2 ? "attn_umma_bf16_kernel" : (d->dtype == SDLLM_BF16 ? "attn_bf16_kernel" : "attn_f32_kernel"));
+                                  : (pl.kind == 4 || pl.kind == 2 ? "attn_umma_bf16_kernel" : (d->dtype == SDLLM_BF16 ? "attn_bf16_kernel" : "attn_f32_kernel"));
   if (pl.kind == 3)
     snprintf(buf, buf_bytes, "%s splits=%d cluster=%d stages=%d softmax_warpgroups=%d threads=%d smem=%zu", name, pl.cluster, pl.cluster,
              pl.stages, pl.c_warps * pl.warp_keys, pl.threads, pl.smem_bytes);
@@ -222,6 +222,7 @@ int32_t sdllm_launch_count(const sdllm_desc* d, int op) {
   const AttnPlan pl = plan_for(d, op);
   const int M = d->n_q_heads / d->n_kv_heads * d->block_len;
   if (pl.kind == 3) return 1;       // the key splits merge, and the scores are pooled, inside the one launch
+  if (pl.kind == 4) return pl.splits > 1 || refresh ? 2 : 1;       // the fold of the key splits and the pooling are one launch
   if (pl.kind == 2) {
     const int n1 = refresh ? d->seq_len_max : d->n_keep_max;
     if (refresh && d->score == SDLLM_SCORE_PROB_MEAN)     // attention pass (+ its merge) and saliency pass (+ its pooling)

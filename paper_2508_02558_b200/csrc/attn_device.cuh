@@ -100,6 +100,47 @@ __device__ __forceinline__ void compute_qbar(const AttnParams& p, const CtaRange
   }
 }
 
+// Importance of one absolute position: Algorithm 1, MaxPool1D(A, kernel_size = s, padding = s/2) over the candidate
+// axis Concat(prefix, suffix) (AvgPool for the ablation); block positions and padding get -inf. `a` holds the raw
+// saliency by absolute position.
+__device__ __forceinline__ float pool_at(const AttnParams& p, const float* a, int L, int o_in, int pos, int n_arr = 1,
+                                         int64_t arr_stride = 0) {
+  const int b = p.b;
+  const int o = min(max(o_in, 0), max(L - b, 0));
+  if (pos >= L || (pos >= o && pos < o + b)) return -INFINITY;
+  const int C = max(L - b, 0), w = (p.window - 1) / 2;
+  const int c = pos < o ? pos : pos - b;
+  int lo = 0, hi = C;
+  if (p.per_region) { if (c < o) hi = o; else lo = o; }
+  float mx = -INFINITY, sum = 0.f;
+  for (int t = c - w; t <= c + w; ++t) {
+    if (t < lo || t >= hi) continue;
+    float x = a[t < o ? t : t + b];
+    for (int r2 = 1; r2 < n_arr; ++r2) x += a[r2 * arr_stride + (t < o ? t : t + b)];   // one array per row tile
+    mx = fmaxf(mx, x);
+    sum += x;
+  }
+  return p.pool_kind == SDLLM_POOL_MAX ? mx : sum / (float)p.window;
+}
+
+// Importance of one absolute position as pool_at, reading the raw saliency from global memory through L2 (other CTAs wrote it during this launch).
+__device__ __forceinline__ float pool_at_ldcg(const AttnParams& p, const float* a, int L, int o_in, int pos) {
+  const int b = p.b;
+  const int o = min(max(o_in, 0), max(L - b, 0));
+  if (pos >= L || (pos >= o && pos < o + b)) return -INFINITY;
+  const int C = max(L - b, 0), w = (p.window - 1) / 2;
+  const int c = pos < o ? pos : pos - b;
+  int lo = 0, hi = C;
+  if (p.per_region) { if (c < o) hi = o; else lo = o; }
+  float mx = -INFINITY, sum = 0.f;
+  for (int t = c - w; t <= c + w; ++t) {
+    if (t < lo || t >= hi) continue;
+    const float x = __ldcg(a + (t < o ? t : t + b));
+    mx = fmaxf(mx, x);
+    sum += x;
+  }
+  return p.pool_kind == SDLLM_POOL_MAX ? mx : sum / (float)p.window;
+}
 
 }  // namespace dev
 }  // namespace sdllm

@@ -827,29 +827,24 @@ bool kt_supported(int dtype, int D, int M, int b) {
   return umma_supported(dtype, D, M, b) && M <= 128;
 }
 
-// Whether the planner picks it among the shapes it covers. A unit's key splits are the CTAs of one cluster, eight at
-// most. With up to 32 query rows that is enough everywhere. With more, a CTA takes a whole SM, and a few units with
-// long key ranges (8 KV heads, one sequence, 16k keys: 64 CTAs) would leave most SMs idle; the query-row kernel splits
-// those further through its workspace and measured faster there (25 against 38 us), slower with 64 units and more.
-// Short walks are latency chains whatever the number of CTAs, and this kernel's chain is the shorter one: up to six
-// tiles per CTA at 64 query columns (8 KV heads x 1024 keys: 8.1 against 14.5 us; x 4096: 12.2 against 15.2), up to two
-// with more columns (12.1 against 13.0 us at 128 columns x 1024 keys; at 4096 keys the query-row kernel is ahead).
-bool kt_preferred(int M, int B, int Hkv, int n1_max, int n2) {
+// Whether the planner picks it among the shapes it covers: against the query-row kernel with two softmax warpgroups
+// (attn_pair.cu), from a sweep of both calls over 8 to 512 units of 3 to 128 tiles.
+// Up to 32 query rows it is ahead nearly everywhere (the query-row kernel pads them to 128); with more than 64 the query-row
+// kernel is (1.1 to 1.9 times). In between it loses
+//   - a reuse step of up to three tiles (7.7 against 8.4 us), or of more heads than half the SMs, which get one CTA each either
+//     way (22.6 against 28.1 us at 128 heads x 17 tiles);
+//   - long walks of few heads, which its clusters of at most eight CTAs cannot spread over the GPU (11.7 against 12.6 us at 8
+//     heads x 33 tiles, refresh 25.7 against 34.3 at 8 heads x 128; head dimension 64 from half that length on).
+bool kt_preferred(int D, int M, int B, int Hkv, int n1_max, int n2) {
   if (M <= 32) return true;
+  if (M > 64) return false;
   const long long units = (long long)B * Hkv;
-  const int sms = sm_count();
-  long long S = sms / units;
-  const long long by_tiles = ((n1_max + 31) / 32 + (n2 + 31) / 32 + 3) / 4;
-  if (S > by_tiles) S = by_tiles;
-  if (S > 8) S = 8;
-  if (S < 1) S = 1;
-  const long long tiles_cta = (by_tiles + S - 1) / S;
-  // (three or four column groups walk a tile in 2 us, the query-row kernel in 1.5: long walks go there even when the
-  // SMs are filled - 32 units x 128 tiles: 70.7 against 79.6 us)
-  // (with 16 to 24 units the query-row kernel, which can use more CTAs, is ahead from five tiles per CTA on: 19.7 against
-  // 22.3 us at 16 units x 33 tiles)
-  if (units * S * 4 >= (long long)sms * 3) return M <= 64 || tiles_cta <= (units >= 32 ? 16 : 4);
-  return tiles_cta <= (M <= 64 ? 6 : 2);
+  const int sms = sm_count(), tiles = (n1_max + 127) / 128 + (n2 > 0 ? (n2 + 127) / 128 : 0);
+  if (n2 > 0) {
+    if (units * 2 > sms) return tiles <= 3;
+    return tiles > 3 && !(units * 8 <= sms && tiles >= 24);
+  }
+  return !(units * 8 <= sms && tiles > (D == 64 ? 20 : 40));
 }
 
 AttnPlan plan_attention_kt(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn) {

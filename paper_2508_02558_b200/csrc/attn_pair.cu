@@ -1,0 +1,671 @@
+// bf16 block-query attention for wide heads (more than 32 query rows per KV head) on tcgen05, two softmax warpgroups.
+//
+// The queries lie on the 128 accumulator rows, so a softmax thread owns a query row and nothing is exchanged between threads;
+// P stays in tensor memory (A operand of P V). A CTA owns (sequence, KV head, key split) and streams its share of the key axis
+//   [source 1 rows 0..n1) ++ [source 2 rows 0..n2)     (refresh: the full K/V; reuse: the compacted cache ++ the block's rows)
+// once. What limited the one-warpgroup kernel (attn_umma.cu) on long walks was the chain S -> softmax -> P V of a tile, about
+// 2.8 us per 128 keys against the 1.45 us that an SM's share of HBM takes for the 64 KB of K and V. Here two tiles are always
+// in flight on the chain of the dense kernel (attn_dense.cu):
+//   TWO = false (at most 128 query rows): one Q tile; the warpgroups take the key tiles in turn, each with its own S / P
+//               buffer, accumulator, maxima and sums, which are folded once at the end;
+//   TWO = true  (129 to 256 rows): two Q tiles, one per warpgroup, both fed by every key tile.
+// Roles (384 threads):
+//   warp 0       TMA producer: K and V tiles (128 keys, 128-byte swizzle) into a ring of two to four slots
+//   warp 1       tcgen05.mma issuer, warp-uniform: S_w = Q K_j^T, O_w += P_w V_j
+//   warps 2-3    refresh only: mean-query saliency of every streamed key (Algorithm 1, "qbar <- Mean(Q_b)",
+//                "A <- MatMul(qbar, K_f^T)") from the K tile in shared memory, fp32
+//   warps 4-7, 8-11   the softmax warpgroups
+// Tensor memory (512 columns): S0 | S1 | O0 | O1, 128 columns each. Key splits leave un-normalised rows in the workspace, float4
+// columns apart ([D / 4][128 rows], so that the lanes of a warp - one row each - write and read in a row); pair_tail_kernel
+// folds them and pools the saliency. (Measured against it and dropped: splits meeting inside a cluster, by 16-byte pushes into
+// distributed shared memory - 25 bytes per ns and SM - or through L2 behind a cluster barrier: 31 to 33 us against 22.4 on 8 heads
+// x 16 k keys, 13.7 against 10.5 on 4 heads x 1 k keys.)
+// Every mbarrier wait is bounded; on expiry the CTA sets an abort flag, records a code in the status word and runs to its end.
+#include <cuda.h>
+#include <string.h>
+
+#include "attn_device.cuh"
+#include "tuning.cuh"
+#include "umma_host.cuh"
+
+namespace sdllm {
+using namespace dev;
+namespace {
+
+constexpr int PR_THREADS = 384;
+constexpr int PR_POLY = 4;             // one pair of exponentials in PR_POLY is a polynomial
+
+struct PairMaps {
+  CUtensorMap q, k1, v1, k2, v2;
+};
+struct PairParams {
+  AttnParams a;
+  int KT2;           // rows of a source-2 tile (<= 128, multiple of 16)
+  int heads_rt;      // query heads per Q tile
+  int early_src1;    // 1: source 1 and its count are older than the previous kernel in the stream (reuse step)
+  int lpt;           // 1: grid z counts the sequences from the longest to the shortest (several waves of ragged work)
+};
+
+#include "umma_ptx.cuh"
+
+template <int D, bool TWO>
+struct PairShape {
+  static constexpr int H = D / 64;                        // 64-column halves of a row (128 bytes each: one swizzle atom wide)
+  static constexpr int HALF = 128 * 128;                  // bytes of one 64-column half of a 128-row tile
+  static constexpr int TILE = H * HALF;                   // bytes of a Q, K or V tile
+  static constexpr int QT = TWO ? 2 : 1;                  // Q tiles
+  static constexpr int NS = D == 64 ? 4 : (TWO ? 2 : 3);  // ring slots: what fits beside Q
+  static constexpr size_t SMEM = 1024 /*alignment slack*/ + 1024 /*barriers, qbar*/ + (size_t)QT * TILE + (size_t)NS * 2 * TILE;
+};
+
+template <int D, bool TWO>
+__global__ void __launch_bounds__(PR_THREADS, 1) attn_pair_kernel(const __grid_constant__ PairMaps tm, const PairParams pp) {
+  using Sh = PairShape<D, TWO>;
+  constexpr int H = Sh::H, HALF = Sh::HALF, TILE = Sh::TILE, NS = Sh::NS, KT = 128;
+  constexpr uint32_t S_COL0 = 0, O_COL0 = 256, T_STRIDE = 128;
+  const AttnParams& p = pp.a;
+  extern __shared__ unsigned char smem_raw[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int split = blockIdx.x, g = blockIdx.y;
+  int bi = blockIdx.z;
+  if (pp.lpt) {
+    if (!pp.early_src1) grid_dependency_wait();           // the lengths may come from the kernel in front
+    bi = sequence_of_rank(p.n1_per_seq, p.B, blockIdx.z);
+  }
+  const int n2 = p.n2, tiles2 = (n2 + pp.KT2 - 1) / pp.KT2;
+  const bool do_attn = p.out != nullptr, do_scores = p.want_scores != 0;
+
+  const uint32_t raw_addr = smem_u32(smem_raw);
+  unsigned char* smem = smem_raw + (((raw_addr + 1023u) & ~1023u) - raw_addr);
+  const uint32_t bars = smem_u32(smem);
+  auto BAR = [&](int i) { return bars + 8u * (uint32_t)i; };
+  const int Q_FULL = 0, FULL_K = 1, FULL_V = 1 + NS, EMPTY_K = 1 + 2 * NS, EMPTY_V = 1 + 3 * NS;
+  const int S_FULL = 1 + 4 * NS, P_FULL = S_FULL + 2, PV_DONE = S_FULL + 6, DRAIN = S_FULL + 8;   // P_FULL: two parts per warpgroup
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + 256);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + 260);
+  float* qbar_s = reinterpret_cast<float*>(smem + 512);
+  unsigned char* q_s = smem + 1024;
+  unsigned char* stage0 = q_s + Sh::QT * TILE;
+
+  // This CTA's tiles: an even share of the sequence's own tiles (not of the longest one's).
+  int n1 = 0, tiles1 = 0, t_begin = 0, t_end = 0;
+  auto place = [&]() {
+    n1 = p.n1_per_seq ? __ldcg(p.n1_per_seq + bi) : p.n1_max;
+    n1 = min(max(n1, 0), p.n1_max);
+    tiles1 = (n1 + KT - 1) / KT;
+    const int all = tiles1 + tiles2;
+    t_begin = split * all / p.splits;
+    t_end = (split + 1) * all / p.splits;
+  };
+  auto tile_at = [&](int t) { return tile_of(t, tiles1, KT, pp.KT2, n1, n2); };
+
+  int prod_it = 0;
+  bool prod_ok = true, v_missing = false, q_issued = false;
+  auto issue_q = [&]() {
+    mbar_expect_tx(BAR(Q_FULL), (uint32_t)(Sh::QT * H * p.b * pp.heads_rt * 128));
+    for (int t = 0; t < Sh::QT; ++t)
+      for (int h = 0; h < H; ++h)
+        tma_load_4d(smem_u32(q_s + t * TILE + h * HALF), &tm.q, BAR(Q_FULL), h * 64, 0, g * p.G + t * pp.heads_rt, bi);
+    q_issued = true;
+  };
+  // loads of further tiles (producer lane only); first: only what fits the ring without waiting, source 1 only
+  auto produce = [&](bool first) {
+    while (t_begin + prod_it < t_end && prod_ok) {
+      const int it = prod_it, s = it % NS;
+      const Tile x = tile_at(t_begin + it);
+      if (first && (it >= NS || !x.src1)) return;
+      const uint32_t ph = ((it / NS) - 1) & 1;
+      const uint32_t kdst = smem_u32(stage0 + (size_t)s * 2 * TILE), vdst = kdst + TILE;
+      const uint32_t tx = (uint32_t)(H * (x.src1 ? KT : pp.KT2) * 128);
+      if (it >= NS && !wait_bar(BAR(EMPTY_K + s), ph, abort_flag, p.status, 41, p.wait_cycles)) { prod_ok = false; return; }
+      mbar_expect_tx(BAR(FULL_K + s), tx);
+      for (int h = 0; h < H; ++h) tma_load_4d(kdst + h * HALF, x.src1 ? &tm.k1 : &tm.k2, BAR(FULL_K + s), h * 64, x.row0, g, bi);
+      ++prod_it;
+      if (do_attn) {
+        if (it >= NS && !wait_bar(BAR(EMPTY_V + s), ph, abort_flag, p.status, 42, p.wait_cycles)) { prod_ok = false; v_missing = true; return; }
+        mbar_expect_tx(BAR(FULL_V + s), tx);
+        for (int h = 0; h < H; ++h) tma_load_4d(vdst + h * HALF, x.src1 ? &tm.v1 : &tm.v2, BAR(FULL_V + s), h * 64, x.row0, g, bi);
+      }
+    }
+  };
+
+  if (tid == 0) {
+    prefetch_tmap(&tm.k1); prefetch_tmap(&tm.v1); prefetch_tmap(&tm.q);
+    if (n2 > 0) { prefetch_tmap(&tm.k2); prefetch_tmap(&tm.v2); }
+    mbar_init(BAR(Q_FULL), 1);
+    for (int s = 0; s < NS; ++s) {
+      mbar_init(BAR(FULL_K + s), 1); mbar_init(BAR(FULL_V + s), 1);
+      mbar_init(BAR(EMPTY_K + s), (do_attn ? 1 : 0) + (do_scores ? 2 : 0)); mbar_init(BAR(EMPTY_V + s), 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(BAR(S_FULL + i), 1);
+      mbar_init(BAR(P_FULL + 2 * i), 4);                  // the four warps of a softmax warpgroup
+      mbar_init(BAR(P_FULL + 2 * i + 1), 4);
+      mbar_init(BAR(PV_DONE + i), 1);
+    }
+    mbar_init(BAR(DRAIN), 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    // The loads need nothing but the barriers: the first ones go out before the rest of the CTA is set up, at a reuse step even
+    // ahead of the grid dependency (the compacted cache and its count are older than any kernel that may still run).
+    if (pp.early_src1) { place(); produce(true); }
+    grid_dependency_wait();
+    if (!pp.early_src1) place();
+    issue_q();
+    produce(true);
+  }
+  if (warp == 1) {                                        // the MMA warp owns the tensor memory
+    tmem_alloc(smem_u32(tmem_slot), 512);
+    tmem_relinquish();
+  }
+  fence_proxy_async();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  grid_dependency_wait();                                 // everything below may read what earlier kernels in the stream wrote
+  grid_launch_dependents();
+  if (tid != 0) place();
+  const int nt = t_end - t_begin;
+
+  if (warp < 4) {
+    regs_dec_80();
+    if (warp == 0) {
+      // ======================================= TMA producer =======================================
+      if (lane == 0) {
+        produce(false);
+        if (*abort_flag) {                  // let the copies that were issued land before the CTA retires
+          for (int j = max(prod_it - NS, 0); j < prod_it; ++j) {
+            drain_bar(BAR(FULL_K + j % NS), (j / NS) & 1);
+            if (do_attn && !(v_missing && j == prod_it - 1)) drain_bar(BAR(FULL_V + j % NS), (j / NS) & 1);
+          }
+          drain_bar(BAR(Q_FULL), 0);
+        }
+      }
+    } else if (warp == 1) {
+      // ======================================= MMA issuer =======================================
+      const bool leader = elect_one();
+      bool ok = wait_bar_warp(BAR(Q_FULL), 0, abort_flag, p.status, 43, p.wait_cycles);
+      if (do_attn) {
+        const uint32_t idesc_pv = instr_desc(D, true);
+        const uint64_t q_desc = smem_desc(smem_u32(q_s), 16u, 1024u), k_desc = smem_desc(smem_u32(stage0), 16u, 1024u);
+        const uint64_t v_desc = smem_desc(smem_u32(stage0) + TILE, (uint32_t)HALF, 1024u);
+        // S of tile it for warpgroup w
+        auto issue_s = [&](int w, int it, int n_mma) {
+          const uint32_t idesc_s = instr_desc(n_mma, false);
+          const uint32_t d_t = tmem_base + S_COL0 + (uint32_t)w * T_STRIDE;
+          const uint64_t qd = q_desc + (uint64_t)(TWO ? w * (TILE >> 4) : 0), kd = k_desc + (uint64_t)((it % NS) * (2 * TILE >> 4));
+          if (leader) {
+#pragma unroll
+            for (int ks = 0; ks < D / 16; ++ks) {
+              const uint64_t off = (uint64_t)(((ks >> 2) * HALF + (ks & 3) * 32) >> 4);
+              mma_ss(d_t, qd + off, kd + off, idesc_s, ks > 0 ? 1u : 0u);
+            }
+            tc_commit(BAR(S_FULL + w));
+          }
+          __syncwarp();
+        };
+        // O_w += P_w V of tile it as warpgroup w hands P over; k counts its tiles
+        auto issue_pv = [&](int w, int it, int k, int n_mma, bool release) -> bool {
+          const int s = it % NS;
+          if (!wait_bar_warp(BAR(FULL_V + s), (it / NS) & 1, abort_flag, p.status, 45, p.wait_cycles)) return false;
+          const uint64_t vd = v_desc + (uint64_t)(s * (2 * TILE >> 4));
+          const uint32_t a_t = tmem_base + S_COL0 + (uint32_t)w * T_STRIDE, o_t = tmem_base + O_COL0 + (uint32_t)w * T_STRIDE;
+          const int n_ks = n_mma >> 4;
+#pragma unroll
+          for (int part = 0; part < 2; ++part) {          // the first 96 keys start while P of the other 32 is still being made
+            if (!wait_bar_warp(BAR(P_FULL + 2 * w + part), k & 1, abort_flag, p.status, 44, p.wait_cycles)) return false;
+            tc_fence_after();
+            if (leader) {
+#pragma unroll
+              for (int ks = part * 6; ks < 6 + 2 * part; ++ks)
+                if (ks < n_ks) mma_ts(o_t, a_t + ks * 8, vd + ks * (2048 >> 4), idesc_pv, (k > 0 || ks > 0) ? 1u : 0u);
+            }
+          }
+          if (leader) {
+            tc_commit(BAR(PV_DONE + w));
+            if (release) tc_commit(BAR(EMPTY_V + s));
+          }
+          __syncwarp();
+          return true;
+        };
+        int n_prev = 0;
+        for (int it = 0; it < nt && ok; ++it) {
+          const int s = it % NS, n_mma = tile_at(t_begin + it).n_mma;
+          if (!wait_bar_warp(BAR(FULL_K + s), (it / NS) & 1, abort_flag, p.status, 46, p.wait_cycles)) { ok = false; break; }
+          tc_fence_after();
+          if constexpr (TWO) {
+            issue_s(0, it, n_mma);
+            if (it > 0 && !issue_pv(1, it - 1, it - 1, n_prev, true)) { ok = false; break; }
+            issue_s(1, it, n_mma);
+            if (leader) tc_commit(BAR(EMPTY_K + s));
+            if (!issue_pv(0, it, it, n_mma, false)) { ok = false; break; }
+          } else {
+            issue_s(it & 1, it, n_mma);
+            if (leader) tc_commit(BAR(EMPTY_K + s));
+            if (it > 0 && !issue_pv((it - 1) & 1, it - 1, (it - 1) >> 1, n_prev, true)) { ok = false; break; }
+          }
+          n_prev = n_mma;
+        }
+        if (ok && nt > 0) ok = TWO ? issue_pv(1, nt - 1, nt - 1, n_prev, true) : issue_pv((nt - 1) & 1, nt - 1, (nt - 1) >> 1, n_prev, true);
+        if (*abort_flag && leader) {        // wait for the tensor pipe to finish what was issued before TMEM is freed
+          tc_commit(BAR(DRAIN));
+          drain_bar(BAR(DRAIN), 0);
+        }
+        __syncwarp();
+      }
+    } else if (do_scores) {
+      // ======================================= saliency warps (refresh) =======================================
+      // qbar <- Mean(Q_b) over the b*G rows of the KV head, fp32, in row order, from the Q tiles in shared memory
+      bool ok = wait_bar_warp(BAR(Q_FULL), 0, abort_flag, p.status, 47, p.wait_cycles);
+      const int st = tid - 64;                            // 0..63
+      if (ok && 2 * st < D) {
+        float a0 = 0.f, a1 = 0.f;
+        const int chunk = (2 * st & 63) >> 3, in_chunk = (2 * st & 7) * 2, half = (2 * st) >> 6;
+#pragma unroll 8
+        for (int m = 0; m < p.M; ++m) {
+          const int r = m & 127;
+          const uint32_t v = *reinterpret_cast<const uint32_t*>(q_s + (m >> 7) * TILE + half * HALF + r * 128 + ((chunk ^ (r & 7)) << 4) + in_chunk);
+          a0 += __uint_as_float(v << 16);
+          a1 += __uint_as_float(v & 0xffff0000u);
+        }
+        qbar_s[2 * st] = a0 / (float)p.M;
+        qbar_s[2 * st + 1] = a1 / (float)p.M;
+      }
+      asm volatile("bar.sync 2, 64;\n" ::: "memory");
+      float* raw_scores = p.raw_scores + (int64_t)(bi * p.Hkv + g) * p.n1_max;
+      for (int it = 0; it < nt; ++it) {
+        const int s = it % NS;
+        const Tile x = tile_at(t_begin + it);
+        if (!wait_bar_warp(BAR(FULL_K + s), (it / NS) & 1, abort_flag, p.status, 48, p.wait_cycles)) break;
+        // two keys per lane: a_j = scale * <qbar, k_j>; the 128-byte swizzle keeps 32 consecutive rows conflict-free
+        const unsigned char* kst = stage0 + (size_t)s * 2 * TILE;
+        const int k0 = st, k1 = st + 64;
+        uint64_t a[2][2] = {{0ull, 0ull}, {0ull, 0ull}};   // per key four sums, as two pairs
+#pragma unroll 4
+        for (int c = 0; c < H * 8; ++c) {
+          const ulonglong2 qa = *reinterpret_cast<const ulonglong2*>(qbar_s + c * 8), qc = *reinterpret_cast<const ulonglong2*>(qbar_s + c * 8 + 4);
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const int kk = u ? k1 : k0;
+            const uint4 raw = *reinterpret_cast<const uint4*>(kst + (c >> 3) * HALF + kk * 128 + (((c & 7) ^ (kk & 7)) << 4));
+            auto wide = [](uint32_t v) { return pack_f2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u)); };
+            a[u][0] = fma_f2(qa.x, wide(raw.x), a[u][0]);
+            a[u][1] = fma_f2(qa.y, wide(raw.y), a[u][1]);
+            a[u][0] = fma_f2(qc.x, wide(raw.z), a[u][0]);
+            a[u][1] = fma_f2(qc.y, wide(raw.w), a[u][1]);
+          }
+        }
+        float r[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          float a0, a1, a2, a3;
+          unpack_f2(a[u][0], a0, a1);
+          unpack_f2(a[u][1], a2, a3);
+          r[u] = ((a0 + a1) + (a2 + a3)) * p.scale;
+        }
+        if (k0 < x.nv) raw_scores[x.row0 + k0] = r[0];
+        if (k1 < x.nv) raw_scores[x.row0 + k1] = r[1];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(BAR(EMPTY_K + s));
+      }
+      if (do_attn) asm volatile("bar.arrive 3, 320;\n" ::: "memory");     // the ring is no longer read here
+    }
+  } else if (do_attn) {
+    // ======================================= softmax warpgroups =======================================
+    regs_inc_208();
+    const int w = (warp - 4) >> 2;                        // warpgroup: Q tile (TWO) or tile parity
+    const int q4 = warp & 3;                              // TMEM lane quadrant this warp may access
+    const int row = q4 * 32 + lane;
+    const uint32_t lane_addr = tmem_base + ((uint32_t)(q4 * 32) << 16);
+    const uint32_t s_addr = lane_addr + S_COL0 + (uint32_t)w * T_STRIDE;
+    const uint32_t o_addr = lane_addr + O_COL0 + (uint32_t)w * T_STRIDE;
+    float m_run = -INFINITY, l_run = 0.f;
+    bool ok = true;
+    int k = 0;                                            // tiles of this warpgroup so far
+    for (int it = TWO ? 0 : w; it < nt && ok; it += TWO ? 1 : 2, ++k) {
+      const Tile x = tile_at(t_begin + it);
+      const int nv = x.nv;
+      if (!wait_bar_warp(BAR(S_FULL + w), k & 1, abort_flag, p.status, 49, p.wait_cycles)) { ok = false; break; }
+      tc_fence_after();
+      uint32_t sv[4][32];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) tmem_ld32(s_addr + c * 32, sv[c]);
+      tc_wait_ld();
+      if (nv < KT) {                                      // a ragged tile: keys past its end count as -inf
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+          for (int e = 0; e < 32; ++e)
+            if (c * 32 + e >= nv) sv[c][e] = __float_as_uint(-INFINITY);
+      }
+      float m8[8];
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+          const float a = __uint_as_float(sv[c][2 * e]), b = __uint_as_float(sv[c][2 * e + 1]);
+          m8[e & 7] = c == 0 && e < 8 ? fmaxf(a, b) : max3(m8[e & 7], a, b);
+        }
+      const float mx = max3(max3(m8[0], m8[1], m8[2]), max3(m8[3], m8[4], m8[5]), fmaxf(m8[6], m8[7]));
+      // running maximum: O (in TMEM) and l are rescaled only when the maximum grows by more than 2^8
+      const float m_new = fmaxf(m_run, mx * p.scale_log2);
+      const bool grow = m_new > m_run + 8.f;              // also true on the first finite maximum
+      if (__any_sync(0xffffffffu, grow)) {
+        const float alpha = grow ? fast_exp2(m_run - m_new) : 1.f;        // 0 when m_run is -inf
+        if (grow) m_run = m_new;
+        l_run *= alpha;
+        if (k > 0) {
+          // every P V of this warpgroup issued so far must have landed before its rows are rewritten
+          if (!wait_bar_warp(BAR(PV_DONE + w), (k - 1) & 1, abort_flag, p.status, 50, p.wait_cycles)) { ok = false; break; }
+          tc_fence_after();
+#pragma unroll 1
+          for (int c = 0; c < D / 16; ++c) {
+            uint32_t ov[16];
+            tmem_ld16(o_addr + c * 16, ov);
+            tc_wait_ld();
+#pragma unroll
+            for (int e = 0; e < 16; ++e) ov[e] = __float_as_uint(__uint_as_float(ov[e]) * alpha);
+            tmem_st16(o_addr + c * 16, ov);
+          }
+        }
+      }
+      const float mu = (m_run == -INFINITY) ? 0.f : m_run;
+      // V rows past the tile's end may hold anything: they are zeroed so that 0 * V stays 0
+      if ((!TWO || w == 0) && nv < x.n_mma) {
+        const int s = it % NS;
+        if (!wait_bar_warp(BAR(FULL_V + s), (it / NS) & 1, abort_flag, p.status, 51, p.wait_cycles)) { ok = false; break; }
+        unsigned char* vs = stage0 + (size_t)s * 2 * TILE + TILE;
+        const int nz = (x.n_mma - nv) * H * 8;            // 16-byte chunks to clear
+        for (int e = row; e < nz; e += 128) {
+          const int rr = nv + e / (H * 8), c = e % (H * 8);
+          *reinterpret_cast<uint4*>(vs + (c >> 3) * HALF + rr * 128 + (((c & 7) ^ (rr & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
+        }
+        fence_proxy_async();
+      }
+      // P = exp2(S * scale_log2 - mu) as bf16 over the first 64 columns of the S buffer, handed over in two parts
+      const uint64_t scale2 = pack_f2(p.scale_log2, p.scale_log2), mu2 = pack_f2(-mu, -mu);
+      uint64_t ps[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        uint32_t pk[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+          float x0, x1, e0, e1;
+          unpack_f2(fma_f2(pack_f2(__uint_as_float(sv[c][2 * e]), __uint_as_float(sv[c][2 * e + 1])), scale2, mu2), x0, x1);
+          if (e % PR_POLY == PR_POLY - 1) {
+            poly_exp2(x0, x1, e0, e1);
+          } else {
+            e0 = fast_exp2(x0);
+            e1 = fast_exp2(x1);
+          }
+          ps[e & 3] = add_f2(ps[e & 3], pack_f2(e0, e1));
+          pk[e] = pack_bf16(e0, e1);
+        }
+        tmem_st16(s_addr + c * 16, pk);
+        if (c >= 2) {
+          tc_wait_st();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(BAR(P_FULL + 2 * w + (c - 2)));
+        }
+      }
+      float a, b;
+      unpack_f2(add_f2(add_f2(ps[0], ps[1]), add_f2(ps[2], ps[3])), a, b);
+      l_run += a + b;
+    }
+    // ---- the way out ----
+    if (ok && k > 0) ok = wait_bar_warp(BAR(PV_DONE + w), (k - 1) & 1, abort_flag, p.status, 52, p.wait_cycles);
+    tc_fence_after();
+    const bool have = ok && k > 0;                        // this warpgroup has rows in its accumulator
+    const int m = (TWO ? w * 128 : 0) + row;              // query row within the KV head: head_in_group * b + i
+    const int hg = m / p.b, i_row = m - hg * p.b;
+    __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(p.out) + (int64_t)bi * p.o_stride[0] + (int64_t)(g * p.G + hg) * p.o_stride[1] +
+                         (int64_t)i_row * p.o_stride[2];
+    float* lse = p.lse ? p.lse + ((int64_t)bi * p.Hq + g * p.G + hg) * p.b + i_row : nullptr;
+    const int64_t part = ((int64_t)((bi * p.Hkv + g) * Sh::QT + (TWO ? w : 0)) * p.splits + split) * 128;     // rows of partials in front
+    float4* part_o = reinterpret_cast<float4*>(p.part_o) + part * (D / 4) + row;
+    float2* part_ml = reinterpret_cast<float2*>(p.part_ml) + part + row;
+    float m_row = m_run, l_row = have ? l_run : 0.f, w_own = 1.f, w_other = 0.f;
+    int c_lo = 0, c_hi = D / 16;                          // columns, in chunks of 16, that this warpgroup carries out
+    const float4* other = nullptr;                        // the other warpgroup's accumulator for them
+    if constexpr (!TWO) {
+      // Both warpgroups hold the same query rows: each leaves the half of its columns that the other carries out, and its
+      // (maximum, sum), in the ring, which nobody reads any more once all eight warps (and the saliency warps) are here.
+      if (do_scores) asm volatile("bar.sync 3, 320;\n" ::: "memory");
+      else asm volatile("bar.sync 1, 256;\n" ::: "memory");
+      float4* box = reinterpret_cast<float4*>(stage0);    // [2 warpgroups][D / 8][128] float4, then [2][128] float2
+      float2* ml_s = reinterpret_cast<float2*>(stage0 + D * 128 * 4);
+      const int give = (1 - w) * (D / 32);
+      if (have) {
+#pragma unroll 1
+        for (int c = 0; c < D / 32; ++c) {
+          uint32_t ov[16];
+          tmem_ld16(o_addr + (give + c) * 16, ov);
+          tc_wait_ld();
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            box[(w * (D / 8) + c * 4 + e) * 128 + row] = make_float4(__uint_as_float(ov[4 * e]), __uint_as_float(ov[4 * e + 1]),
+                                                                    __uint_as_float(ov[4 * e + 2]), __uint_as_float(ov[4 * e + 3]));
+        }
+      }
+      ml_s[w * 128 + row] = make_float2(m_row, l_row);
+      asm volatile("bar.sync 1, 256;\n" ::: "memory");
+      const float2 o2 = ml_s[(1 - w) * 128 + row];
+      const float mm = fmaxf(l_row > 0.f ? m_row : -INFINITY, o2.y > 0.f ? o2.x : -INFINITY);
+      w_own = l_row > 0.f ? fast_exp2(m_row - mm) : 0.f;
+      w_other = o2.y > 0.f ? fast_exp2(o2.x - mm) : 0.f;
+      l_row = l_row * w_own + (o2.y > 0.f ? o2.y * w_other : 0.f);
+      m_row = mm;
+      c_lo = w * (D / 32); c_hi = c_lo + D / 32;
+      other = box + (1 - w) * (D / 8) * 128 + row;
+    }
+    const bool first_half = TWO || w == 0;                // who writes the row's sum
+    const float inv = p.splits == 1 ? (l_row > 0.f ? 1.f / l_row : 0.f) : 1.f;
+    if (!*abort_flag) {
+#pragma unroll 1
+      for (int c = c_lo; c < c_hi; ++c) {
+        uint32_t ov[16];
+        float4 v[4];
+        if (have) {
+          tmem_ld16(o_addr + c * 16, ov);
+          tc_wait_ld();
+        } else {
+#pragma unroll
+          for (int e = 0; e < 16; ++e) ov[e] = 0u;
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          v[e] = make_float4(__uint_as_float(ov[4 * e]), __uint_as_float(ov[4 * e + 1]), __uint_as_float(ov[4 * e + 2]), __uint_as_float(ov[4 * e + 3]));
+          if constexpr (!TWO) {
+            v[e].x *= w_own; v[e].y *= w_own; v[e].z *= w_own; v[e].w *= w_own;
+            if (w_other > 0.f) {
+              const float4 y = other[((c - c_lo) * 4 + e) * 128];
+              v[e].x = fmaf(y.x, w_other, v[e].x); v[e].y = fmaf(y.y, w_other, v[e].y);
+              v[e].z = fmaf(y.z, w_other, v[e].z); v[e].w = fmaf(y.w, w_other, v[e].w);
+            }
+          }
+        }
+        if (m < p.M) {
+          if (p.splits == 1) {
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+              *reinterpret_cast<uint4*>(out + c * 16 + e * 8) =
+                  make_uint4(pack_bf16(v[2 * e].x * inv, v[2 * e].y * inv), pack_bf16(v[2 * e].z * inv, v[2 * e].w * inv),
+                             pack_bf16(v[2 * e + 1].x * inv, v[2 * e + 1].y * inv), pack_bf16(v[2 * e + 1].z * inv, v[2 * e + 1].w * inv));
+          } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) __stcg(part_o + (c * 4 + e) * 128, v[e]);
+          }
+        }
+      }
+      if (first_half && m < p.M) {
+        if (p.splits > 1) __stcg(part_ml, make_float2(m_row, l_row));
+        else if (lse) *lse = (m_row + log2f(l_row)) * kLn2;
+      }
+    }
+  }
+
+  // ---- free the tensor memory ----
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    __syncwarp();
+    tc_fence_after();
+    tmem_dealloc(tmem_base, 512);
+  }
+}
+
+// Fold of the key splits (one thread per query row and float4 column, lanes along the rows, the loads of all splits in flight
+// together) and pooling of the saliency (one thread per position).
+template <int D>
+__global__ void __launch_bounds__(128) pair_tail_kernel(const PairParams pp, const int q_tiles, const int merge_blocks) {
+  const AttnParams& p = pp.a;
+  constexpr int C4 = D / 4, MB = 18;
+  const int row = threadIdx.x, c4 = blockIdx.x % C4, tile = blockIdx.x / C4;      // tile: (sequence, KV head, Q tile)
+  const int m = (tile % q_tiles) * 128 + row, bg = tile / q_tiles;
+  const int bi = bg / p.Hkv, g = bg - bi * p.Hkv, hg = m / p.b, i = m - hg * p.b;
+  const float4* po = reinterpret_cast<const float4*>(p.part_o) + ((int64_t)tile * p.splits * C4 + c4) * 128 + row;
+  const float2* pm = reinterpret_cast<const float2*>(p.part_ml) + (int64_t)tile * p.splits * 128 + row;
+  grid_dependency_wait();
+  grid_launch_dependents();
+  if ((int)blockIdx.x < merge_blocks) {
+    if (m >= p.M) return;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    float m_run = -INFINITY, l = 0.f;
+    for (int s0 = 0; s0 < p.splits; s0 += MB) {
+      float2 ml[MB];
+      float4 v[MB];
+#pragma unroll
+      for (int u = 0; u < MB; ++u)
+        if (s0 + u < p.splits) {
+          ml[u] = __ldcg(pm + (s0 + u) * 128);
+          v[u] = __ldcg(po + (int64_t)(s0 + u) * C4 * 128);
+        } else {
+          ml[u] = make_float2(-INFINITY, 0.f);
+          v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+      float bm = m_run;
+#pragma unroll
+      for (int u = 0; u < MB; ++u)
+        if (ml[u].y > 0.f) bm = fmaxf(bm, ml[u].x);
+      const float a = (bm == -INFINITY) ? 1.f : fast_exp2(m_run - bm);    // 0 on the first batch with data
+      l *= a; acc.x *= a; acc.y *= a; acc.z *= a; acc.w *= a;
+      m_run = bm;
+#pragma unroll
+      for (int u = 0; u < MB; ++u) {
+        if (!(ml[u].y > 0.f)) continue;
+        const float w = fast_exp2(ml[u].x - bm);
+        l = fmaf(ml[u].y, w, l);
+        acc.x = fmaf(v[u].x, w, acc.x); acc.y = fmaf(v[u].y, w, acc.y); acc.z = fmaf(v[u].z, w, acc.z); acc.w = fmaf(v[u].w, w, acc.w);
+      }
+    }
+    const float inv = l > 0.f ? 1.f / l : 0.f;
+    __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(p.out) + (int64_t)bi * p.o_stride[0] + (int64_t)(g * p.G + hg) * p.o_stride[1] +
+                         (int64_t)i * p.o_stride[2] + c4 * 4;
+    *reinterpret_cast<uint2*>(out) = make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
+    if (c4 == 0 && p.lse) p.lse[((int64_t)bi * p.Hq + g * p.G + hg) * p.b + i] = (m_run + log2f(l)) * kLn2;
+    return;
+  }
+  const int64_t idx = (int64_t)(blockIdx.x - merge_blocks) * 128 + threadIdx.x;
+  if (idx >= (int64_t)p.B * p.Hkv * p.n1_max) return;
+  const int pos = (int)(idx % p.n1_max);
+  const int64_t bh = idx / p.n1_max;
+  const int seq = (int)(bh / p.Hkv);
+  int L = p.n1_per_seq ? p.n1_per_seq[seq] : p.n1_max;
+  L = min(max(L, 0), p.n1_max);
+  p.pooled[idx] = pool_at_ldcg(p, p.raw_scores + bh * p.n1_max, L, p.block_off[seq], pos);
+}
+
+template <int D, bool TWO>
+cudaError_t launch_pair_shape(const PairMaps& tm, const PairParams& pp, bool pdl, cudaStream_t st) {
+  auto kern = attn_pair_kernel<D, TWO>;
+  static SmemConfig configured;
+  const size_t smem = PairShape<D, TWO>::SMEM > 120 * 1024 ? PairShape<D, TWO>::SMEM : 120 * 1024;    // one CTA per SM: it takes all TMEM
+  cudaError_t e = configure_smem(reinterpret_cast<const void*>(kern), smem, configured, true);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(pp.a.splits, pp.a.Hkv, pp.a.B);
+  cfg.blockDim = dim3(PR_THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = pdl ? 1 : 0;
+  e = cudaLaunchKernelEx(&cfg, kern, tm, pp);
+  if (e != cudaSuccess) return e;
+  const bool merge = pp.a.out != nullptr && pp.a.splits > 1, pool = pp.a.want_scores && pp.a.pooled != nullptr;
+  if (!merge && !pool) return cudaSuccess;
+  const int merge_blocks = merge ? pp.a.B * pp.a.Hkv * (TWO ? 2 : 1) * (D / 4) : 0;
+  const long long pool_threads = pool ? (long long)pp.a.B * pp.a.Hkv * pp.a.n1_max : 0;
+  cfg.gridDim = dim3((unsigned)(merge_blocks + (pool_threads + 127) / 128));
+  cfg.blockDim = dim3(128);
+  cfg.dynamicSmemBytes = 0;
+  return cudaLaunchKernelEx(&cfg, pair_tail_kernel<D>, pp, TWO ? 2 : 1, merge_blocks);
+}
+
+}  // namespace
+
+// The key splits of a unit, at most one wave of CTAs in all. Costs in us, fitted to sweeps over 1 to 16 units of 5 to 256 tiles:
+// a tile takes 1.0 (one Q tile) or 1.55 (two), the partial rows 0.43 per MB on their way to the fold and back, and a reuse step
+// without splits saves the second launch. (8 units x 17 tiles: 9 splits of two tiles 10.4, 17 of one 11.2; 4 units x 9 tiles of
+// two Q tiles: 9 splits 10.5, 6 splits 11.9; 8 units x 129 tiles: flat from 12 to 18, 22.4.)
+AttnPlan plan_attention_pair(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn) {
+  (void)b;
+  AttnPlan pl{};
+  pl.kind = 4; pl.tma = true; pl.cluster = 1; pl.fused_tail = true;
+  pl.threads = PR_THREADS; pl.key_tile = 128; pl.key_tile2 = n2 > 0 ? (n2 < 128 ? n2 : 128) : 128;
+  pl.row_tiles = M > 128 ? 2 : 1; pl.rep = 1; pl.rows_rep = 128;
+  pl.stages = D == 64 ? 4 : (M > 128 ? 2 : 3);
+  const long long units = (long long)B * Hkv;
+  const int tiles = (n1_max + 127) / 128 + (n2 > 0 ? (n2 + pl.key_tile2 - 1) / pl.key_tile2 : 0);
+  long long most = sm_count() / units;
+  if (most > tiles) most = tiles;
+  if (most > kMaxSplits) most = kMaxSplits;
+  pl.splits = 1;
+  double least = 1e30;
+  for (int s = 1; s == 1 || s <= most; ++s) {
+    const double cost = (tiles + s - 1) / s * (pl.row_tiles == 2 ? 1.55 : 1.0) +
+                        (s > 1 ? 0.43e-6 * (double)units * s * pl.row_tiles * 128 * D * 4 + (n2 > 0 ? 2.5 : 0.) : 0.);
+    if (cost < least) { least = cost; pl.splits = s; }
+  }
+  if (tn.splits > 0) pl.splits = tn.splits < tiles ? tn.splits : (tiles > 0 ? tiles : 1);
+  pl.parts = pl.splits;
+  pl.part_rows = pl.splits > 1 ? (size_t)pl.row_tiles * pl.splits * 128 : 0;
+  pl.n_counters = 0;
+  return pl;
+}
+
+cudaError_t launch_attn_pair(const AttnParams& p, const AttnPlan& pl, int D, cudaStream_t st) {
+  const Tuning tn = tuning();
+  PairMaps tm;
+  PairParams pp{};
+  pp.a = p;
+  pp.a.splits = pl.splits;
+  pp.KT2 = pl.key_tile2;
+  pp.heads_rt = pl.row_tiles == 1 ? p.G : 128 / p.b;
+  pp.early_src1 = (p.n2 > 0 && p.n1_max > 0 && tn.early_loads != 0) ? 1 : 0;
+  const long long ctas = (long long)pl.splits * p.Hkv * p.B;
+  pp.lpt = (p.n1_per_seq != nullptr && p.B >= 4 && p.B <= 64 && ctas > sm_count()) ? 1 : 0;
+  if (tn.lpt >= 0) pp.lpt = (tn.lpt == 1 && p.n1_per_seq != nullptr && p.B >= 2 && p.B <= 64) ? 1 : 0;
+  memset(&tm, 0, sizeof(tm));
+  bool ok = umma_make_map(&tm.q, p.q, D, p.b, p.Hq, p.B, p.q_stride, p.b, pp.heads_rt);
+  if (p.n1_max > 0) {
+    ok = ok && umma_make_map(&tm.k1, p.k1, D, p.n1_max, p.Hkv, p.B, p.k1_stride, 128, 1);
+    ok = ok && umma_make_map(&tm.v1, p.v1, D, p.n1_max, p.Hkv, p.B, p.k1_stride, 128, 1);
+  }
+  if (p.n2 > 0) {
+    ok = ok && umma_make_map(&tm.k2, p.k2, D, p.n2, p.Hkv, p.B, p.k2_stride, pl.key_tile2, 1);
+    ok = ok && umma_make_map(&tm.v2, p.v2, D, p.n2, p.Hkv, p.B, p.k2_stride, pl.key_tile2, 1);
+    if (p.n1_max <= 0) { tm.k1 = tm.k2; tm.v1 = tm.v2; }
+  } else {
+    tm.k2 = tm.k1; tm.v2 = tm.v1;
+  }
+  if (!ok) return cudaErrorInvalidValue;
+  const bool pdl = tn.pdl != 0;
+  if (pl.row_tiles == 2) return D == 128 ? launch_pair_shape<128, true>(tm, pp, pdl, st) : launch_pair_shape<64, true>(tm, pp, pdl, st);
+  return D == 128 ? launch_pair_shape<128, false>(tm, pp, pdl, st) : launch_pair_shape<64, false>(tm, pp, pdl, st);
+}
+
+}  // namespace sdllm

@@ -57,48 +57,6 @@ struct UmmaParams {
 
 #include "umma_ptx.cuh"
 
-// Importance of one absolute position: Algorithm 1, MaxPool1D(A, kernel_size = s, padding = s/2) over the candidate
-// axis Concat(prefix, suffix) (AvgPool for the ablation); block positions and padding get -inf. `a` holds the raw
-// saliency by absolute position.
-__device__ __forceinline__ float pool_at(const AttnParams& p, const float* a, int L, int o_in, int pos, int n_arr = 1,
-                                         int64_t arr_stride = 0) {
-  const int b = p.b;
-  const int o = min(max(o_in, 0), max(L - b, 0));
-  if (pos >= L || (pos >= o && pos < o + b)) return -INFINITY;
-  const int C = max(L - b, 0), w = (p.window - 1) / 2;
-  const int c = pos < o ? pos : pos - b;
-  int lo = 0, hi = C;
-  if (p.per_region) { if (c < o) hi = o; else lo = o; }
-  float mx = -INFINITY, sum = 0.f;
-  for (int t = c - w; t <= c + w; ++t) {
-    if (t < lo || t >= hi) continue;
-    float x = a[t < o ? t : t + b];
-    for (int r2 = 1; r2 < n_arr; ++r2) x += a[r2 * arr_stride + (t < o ? t : t + b)];   // one array per row tile
-    mx = fmaxf(mx, x);
-    sum += x;
-  }
-  return p.pool_kind == SDLLM_POOL_MAX ? mx : sum / (float)p.window;
-}
-
-// The same, reading the raw saliency from global memory through L2 (other CTAs wrote it during this launch).
-__device__ __forceinline__ float pool_at_ldcg(const AttnParams& p, const float* a, int L, int o_in, int pos) {
-  const int b = p.b;
-  const int o = min(max(o_in, 0), max(L - b, 0));
-  if (pos >= L || (pos >= o && pos < o + b)) return -INFINITY;
-  const int C = max(L - b, 0), w = (p.window - 1) / 2;
-  const int c = pos < o ? pos : pos - b;
-  int lo = 0, hi = C;
-  if (p.per_region) { if (c < o) hi = o; else lo = o; }
-  float mx = -INFINITY, sum = 0.f;
-  for (int t = c - w; t <= c + w; ++t) {
-    if (t < lo || t >= hi) continue;
-    const float x = __ldcg(a + (t < o ? t : t + b));
-    mx = fmaxf(mx, x);
-    sum += x;
-  }
-  return p.pool_kind == SDLLM_POOL_MAX ? mx : sum / (float)p.window;
-}
-
 // Merge of the key-split partials of S (row, float4 column) slots of a unit and the final stores. slot[s] < 0 marks
 // an unused entry. The partials are read in batches of MB per slot with the loads of all slots and of the whole batch
 // in flight together (one L2 latency per batch) and folded with a running maximum, so that four splits cost a single
@@ -1179,19 +1137,23 @@ cudaError_t launch_attn_umma(const AttnParams& p, const AttnPlan& pl, int D, cud
 AttnPlan plan_attention_legacy(int dtype, int D, int M, int B, int Hkv, int n_keys_max, const Tuning& tn);
 cudaError_t launch_attn_legacy(const AttnParams& p, const AttnPlan& plan, int dtype, int D, cudaStream_t st);
 bool kt_supported(int dtype, int D, int M, int b);
-bool kt_preferred(int M, int B, int Hkv, int n1_max, int n2);
+bool kt_preferred(int D, int M, int B, int Hkv, int n1_max, int n2);
 AttnPlan plan_attention_kt(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn);
 cudaError_t launch_attn_kt(const AttnParams& p, const AttnPlan& pl, int D, cudaStream_t st);
 
+AttnPlan plan_attention_pair(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn);
+cudaError_t launch_attn_pair(const AttnParams& p, const AttnPlan& pl, int D, cudaStream_t st);
+
 AttnPlan plan_attention(int dtype, int D, int M, int b, int B, int Hkv, int n1_max, int n2, bool prob_scores) {
-  // bf16 goes to the tcgen05 kernels wherever they apply: heads with at most 128 query rows to the kernel that puts the
-  // keys on the accumulator rows (it has no softmax-probability saliency pass) unless its cluster limit would leave most
-  // SMs idle, the rest to the one that puts the queries there; fp32 and the remaining bf16 shapes go to the cp.async
-  // kernels. Tuning::kernel forces a family.
+  // bf16 goes to the tcgen05 kernels wherever they apply: heads with few query rows to the kernel that puts the keys on the
+  // accumulator rows, the rest to the one that puts the queries there and has two softmax warpgroups (attn_pair.cu); the
+  // probability saliency has its own second pass in the older query-row kernel of this file. fp32 and the remaining bf16
+  // shapes go to the cp.async kernels. Tuning::kernel forces a family.
   const Tuning tn = tuning();
   const bool kt_ok = kt_supported(dtype, D, M, b) && !prob_scores;
-  if (kt_ok && (tn.kernel == 3 || (tn.kernel == 0 && kt_preferred(M, B, Hkv, n1_max, n2))))
+  if (kt_ok && (tn.kernel == 3 || (tn.kernel == 0 && kt_preferred(D, M, B, Hkv, n1_max, n2))))
     return plan_attention_kt(D, M, b, B, Hkv, n1_max, n2, tn);
+  if ((tn.kernel == 0 || tn.kernel == 4) && umma_supported(dtype, D, M, b) && !prob_scores) return plan_attention_pair(D, M, b, B, Hkv, n1_max, n2, tn);
   if (tn.kernel != 1 && umma_supported(dtype, D, M, b)) return plan_attention_umma(D, M, b, B, Hkv, n1_max, n2, tn);
   AttnPlan pl = plan_attention_legacy(dtype, D, M, B, Hkv, n1_max + n2, tn);
   pl.tma = false; pl.cluster = 1; pl.warp_keys = 32; pl.kind = 0;
@@ -1203,6 +1165,7 @@ AttnPlan plan_attention(int dtype, int D, int M, int b, int B, int Hkv, int n1_m
 
 cudaError_t launch_attn_partial(const AttnParams& p, const AttnPlan& plan, int dtype, int D, cudaStream_t st) {
   if (plan.kind == 3) return launch_attn_kt(p, plan, D, st);
+  if (plan.kind == 4) return launch_attn_pair(p, plan, D, st);
   if (plan.kind == 2) return launch_attn_umma(p, plan, D, st);
   return launch_attn_legacy(p, plan, dtype, D, st);
 }

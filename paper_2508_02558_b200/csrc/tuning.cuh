@@ -14,7 +14,8 @@ constexpr int kMaxDevices = 64;
 struct Tuning {
   int splits = 0;            // > 0: key splits per (sequence, KV head)
   int kernel = 0;            // 0: automatic; 1: cp.async kernels; 2: tcgen05 kernel with the queries on the accumulator
-                             // rows; 3: tcgen05 kernel with the keys on the accumulator rows
+                             // rows, one softmax warpgroup; 3: tcgen05 kernel with the keys on the accumulator rows; 4: as 2,
+                             // two softmax warpgroups
   int pdl = 1;               // 0: no programmatic dependent launch
   int early_loads = 1;       // 0: no loads ahead of the grid dependency
   int cluster = 1;           // query-row kernel: 2 merges few key splits through a cluster where the shape allows (off otherwise)

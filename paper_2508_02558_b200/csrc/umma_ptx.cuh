@@ -144,6 +144,7 @@ __device__ __forceinline__ void poly_exp2(float x0, float x1, float& e0, float& 
   e1 = __uint_as_float(__float_as_uint(y1) + (__float_as_uint(t1) << 23));
 }
 __device__ __forceinline__ void regs_dec_72() { asm volatile("setmaxnreg.dec.sync.aligned.u32 72;\n"); }
+__device__ __forceinline__ void regs_dec_80() { asm volatile("setmaxnreg.dec.sync.aligned.u32 80;\n"); }
 __device__ __forceinline__ void regs_inc_208() { asm volatile("setmaxnreg.inc.sync.aligned.u32 208;\n"); }
 
 __device__ __forceinline__ void cluster_sync_all() {
@@ -175,6 +176,21 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes,
 // Instruction descriptor, kind::f16: fp32 accumulator, bf16 A and B, M = 128, N = n, A K-major, B K- or MN-major.
 __device__ __forceinline__ uint32_t instr_desc(int n, bool b_mn_major) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((b_mn_major ? 1u : 0u) << 16) | ((uint32_t)(n >> 3) << 17) | ((128u >> 4) << 24);
+}
+
+// The sequence of rank `rank` when a batch of at most 64 is ordered from the longest to the shortest (equal lengths in batch
+// order). A whole warp calls this; every lane gets the answer.
+__device__ __forceinline__ int sequence_of_rank(const int32_t* lengths, int B, int rank) {
+  const int lane = threadIdx.x & 31;
+  const int l0 = lane < B ? lengths[lane] : -1, l1 = lane + 32 < B ? lengths[lane + 32] : -1;
+  int r0 = 0, r1 = 0;                                  // how many sequences come before mine
+  for (int i = 0; i < B; ++i) {
+    const int li = __shfl_sync(0xffffffffu, i < 32 ? l0 : l1, i & 31);
+    r0 += (li > l0 || (li == l0 && i < lane)) ? 1 : 0;
+    r1 += (li > l1 || (li == l1 && i < lane + 32)) ? 1 : 0;
+  }
+  const unsigned hit0 = __ballot_sync(0xffffffffu, lane < B && r0 == rank), hit1 = __ballot_sync(0xffffffffu, lane + 32 < B && r1 == rank);
+  return hit0 ? __ffs(hit0) - 1 : (hit1 ? __ffs(hit1) + 31 : rank);
 }
 
 // Which tile (source, first row, valid rows, MMA width) a CTA-local ordinal refers to.

@@ -35,8 +35,8 @@ def test_select_compact_at_the_ends_of_each_variant(cand, heads, mode, r):
     n, n_pre, n_suf = B.keep_count(d, L, o)
     assert cnt.item() == n
     pos = oracle.candidate_positions(L, b, o)
-    x = np.where(np.isnan(sc), -np.inf, sc)[0][:, pos]
-    x = np.where(np.isnan(sc[0][:, pos]), np.finfo(np.float64).min * np.ones_like(x, np.float64), np.maximum(x, -1e300).astype(np.float64))
+    x = sc[0][:, pos].astype(np.float64)
+    x = np.where(np.isnan(x), -1e301, np.maximum(x, -1e300))            # NaN below everything
     for h in range(heads):
         segments = [(0, cand, n)] if mode == B.SELECT_JOINT_FLOOR else [(0, o, n_pre), (o, cand, n_suf)]
         want = np.concatenate([pos[lo + np.sort(np.argsort(-x[h, lo:hi], kind="stable")[:m])] for lo, hi, m in segments])
@@ -45,3 +45,34 @@ def test_select_compact_at_the_ends_of_each_variant(cand, heads, mode, r):
         assert (got[n:] == -1).all()
         rows = np.where(np.arange(cand) < n, h * L + got, 0)
         assert (kc[0, h, :, 0].cpu().numpy() == rows).all() and (vc[0, h, :, -1].cpu().numpy() == -rows).all()
+
+
+def _wide(name, Hq, Hkv, D, p, gen, b=32):
+    from test_gpu_parity import _small
+    return _small(name, "bf16", Hq, Hkv, D, p, gen, block_len=b, salient_frac=0.02)
+
+
+@pytest.mark.parametrize("cfg,block", [
+    (_wide("m128", 8, 2, 128, 700, 64), 1), (_wide("m224", 14, 2, 128, 1000, 64), 0), (_wide("m256_d64", 4, 1, 64, 500, 128, 64), 1),
+    (_wide("m96", 3, 1, 128, 300, 32), 0), (_wide("m112_blk16", 7, 1, 64, 640, 32, 16), 1), (_wide("m64_short", 4, 2, 128, 40, 32), 0),
+])
+@pytest.mark.parametrize("splits", [0, 1, 2, 5, 19])
+def test_two_warpgroup_query_row_kernel(cfg, block, splits, tuning):
+    """One and two Q tiles, partly filled row tiles, one tile per CTA and several, more splits than a fold batch holds."""
+    from test_gpu_parity import _run_sequence_case
+    tuning(kernel=4, **(dict(splits=splits) if splits else {}))
+    _run_sequence_case(cfg, seed=17, block=block)
+
+
+@pytest.mark.parametrize("lens", [[900, 300, 64, 1300, 33], [640, 640]])
+def test_two_warpgroup_query_row_kernel_on_ragged_batches(lens, tuning):
+    import parity_util as U
+    from paper_2508_02558_b200 import workloads as W
+    for plan in (dict(kernel=4), dict(kernel=4, lpt=1), dict(kernel=4, lpt=1, early_loads=0, splits=3)):
+        tuning(**plan)
+        bw = W.make_batch(_wide("ragged", 8, 2, 128, 100, 32), [n - 32 for n in lens], seed=5)
+        q, k, v = bw.refresh_inputs(1, pad_value=np.nan)
+        g = U.gpu_refresh(q, k, v, bw.seq_len, bw.block_off, "bf16", 0.5, 3)
+        U.check_refresh_against_oracle(g, q, np.nan_to_num(k), np.nan_to_num(v), bw.seq_len, bw.block_off, "bf16", 0.5, 3)
+        q2, kn, vn = bw.sparse_inputs(2)
+        U.check_sparse_against_oracle(g, U.gpu_sparse_step(g, q2, kn, vn, "bf16"), q2, kn, vn, "bf16")
