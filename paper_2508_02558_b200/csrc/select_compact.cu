@@ -95,8 +95,7 @@ __device__ __forceinline__ void select_barrier() {
 }
 
 // The threads of the SW selecting warps call this with their keys (item j is candidate c0 + 32 j; key 0: none).
-// emit(w, c) is called for every kept candidate c with its rank w in the head's ascending list. A threshold is never 0 (a
-// quota does not exceed its segment), so items without a candidate need no test anywhere.
+// emit(w, c) is called for every kept candidate c with its rank w in the head's ascending list.
 template <int SW, int KPT, int CS, typename Emit>
 __device__ __forceinline__ void select_head(const HeadPlace& h, const uint32_t (&key)[KPT], int c0, SelectShared<SW, CS>& sh, int rank, Emit emit) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -105,9 +104,9 @@ __device__ __forceinline__ void select_head(const HeadPlace& h, const uint32_t (
   for (int si = 0; si < 2; ++si) {
     const int c_lo = si == 0 ? 0 : h.c1, c_hi = si == 0 ? h.c1 : h.C, n = si == 0 ? h.n0 : h.n1;
     if (n <= 0 || c_hi <= c_lo) continue;              // (the same decision in every CTA of a cluster)
-    uint32_t k[KPT];                                   // the segment's keys
+    uint32_t in = 0u;                                  // items with a candidate of the segment
 #pragma unroll
-    for (int j = 0; j < KPT; ++j) k[j] = c0 + 32 * j >= c_lo && c0 + 32 * j < c_hi ? key[j] : 0u;
+    for (int j = 0; j < KPT; ++j) in |= key[j] != 0u && c0 + 32 * j >= c_lo && c0 + 32 * j < c_hi ? 1u << j : 0u;
     uint32_t thr = 0u, need_eq = 0u;                   // (as they stand: everything is kept)
     if (n < c_hi - c_lo) {
       uint32_t remaining = (uint32_t)n;
@@ -118,7 +117,7 @@ __device__ __forceinline__ void select_head(const HeadPlace& h, const uint32_t (
         uint32_t* hist = sh.hist[si][pass];
 #pragma unroll
         for (int j = 0; j < KPT; ++j)
-          if ((k[j] & himask) == thr && k[j] != 0u) atomicAdd(&hist[(k[j] >> shift) & 0xFFu], 1u);
+          if ((in >> j & 1u) != 0u && (key[j] & himask) == thr) atomicAdd(&hist[(key[j] >> shift) & 0xFFu], 1u);
         if constexpr (CS > 1) {
           __syncthreads();
           for (int i = tid; i < 256 * CS; i += 32 * SW) {
@@ -160,8 +159,8 @@ __device__ __forceinline__ void select_head(const HeadPlace& h, const uint32_t (
     uint32_t n_gt = 0, n_eq = 0;
 #pragma unroll
     for (int j = 0; j < KPT; ++j) {
-      n_gt += k[j] > thr ? 1u : 0u;
-      n_eq += k[j] == thr ? 1u : 0u;
+      n_gt += (in >> j & 1u) != 0u && key[j] > thr ? 1u : 0u;
+      n_eq += (in >> j & 1u) != 0u && key[j] == thr ? 1u : 0u;
     }
     n_gt = __reduce_add_sync(0xffffffffu, n_gt);
     n_eq = __reduce_add_sync(0xffffffffu, n_eq);
@@ -185,7 +184,7 @@ __device__ __forceinline__ void select_head(const HeadPlace& h, const uint32_t (
     const uint32_t below = (1u << lane) - 1u;
 #pragma unroll
     for (int j = 0; j < KPT; ++j) {
-      const bool gt = k[j] > thr, eq = k[j] == thr;
+      const bool mine = (in >> j & 1u) != 0u, gt = mine && key[j] > thr, eq = mine && key[j] == thr;
       const uint32_t m_gt = __ballot_sync(0xffffffffu, gt), m_eq = __ballot_sync(0xffffffffu, eq);
       const uint32_t eq_rank = eq_before + __popc(m_eq & below);              // ties go to the lowest positions
       if (gt || (eq && eq_rank < need_eq)) emit((int)(run_out + gt_before + __popc(m_gt & below) + min(eq_rank, need_eq)), c0 + 32 * j);
@@ -464,16 +463,22 @@ cudaError_t launch_select_topk_shape(const SelectParams& p, bool pdl, cudaStream
   return cudaLaunchKernelEx(&lc.cfg, select_topk_kernel<SW, KPT, CS>, p);
 }
 
-// Candidates in the registers of one CTA up to 8192 per head, of a cluster of eight CTAs up to 65536, and in global memory
-// beyond. Tuning::select forces one CTA (1) or a cluster (2) per head.
+// Candidates in the registers of one CTA up to 8192 per head; beyond that, for up to a quarter as many heads as SMs (two waves
+// of clusters), in those of a cluster of eight CTAs (up to 65536), else again of one CTA, of 1024 threads (up to 32768); in
+// global memory where neither fits. (30000 candidates: 32 heads 16.5 us with clusters, 39 without; 128 heads 61 and 39.) Tuning::select forces one CTA (1) or a cluster (2) per head.
 cudaError_t launch_topk(const SelectParams& p, bool pdl, cudaStream_t st) {
   const int cand = p.Lmax - p.b, forced = tuning().select;
+  const bool few = (long long)p.B * p.Hkv * 4 <= sm_count();
   if (forced != 2) {
     if (cand <= 512) return launch_select_topk_shape<8, 2, 1>(p, pdl, st);
     if (cand <= 1536) return launch_select_topk_shape<8, 6, 1>(p, pdl, st);
     if (cand <= 3072) return launch_select_topk_shape<16, 6, 1>(p, pdl, st);
     if (cand <= 5120) return launch_select_topk_shape<16, 10, 1>(p, pdl, st);
     if (cand <= 8192) return launch_select_topk_shape<16, 16, 1>(p, pdl, st);
+    if (!few || forced == 1) {
+      if (cand <= 16384) return launch_select_topk_shape<32, 16, 1>(p, pdl, st);
+      if (cand <= 32768) return launch_select_topk_shape<32, 32, 1>(p, pdl, st);
+    }
   }
   if (forced != 1) {
     if (cand <= SEL_CLUSTER * 4096) return launch_select_topk_shape<16, 8, SEL_CLUSTER>(p, pdl, st);
