@@ -821,10 +821,11 @@ int kt_resident_clusters(int D, int CG, int S) {
 
 }  // namespace
 
-// Whether the key-row kernel covers a shape: bf16, D in {64, 128}, at most 128 query rows per KV head, block length a
-// multiple of 16.
+// Whether the key-row kernel covers a shape: bf16, D in {64, 128}, at most 128 query rows per KV head, a multiple of four (the
+// way out stores four rows at a time). The block length is otherwise free: query rows are padded to a multiple of 32 with zeros,
+// the block's own keys to a group of 32.
 bool kt_supported(int dtype, int D, int M, int b) {
-  return umma_supported(dtype, D, M, b) && M <= 128;
+  return umma_supported(dtype, D, 16, 16) && M <= 128 && M % 4 == 0 && b <= 128;
 }
 
 // Whether the planner picks it among the shapes it covers: against the query-row kernel with two softmax warpgroups

@@ -40,7 +40,7 @@ struct PairMaps {
 };
 struct PairParams {
   AttnParams a;
-  int KT2;           // rows of a source-2 tile (<= 128, multiple of 16)
+  int KT2;           // rows of a source-2 tile (<= 128)
   int heads_rt;      // query heads per Q tile
   int early_src1;    // 1: source 1 and its count are older than the previous kernel in the stream (reuse step)
   int lpt;           // 1: grid z counts the sequences from the longest to the shortest (several waves of ragged work)
@@ -606,6 +606,11 @@ cudaError_t launch_pair_shape(const PairMaps& tm, const PairParams& pp, bool pdl
 }
 
 }  // namespace
+
+// Whether this kernel covers a shape: bf16, D in {64, 128}, and whole query heads in every Q tile.
+bool pair_supported(int dtype, int D, int M, int b) {
+  return umma_supported(dtype, D, 16, 16) && b <= 128 && (M <= 128 || (M <= 256 && 128 % b == 0));
+}
 
 // The key splits of a unit, at most one wave of CTAs in all. Costs in us, fitted to sweeps over 1 to 16 units of 5 to 256 tiles:
 // a tile takes 1.0 (one Q tile) or 1.55 (two), the partial rows 0.43 per MB on their way to the fold and back, and a reuse step

@@ -1141,6 +1141,7 @@ bool kt_preferred(int D, int M, int B, int Hkv, int n1_max, int n2);
 AttnPlan plan_attention_kt(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn);
 cudaError_t launch_attn_kt(const AttnParams& p, const AttnPlan& pl, int D, cudaStream_t st);
 
+bool pair_supported(int dtype, int D, int M, int b);
 AttnPlan plan_attention_pair(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn);
 cudaError_t launch_attn_pair(const AttnParams& p, const AttnPlan& pl, int D, cudaStream_t st);
 
@@ -1153,7 +1154,7 @@ AttnPlan plan_attention(int dtype, int D, int M, int b, int B, int Hkv, int n1_m
   const bool kt_ok = kt_supported(dtype, D, M, b) && !prob_scores;
   if (kt_ok && (tn.kernel == 3 || (tn.kernel == 0 && kt_preferred(D, M, B, Hkv, n1_max, n2))))
     return plan_attention_kt(D, M, b, B, Hkv, n1_max, n2, tn);
-  if ((tn.kernel == 0 || tn.kernel == 4) && umma_supported(dtype, D, M, b) && !prob_scores) return plan_attention_pair(D, M, b, B, Hkv, n1_max, n2, tn);
+  if ((tn.kernel == 0 || tn.kernel == 4) && pair_supported(dtype, D, M, b) && !prob_scores) return plan_attention_pair(D, M, b, B, Hkv, n1_max, n2, tn);
   if (tn.kernel != 1 && umma_supported(dtype, D, M, b)) return plan_attention_umma(D, M, b, B, Hkv, n1_max, n2, tn);
   AttnPlan pl = plan_attention_legacy(dtype, D, M, B, Hkv, n1_max + n2, tn);
   pl.tma = false; pl.cluster = 1; pl.warp_keys = 32; pl.kind = 0;

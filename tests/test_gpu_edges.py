@@ -76,3 +76,15 @@ def test_two_warpgroup_query_row_kernel_on_ragged_batches(lens, tuning):
         U.check_refresh_against_oracle(g, q, np.nan_to_num(k), np.nan_to_num(v), bw.seq_len, bw.block_off, "bf16", 0.5, 3)
         q2, kn, vn = bw.sparse_inputs(2)
         U.check_sparse_against_oracle(g, U.gpu_sparse_step(g, q2, kn, vn, "bf16"), q2, kn, vn, "bf16")
+
+
+@pytest.mark.parametrize("b,Hq,Hkv,D", [(8, 4, 4, 128), (8, 8, 2, 64), (1, 2, 2, 128), (20, 6, 2, 128), (37, 2, 1, 64), (100, 1, 1, 128), (8, 28, 1, 128), (24, 5, 1, 128)])
+def test_block_lengths_that_fill_no_tile(b, Hq, Hkv, D, tuning):
+    """Any block length runs on the tensor cores: query rows and the block's own keys are padded inside the kernels."""
+    from test_gpu_parity import _run_sequence_case
+    from paper_2508_02558_b200 import binding as B
+    cfg = _wide("odd_block", Hq, Hkv, D, 333, 2 * b, b)
+    for plan in ({}, dict(kernel=3), dict(kernel=4), dict(persist=2)):
+        tuning(**plan)
+        _run_sequence_case(cfg, seed=23, block=1)
+        B.tuning_reset()
