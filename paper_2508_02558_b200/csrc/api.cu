@@ -42,7 +42,7 @@ sdllm_status check_desc(const sdllm_desc* d) {
   if (d->head_dim != 64 && d->head_dim != 128) return SDLLM_ERR_UNSUPPORTED;
   if ((int64_t)d->block_len * (d->n_q_heads / d->n_kv_heads) > kMaxRows) return SDLLM_ERR_UNSUPPORTED;
   if (d->batch > 65535 || d->n_kv_heads > 65535) return SDLLM_ERR_UNSUPPORTED;
-  // the softmax-probability saliency exists in the tcgen05 kernel only
+  // the softmax-probability saliency exists for the shapes of the tcgen05 kernels only
   if (d->score == SDLLM_SCORE_PROB_MEAN &&
       !umma_supported(d->dtype, d->head_dim, d->n_q_heads / d->n_kv_heads * d->block_len, d->block_len))
     return SDLLM_ERR_UNSUPPORTED;
@@ -96,7 +96,7 @@ WsLayout attn_ws(const sdllm_desc* d, const AttnPlan& pl, bool scores) {
   off += align_up((size_t)d->batch * d->n_kv_heads * pl.part_rows * 2 * 4, 256);
   w.raw = off;
   const bool prob = d->score == SDLLM_SCORE_PROB_MEAN;
-  if (scores) off += align_up((size_t)d->batch * d->n_kv_heads * d->seq_len_max * 4 * (prob ? pl.row_tiles : 1), 256);
+  if (scores) off += align_up((size_t)d->batch * d->n_kv_heads * d->seq_len_max * 4, 256);
   w.lse = off;                         // probability saliency: the rows' log-sum-exp between its two passes
   if (scores && prob) off += align_up((size_t)d->batch * d->n_q_heads * d->block_len * 4, 256);
   w.total = off;
@@ -107,8 +107,7 @@ AttnPlan plan_for(const sdllm_desc* d, int op) {
   const int G = d->n_q_heads / d->n_kv_heads;
   const bool refresh = op == SDLLM_OP_REFRESH_SCORES;
   return plan_attention(d->dtype, d->head_dim, G * d->block_len, d->block_len, d->batch, d->n_kv_heads,
-                        refresh ? d->seq_len_max : d->n_keep_max, refresh ? 0 : d->block_len,
-                        refresh && d->score == SDLLM_SCORE_PROB_MEAN);
+                        refresh ? d->seq_len_max : d->n_keep_max, refresh ? 0 : d->block_len);
 }
 
 void fill_common(AttnParams& p, const sdllm_desc* d, const AttnPlan& pl) {
@@ -221,13 +220,12 @@ int32_t sdllm_launch_count(const sdllm_desc* d, int op) {
   const bool refresh = op == SDLLM_OP_REFRESH_SCORES;
   const AttnPlan pl = plan_for(d, op);
   const int M = d->n_q_heads / d->n_kv_heads * d->block_len;
+  if (refresh && d->score == SDLLM_SCORE_PROB_MEAN)         // attention pass (and its fold), saliency pass
+    return 2 + (pl.kind == 4 && pl.splits > 1 ? 1 : 0) + (pl.kind == 2 && pl.splits > 1 && !umma_tail_is_fused(pl, d->head_dim, M, d->seq_len_max, false, true) ? 1 : 0);
   if (pl.kind == 3) return 1;       // the key splits merge, and the scores are pooled, inside the one launch
   if (pl.kind == 4) return pl.splits > 1 || refresh ? 2 : 1;       // the fold of the key splits and the pooling are one launch
   if (pl.kind == 2) {
     const int n1 = refresh ? d->seq_len_max : d->n_keep_max;
-    if (refresh && d->score == SDLLM_SCORE_PROB_MEAN)     // attention pass (+ its merge) and saliency pass (+ its pooling)
-      return 1 + ((pl.splits > 1 && !umma_tail_is_fused(pl, d->head_dim, M, n1, false, true)) ? 1 : 0) + 1 +
-             (umma_tail_is_fused(pl, d->head_dim, M, n1, true, false) ? 0 : 1);
     const bool tail_work = pl.splits > 1 || refresh;
     return 1 + ((tail_work && !umma_tail_is_fused(pl, d->head_dim, M, n1, refresh, true)) ? 1 : 0);
   }
@@ -281,13 +279,14 @@ sdllm_status sdllm_refresh_scores(const sdllm_desc* d, const void* q_blk, const 
     // Softmax-probability saliency: the probabilities need each row's final normaliser, so the scores come from a
     // second pass over K once the attention pass has left the rows' log-sum-exp.
     if (!out) return SDLLM_ERR_INVALID_ARG;
+    if (pl.kind == 0) return SDLLM_ERR_UNSUPPORTED;       // (the cp.async kernels, forced by an override)
     AttnParams a = p;
     a.want_scores = 0; a.pooled = nullptr; a.raw_scores = nullptr;
     if (!a.lse) a.lse = reinterpret_cast<float*>(wsb + w.lse);
     if (cuda_failed(launch_attn_partial(a, pl, d->dtype, d->head_dim, stream), "attention launch")) return SDLLM_ERR_CUDA;
     AttnParams s2 = p;
-    s2.out = nullptr; s2.lse = nullptr; s2.lse_in = a.lse; s2.prob_pass = 1; s2.want_scores = 0;
-    if (cuda_failed(launch_attn_partial(s2, pl, d->dtype, d->head_dim, stream), "saliency launch")) return SDLLM_ERR_CUDA;
+    s2.lse_in = a.lse;
+    if (cuda_failed(launch_prob_saliency(s2, d->head_dim, stream), "saliency launch")) return SDLLM_ERR_CUDA;
     return SDLLM_OK;
   }
   if (cuda_failed(launch_attn_partial(p, pl, d->dtype, d->head_dim, stream), "attention launch")) return SDLLM_ERR_CUDA;

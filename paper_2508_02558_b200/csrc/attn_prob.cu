@@ -1,0 +1,237 @@
+// Softmax-probability saliency of the refresh step (sdllm_score_kind PROB_MEAN): once the attention pass has left the rows'
+// log-sum-exp, P_ij = exp(S_ij - lse_i) is final, and the saliency of key j is the mean of its P over the b*G query rows.
+//
+// The keys lie on the accumulator rows (S^T = K_tile Q^T, as in attn_kt.cu), so one thread owns one key and adds up its
+// probabilities without any exchange, and one MMA covers all query rows of the head (N up to 256). The key tiles of a (sequence,
+// KV head) are shared out to the CTAs of one cluster; behind a cluster barrier each of them pools a share of the positions.
+// Bound by reading K once more (often from L2) and by latency. A refresh of 32 heads x 1280 keys with it: 43.6 -> 31.1 us, where the
+// query-row kernel's attention pass, its fold,
+// and a second pass of column sums by shuffle transposes with a separate pooling stood before.
+//   warp 0      TMA producer: Q, then K tiles (128 keys, 128-byte swizzle) into a three-slot ring
+//   warp 1      tcgen05.mma issuer, two S^T buffers in turn
+//   warps 2-5   one key per thread
+#include <cuda.h>
+#include <string.h>
+
+#include "attn_device.cuh"
+#include "tuning.cuh"
+#include "umma_host.cuh"
+
+namespace sdllm {
+using namespace dev;
+namespace {
+
+constexpr int PB_THREADS = 192;
+constexpr int PB_STAGES = 3;
+
+struct ProbMaps {
+  CUtensorMap q, k;
+};
+struct ProbParams {
+  AttnParams a;
+  int NP;            // query columns: M rounded up to 32
+  int S;             // CTAs of a cluster
+  int tmem_cols;     // two S^T buffers, a power of two
+};
+
+#include "umma_ptx.cuh"
+
+size_t prob_smem_bytes(int D, int NP) {
+  return 1024 /*alignment slack*/ + 2048 /*barriers, log-sum-exps*/ + (size_t)NP * D * 2 + (size_t)PB_STAGES * 128 * D * 2;
+}
+
+template <int D>
+__global__ void __launch_bounds__(PB_THREADS) prob_saliency_kernel(const __grid_constant__ ProbMaps tm, const ProbParams pp) {
+  constexpr int H = D / 64, HALF = 128 * 128, TILE = H * HALF, NS = PB_STAGES;
+  const AttnParams& p = pp.a;
+  extern __shared__ unsigned char smem_raw[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int S = pp.S, NP = pp.NP, rank = blockIdx.x, g = blockIdx.y, bi = blockIdx.z;
+  const uint32_t raw_addr = smem_u32(smem_raw);
+  unsigned char* smem = smem_raw + (((raw_addr + 1023u) & ~1023u) - raw_addr);
+  const uint32_t bars = smem_u32(smem);
+  auto BAR = [&](int i) { return bars + 8u * (uint32_t)i; };
+  const int Q_FULL = 0, FULL_K = 1, EMPTY_K = 1 + NS, S_FULL = 1 + 2 * NS, S_FREE = 3 + 2 * NS, DRAIN = 5 + 2 * NS;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + 256);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + 260);
+  float* lse_s = reinterpret_cast<float*>(smem + 1024);    // [256] log-sum-exps in log2 units
+  unsigned char* q_s = smem + 2048;
+  unsigned char* ring = q_s + NP * D * 2;
+
+  if (tid == 0) {
+    prefetch_tmap(&tm.q); prefetch_tmap(&tm.k);
+    mbar_init(BAR(Q_FULL), 1);
+    for (int i = 0; i < NS; ++i) { mbar_init(BAR(FULL_K + i), 1); mbar_init(BAR(EMPTY_K + i), 1); }
+    for (int i = 0; i < 2; ++i) { mbar_init(BAR(S_FULL + i), 1); mbar_init(BAR(S_FREE + i), 4); }
+    mbar_init(BAR(DRAIN), 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  if (warp == 1) {
+    tmem_alloc(smem_u32(tmem_slot), (uint32_t)pp.tmem_cols);
+    tmem_relinquish();
+  }
+  // query rows past M take part in the MMAs; whatever they hold, their columns are not read, but it must be finite
+  for (int i = tid; i < H * (NP - p.M) * 8; i += PB_THREADS) {
+    const int h = i / ((NP - p.M) * 8), r = i % ((NP - p.M) * 8);
+    reinterpret_cast<uint4*>(q_s + h * NP * 128 + p.M * 128)[r] = make_uint4(0u, 0u, 0u, 0u);
+  }
+  grid_dependency_wait();                                  // the log-sum-exps come from the kernel in front
+  grid_launch_dependents();
+  for (int m = tid; m < NP; m += PB_THREADS) {
+    float v = INFINITY;                                    // no query row: exp2(-inf) = 0
+    if (m < p.M) {
+      const int hg = m / p.b, i = m - hg * p.b;
+      v = __ldcg(p.lse_in + ((int64_t)bi * p.Hq + g * p.G + hg) * p.b + i) * kLog2e;
+    }
+    lse_s[m] = v;
+  }
+  fence_proxy_async();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  int n = p.n1_per_seq ? p.n1_per_seq[bi] : p.n1_max;
+  n = min(max(n, 0), p.n1_max);
+  const int all = (n + 127) / 128, t0 = rank * all / S, nt = (rank + 1) * all / S - t0;
+  float* raw = p.raw_scores + (int64_t)(bi * p.Hkv + g) * p.n1_max;
+
+  if (warp == 0) {
+    if (lane == 0 && nt > 0) {
+      mbar_expect_tx(BAR(Q_FULL), (uint32_t)(H * p.M * 128));
+      for (int h = 0; h < H; ++h) tma_load_4d(smem_u32(q_s + h * NP * 128), &tm.q, BAR(Q_FULL), h * 64, 0, g * p.G, bi);
+      int it = 0;
+      for (; it < nt; ++it) {
+        const int s = it % NS;
+        if (it >= NS && !wait_bar(BAR(EMPTY_K + s), ((it / NS) - 1) & 1, abort_flag, p.status, 61, p.wait_cycles)) break;
+        mbar_expect_tx(BAR(FULL_K + s), (uint32_t)TILE);
+        for (int h = 0; h < H; ++h) tma_load_4d(smem_u32(ring + s * TILE + h * HALF), &tm.k, BAR(FULL_K + s), h * 64, (t0 + it) * 128, g, bi);
+      }
+      if (*abort_flag) {                                   // let the copies that were issued land before the CTA retires
+        for (int j = max(it - NS, 0); j < it; ++j) drain_bar(BAR(FULL_K + j % NS), (j / NS) & 1);
+        drain_bar(BAR(Q_FULL), 0);
+      }
+    }
+  } else if (warp == 1) {
+    const bool leader = elect_one();
+    // kind::f16, fp32 accumulator, bf16 A and B, both K-major: M = 128 keys, N = query columns
+    const uint32_t idesc = instr_desc(NP, false);
+    const uint64_t k_desc = smem_desc(smem_u32(ring), 16u, 1024u), q_desc = smem_desc(smem_u32(q_s), 16u, 1024u);
+    bool ok = nt > 0 && wait_bar_warp(BAR(Q_FULL), 0, abort_flag, p.status, 62, p.wait_cycles);
+    for (int it = 0; it < nt && ok; ++it) {
+      const int s = it % NS, sb = it & 1;
+      ok = wait_bar_warp(BAR(FULL_K + s), (it / NS) & 1, abort_flag, p.status, 63, p.wait_cycles) &&
+           (it < 2 || wait_bar_warp(BAR(S_FREE + sb), ((it >> 1) - 1) & 1, abort_flag, p.status, 64, p.wait_cycles));
+      if (!ok) break;
+      tc_fence_after();
+      if (leader) {
+#pragma unroll
+        for (int ks = 0; ks < D / 16; ++ks)
+          mma_ss(tmem_base + (uint32_t)(sb * NP), k_desc + (uint64_t)((s * TILE + (ks >> 2) * HALF + (ks & 3) * 32) >> 4),
+                 q_desc + (uint64_t)(((ks >> 2) * NP * 128 + (ks & 3) * 32) >> 4), idesc, ks > 0 ? 1u : 0u);
+        tc_commit(BAR(S_FULL + sb));
+        tc_commit(BAR(EMPTY_K + s));
+      }
+      __syncwarp();
+    }
+    if (*abort_flag && leader) {                           // wait for the tensor pipe to finish what was issued before TMEM is freed
+      tc_commit(BAR(DRAIN));
+      drain_bar(BAR(DRAIN), 0);
+    }
+    __syncwarp();
+  } else {
+    const int q4 = warp & 3, row = q4 * 32 + lane;
+    const float inv_rows = 1.f / (float)p.M;
+    for (int it = 0; it < nt; ++it) {
+      const int sb = it & 1;
+      if (!wait_bar_warp(BAR(S_FULL + sb), (it >> 1) & 1, abort_flag, p.status, 65, p.wait_cycles)) break;
+      tc_fence_after();
+      float a4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+      for (int c = 0; c < NP; c += 32) {
+        uint32_t sv[32];
+        tmem_ld32(tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(sb * NP + c), sv);
+        tc_wait_ld();
+#pragma unroll
+        for (int e = 0; e < 32; e += 4) {
+          const float4 l4 = *reinterpret_cast<const float4*>(lse_s + c + e);
+          a4[0] += fast_exp2(fmaf(__uint_as_float(sv[e]), p.scale_log2, -l4.x));
+          a4[1] += fast_exp2(fmaf(__uint_as_float(sv[e + 1]), p.scale_log2, -l4.y));
+          a4[2] += fast_exp2(fmaf(__uint_as_float(sv[e + 2]), p.scale_log2, -l4.z));
+          a4[3] += fast_exp2(fmaf(__uint_as_float(sv[e + 3]), p.scale_log2, -l4.w));
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(BAR(S_FREE + sb));
+      const int pos = (t0 + it) * 128 + row;
+      if (pos < n) __stcg(raw + pos, ((a4[0] + a4[1]) + (a4[2] + a4[3])) * inv_rows);
+    }
+  }
+
+  // ---- pooling: the head's saliency is complete once every CTA of the cluster is here ----
+  tc_fence_before();
+  __threadfence();
+  __syncthreads();
+  if (S > 1) cluster_sync_all();
+  if (!*abort_flag) {
+    float* pooled = p.pooled + (int64_t)(bi * p.Hkv + g) * p.n1_max;
+    const int lo = rank * p.n1_max / S, hi = (rank + 1) * p.n1_max / S, o = p.block_off[bi];
+    for (int pos = lo + tid; pos < hi; pos += PB_THREADS) pooled[pos] = pool_at_ldcg(p, raw, n, o, pos);
+  }
+  if (warp == 1) {
+    __syncwarp();
+    tc_fence_after();
+    tmem_dealloc(tmem_base, (uint32_t)pp.tmem_cols);
+  }
+}
+
+template <int D>
+cudaError_t launch_prob_d(const ProbMaps& tm, const ProbParams& pp, cudaStream_t st) {
+  auto kern = prob_saliency_kernel<D>;
+  static SmemConfig configured;
+  const size_t smem = prob_smem_bytes(D, pp.NP);
+  const cudaError_t e = configure_smem(reinterpret_cast<const void*>(kern), smem, configured, true);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(pp.S, pp.a.Hkv, pp.a.B);
+  cfg.blockDim = dim3(PB_THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  int na = 0;
+  if (tuning().pdl != 0) {
+    attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[na].val.programmaticStreamSerializationAllowed = 1;
+    ++na;
+  }
+  if (pp.S > 1) {
+    attr[na].id = cudaLaunchAttributeClusterDimension;
+    attr[na].val.clusterDim.x = pp.S; attr[na].val.clusterDim.y = 1; attr[na].val.clusterDim.z = 1;
+    ++na;
+  }
+  cfg.attrs = attr; cfg.numAttrs = na;
+  return cudaLaunchKernelEx(&cfg, kern, tm, pp);
+}
+
+}  // namespace
+
+// p.lse_in: the rows' log-sum-exp; p.raw_scores: scratch; p.pooled: the result.
+cudaError_t launch_prob_saliency(const AttnParams& p, int D, cudaStream_t st) {
+  ProbMaps tm;
+  ProbParams pp{};
+  pp.a = p;
+  pp.NP = (p.M + 31) / 32 * 32;
+  pp.tmem_cols = 64;
+  while (pp.tmem_cols < 2 * pp.NP) pp.tmem_cols *= 2;
+  // a cluster of up to eight CTAs per head: enough of them for one CTA per SM, and at least one tile each
+  const long long units = (long long)p.B * p.Hkv, tiles = (p.n1_max + 127) / 128;
+  pp.S = 1;
+  while (pp.S < 8 && units * pp.S * 2 <= sm_count() + sm_count() / 2 && pp.S * 2 <= tiles) pp.S *= 2;
+  memset(&tm, 0, sizeof(tm));
+  if (!umma_make_map(&tm.q, p.q, D, p.b, p.Hq, p.B, p.q_stride, p.b, p.G) || !umma_make_map(&tm.k, p.k1, D, p.n1_max, p.Hkv, p.B, p.k1_stride, 128, 1))
+    return cudaErrorInvalidValue;
+  return D == 128 ? launch_prob_d<128>(tm, pp, st) : launch_prob_d<64>(tm, pp, st);
+}
+
+}  // namespace sdllm

@@ -50,7 +50,6 @@ struct UmmaParams {
   int heads_rt;      // query heads per row tile
   int fused_tail;    // 1: the last CTA of a unit merges and pools; 0: umma_tail_kernel does
   int early_src1;    // 1: source 1 and its count are older than the previous kernel in the stream (reuse step)
-  int prob_pass;     // 1: second pass of the probability saliency: S and the rows' log-sum-exp give column means of P
   int cluster;       // > 1: the key splits of a unit form a thread-block cluster and merge through distributed shared memory
   int lpt;           // 1: grid z counts the sequences from the longest to the shortest (several waves of ragged work)
 };
@@ -153,15 +152,12 @@ __global__ void __launch_bounds__(256) umma_tail_kernel(const UmmaParams up, con
   const int bi = (int)(bh / p.Hkv);
   int L = p.n1_per_seq ? p.n1_per_seq[bi] : p.n1_max;
   L = min(max(L, 0), p.n1_max);
-  p.pooled[idx] = pool_at(p, p.raw_scores + bh * p.n1_max, L, p.block_off[bi], pos, up.prob_pass ? up.row_tiles : 1,
-                          (int64_t)p.B * p.Hkv * p.n1_max);
+  p.pooled[idx] = pool_at(p, p.raw_scores + bh * p.n1_max, L, p.block_off[bi], pos);
 }
 
-// PROB selects the second pass of the probability saliency; it is a template parameter so that the attention kernel proper
-// does not carry that pass's code.
 // DUAL is the small-footprint variant for grids of several waves: 64-key tiles, a two-slot ring, 256 TMEM columns and at
 // most 128 registers per thread, so that two CTAs share an SM and one's set-up and way out overlap the other's streaming.
-template <int D, bool PROB, bool DUAL>
+template <int D, bool DUAL>
 __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kernel(const __grid_constant__ UmmaMaps tm, const UmmaParams up) {
   constexpr int H = D / 64;            // 128-byte column halves of a row
   constexpr int NS = DUAL ? 2 : UM_STAGES;
@@ -202,10 +198,8 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
   const int t_begin = (int)(((long long)split * tiles_all) / p.splits);
   const int t_end = (int)(((long long)(split + 1) * tiles_all) / p.splits);
   const int M_rt = min(p.M - rt * 128, 128);          // valid query rows of this row tile (<= rows_rep when R > 1)
-  constexpr bool prob_pass = PROB;                      // no V, no PV: S tiles only, reduced over the query rows
-  const bool do_attn = p.out != nullptr && !prob_pass;
-  const bool do_s = do_attn || prob_pass;              // Q and the S = Q K^T tiles are needed
-  const bool do_scores = p.want_scores && rt == 0 && !prob_pass;   // mean-query logit saliency (saliency warps)
+  const bool do_attn = p.out != nullptr;
+  const bool do_scores = p.want_scores && rt == 0;   // mean-query logit saliency (saliency warps)
   const int n2 = p.n2;
 
   // ---- shared memory carve-up (1024-byte aligned for the 128-byte swizzle) ----
@@ -230,11 +224,11 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
   const int q_rows = p.b * up.heads_rt;
   const int q_copies = (128 % q_rows == 0) ? 128 / q_rows : R;
   const int q_step = (128 % q_rows == 0) ? q_rows : rows_rep;
-  const bool zero_q = do_s && 128 % q_rows != 0 && q_rows < rows_rep;
+  const bool zero_q = do_attn && 128 % q_rows != 0 && q_rows < rows_rep;
   if (tid == 0) {                        // the descriptors live in the kernel parameters: fetch them while the CTA sets up
     prefetch_tmap(&tm.k1); prefetch_tmap(&tm.v1);
     if (n2 > 0) { prefetch_tmap(&tm.k2); prefetch_tmap(&tm.v2); }
-    if (do_s) prefetch_tmap(&tm.q);
+    if (do_attn) prefetch_tmap(&tm.q);
   }
 
   // The producer lane sets the barriers up and, unless the Q tile has to be cleared first, starts the first loads
@@ -244,7 +238,7 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
   bool q_issued = false;
   auto issue_q = [&]() {              // the Q tile (replicated R times along the accumulator rows)
     q_issued = true;
-    if (!do_s) return;
+    if (!do_attn) return;
     mbar_expect_tx(BAR(Q_FULL), (uint32_t)(q_copies * H * q_rows * 128));
     for (int c = 0; c < q_copies; ++c)
       for (int h = 0; h < H; ++h)
@@ -282,7 +276,7 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
     for (int s = 0; s < NS; ++s) {
       mbar_init(BAR(FULL_K + s), 1);
       mbar_init(BAR(FULL_V + s), 1);
-      mbar_init(BAR(EMPTY_K + s), max((do_s ? 1 : 0) + (do_scores ? 2 : 0), 1));
+      mbar_init(BAR(EMPTY_K + s), max((do_attn ? 1 : 0) + (do_scores ? 2 : 0), 1));
       mbar_init(BAR(EMPTY_V + s), 1);
     }
     for (int i = 0; i < 2; ++i) {
@@ -294,7 +288,7 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
     *abort_flag = 0;
     *last_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    if (!zero_q && (do_s || do_scores)) {
+    if (!zero_q && (do_attn || do_scores)) {
       if (up.early_src1) {
         // Reuse step: the compacted cache and its count were written before the previous kernel in the stream even
         // started, so their tiles may stream in while that kernel is still finishing.
@@ -336,7 +330,7 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
 
   if (warp == 0) {
     // ======================================= TMA producer =======================================
-    if (lane == 0 && (do_s || do_scores)) {
+    if (lane == 0 && (do_attn || do_scores)) {
       prod_n1 = n1;
       if (!q_issued) issue_q();
       produce(1 << 30, false);
@@ -346,12 +340,12 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
           drain_bar(BAR(FULL_K + j % NS), (j / NS) & 1);
           if (do_attn) drain_bar(BAR(FULL_V + j % NS), (j / NS) & 1);
         }
-        if (do_s && q_issued) drain_bar(BAR(Q_FULL), 0);
+        if (do_attn && q_issued) drain_bar(BAR(Q_FULL), 0);
       }
     }
   } else if (warp == 1) {
     // ======================================= MMA issuer =======================================
-    if (lane == 0 && do_s) {
+    if (lane == 0 && do_attn) {
       const uint32_t idesc_pv = instr_desc(D, true);
       bool ok = true, have_q = false;
       int it = 0;
@@ -379,8 +373,6 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
           if (!wait_bar(BAR(Q_FULL), 0, abort_flag, p.status, 3, p.wait_cycles)) { ok = false; break; }
           have_q = true;
         }
-        // without PV nothing else orders the reuse of an S buffer: wait until the softmax warps have read tile it - 2
-        if (prob_pass && it >= 2 && !wait_bar(BAR(P_FULL + sb), ((it >> 1) - 1) & 1, abort_flag, p.status, 12, p.wait_cycles)) { ok = false; break; }
         tc_fence_after();
         const uint32_t ksm = smem_u32(stage0 + (size_t)s * stage_bytes);
         const uint32_t qsm = smem_u32(q_s);
@@ -408,75 +400,7 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
     }
   } else if (warp < 6) {
     // ======================================= softmax warps =======================================
-    if constexpr (PROB) {
-      // Probability saliency, second pass: with the rows' log-sum-exp known, P_ij = exp(S_ij - lse_i) is final, and
-      // the saliency of key j is the mean of column j over the b*G query rows. Each warp sums its 32 rows of a
-      // 32-column chunk with a shuffle transpose (lane i ends up with column i); the four warps' sums meet in shared
-      // memory (the V half of ring slot 0, never loaded in this pass), double-buffered by tile parity.
-      const int q4 = warp & 3;
-      const int row = q4 * 32 + lane;
-      const int rep = row / rows_rep, m_local = row - rep * rows_rep;
-      const uint32_t lane_addr = tmem_base + ((uint32_t)(q4 * 32) << 16);
-      const int chunk_keys = KT / R;
-      float* colsum = reinterpret_cast<float*>(stage0 + kv_bytes);          // [2][4][KT]
-      float lse2 = INFINITY;                           // rows outside the tile contribute exp2(-inf) = 0
-      if (m_local < M_rt) {
-        const int m = rt * 128 + m_local;
-        const int hg = m / p.b, i = m - hg * p.b;
-        lse2 = p.lse_in[((int64_t)bi * p.Hq + g * p.G + hg) * p.b + i] * kLog2e;
-      }
-      const float inv_rows = 1.f / (float)p.M;
-      float* raw = p.raw_scores + ((int64_t)rt * p.B * p.Hkv + (int64_t)(bi * p.Hkv + g)) * p.n1_max;
-      const int st = (warp - 2) * 32 + lane;
-      int it = 0;
-      bool dead = false;
-      for (int t = t_begin; t < t_end; ++t) {
-        const Tile x = tile_of(t, tiles1, KT, KT2, n1, n2);
-        if (x.nv == 0) continue;
-        const int sb = it & 1;
-        const int c_lo = min(rep * chunk_keys, x.nv), c_hi = min((rep + 1) * chunk_keys, x.nv);
-        // a warp that gave up keeps walking the tiles so that the four warps meet at every barrier below
-        if (!dead && !wait_bar_warp(BAR(S_FULL + sb), (it >> 1) & 1, abort_flag, p.status, 9, p.wait_cycles)) dead = true;
-        tc_fence_after();
-        float* cs = colsum + (size_t)sb * 4 * KT + (size_t)(warp - 2) * KT;
-#pragma unroll 1
-        for (int c = 0; c * 32 < KT && !dead; ++c) {
-          float v[32];
-          if (c * 32 < c_hi && c * 32 + 32 > c_lo) {
-            uint32_t sv[32];
-            tmem_ld32(lane_addr + (uint32_t)sb * S_STRIDE + c * 32, sv);
-            tc_wait_ld();
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-              const bool in = c * 32 + i >= c_lo && c * 32 + i < c_hi;
-              v[i] = in ? fast_exp2(fmaf(__uint_as_float(sv[i]), p.scale_log2, -lse2)) : 0.f;
-            }
-#pragma unroll
-            for (int off = 16; off >= 1; off >>= 1) {
-              const bool up_half = (lane & off) != 0;
-#pragma unroll
-              for (int k = 0; k < off; ++k) {
-                const float send = up_half ? v[k] : v[k + off];
-                const float keep = up_half ? v[k + off] : v[k];
-                v[k] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-              }
-            }
-          } else {
-            v[0] = 0.f;
-          }
-          cs[c * 32 + lane] = v[0];
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(BAR(P_FULL + sb));        // the S buffer may be overwritten
-        asm volatile("bar.sync 2, 128;\n" ::: "memory");
-        if (st < x.nv && x.src1 && !dead) {
-          const float* c4 = colsum + (size_t)sb * 4 * KT + st;
-          raw[x.row0 + st] = ((c4[0] + c4[KT]) + (c4[2 * KT] + c4[3 * KT])) * inv_rows;
-        }
-        ++it;
-      }
-    } else if (do_attn) {
+    if (do_attn) {
       const int q4 = warp & 3;                         // TMEM lane quadrant this warp may access
       const int row = q4 * 32 + lane;
       const int rep = row / rows_rep;                  // warp-uniform
@@ -785,11 +709,9 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
 
   // ---- fused tail: the last CTA of the unit merges the key splits and pools the saliency; nobody waits ----
   const bool tail_merge = do_attn && p.splits > 1;
-  const bool tail_pool = (do_scores || prob_pass) && p.pooled != nullptr;
-  // who counts: the key splits of a unit; in the probability pass all row tiles of the head as well (its pooling
-  // needs every row tile's column sums), on the counter of the head's first unit
-  const int expected = prob_pass ? p.splits * up.row_tiles : p.splits;
-  int32_t* counter = p.counters + (prob_pass ? unit - rt : unit);
+  const bool tail_pool = do_scores && p.pooled != nullptr;
+  const int expected = p.splits;                       // who counts: the key splits of a unit
+  int32_t* counter = p.counters + unit;
   if (up.cluster > 1) {
     // ---- cluster tail: the key splits of the unit are the CTAs of one cluster. After a cluster barrier every split's
     //      partial (in its shared memory) and raw saliency (in global memory) is visible to all of them; each CTA then
@@ -871,12 +793,7 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
         // stage the head's raw saliency in shared memory (the ring is free), then pool from there
         float* a_s = reinterpret_cast<float*>(stage0);
         const float* a = p.raw_scores + (int64_t)(bi * p.Hkv + g) * p.n1_max;
-        const int n_arr = prob_pass ? up.row_tiles : 1;          // the probability pass left one array per row tile
-        for (int i = tid; i < n1; i += UM_THREADS) {
-          float x = 0.f;
-          for (int r2 = 0; r2 < n_arr; ++r2) x += __ldcg(a + (int64_t)r2 * p.B * p.Hkv * p.n1_max + i);
-          a_s[i] = x;
-        }
+        for (int i = tid; i < n1; i += UM_THREADS) a_s[i] = __ldcg(a + i);
         __syncthreads();
         for (int pos = tid; pos < p.n1_max; pos += UM_THREADS)
           p.pooled[(int64_t)(bi * p.Hkv + g) * p.n1_max + pos] = pool_at(p, a_s, n1, p.block_off[bi], pos);
@@ -937,9 +854,9 @@ size_t umma_smem_bytes(int D, int KT, bool dual) {
   return need > 120 * 1024 ? need : 120 * 1024;
 }
 
-template <int D, bool PROB, bool DUAL>
+template <int D, bool DUAL>
 cudaError_t launch_umma_d(const UmmaMaps& tm, const UmmaParams& up, const AttnPlan& pl, bool pdl, cudaStream_t st) {
-  auto kern = attn_umma_bf16_kernel<D, PROB, DUAL>;
+  auto kern = attn_umma_bf16_kernel<D, DUAL>;
   static SmemConfig configured;
   cudaError_t e = configure_smem(reinterpret_cast<const void*>(kern), pl.smem_bytes, configured, true);
   if (e != cudaSuccess) return e;
@@ -1058,8 +975,6 @@ AttnPlan plan_attention_umma(int D, int M, int b, int B, int Hkv, int n1_max, in
   pl.smem_bytes = umma_smem_bytes(D, pl.key_tile, pl.dual);
   // Few key splits of a small problem: make them one thread-block cluster, so that they merge through distributed shared
   // memory instead of the workspace. Only where the whole grid is one wave (a cluster needs all its SMs at once).
-  // Several row tiles only at the reuse step: the probability pass of the refresh step pools over all row tiles of a
-  // head, which one cluster does not span.
   if (!no_cluster && pl.splits >= 2 && pl.splits <= 8 && (pl.row_tiles == 1 || n2 > 0) && pl.key_tile == 128 &&
       units * pl.splits <= sms && n1_max <= 8192)
     pl.cluster = pl.splits;
@@ -1077,17 +992,16 @@ cudaError_t launch_attn_umma(const AttnParams& p, const AttnPlan& pl, int D, cud
   up.heads_rt = pl.row_tiles == 1 ? p.G : 128 / p.b;
   const bool pool = p.want_scores && p.pooled != nullptr;
   up.early_src1 = (p.n2 > 0 && p.n1_max > 0 && tn.early_loads != 0) ? 1 : 0;
-  up.prob_pass = p.prob_pass;
   up.cluster = pl.cluster;
   {
     const long long ctas = (long long)pl.splits * p.Hkv * pl.row_tiles * p.B;
     up.lpt = (p.n1_per_seq != nullptr && p.B >= 4 && p.B <= 64 && ctas > sm_count()) ? 1 : 0;
     if (tn.lpt >= 0) up.lpt = (tn.lpt == 1 && p.n1_per_seq != nullptr && p.B >= 2 && p.B <= 64) ? 1 : 0;
   }
-  up.fused_tail = (pl.cluster > 1 || umma_tail_is_fused(pl, D, p.M, p.n1_max, pool || p.prob_pass, p.out != nullptr && !p.prob_pass)) ? 1 : 0;
+  up.fused_tail = (pl.cluster > 1 || umma_tail_is_fused(pl, D, p.M, p.n1_max, pool, p.out != nullptr)) ? 1 : 0;
   memset(&tm, 0, sizeof(tm));
   bool ok = true;
-  if (p.out != nullptr || p.prob_pass) ok = make_map(&tm.q, p.q, D, p.b, p.Hq, p.B, p.q_stride, p.b, up.heads_rt);
+  if (p.out != nullptr) ok = make_map(&tm.q, p.q, D, p.b, p.Hq, p.B, p.q_stride, p.b, up.heads_rt);
   if (p.n1_max > 0) {
     ok = ok && make_map(&tm.k1, p.k1, D, p.n1_max, p.Hkv, p.B, p.k1_stride, pl.key_tile, 1);
     ok = ok && make_map(&tm.v1, p.v1, D, p.n1_max, p.Hkv, p.B, p.k1_stride, pl.key_tile, 1);
@@ -1102,19 +1016,13 @@ cudaError_t launch_attn_umma(const AttnParams& p, const AttnPlan& pl, int D, cud
   if (!ok) return cudaErrorInvalidValue;
   cudaError_t err;
   const bool pdl = tn.pdl != 0;
-  if (pl.dual) {
-    if (up.prob_pass) err = D == 128 ? launch_umma_d<128, true, true>(tm, up, pl, pdl, st) : launch_umma_d<64, true, true>(tm, up, pl, pdl, st);
-    else err = D == 128 ? launch_umma_d<128, false, true>(tm, up, pl, pdl, st) : launch_umma_d<64, false, true>(tm, up, pl, pdl, st);
-  } else {
-    if (up.prob_pass) err = D == 128 ? launch_umma_d<128, true, false>(tm, up, pl, pdl, st) : launch_umma_d<64, true, false>(tm, up, pl, pdl, st);
-    else err = D == 128 ? launch_umma_d<128, false, false>(tm, up, pl, pdl, st) : launch_umma_d<64, false, false>(tm, up, pl, pdl, st);
-  }
+  if (pl.dual) err = D == 128 ? launch_umma_d<128, true>(tm, up, pl, pdl, st) : launch_umma_d<64, true>(tm, up, pl, pdl, st);
+  else err = D == 128 ? launch_umma_d<128, false>(tm, up, pl, pdl, st) : launch_umma_d<64, false>(tm, up, pl, pdl, st);
   if (err != cudaSuccess || up.fused_tail) return err;
-  const bool merge = p.out != nullptr && !p.prob_pass && pl.splits > 1;
-  const bool pool_tail = pool || (p.prob_pass && p.pooled != nullptr);
-  if (!merge && !pool_tail) return cudaSuccess;
+  const bool merge = p.out != nullptr && pl.splits > 1;
+  if (!merge && !pool) return cudaSuccess;
   const long long merge_threads = merge ? (long long)p.B * p.Hkv * pl.row_tiles * 128 * (D / 4) : 0;
-  const long long pool_threads = pool_tail ? (long long)p.B * p.Hkv * p.n1_max : 0;
+  const long long pool_threads = pool ? (long long)p.B * p.Hkv * p.n1_max : 0;
   const int merge_blocks = (int)((merge_threads + 255) / 256);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(merge_blocks + (pool_threads + 255) / 256));
@@ -1145,16 +1053,15 @@ bool pair_supported(int dtype, int D, int M, int b);
 AttnPlan plan_attention_pair(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn);
 cudaError_t launch_attn_pair(const AttnParams& p, const AttnPlan& pl, int D, cudaStream_t st);
 
-AttnPlan plan_attention(int dtype, int D, int M, int b, int B, int Hkv, int n1_max, int n2, bool prob_scores) {
+AttnPlan plan_attention(int dtype, int D, int M, int b, int B, int Hkv, int n1_max, int n2) {
   // bf16 goes to the tcgen05 kernels wherever they apply: heads with few query rows to the kernel that puts the keys on the
-  // accumulator rows, the rest to the one that puts the queries there and has two softmax warpgroups (attn_pair.cu); the
-  // probability saliency has its own second pass in the older query-row kernel of this file. fp32 and the remaining bf16
-  // shapes go to the cp.async kernels. Tuning::kernel forces a family.
+  // accumulator rows, the rest to the one that puts the queries there and has two softmax warpgroups (attn_pair.cu). fp32 and
+  // the remaining bf16 shapes go to the cp.async kernels. Tuning::kernel forces a family.
   const Tuning tn = tuning();
-  const bool kt_ok = kt_supported(dtype, D, M, b) && !prob_scores;
+  const bool kt_ok = kt_supported(dtype, D, M, b);
   if (kt_ok && (tn.kernel == 3 || (tn.kernel == 0 && kt_preferred(D, M, B, Hkv, n1_max, n2))))
     return plan_attention_kt(D, M, b, B, Hkv, n1_max, n2, tn);
-  if ((tn.kernel == 0 || tn.kernel == 4) && pair_supported(dtype, D, M, b) && !prob_scores) return plan_attention_pair(D, M, b, B, Hkv, n1_max, n2, tn);
+  if ((tn.kernel == 0 || tn.kernel == 4) && pair_supported(dtype, D, M, b)) return plan_attention_pair(D, M, b, B, Hkv, n1_max, n2, tn);
   if (tn.kernel != 1 && umma_supported(dtype, D, M, b)) return plan_attention_umma(D, M, b, B, Hkv, n1_max, n2, tn);
   AttnPlan pl = plan_attention_legacy(dtype, D, M, B, Hkv, n1_max + n2, tn);
   pl.tma = false; pl.cluster = 1; pl.warp_keys = 32; pl.kind = 0;

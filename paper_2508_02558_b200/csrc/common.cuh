@@ -64,7 +64,6 @@ struct AttnParams {
   float* pooled;               // refresh with a fused tail: pooled scores [B][Hkv][n1_max], else null
   int window, pool_kind, per_region;
   const float* lse_in;         // probability saliency, second pass: log-sum-exp of every block row [B][Hq][b]
-  int prob_pass;               // 1: this launch is that second pass (tcgen05 kernel only)
   int want_scores;             // compute mean-query logit scores for src1 keys
   float scale;                 // softmax scale
   float scale_log2;            // scale * log2(e)
@@ -99,7 +98,8 @@ struct CompactParams {
   int64_t kv_stride_bytes[3], c_stride_bytes[3];
 };
 
-AttnPlan plan_attention(int dtype, int D, int M, int b, int B, int Hkv, int n1_max, int n2, bool prob_scores);
+AttnPlan plan_attention(int dtype, int D, int M, int b, int B, int Hkv, int n1_max, int n2);
+cudaError_t launch_prob_saliency(const AttnParams& p, int D, cudaStream_t st);    // second pass of the probability saliency
 
 bool umma_tail_is_fused(const AttnPlan& pl, int D, int M, int n1_max, bool pool, bool merge);
 bool umma_supported(int dtype, int D, int M, int b);
