@@ -94,7 +94,15 @@ __device__ __forceinline__ void compute_qbar(const AttnParams& p, const CtaRange
     float acc = 0.f;
     for (int hg = 0; hg < p.G; ++hg) {
       const T* qh = reinterpret_cast<const T*>(p.q) + (int64_t)r.bi * p.q_stride[0] + (int64_t)(r.g * p.G + hg) * p.q_stride[1];
-      for (int i = 0; i < p.b; ++i) acc += to_f32<T>(qh[(int64_t)i * p.q_stride[2] + d]);
+      int i = 0;
+      for (; i + 16 <= p.b; i += 16) {                    // sixteen loads in flight, added up in row order
+        T x[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) x[u] = qh[(int64_t)(i + u) * p.q_stride[2] + d];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) acc += to_f32<T>(x[u]);
+      }
+      for (; i < p.b; ++i) acc += to_f32<T>(qh[(int64_t)i * p.q_stride[2] + d]);
     }
     qbar_s[d] = acc / (float)p.M;
   }

@@ -88,3 +88,10 @@ def test_block_lengths_that_fill_no_tile(b, Hq, Hkv, D, tuning):
         tuning(**plan)
         _run_sequence_case(cfg, seed=23, block=1)
         B.tuning_reset()
+
+
+@pytest.mark.parametrize("H,D,p,gen", [(2, 64, 20, 32), (2, 64, 1000, 64), (3, 128, 300, 32), (40, 64, 300, 32), (1, 128, 2000, 32)])
+def test_fp32_key_tiles(H, D, p, gen):
+    """16, 32 and 64 keys per tile, ragged last tiles, more splits than a fold batch holds."""
+    from test_gpu_parity import _run_sequence_case, _small
+    _run_sequence_case(_small("f32_tiles", "f32", H, H, D, p, gen, salient_frac=0.02), seed=3, block=0)
