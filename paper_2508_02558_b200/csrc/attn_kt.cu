@@ -267,58 +267,70 @@ __global__ void __launch_bounds__(64 + 128 * WG * CG, (WG == 1 && CG == 1) ? 2 :
     }
   } else if (warp == 1) {
     // ======================================= MMA issuer =======================================
-    if (lane == 0) {
+    // The whole warp walks the tiles and one elected lane issues: with everything around the MMAs warp-uniform, their
+    // descriptors live in uniform registers (a loop run by one lane alone takes about 75 cycles per MMA, several times what
+    // these narrow ones execute).
+    {
+      const bool leader = elect_one();
       const uint32_t idesc_s = kt_idesc(NPT, false, false);
       const uint32_t idesc_pv = kt_idesc(NPT, true, true);
       const uint32_t qsm = smem_u32(q_s);
-      bool ok = wait_bar(BAR(Q_FULL), 0, abort_flag, p.status, 3, wlim);
+      bool ok = wait_bar_warp(BAR(Q_FULL), 0, abort_flag, p.status, 3, wlim);
       const uint32_t ring_a = smem_u32(ring), p_a = smem_u32(p_s);
       const bool two_p = kp.PB == 2;
       auto issue_pv = [&](int j, int s, uint32_t par) -> bool {       // tile j lives in ring slot s, in its use of parity par
         const int pb = j & 1;
         const int ng = min(GPT, ge - (gb + GPT * j));
-        if (!wait_bar(BAR(P_FULL + pb), (j >> 1) & 1, abort_flag, p.status, 4, wlim)) return false;
-        if (!wait_bar(BAR(FULL_V + s), par, abort_flag, p.status, 5, wlim)) return false;
+        if (!wait_bar_warp(BAR(P_FULL + pb), (j >> 1) & 1, abort_flag, p.status, 4, wlim)) return false;
+        if (!wait_bar_warp(BAR(FULL_V + s), par, abort_flag, p.status, 5, wlim)) return false;
         tc_fence_after();
         const uint32_t vsm = ring_a + (uint32_t)s * SLOT + KV_BYTES;
         const uint32_t psm = p_a + ((two_p && pb) ? (uint32_t)PBUF : 0u);
         // O^T += V^T P^T, 16 keys per instruction. A: the V tile read MN-major (the head dimension runs along M; its two
         // 64-element halves lie HALF bytes apart; with D = 64 both halves alias the same data and rows 64..127 of O^T
         // are duplicates nobody reads). B: P^T, MN-major, 8 keys per swizzle atom; its 64-column halves lie 16 KB apart.
-        for (int ks = 0; ks < 2 * ng; ++ks)
-          mma_ss(tmem_base + O_COL + (uint32_t)(j % WG) * NPT, smem_desc(vsm + ks * 2048, H == 2 ? (uint32_t)HALF : 0u, 1024u),
-                 CG > 1 ? smem_desc(psm + ks * 2048, 128u * 128u, 1024u) : smem_desc_sw64(psm + ks * 1024, (uint32_t)PBUF, 512u),
-                 idesc_pv, (j >= WG || ks > 0) ? 1u : 0u);
-        tc_commit(BAR(PV_DONE + pb));    // two alternating barriers: a waiter is never a whole phase ahead of either
-        tc_commit(BAR(EMPTY_V + s));
+        const uint64_t vd = smem_desc(vsm, H == 2 ? (uint32_t)HALF : 0u, 1024u);
+        const uint64_t pd = CG > 1 ? smem_desc(psm, 128u * 128u, 1024u) : smem_desc_sw64(psm, (uint32_t)PBUF, 512u);
+        if (leader) {
+#pragma unroll
+          for (int ks = 0; ks < 2 * GPT; ++ks)
+            if (ks < 2 * ng)
+              mma_ss(tmem_base + O_COL + (uint32_t)(j % WG) * NPT, vd + ks * (2048 >> 4), pd + ks * ((CG > 1 ? 2048 : 1024) >> 4), idesc_pv,
+                     (j >= WG || ks > 0) ? 1u : 0u);
+          tc_commit(BAR(PV_DONE + pb));    // two alternating barriers: a waiter is never a whole phase ahead of either
+          tc_commit(BAR(EMPTY_V + s));
+        }
+        __syncwarp();
         return true;
       };
       int s = 0, s_prev = 0;               // ring slot of tile t and of tile t - 1, and the parities of their uses
       uint32_t par = 0, par_prev = 0;
       for (int t = 0; t < T && ok; ++t) {
         const int sb = t & 1;
-        if (!wait_bar(BAR(FULL_K + s), par, abort_flag, p.status, 7, wlim)) { ok = false; break; }
+        if (!wait_bar_warp(BAR(FULL_K + s), par, abort_flag, p.status, 7, wlim)) { ok = false; break; }
         tc_fence_after();
         const uint32_t ksm = ring_a + (uint32_t)s * SLOT;
         const uint32_t d_t = tmem_base + (uint32_t)sb * NPT;
         // S^T = K_tile Q^T: the S^T buffer of tile t - 2 is free, its softmax arrived before PV(t - 2) was issued
+        const uint64_t kd = smem_desc(ksm, 16u, 1024u), qd = smem_desc(qsm, 16u, 1024u);
+        if (leader) {
 #pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) {
-          const uint32_t hk = (ks >> 2) * HALF + (ks & 3) * 32;
-          const uint32_t hq = (ks >> 2) * (NPT * 128) + (ks & 3) * 32;
-          mma_ss(d_t, smem_desc(ksm + hk, 16u, 1024u), smem_desc(qsm + hq, 16u, 1024u), idesc_s, ks > 0 ? 1u : 0u);
+          for (int ks = 0; ks < D / 16; ++ks)
+            mma_ss(d_t, kd + (((ks >> 2) * HALF + (ks & 3) * 32) >> 4), qd + (((ks >> 2) * (NPT * 128) + (ks & 3) * 32) >> 4), idesc_s, ks > 0 ? 1u : 0u);
+          tc_commit(BAR(S_FULL + sb));
+          tc_commit(BAR(EMPTY_K + s));
         }
-        tc_commit(BAR(S_FULL + sb));
-        tc_commit(BAR(EMPTY_K + s));
+        __syncwarp();
         if (t > 0 && !issue_pv(t - 1, s_prev, par_prev)) { ok = false; break; }
         s_prev = s; par_prev = par;
         if (++s == NS) { s = 0; par ^= 1u; }
       }
       if (ok && T > 0) ok = issue_pv(T - 1, s_prev, par_prev);
-      if (*abort_flag) {                 // wait for the tensor pipe to finish what was issued before TMEM is freed
+      if (*abort_flag && leader) {       // wait for the tensor pipe to finish what was issued before TMEM is freed
         tc_commit(BAR(DRAIN));
         drain_bar(BAR(DRAIN), 0);
       }
+      __syncwarp();
     }
   } else {
     // ======================================= softmax warps =======================================

@@ -260,7 +260,9 @@ __global__ void __launch_bounds__(KS_THREADS, 1) attn_kt_stream_kernel(const __g
     }
   } else if (warp == 1) {
     // ======================================= MMA issuer =======================================
-    if (lane == 0) {
+    // warp-uniform, one elected lane issues (see attn_kt.cu)
+    {
+      const bool leader = elect_one();
       const uint32_t idesc_s = kt_idesc(NP, false, false);
       const uint32_t idesc_pv = kt_idesc(NP, true, true);
       const uint32_t qsm = smem_u32(q_s), ring_a = smem_u32(ring), p_a = smem_u32(p_s);
@@ -270,53 +272,60 @@ __global__ void __launch_bounds__(KS_THREADS, 1) attn_kt_stream_kernel(const __g
       int pv_G = -1, pv_ng = 0; bool pv_first = false;
       auto issue_pv = [&]() -> bool {
         const int j = pv_G, pb = j & 1, s = j % NS;
-        if (!wait_bar(BAR(P_FULL + pb), (uint32_t)(j >> 1) & 1u, abort_flag, p.status, 4, wlim)) return false;
-        if (!wait_bar(BAR(FULL_V + s), (uint32_t)(j / NS) & 1u, abort_flag, p.status, 5, wlim)) return false;
+        if (!wait_bar_warp(BAR(P_FULL + pb), (uint32_t)(j >> 1) & 1u, abort_flag, p.status, 4, wlim)) return false;
+        if (!wait_bar_warp(BAR(FULL_V + s), (uint32_t)(j / NS) & 1u, abort_flag, p.status, 5, wlim)) return false;
         tc_fence_after();
         const uint32_t vsm = ring_a + (uint32_t)s * SLOT + KV_BYTES;
         const uint32_t psm = p_a + (pb ? (uint32_t)PBUF : 0u);
         // O^T_w += V^T P^T, 16 keys per instruction. A: the V tile read MN-major (its two 64-element halves lie HALF bytes
         // apart; with D = 64 both halves alias the same data and rows 64..127 of O^T are duplicates nobody reads).
         // B: P^T, MN-major, 64-byte rows, 8 keys per swizzle atom.
-        for (int ks = 0; ks < 2 * pv_ng; ++ks)
-          mma_ss(tmem_base + O_COL + (uint32_t)pb * NP, smem_desc(vsm + ks * 2048, H == 2 ? (uint32_t)HALF : 0u, 1024u),
-                 smem_desc_sw64(psm + ks * 1024, (uint32_t)PBUF, 512u), idesc_pv, (!pv_first || ks > 0) ? 1u : 0u);
-        tc_commit(BAR(PV_DONE + pb));
-        tc_commit(BAR(EMPTY_V + s));
+        const uint64_t vd = smem_desc(vsm, H == 2 ? (uint32_t)HALF : 0u, 1024u), pd = smem_desc_sw64(psm, (uint32_t)PBUF, 512u);
+        if (leader) {
+#pragma unroll
+          for (int ks = 0; ks < 2 * GPT; ++ks)
+            if (ks < 2 * pv_ng)
+              mma_ss(tmem_base + O_COL + (uint32_t)pb * NP, vd + ks * (2048 >> 4), pd + ks * (1024 >> 4), idesc_pv, (!pv_first || ks > 0) ? 1u : 0u);
+          tc_commit(BAR(PV_DONE + pb));
+          tc_commit(BAR(EMPTY_V + s));
+        }
+        __syncwarp();
         return true;
       };
       for (int k = 0; ok; ++k) {
-        const int u = unit_at(k);
+        const int u = __shfl_sync(0xffffffffu, unit_at(k), 0);      // (one lane's answer for all)
         if (u < 0) break;
         const Unit x = unit_of(u);
         if (x.T == 0) continue;
-        if (!wait_bar(BAR(Q_FULL), (uint32_t)qn & 1u, abort_flag, p.status, 3, wlim)) { ok = false; break; }
+        if (!wait_bar_warp(BAR(Q_FULL), (uint32_t)qn & 1u, abort_flag, p.status, 3, wlim)) { ok = false; break; }
         ++qn;
         for (int t = 0; t < x.T && ok; ++t, ++G) {
           const int s = G % NS, sb = G & 1;
-          if (!wait_bar(BAR(FULL_K + s), (uint32_t)(G / NS) & 1u, abort_flag, p.status, 7, wlim)) { ok = false; break; }
+          if (!wait_bar_warp(BAR(FULL_K + s), (uint32_t)(G / NS) & 1u, abort_flag, p.status, 7, wlim)) { ok = false; break; }
           tc_fence_after();
           const uint32_t ksm = ring_a + (uint32_t)s * SLOT;
           const uint32_t d_t = tmem_base + (uint32_t)sb * NP;
           // S^T = K_tile Q^T: the S^T buffer of tile G - 2 is free, its softmax arrived before PV(G - 2) was issued
+          const uint64_t kd = smem_desc(ksm, 16u, 1024u), qd = smem_desc(qsm, 16u, 1024u);
+          if (leader) {
 #pragma unroll
-          for (int ks = 0; ks < D / 16; ++ks) {
-            const uint32_t hk = (ks >> 2) * HALF + (ks & 3) * 32;
-            const uint32_t hq = (ks >> 2) * (NP * 128) + (ks & 3) * 32;
-            mma_ss(d_t, smem_desc(ksm + hk, 16u, 1024u), smem_desc(qsm + hq, 16u, 1024u), idesc_s, ks > 0 ? 1u : 0u);
+            for (int ks = 0; ks < D / 16; ++ks)
+              mma_ss(d_t, kd + (((ks >> 2) * HALF + (ks & 3) * 32) >> 4), qd + (((ks >> 2) * (NP * 128) + (ks & 3) * 32) >> 4), idesc_s, ks > 0 ? 1u : 0u);
+            tc_commit(BAR(S_FULL + sb));
+            tc_commit(BAR(EMPTY_K + s));
+            if (t == x.T - 1) tc_commit(BAR(Q_EMPTY));   // the unit's last use of Q
           }
-          tc_commit(BAR(S_FULL + sb));
-          tc_commit(BAR(EMPTY_K + s));
-          if (t == x.T - 1) tc_commit(BAR(Q_EMPTY));   // the unit's last use of Q
+          __syncwarp();
           if (pv_G >= 0 && !issue_pv()) { ok = false; break; }
           pv_G = G; pv_ng = min(GPT, x.ge - GPT * t); pv_first = t < 2;
         }
       }
       if (ok && pv_G >= 0) ok = issue_pv();
-      if (*abort_flag) {                 // wait for the tensor pipe to finish what was issued before TMEM is freed
+      if (*abort_flag && leader) {       // wait for the tensor pipe to finish what was issued before TMEM is freed
         tc_commit(BAR(DRAIN));
         drain_bar(BAR(DRAIN), 0);
       }
+      __syncwarp();
     }
   } else {
     // ======================================= softmax warps =======================================

@@ -23,6 +23,14 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
       : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
 }
+// ... without the suspension that try_wait may take while the phase is open
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+  return ok != 0;
+}
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int x, int y, int z, int w) {
   asm volatile(
       "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];\n"
@@ -212,6 +220,14 @@ __device__ __forceinline__ Tile tile_of(int t, int tiles1, int KT, int KT2, int 
 // one expired).
 __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status, int code,
                                          long long limit) {
+#ifdef SDLLM_ZERO_LIMIT_NEVER_WAITS
+  if (limit == 0) {                                      // try_wait alone may outlast every short wait of a small problem
+    if (mbar_test_wait(bar, parity)) return true;
+    *abort_flag = 1;
+    atomicExch(status, code);
+    return false;
+  }
+#endif
   if (mbar_try_wait(bar, parity)) return true;
   const long long t0 = clock64();
   for (;;) {
