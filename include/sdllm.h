@@ -201,8 +201,9 @@ sdllm_status sdllm_sparse_block_attn(const sdllm_desc* desc, const void* q_blk, 
  * seq_len NULL means every sequence has seq_len_max rows. desc->block_len, retention and the selection fields are
  * not used. bf16 only, D in {64, 128}, at most 65535 query heads; anything else returns
  * SDLLM_ERR_UNSUPPORTED. The probability matrix is never written to memory. Workspace:
- * sdllm_workspace_bytes(desc, SDLLM_OP_DENSE_ATTN) bytes (the status word), zeroed once by the caller; a workspace of
- * the other attention calls serves as well. */
+ * sdllm_workspace_bytes(desc, SDLLM_OP_DENSE_ATTN) bytes (the status word, and rows of units whose keys are shared out between
+ * CTAs), zeroed once by the caller; a smaller one, down to 256 bytes, works too, without that sharing, and so does a workspace
+ * of the other attention calls. */
 sdllm_status sdllm_dense_attn(const sdllm_desc* desc, const void* q, const int64_t* q_stride, const void* k, const void* v,
                               const int32_t* seq_len, void* out, const int64_t* o_stride, float* lse, void* workspace,
                               size_t workspace_bytes, void* cuda_stream);

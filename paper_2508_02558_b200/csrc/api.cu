@@ -121,8 +121,8 @@ void fill_common(AttnParams& p, const sdllm_desc* d, const AttnPlan& pl) {
 }
 
 // Full-sequence attention runs on its own tcgen05 kernel: bf16, D in {64, 128}, one grid row per query head.
-// Its workspace is the status word alone.
-constexpr size_t kDenseWorkspaceBytes = 256;
+// Of its workspace the status block is required; the partial rows behind it let the call share out its last units.
+constexpr size_t kDenseStatusBytes = 256;
 bool dense_supported(const sdllm_desc* d) {
   return umma_supported(d->dtype, d->head_dim, 128, 128) && d->n_q_heads <= 65535;
 }
@@ -176,7 +176,7 @@ size_t sdllm_workspace_bytes(const sdllm_desc* d, int op) {
   if (check_desc(d) != SDLLM_OK) return 0;
   if (op == SDLLM_OP_REFRESH_SCORES) return attn_ws(d, plan_for(d, op), true).total;
   if (op == SDLLM_OP_SPARSE_BLOCK_ATTN) return attn_ws(d, plan_for(d, op), false).total;
-  if (op == SDLLM_OP_DENSE_ATTN && dense_supported(d)) return kDenseWorkspaceBytes;
+  if (op == SDLLM_OP_DENSE_ATTN && dense_supported(d)) return dense_workspace_bytes(d->batch, d->n_q_heads, d->seq_len_max, d->head_dim);
   return 0;
 }
 
@@ -215,7 +215,7 @@ int32_t sdllm_launch_count(const sdllm_desc* d, int op) {
   if (op == SDLLM_OP_COMPACT_KV) return d->n_keep_max > 0 ? 1 : 0;
   if (op == SDLLM_OP_SELECT_COMPACT)
     return select_compact_is_fused(d->batch, d->n_kv_heads, d->seq_len_max, d->block_len, d->n_keep_max) ? 1 : 1 + (d->n_keep_max > 0 ? 1 : 0);
-  if (op == SDLLM_OP_DENSE_ATTN) return dense_supported(d) ? 1 : -1;
+  if (op == SDLLM_OP_DENSE_ATTN) return dense_supported(d) ? dense_launches(d->batch, d->n_q_heads, d->seq_len_max) : -1;
   if (op != SDLLM_OP_REFRESH_SCORES && op != SDLLM_OP_SPARSE_BLOCK_ATTN) return -1;
   const bool refresh = op == SDLLM_OP_REFRESH_SCORES;
   const AttnPlan pl = plan_for(d, op);
@@ -406,11 +406,11 @@ sdllm_status sdllm_dense_attn(const sdllm_desc* d, const void* q, const int64_t*
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(out) || !aligned16(lse)) return SDLLM_ERR_INVALID_ARG;
   if (!strides_ok(q_stride, elem_size(d->dtype)) || !strides_ok(o_stride, elem_size(d->dtype))) return SDLLM_ERR_INVALID_ARG;
   if (!dense_supported(d)) return SDLLM_ERR_UNSUPPORTED;
-  if (ws == nullptr || ws_bytes < kDenseWorkspaceBytes || (reinterpret_cast<uintptr_t>(ws) & 255u)) return SDLLM_ERR_WORKSPACE;
+  if (ws == nullptr || ws_bytes < kDenseStatusBytes || (reinterpret_cast<uintptr_t>(ws) & 255u)) return SDLLM_ERR_WORKSPACE;
   if ((st = check_device()) != SDLLM_OK) return st;
-  if (cuda_failed(launch_dense_pair(q, q_stride, k, v, d->kv_stride, seq_len, out, o_stride, lse, reinterpret_cast<int32_t*>(ws),
-                                    d->batch, d->n_q_heads, d->n_kv_heads, d->seq_len_max, d->head_dim, scale_of(d),
-                                    reinterpret_cast<cudaStream_t>(cuda_stream)), "dense attention launch"))
+  const DenseCall c{q, k, v, q_stride, d->kv_stride, o_stride, seq_len, out, lse, ws, ws_bytes,
+                    d->batch, d->n_q_heads, d->n_kv_heads, d->seq_len_max, d->head_dim, scale_of(d)};
+  if (cuda_failed(launch_dense(c, reinterpret_cast<cudaStream_t>(cuda_stream)), "dense attention launch"))
     return SDLLM_ERR_CUDA;
   return SDLLM_OK;
 }

@@ -45,7 +45,12 @@ struct DenseParams {
   void* out;                // [B, Hq, L, D] bf16 with o_stride
   float* lse;               // [B, Hq, L], nullable
   int32_t* status;          // device status word
+  float* part_o;            // rows of the cut units: [unit][part][D / 4][256] float4
+  float* part_ml;           // [unit][part][256] (maximum, sum)
   int B, Hq, G, L;
+  int pairs;                // units of a head at full length
+  int unit0, parts;         // units in front of the cut ones; CTAs that share the key tiles of a cut unit
+  int second;               // 1: the launch in front is the first part of the same call (see launch_dense)
   float scale_log2;         // softmax scale * log2(e)
   int64_t o_stride[3];
   long long wait_cycles;    // limit of every abortable mbarrier wait
@@ -53,7 +58,8 @@ struct DenseParams {
 
 #include "umma_ptx.cuh"
 
-template <int D>
+// CUT: the CTA takes a share of a unit's key tiles (a variant of its own: the plain one has no register to spare for it).
+template <int D, bool CUT>
 __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __grid_constant__ DenseMaps tm, const DenseParams p) {
   extern __shared__ unsigned char smem_raw[];
   constexpr int H = D / 64;                 // 64-column halves of a row (128 bytes each: one swizzle atom wide)
@@ -63,16 +69,25 @@ __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __
   constexpr int TILE = H * HALF;            // bytes of a Q, K or V tile
   constexpr uint32_t S_COL0 = 0, O_COL0 = 256, T_STRIDE = 128;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int bi = blockIdx.z, h = blockIdx.y, g = h / p.G, jp = blockIdx.x;
+  // (the plain variant takes its place from the grid as it is: values that the compiler knows to be warp-uniform, sequence length
+  // and loop bounds included, stay in uniform registers; from a linear index it ran 2.5 % slower)
+  const int part = CUT ? blockIdx.x % (unsigned)p.parts : 0, unit = CUT ? p.unit0 + (int)(blockIdx.x / (unsigned)p.parts) : 0;
+  const int jp = CUT ? unit % p.pairs : blockIdx.x, h = CUT ? (unit / p.pairs) % p.Hq : blockIdx.y, g = h / p.G;
+  const int bi = CUT ? unit / (p.pairs * p.Hq) : blockIdx.z;
 
-  grid_dependency_wait();                   // everything this kernel reads may come from the kernel in front of it
+  if (!CUT && (bi * p.Hq + h) * p.pairs + jp >= p.unit0) return;          // one of the units that are cut
+  if (!CUT || !p.second) grid_dependency_wait();    // everything this kernel reads may come from the kernel in front of it
   grid_launch_dependents();
   int n = p.seq_len ? p.seq_len[bi] : p.L;
   n = min(max(n, 0), p.L);
   const int row00 = 2 * jp * 128;           // first row of query tile 0; query tile 1 starts 128 rows further
-  if (row00 >= n) return;                   // both query tiles lie past the sequence's end (whole CTA, before any set-up)
+  if (row00 >= n) {                         // both query tiles lie past the sequence's end (whole CTA, before any set-up)
+    if (CUT && p.second) grid_dependency_wait();
+    return;
+  }
   const bool act1 = row00 + 128 < n;
-  const int nt = (n + KT - 1) / KT;         // key tiles
+  const int nt_all = (n + KT - 1) / KT;     // key tiles of the unit; this CTA takes [t0, t0 + nt)
+  const int t0 = CUT ? part * nt_all / p.parts : 0, nt = CUT ? (part + 1) * nt_all / p.parts - t0 : nt_all;
 
   const uint32_t raw_addr = smem_u32(smem_raw);
   unsigned char* smem = smem_raw + (((raw_addr + 1023u) & ~1023u) - raw_addr);
@@ -112,14 +127,14 @@ __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  auto tile_nv = [&](int j) { return min(n - j * KT, KT); };     // valid keys of tile j (> 0 for j < nt)
+  auto tile_nv = [&](int j) { return min(n - (t0 + j) * KT, KT); };     // valid keys of this CTA's tile j (> 0 for j < nt)
 
   // Registers move from the first warpgroup to the softmax warps: 128 * (72 + 2 * 208) of the 384 * 168 at launch.
   if (warp < 4) {
     regs_dec_72();
     if (warp == 0) {
       // ======================================= TMA producer =======================================
-      if (lane == 0) {
+      if (lane == 0 && (!CUT || nt > 0)) {
         mbar_expect_tx(BAR(Q_FULL), (uint32_t)((act1 ? 2 : 1) * TILE));
         for (int t = 0; t < (act1 ? 2 : 1); ++t)
           for (int hh = 0; hh < H; ++hh)
@@ -132,13 +147,13 @@ __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __
           const uint32_t kdst = smem_u32(stage0 + (size_t)s * 2 * TILE), vdst = kdst + TILE;
           if (j >= NS && !wait_bar(BAR(EMPTY_K + s), ph, abort_flag, p.status, 21, p.wait_cycles)) { ok = false; break; }
           mbar_expect_tx(BAR(FULL_K + s), (uint32_t)TILE);
-          for (int hh = 0; hh < H; ++hh) tma_load_4d(kdst + hh * HALF, &tm.k, BAR(FULL_K + s), hh * 64, j * KT, g, bi);
+          for (int hh = 0; hh < H; ++hh) tma_load_4d(kdst + hh * HALF, &tm.k, BAR(FULL_K + s), hh * 64, (t0 + j) * KT, g, bi);
           if (j >= NS && !wait_bar(BAR(EMPTY_V + s), ph, abort_flag, p.status, 22, p.wait_cycles)) {
             drain_bar(BAR(FULL_K + s), (j / NS) & 1);                 // the K half of this slot is already on its way
             ok = false; break;
           }
           mbar_expect_tx(BAR(FULL_V + s), (uint32_t)TILE);
-          for (int hh = 0; hh < H; ++hh) tma_load_4d(vdst + hh * HALF, &tm.v, BAR(FULL_V + s), hh * 64, j * KT, g, bi);
+          for (int hh = 0; hh < H; ++hh) tma_load_4d(vdst + hh * HALF, &tm.v, BAR(FULL_V + s), hh * 64, (t0 + j) * KT, g, bi);
           issued = j + 1;
         }
         if (*abort_flag) {                    // let the copies that were issued land before the CTA retires
@@ -158,7 +173,7 @@ __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __
       const uint32_t idesc_pv = instr_desc(D, true);
       const uint64_t q_desc = smem_desc(smem_u32(q_s), 16u, 1024u), k_desc = smem_desc(smem_u32(stage0), 16u, 1024u);
       const uint64_t v_desc = smem_desc(smem_u32(stage0) + TILE, (uint32_t)HALF, 1024u);
-      bool ok = wait_bar_warp(BAR(Q_FULL), 0, abort_flag, p.status, 23, p.wait_cycles);
+      bool ok = (!CUT || nt > 0) && wait_bar_warp(BAR(Q_FULL), 0, abort_flag, p.status, 23, p.wait_cycles);
       // S_t = Q_t K_j^T into the S region of query tile t
       auto issue_s = [&](int t, int j) {
         const uint32_t idesc_s = instr_desc((tile_nv(j) + 15) & ~15, false);
@@ -325,10 +340,28 @@ __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __
         }
       }
       // ---- the finished row: TMEM -> registers -> normalise -> bf16 -> global memory ----
-      if (ok) ok = wait_bar_warp(BAR(PV_DONE + t), (nt - 1) & 1, abort_flag, p.status, 30, p.wait_cycles);
+      if (ok) ok = (!CUT || nt > 0) && wait_bar_warp(BAR(PV_DONE + t), (nt - 1) & 1, abort_flag, p.status, 30, p.wait_cycles);
       tc_fence_after();
       const int r_glob = row00 + t * 128 + row;
-      if (ok) {
+      if constexpr (CUT) {
+        // A share of a unit: un-normalised rows and their (maximum, sum) go to the workspace, float4 columns apart so that the
+        // lanes of a warp write in a row; dense_fold_kernel folds them.
+        const int64_t slot = blockIdx.x;
+        float4* po = reinterpret_cast<float4*>(p.part_o) + slot * (D / 4) * 256 + t * 128 + row;
+        if (ok) {
+#pragma unroll 1
+          for (int c = 0; c < D / 16; ++c) {
+            uint32_t ov[16];
+            tmem_ld16(o_addr + c * 16, ov);
+            tc_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              __stcg(po + (c * 4 + i) * 256, make_float4(__uint_as_float(ov[4 * i]), __uint_as_float(ov[4 * i + 1]), __uint_as_float(ov[4 * i + 2]),
+                                                         __uint_as_float(ov[4 * i + 3])));
+          }
+        }
+        __stcg(reinterpret_cast<float2*>(p.part_ml) + slot * 256 + t * 128 + row, make_float2(m_run, ok ? l_run : 0.f));
+      } else if (ok) {
         const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
         __nv_bfloat16* orow = reinterpret_cast<__nv_bfloat16*>(p.out) + (int64_t)bi * p.o_stride[0] + (int64_t)h * p.o_stride[1] +
                               (int64_t)r_glob * p.o_stride[2];
@@ -355,6 +388,7 @@ __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __
   }
 
   // ---- teardown ----
+  if (CUT && p.second) grid_dependency_wait();      // this launch must not be over before the one in front of it is
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
@@ -369,49 +403,149 @@ size_t dense_smem_bytes(int D) {
   return 1024 /*alignment slack*/ + 1024 /*barriers*/ + 2 * tile + (size_t)DN_STAGES * 2 * tile;
 }
 
+// Fold of the shares of the cut units: one thread per query row and float4 column, lanes along the rows.
 template <int D>
-cudaError_t launch_dense_d(const DenseMaps& tm, const DenseParams& p, int nqb, cudaStream_t st) {
-  auto kern = dense_attn_bf16_kernel<D>;
-  static SmemConfig configured;
-  const size_t smem = dense_smem_bytes(D);
-  const cudaError_t ce = configure_smem(reinterpret_cast<const void*>(kern), smem, configured, true);
-  if (ce != cudaSuccess) return ce;
+__global__ void __launch_bounds__(256) dense_fold_kernel(const DenseParams p) {
+  constexpr int C4 = D / 4, MB = 8;
+  const int c4 = blockIdx.x % C4, cut = blockIdx.x / C4, row = threadIdx.x;
+  const int unit = p.unit0 + cut, jp = unit % p.pairs, h = (unit / p.pairs) % p.Hq;
+  const int bi = unit / (p.pairs * p.Hq);
+  grid_dependency_wait();
+  grid_launch_dependents();
+  int n = p.seq_len ? p.seq_len[bi] : p.L;
+  n = min(max(n, 0), p.L);
+  const int r = jp * 256 + row;
+  if (r >= n) return;
+  const float4* po = reinterpret_cast<const float4*>(p.part_o) + ((int64_t)cut * p.parts * C4 + c4) * 256 + row;
+  const float2* pm = reinterpret_cast<const float2*>(p.part_ml) + (int64_t)cut * p.parts * 256 + row;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  float m = -INFINITY, l = 0.f;
+  for (int s0 = 0; s0 < p.parts; s0 += MB) {
+    float2 x[MB];
+    float4 v[MB];
+#pragma unroll
+    for (int u = 0; u < MB; ++u) {
+      const int s = min(s0 + u, p.parts - 1);
+      x[u] = __ldcg(pm + s * 256);
+      v[u] = __ldcg(po + (int64_t)s * C4 * 256);
+    }
+    float bm = m;
+#pragma unroll
+    for (int u = 0; u < MB; ++u)
+      if (s0 + u < p.parts && x[u].y > 0.f) bm = fmaxf(bm, x[u].x);
+    const float a = bm == -INFINITY ? 1.f : fast_exp2(m - bm);           // 0 on the first batch with data
+    acc.x *= a; acc.y *= a; acc.z *= a; acc.w *= a; l *= a;
+    m = bm;
+#pragma unroll
+    for (int u = 0; u < MB; ++u) {
+      if (s0 + u >= p.parts || !(x[u].y > 0.f)) continue;
+      const float w = fast_exp2(x[u].x - bm);
+      l = fmaf(x[u].y, w, l);
+      acc.x = fmaf(v[u].x, w, acc.x); acc.y = fmaf(v[u].y, w, acc.y); acc.z = fmaf(v[u].z, w, acc.z); acc.w = fmaf(v[u].w, w, acc.w);
+    }
+  }
+  const float inv = l > 0.f ? 1.f / l : 0.f;
+  __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(p.out) + (int64_t)bi * p.o_stride[0] + (int64_t)h * p.o_stride[1] + (int64_t)r * p.o_stride[2] + c4 * 4;
+  *reinterpret_cast<uint2*>(out) = make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
+  if (c4 == 0 && p.lse) p.lse[((int64_t)bi * p.Hq + h) * p.L + r] = (m + log2f(l)) * kLn2;
+}
+
+// How the units (a sequence's head and pair of query tiles) of a call are launched: the first `whole` of them one CTA each, the
+// rest - what the last full wave leaves over, or all of less than a wave - with their key tiles shared out to `parts` CTAs. A
+// unit takes a whole SM, so without that 160 units on 148 SMs run in two waves (32 heads x 1280 rows: 46.2 us, 42.8 so; 28 heads
+// x 4096: 245 us, 200; 16 heads x 3000: 106, 81). Costs in us: a key tile 1.55, a CTA's set-up and way out 6.5, of which a cut unit overlaps 2 with the
+// wave in front, its partial rows and the launch that folds
+// them 9 (3 of it a margin).
+// Batches of several sequences may be ragged, which the host cannot see: they are cut only where all units fit one wave.
+struct DensePlan {
+  int whole, parts;
+};
+DensePlan plan_dense(int B, int Hq, int L) {
+  const int sms = sm_count(), nt = (L + 127) / 128, pairs = (nt + 1) / 2;
+  const long long units = (long long)B * Hq * pairs, rest = units % sms;
+  DensePlan pl{(int)units, 1};
+  if (rest == 0 || (B > 1 && rest != units)) return pl;
+  double least = 6.5 + 1.55 * nt;
+  for (int q = 2; q <= 16 && q <= nt && rest * q <= sms; ++q) {
+    const double cost = (rest == units ? 6.5 : 4.5) + 1.55 * ((nt + q - 1) / q) + 9.;
+    if (cost < least) { least = cost; pl.whole = (int)(units - rest); pl.parts = q; }
+  }
+  return pl;
+}
+constexpr size_t DN_STATUS_BYTES = 256;
+size_t partial_bytes(long long cut, int parts, int D) { return (size_t)cut * parts * 256 * (D + 2) * 4; }
+
+cudaError_t launch_overlapped(const void* kern, void** args, dim3 grid, int threads, size_t smem, cudaStream_t st) {
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((nqb + 1) / 2, p.Hq, p.B);
-  cfg.blockDim = dim3(DN_THREADS);
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
-  int na = 0;
-  if (tuning().pdl != 0) {
-    attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[na].val.programmaticStreamSerializationAllowed = 1;
-    ++na;
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = tuning().pdl != 0 ? 1 : 0;
+  return cudaLaunchKernelExC(&cfg, kern, args);
+}
+
+template <int D>
+cudaError_t launch_dense_d(const DenseMaps& tm, DenseParams p, const DensePlan& pl, int units, cudaStream_t st) {
+  const void *kern = reinterpret_cast<const void*>(dense_attn_bf16_kernel<D, false>), *cut_kern = reinterpret_cast<const void*>(dense_attn_bf16_kernel<D, true>);
+  static SmemConfig configured, cut_configured;
+  const size_t smem = dense_smem_bytes(D);
+  cudaError_t e = configure_smem(kern, smem, configured, true);
+  if (e == cudaSuccess) e = configure_smem(cut_kern, smem, cut_configured, true);
+  if (e != cudaSuccess) return e;
+  void* args[2] = {const_cast<DenseMaps*>(&tm), &p};
+  p.parts = pl.parts; p.unit0 = pl.whole; p.second = 0;
+  if (pl.whole > 0) {
+    e = launch_overlapped(kern, args, dim3(p.pairs, p.Hq, p.B), DN_THREADS, smem, st);
+    if (e != cudaSuccess || pl.whole == units) return e;
+    // The second launch need not wait for the first (it depends on what that one depends on, and every CTA of the first has seen
+    // that complete before it lets the next launch start), so its CTAs take the SMs that the last wave leaves idle; each waits
+    // for the first launch at its own end, so that nothing behind them starts before both are done.
+    p.second = tuning().pdl != 0 ? 1 : 0;
   }
-  cfg.attrs = attr; cfg.numAttrs = na;
-  return cudaLaunchKernelEx(&cfg, kern, tm, p);
+  e = launch_overlapped(cut_kern, args, dim3((unsigned)((units - pl.whole) * pl.parts)), DN_THREADS, smem, st);
+  if (e != cudaSuccess) return e;
+  void* fold_args[1] = {&p};
+  return launch_overlapped(reinterpret_cast<const void*>(dense_fold_kernel<D>), fold_args, dim3((unsigned)((units - pl.whole) * (D / 4))), 256, 0, st);
 }
 
 }  // namespace
 
-cudaError_t launch_dense_pair(const void* q, const int64_t* q_stride, const void* k, const void* v, const int64_t* kv_stride,
-                              const int32_t* seq_len, void* out, const int64_t* o_stride, float* lse, int32_t* status, int B, int Hq,
-                              int Hkv, int L, int D, float scale, cudaStream_t st) {
-  if (Hq > 65535 || B > 65535) return cudaErrorInvalidValue;
+int dense_launches(int B, int Hq, int L) {
+  const DensePlan pl = plan_dense(B, Hq, L);
+  return pl.parts == 1 ? 1 : (pl.whole > 0 ? 3 : 2);
+}
+
+size_t dense_workspace_bytes(int B, int Hq, int L, int D) {
+  const DensePlan pl = plan_dense(B, Hq, L);
+  const long long units = (long long)B * Hq * ((L + 255) / 256);
+  return DN_STATUS_BYTES + (pl.parts > 1 ? partial_bytes(units - pl.whole, pl.parts, D) : 0);
+}
+
+cudaError_t launch_dense(const DenseCall& c, cudaStream_t st) {
+  const int pairs = (c.L + 255) / 256;
+  const long long units = (long long)c.B * c.Hq * pairs;
+  if (c.Hq > 65535 || c.B > 65535 || units > 0x7fffffffLL / 16) return cudaErrorInvalidValue;
   DenseMaps tm;
   memset(&tm, 0, sizeof(tm));
-  bool ok = umma_make_map(&tm.q, q, D, L, Hq, B, q_stride, 128, 1);
-  ok = ok && umma_make_map(&tm.k, k, D, L, Hkv, B, kv_stride, 128, 1);
-  ok = ok && umma_make_map(&tm.v, v, D, L, Hkv, B, kv_stride, 128, 1);
+  bool ok = umma_make_map(&tm.q, c.q, c.D, c.L, c.Hq, c.B, c.q_stride, 128, 1);
+  ok = ok && umma_make_map(&tm.k, c.k, c.D, c.L, c.Hkv, c.B, c.kv_stride, 128, 1);
+  ok = ok && umma_make_map(&tm.v, c.v, c.D, c.L, c.Hkv, c.B, c.kv_stride, 128, 1);
   if (!ok) return cudaErrorInvalidValue;
+  DensePlan pl = plan_dense(c.B, c.Hq, c.L);
+  if (c.workspace_bytes < dense_workspace_bytes(c.B, c.Hq, c.L, c.D)) pl = {(int)units, 1};
   DenseParams p{};
-  p.seq_len = seq_len; p.out = out; p.lse = lse; p.status = status;
-  p.B = B; p.Hq = Hq; p.G = Hq / Hkv; p.L = L;
-  p.scale_log2 = scale * kLog2e;
+  p.seq_len = c.seq_len; p.out = c.out; p.lse = c.lse; p.status = reinterpret_cast<int32_t*>(c.workspace);
+  p.part_o = reinterpret_cast<float*>(reinterpret_cast<char*>(c.workspace) + DN_STATUS_BYTES);
+  p.part_ml = p.part_o + (size_t)(units - pl.whole) * pl.parts * 256 * c.D;
+  p.B = c.B; p.Hq = c.Hq; p.G = c.Hq / c.Hkv; p.L = c.L; p.pairs = pairs;
+  p.scale_log2 = c.scale * kLog2e;
   p.wait_cycles = tuning().wait_cycles;
-  for (int i = 0; i < 3; ++i) p.o_stride[i] = o_stride[i];
-  const int nqb = (L + 127) / 128;
-  return D == 128 ? launch_dense_d<128>(tm, p, nqb, st) : launch_dense_d<64>(tm, p, nqb, st);
+  for (int i = 0; i < 3; ++i) p.o_stride[i] = c.o_stride[i];
+  return c.D == 128 ? launch_dense_d<128>(tm, p, pl, (int)units, st) : launch_dense_d<64>(tm, p, pl, (int)units, st);
 }
 
 }  // namespace sdllm

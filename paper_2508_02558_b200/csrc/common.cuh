@@ -103,10 +103,19 @@ cudaError_t launch_prob_saliency(const AttnParams& p, int D, cudaStream_t st);  
 
 bool umma_tail_is_fused(const AttnPlan& pl, int D, int M, int n1_max, bool pool, bool merge);
 bool umma_supported(int dtype, int D, int M, int b);
-// Full-sequence attention, two query tiles per CTA (attn_dense.cu).
-cudaError_t launch_dense_pair(const void* q, const int64_t* q_stride, const void* k, const void* v, const int64_t* kv_stride,
-                              const int32_t* seq_len, void* out, const int64_t* o_stride, float* lse, int32_t* status, int B, int Hq,
-                              int Hkv, int L, int D, float scale, cudaStream_t st);
+// Full-sequence attention (attn_dense.cu).
+struct DenseCall {
+  const void *q, *k, *v;
+  const int64_t *q_stride, *kv_stride, *o_stride;
+  const int32_t* seq_len;
+  void* out; float* lse;
+  void* workspace; size_t workspace_bytes;
+  int B, Hq, Hkv, L, D;
+  float scale;
+};
+cudaError_t launch_dense(const DenseCall& c, cudaStream_t st);
+int dense_launches(int B, int Hq, int L);             // kernel launches of one call
+size_t dense_workspace_bytes(int B, int Hq, int L, int D);
 cudaError_t launch_attn_partial(const AttnParams& p, const AttnPlan& plan, int dtype, int D, cudaStream_t st);
 cudaError_t launch_merge_pool(const MergeParams& p, cudaStream_t st);
 cudaError_t launch_select_topk(const SelectParams& p, cudaStream_t st);

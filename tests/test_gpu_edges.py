@@ -95,3 +95,18 @@ def test_fp32_key_tiles(H, D, p, gen):
     """16, 32 and 64 keys per tile, ragged last tiles, more splits than a fold batch holds."""
     from test_gpu_parity import _run_sequence_case, _small
     _run_sequence_case(_small("f32_tiles", "f32", H, H, D, p, gen, salient_frac=0.02), seed=3, block=0)
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,lens", [
+    (2, 1, 128, [1100]), (2, 2, 64, [1100]),            # less than a wave of units: all of them cut along the keys
+    (3, 3, 128, [1500, 700, 0, 17]), (2, 1, 64, [2000, 1999, 129, 128]),       # ragged: shares without a key tile
+    (32, 8, 128, [1030]), (32, 4, 64, [1030]),          # a whole wave of units, then the cut ones
+    (10, 5, 64, [600, 300, 900, 40, 1000, 17] * 4),     # several waves of a ragged batch, longest first
+])
+def test_dense_step_schedule(Hq, Hkv, D, lens):
+    import parity_util as U
+    from test_gpu_parity import _dense_case
+    q, k, v = _dense_case(Hq, Hkv, D, lens, seed=33)
+    out, lse = U.gpu_dense(q, k, v, lens)
+    kw = {} if Hq < 10 else dict(rows=[0, 1, 127, 128, 255, 256, 1000, 1029] if len(lens) == 1 else [0, 16], heads=[0, 1, Hkv - 1])
+    U.check_dense_against_oracle(out, lse, np.nan_to_num(q), np.nan_to_num(k), np.nan_to_num(v), lens, **kw)
