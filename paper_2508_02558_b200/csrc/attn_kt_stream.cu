@@ -35,6 +35,7 @@ namespace {
 constexpr int KS_NS = 3;                 // ring slots
 constexpr int KS_THREADS = 64 + 2 * 128;
 constexpr int KS_CTRL = KT_CTRL0 + 2 * KT_GRP;
+constexpr int KS_RAW = 6;                // tiles whose saliency is kept: five are in use at a time (two being written, three being pooled)
 
 // asymmetric named barriers between the two softmax warpgroups (256 threads): one side only announces, the other waits
 __device__ __forceinline__ void pair_arrive(int id) { asm volatile("bar.arrive %0, 256;\n" ::"r"(id) : "memory"); }
@@ -66,7 +67,7 @@ __global__ void __launch_bounds__(KS_THREADS, 1) attn_kt_stream_kernel(const __g
   const uint32_t bars = smem_u32(smem);
   auto BAR = [&](int i) { return bars + 8u * (uint32_t)i; };
   constexpr int Q_FULL = 0, Q_EMPTY = 1, FULL_K = 2, FULL_V = 2 + NS, EMPTY_K = 2 + 2 * NS, EMPTY_V = 2 + 3 * NS;
-  constexpr int S_FULL = 2 + 4 * NS, P_FULL = S_FULL + 2, PV_DONE = S_FULL + 4, DRAIN = S_FULL + 6;
+  constexpr int S_FULL = 2 + 4 * NS, P_FULL = S_FULL + 2, PV_DONE = S_FULL + 4, DRAIN = S_FULL + 6, RAW_DONE = S_FULL + 7;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + 256);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + 260);
   volatile int* unit_list = reinterpret_cast<volatile int*>(smem + 320);   // [16] the units this CTA took, in order (-1: no more)
@@ -87,6 +88,7 @@ __global__ void __launch_bounds__(KS_THREADS, 1) attn_kt_stream_kernel(const __g
   unsigned char* q_s = smem + KS_CTRL;                              // [H][32 rows][128 B]
   unsigned char* p_s = q_s + H * NP * 128;                          // [2][P^T buffer]
   unsigned char* ring = p_s + 2 * PBUF;                             // [NS][K tile | V tile]
+  float* raw_s = reinterpret_cast<float*>(ring + NS * SLOT);        // [KS_RAW][128] saliency of the CTA's last tiles
 
   if (tid == 0) {
     prefetch_tmap(&tm.k1t); prefetch_tmap(&tm.v1t); prefetch_tmap(&tm.k1); prefetch_tmap(&tm.v1);
@@ -104,6 +106,7 @@ __global__ void __launch_bounds__(KS_THREADS, 1) attn_kt_stream_kernel(const __g
       mbar_init(BAR(S_FULL + i), 1);
       mbar_init(BAR(P_FULL + i), 4);
       mbar_init(BAR(PV_DONE + i), 1);
+      mbar_init(BAR(RAW_DONE + i), 4);
     }
     mbar_init(BAR(DRAIN), 1);
     *abort_flag = 0;
@@ -348,12 +351,40 @@ __global__ void __launch_bounds__(KS_THREADS, 1) attn_kt_stream_kernel(const __g
     bool dead = false;
     bool owe_sync = false;                             // warpgroup 1: warpgroup 0 has not yet confirmed the previous unit
     int Gbase = 0;                                     // tiles of the units walked so far
+    // Refresh step: the saliency is pooled while the walk goes on. A tile's positions are complete once the next tile's saliency
+    // is there (a window and the block it jumps over reach no further), so the warpgroup of tile t pools tile t - 2 from the last
+    // tiles' values in shared memory, and the one of a unit's last tile the two that remain. (Pooled at the end of a unit, from
+    // global memory and with both warpgroups standing still, it took 20 of 142 us on 16 ragged sequences x 32 heads; 11 of those are gone.)
+    const int half_w = (p.window - 1) / 2;
+    const bool lagged = scores && half_w + p.b <= 128;
     for (int k = 0;; ++k) {                            // units walked so far
       const int u = __shfl_sync(0xffffffffu, unit_at(k), 0);       // (one answer per warp; all warps read the same list)
       if (u < 0) break;
       const Unit x = unit_of(u);
       const int bi = x.bi, g = x.g;
       float l_lane = 0.f;                              // sum over this warp's key rows of column `lane`
+      const int o_blk = lagged ? min(max(p.block_off[bi], 0), max(x.n1 - p.b, 0)) : 0;
+      float* pooled = p.pooled + (int64_t)(bi * p.Hkv + g) * p.n1_max;
+      auto pool_tile = [&](int t) {                    // this thread's position of tile t
+        const int pos = t * 128 + row, b = p.b;
+        if (pos >= x.n1) return;
+        float v = -INFINITY;                           // the block's own positions
+        if (pos < o_blk || pos >= o_blk + b) {
+          const int C = x.n1 - b, c = pos < o_blk ? pos : pos - b;
+          int lo = 0, hi = C;
+          if (p.per_region) { if (c < o_blk) hi = o_blk; else lo = o_blk; }
+          lo = max(lo, c - half_w); hi = min(hi, c + half_w + 1);
+          float mx = -INFINITY, sum = 0.f;
+          for (int q = lo; q < hi; ++q) {
+            const int rp = q < o_blk ? q : q + b;
+            const float r = raw_s[((Gbase + (rp >> 7)) % KS_RAW) * 128 + (rp & 127)];
+            mx = fmaxf(mx, r);
+            sum += r;
+          }
+          v = p.pool_kind == SDLLM_POOL_MAX ? mx : sum / (float)p.window;
+        }
+        pooled[pos] = v;
+      };
       const int t0 = ((Gbase & 1) == w) ? 0 : 1;       // this warpgroup's first tile of the unit
       int G_last = -1;
       for (int t = t0; t < x.T; t += 2) {
@@ -383,7 +414,8 @@ __global__ void __launch_bounds__(KS_THREADS, 1) attn_kt_stream_kernel(const __g
           for (int c = 0; c < NP; ++c)
             if (c < n_mine) a4[c & 3] += sv[c];
           const float a = (a4[0] + a4[1]) + (a4[2] + a4[3]);
-          if (work && valid && gr.src1)
+          if (lagged) raw_s[(G % KS_RAW) * 128 + row] = a * (p.scale / (float)N);
+          else if (work && valid && gr.src1)
             p.raw_scores[(int64_t)(bi * p.Hkv + g) * p.n1_max + gr.row0 + lane] = a * (p.scale / (float)N);
         }
         // ---- the references: the first key of the warpgroup's first tile of the unit lends its logits ----
@@ -499,11 +531,25 @@ __global__ void __launch_bounds__(KS_THREADS, 1) attn_kt_stream_kernel(const __g
           }
           l_lane += sv[0];
         }
+        if (lagged) {
+          // (the wait in front of the arrive keeps the two warpgroups within one phase of each other)
+          if (G >= 1 && !dead && !wait_bar_warp(BAR(RAW_DONE + (1 - w)), (uint32_t)((G - 1) >> 1) & 1u, abort_flag, p.status, 15, wlim)) dead = true;
+          if (t >= 2 && !dead) pool_tile(t - 2);
+          __syncwarp();
+          if (lane == 0) mbar_arrive(BAR(RAW_DONE + w));
+        }
       }
 
       // ======================================= end of the unit =======================================
       // ---- refresh step: pooling of the head's saliency, once both warpgroups' raw values are in L2 ----
-      if (scores) {
+      if (lagged) {
+        if (x.T == 0 ? w == 0 : ((Gbase + x.T - 1) & 1) == w) {
+          softmax_barrier(bar_id);                     // the last tile's saliency, of all four warps
+          if (x.T >= 2 && !dead) pool_tile(x.T - 2);
+          if (x.T >= 1 && !dead) pool_tile(x.T - 1);
+          for (int pos = x.n1 + row; pos < p.n1_max; pos += 128) pooled[pos] = -INFINITY;       // padding
+        }
+      } else if (scores) {
         __threadfence_block();                         // writers and readers of the unit's raw saliency are this CTA's threads
         asm volatile("bar.sync 5, 256;\n" ::: "memory");
         if (p.pooled != nullptr && !*abort_flag) {
@@ -639,7 +685,7 @@ cudaError_t launch_kt_stream_d(const KtMaps& tm, const KtParams& kp, size_t smem
 
 size_t kt_stream_smem_bytes(int D) {
   const size_t H = D / 64;
-  return 1024 /*alignment slack*/ + KS_CTRL + H * 32 * 128 + 2 * 128 * 64 + (size_t)KS_NS * 2 * H * 128 * 128;
+  return 1024 /*alignment slack*/ + KS_CTRL + H * 32 * 128 + 2 * 128 * 64 + (size_t)KS_NS * 2 * H * 128 * 128 + KS_RAW * 128 * 4;
 }
 
 cudaError_t launch_kt_stream(const KtMaps& tm, const KtParams& kp, int D, size_t smem_bytes, bool pdl, cudaStream_t st) {

@@ -110,3 +110,21 @@ def test_dense_step_schedule(Hq, Hkv, D, lens):
     out, lse = U.gpu_dense(q, k, v, lens)
     kw = {} if Hq < 10 else dict(rows=[0, 1, 127, 128, 255, 256, 1000, 1029] if len(lens) == 1 else [0, 16], heads=[0, 1, Hkv - 1])
     U.check_dense_against_oracle(out, lse, np.nan_to_num(q), np.nan_to_num(k), np.nan_to_num(v), lens, **kw)
+
+
+@pytest.mark.parametrize("lens,window,policy", [
+    ([900, 300, 64, 1300, 33, 129, 128], 9, {}), ([640, 257, 256], 1, dict(select=B.SELECT_PER_REGION_CEIL)),
+    ([513, 384, 96, 160], 31, dict(pool=B.POOL_AVG)), ([700, 300], 301, {}),     # the last one: a window wider than the kept tiles
+])
+@pytest.mark.parametrize("ctas", [1, 2, 3])
+def test_pooling_while_the_resident_walk_goes_on(lens, window, policy, ctas, tuning):
+    import parity_util as U
+    from paper_2508_02558_b200 import workloads as W
+    tuning(splits=1, persist=ctas)
+    bw = W.make_batch(_wide("lagged", 3, 3, 128, 100, 32), [n - 32 for n in lens], seed=9)
+    for off in (0, 17):                                   # the block at the end of a sequence and in front of it
+        bo = np.maximum(np.asarray(bw.block_off) - off, 0).astype(np.int32)
+        q, k, v = bw.refresh_inputs(1, pad_value=np.nan)
+        g = U.gpu_refresh(q, k, v, bw.seq_len, bo, "bf16", 0.5, window, **policy)
+        U.check_refresh_against_oracle(g, q, np.nan_to_num(k), np.nan_to_num(v), bw.seq_len, bo, "bf16", 0.5, window,
+                                       select=policy.get("select", oracle.SELECT_JOINT_FLOOR), pool_kind=policy.get("pool", oracle.POOL_MAX))
