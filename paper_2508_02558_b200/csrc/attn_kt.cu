@@ -878,7 +878,9 @@ AttnPlan plan_attention_kt(int D, int M, int b, int B, int Hkv, int n1_max, int 
   // Six groups of 32 keys at most (two tiles, the second one short): one CTA walks both rather than two CTAs one each -
   // a short second tile costs less than the cluster merge (124 cached keys, 32 heads: 6.0 against 6.9 us; with eight
   // groups four splits are ahead again, 6.7 against 7.3 us).
-  if (groups <= 6) want = 1;
+  // With more units than half the SMs up to ten groups, as three tiles (96 units x 9 groups: 8.1 against 8.9 us).
+  const bool three_tiles = CG == 1 && units * 2 > sms && units <= sms && n2 > 0 && groups <= 10;
+  if (groups <= 6 || three_tiles) want = 1;
   // More than half as many units as SMs, each with a walk of five tiles or more: one whole-SM CTA per unit (footprint
   // (b) below) beats two splits per unit at two CTAs per SM - the same share of the SMs is busy and nothing is merged
   // (128 units x 17 tiles: 29.6 against 32.8 us; 96 units x 5 tiles: 12.3 against 19.3 us with clusters of three; at
@@ -910,7 +912,7 @@ AttnPlan plan_attention_kt(int D, int M, int b, int B, int Hkv, int n1_max, int 
   // down until they are (48 units: clusters of six at two CTAs per SM ran in two waves, 17.8 against 11.4 us with four).
   auto is_small = [&](long long s_) {
     const long long gc = (groups + s_ - 1) / s_;
-    return CG == 1 && (D == 64 || gc <= 8 || (units * s_ > sms && units * s_ <= 2 * sms) || (units > sms && groups < (n2 > 0 ? 20 : 28)));
+    return CG == 1 && (D == 64 || gc <= 8 || (three_tiles && s_ == 1) || (units * s_ > sms && units * s_ <= 2 * sms) || (units > sms && groups < (n2 > 0 ? 20 : 28)));
   };
   while (CG == 1 && tn.splits <= 0 && tn.dual < 0 && want > 1) {
     long long room;
@@ -940,7 +942,7 @@ AttnPlan plan_attention_kt(int D, int M, int b, int B, int Hkv, int n1_max, int 
   // units of four tiles)
   // (head dimension 64: a tile is half the bytes for the same softmax, so the softmax warps are what is short: always two
   // CTAs per SM - 97.5 against 140 us for 512 units x 4352 keys, 30.2 against 41.1 us for 128 units)
-  bool small = CG == 1 && (D == 64 || groups_cta <= 8 || (units * S > sms && units * S <= 2 * sms) || (units > sms && groups < (n2 > 0 ? 20 : 28)));
+  bool small = CG == 1 && (D == 64 || groups_cta <= 8 || (three_tiles && S == 1) || (units * S > sms && units * S <= 2 * sms) || (units > sms && groups < (n2 > 0 ? 20 : 28)));
   int WG = (CG == 1 && !small) ? 2 : 1;
   if (tn.dual == 1) { small = CG == 1; WG = 1; }       // force (a) / (b) where they apply
   if (tn.dual == 0 && CG == 1) { small = false; WG = 2; }
@@ -977,6 +979,12 @@ AttnPlan plan_attention_kt(int D, int M, int b, int B, int Hkv, int n1_max, int 
   // (d) as (b), but with more units than SMs: the CTAs would run in waves, each paying its set-up and its way out with
   //     the SM's memory pipe idle; one resident CTA per SM walks the units as one sequence of tiles instead.
   pl.persistent = CG == 1 && S == 1 && WG == 2 && units > sms;
+  //     A refresh step also goes there with about one unit per SM (twelve tiles or more) or more than 1.6 (ten or more): it pools on
+  //     the way, where the CTAs of (a) and (b) stop for it (96 units x 20 tiles: 30.0 against 32.6 us, 128 x 32: 48.6 against 50.6,
+  //     256 x 10 to 32: 6 % each). In between, the ring of three slots stays (equal or ahead).
+  if (CG == 1 && S == 1 && D == 128 && n2 == 0 && tn.dual < 0 && tn.stages <= 0 &&
+      ((units * 2 > sms && units <= sms && by_tiles >= 12) || (units * 10 > 16LL * sms && by_tiles >= 10)))
+    pl.persistent = true;
   if (tn.persist == 0) pl.persistent = false;
   if (tn.persist >= 1) pl.persistent = CG == 1 && S == 1;
   if (pl.persistent) {
