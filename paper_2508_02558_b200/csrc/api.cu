@@ -107,7 +107,8 @@ AttnPlan plan_for(const sdllm_desc* d, int op) {
   const int G = d->n_q_heads / d->n_kv_heads;
   const bool refresh = op == SDLLM_OP_REFRESH_SCORES;
   return plan_attention(d->dtype, d->head_dim, G * d->block_len, d->block_len, d->batch, d->n_kv_heads,
-                        refresh ? d->seq_len_max : d->n_keep_max, refresh ? 0 : d->block_len);
+                        refresh ? d->seq_len_max : d->n_keep_max, refresh ? 0 : d->block_len,
+                        refresh && d->score == SDLLM_SCORE_PROB_MEAN);
 }
 
 void fill_common(AttnParams& p, const sdllm_desc* d, const AttnPlan& pl) {

@@ -4,9 +4,10 @@
 // The keys lie on the accumulator rows (S^T = K_tile Q^T, as in attn_kt.cu), so one thread owns one key and adds up its
 // probabilities without any exchange, and one MMA covers all query rows of the head (N up to 256). The key tiles of a (sequence,
 // KV head) are shared out to the CTAs of one cluster; behind a cluster barrier each of them pools a share of the positions.
-// Bound by reading K once more (often from L2) and by latency. A refresh of 32 heads x 1280 keys with it: 43.6 -> 31.1 us, where the
-// query-row kernel's attention pass, its fold,
-// and a second pass of column sums by shuffle transposes with a separate pooling stood before.
+// Bound by reading K once more (often from L2) and by latency: 32 heads x 1280 keys 10 us alone, where a second pass on the
+// query-row kernel, its column sums by shuffle transposes over all replicated rows and its pooling took 14.5.
+// Probabilities of neighbouring ranks differ by as little as their fp32 rounding, so the order of every sum is fixed: 32 rows as a
+// tree of halves, the four trees of 128 rows in pairs, further 128 rows added at the end.
 //   warp 0      TMA producer: Q, then K tiles (128 keys, 128-byte swizzle) into a three-slot ring
 //   warp 1      tcgen05.mma issuer, two S^T buffers in turn
 //   warps 2-5   one key per thread
@@ -146,26 +147,38 @@ __global__ void __launch_bounds__(PB_THREADS) prob_saliency_kernel(const __grid_
       const int sb = it & 1;
       if (!wait_bar_warp(BAR(S_FULL + sb), (it >> 1) & 1, abort_flag, p.status, 65, p.wait_cycles)) break;
       tc_fence_after();
-      float a4[4] = {0.f, 0.f, 0.f, 0.f};
+      float total = 0.f;
 #pragma unroll 1
-      for (int c = 0; c < NP; c += 32) {
-        uint32_t sv[32];
-        tmem_ld32(tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(sb * NP + c), sv);
-        tc_wait_ld();
+      for (int c0 = 0; c0 < NP; c0 += 128) {
+        float part[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int e = 0; e < 32; e += 4) {
-          const float4 l4 = *reinterpret_cast<const float4*>(lse_s + c + e);
-          a4[0] += fast_exp2(fmaf(__uint_as_float(sv[e]), p.scale_log2, -l4.x));
-          a4[1] += fast_exp2(fmaf(__uint_as_float(sv[e + 1]), p.scale_log2, -l4.y));
-          a4[2] += fast_exp2(fmaf(__uint_as_float(sv[e + 2]), p.scale_log2, -l4.z));
-          a4[3] += fast_exp2(fmaf(__uint_as_float(sv[e + 3]), p.scale_log2, -l4.w));
+        for (int c = 0; c < 4; ++c) {
+          if (c0 + 32 * c >= NP) break;
+          uint32_t sv[32];
+          float v[32];
+          tmem_ld32(tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(sb * NP + c0 + 32 * c), sv);
+          tc_wait_ld();
+#pragma unroll
+          for (int e = 0; e < 32; e += 4) {
+            const float4 l4 = *reinterpret_cast<const float4*>(lse_s + c0 + 32 * c + e);
+            v[e] = fast_exp2(fmaf(__uint_as_float(sv[e]), p.scale_log2, -l4.x));
+            v[e + 1] = fast_exp2(fmaf(__uint_as_float(sv[e + 1]), p.scale_log2, -l4.y));
+            v[e + 2] = fast_exp2(fmaf(__uint_as_float(sv[e + 2]), p.scale_log2, -l4.z));
+            v[e + 3] = fast_exp2(fmaf(__uint_as_float(sv[e + 3]), p.scale_log2, -l4.w));
+          }
+#pragma unroll
+          for (int half = 16; half >= 1; half >>= 1)
+#pragma unroll
+            for (int e = 0; e < half; ++e) v[e] += v[e + half];
+          part[c] = v[0];
         }
+        total = __fadd_rn(total, __fmul_rn((part[0] + part[1]) + (part[2] + part[3]), inv_rows));      // (not contracted)
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(BAR(S_FREE + sb));
       const int pos = (t0 + it) * 128 + row;
-      if (pos < n) __stcg(raw + pos, ((a4[0] + a4[1]) + (a4[2] + a4[3])) * inv_rows);
+      if (pos < n) __stcg(raw + pos, total);
     }
   }
 

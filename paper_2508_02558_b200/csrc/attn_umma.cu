@@ -54,6 +54,7 @@ struct UmmaParams {
   int lpt;           // 1: grid z counts the sequences from the longest to the shortest (several waves of ragged work)
 };
 
+#define SDLLM_ZERO_LIMIT_NEVER_WAITS
 #include "umma_ptx.cuh"
 
 // Merge of the key-split partials of S (row, float4 column) slots of a unit and the final stores. slot[s] < 0 marks
@@ -345,32 +346,36 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
     }
   } else if (warp == 1) {
     // ======================================= MMA issuer =======================================
-    if (lane == 0 && do_attn) {
+    // warp-uniform, one elected lane issues (see attn_kt.cu)
+    if (do_attn) {
+      const bool leader = elect_one();
       const uint32_t idesc_pv = instr_desc(D, true);
       bool ok = true, have_q = false;
       int it = 0;
       Tile prev{}; int prev_it = -1;
       auto issue_pv = [&](const Tile& x, int j) -> bool {
         const int s = j % NS, pb = j & 1;
-        if (!wait_bar(BAR(P_FULL + pb), (j >> 1) & 1, abort_flag, p.status, 4, p.wait_cycles)) return false;
-        if (!wait_bar(BAR(FULL_V + s), (j / NS) & 1, abort_flag, p.status, 5, p.wait_cycles)) return false;
+        if (!wait_bar_warp(BAR(P_FULL + pb), (j >> 1) & 1, abort_flag, p.status, 4, p.wait_cycles)) return false;
+        if (!wait_bar_warp(BAR(FULL_V + s), (j / NS) & 1, abort_flag, p.status, 5, p.wait_cycles)) return false;
         tc_fence_after();
         const uint32_t vsm = smem_u32(stage0 + (size_t)s * stage_bytes) + kv_bytes;
         const uint32_t a_t = tmem_base + (uint32_t)pb * S_STRIDE;
-        for (int ks = 0; ks < x.n_mma / 16; ++ks)
-          mma_ts(tmem_base + O_COL, a_t + ks * 8, smem_desc(vsm + ks * 2048, (uint32_t)half_bytes, 1024u), idesc_pv,
-                 (j > 0 || ks > 0) ? 1u : 0u);
-        tc_commit(BAR(PV_DONE + pb));  // two alternating barriers: a waiter is never a whole phase ahead of either
-        tc_commit(BAR(EMPTY_V + s));
+        const uint64_t vd = smem_desc(vsm, (uint32_t)half_bytes, 1024u);
+        if (leader) {
+          for (int ks = 0; ks < x.n_mma / 16; ++ks) mma_ts(tmem_base + O_COL, a_t + ks * 8, vd + ks * (2048 >> 4), idesc_pv, (j > 0 || ks > 0) ? 1u : 0u);
+          tc_commit(BAR(PV_DONE + pb));  // two alternating barriers: a waiter is never a whole phase ahead of either
+          tc_commit(BAR(EMPTY_V + s));
+        }
+        __syncwarp();
         return true;
       };
       for (int t = t_begin; t < t_end && ok; ++t) {
         const Tile x = tile_of(t, tiles1, KT, KT2, n1, n2);
         if (x.nv == 0) continue;
         const int s = it % NS, sb = it & 1;
-        if (!wait_bar(BAR(FULL_K + s), (it / NS) & 1, abort_flag, p.status, 7, p.wait_cycles)) { ok = false; break; }
+        if (!wait_bar_warp(BAR(FULL_K + s), (it / NS) & 1, abort_flag, p.status, 7, p.wait_cycles)) { ok = false; break; }
         if (!have_q) {
-          if (!wait_bar(BAR(Q_FULL), 0, abort_flag, p.status, 3, p.wait_cycles)) { ok = false; break; }
+          if (!wait_bar_warp(BAR(Q_FULL), 0, abort_flag, p.status, 3, p.wait_cycles)) { ok = false; break; }
           have_q = true;
         }
         tc_fence_after();
@@ -378,25 +383,27 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
         const uint32_t qsm = smem_u32(q_s);
         const uint32_t idesc_s = instr_desc(x.n_mma, false);
         const uint32_t d_t = tmem_base + (uint32_t)sb * S_STRIDE;
+        const uint64_t qd = smem_desc(qsm, 16u, 1024u), kd = smem_desc(ksm, 16u, 1024u);
+        if (leader) {
 #pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) {
-          const uint32_t hq = (ks >> 2) * (128 * 128) + (ks & 3) * 32;
-          const uint32_t hk = (ks >> 2) * half_bytes + (ks & 3) * 32;
-          mma_ss(d_t, smem_desc(qsm + hq, 16u, 1024u), smem_desc(ksm + hk, 16u, 1024u), idesc_s, ks > 0 ? 1u : 0u);
+          for (int ks = 0; ks < D / 16; ++ks)
+            mma_ss(d_t, qd + (((ks >> 2) * (128 * 128) + (ks & 3) * 32) >> 4), kd + (((ks >> 2) * half_bytes + (ks & 3) * 32) >> 4), idesc_s, ks > 0 ? 1u : 0u);
+          tc_commit(BAR(S_FULL + sb));
+          tc_commit(BAR(EMPTY_K + s));
         }
-        tc_commit(BAR(S_FULL + sb));
-        tc_commit(BAR(EMPTY_K + s));
+        __syncwarp();
         if (do_attn && prev_it >= 0 && !issue_pv(prev, prev_it)) { ok = false; break; }
         prev = x; prev_it = it;
         ++it;
       }
       if (do_attn && ok && prev_it >= 0) ok = issue_pv(prev, prev_it);
       // a CTA whose slice holds no valid key never used Q: its load must still have landed before the CTA retires
-      if (ok && !have_q) ok = wait_bar(BAR(Q_FULL), 0, abort_flag, p.status, 3, p.wait_cycles);
-      if (*abort_flag) {               // wait for the tensor pipe to finish what was issued before TMEM is freed
+      if (ok && !have_q) ok = wait_bar_warp(BAR(Q_FULL), 0, abort_flag, p.status, 3, p.wait_cycles);
+      if (*abort_flag && leader) {     // wait for the tensor pipe to finish what was issued before TMEM is freed
         tc_commit(BAR(DRAIN));
         drain_bar(BAR(DRAIN), 0);
       }
+      __syncwarp();
     }
   } else if (warp < 6) {
     // ======================================= softmax warps =======================================
@@ -1053,11 +1060,15 @@ bool pair_supported(int dtype, int D, int M, int b);
 AttnPlan plan_attention_pair(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn);
 cudaError_t launch_attn_pair(const AttnParams& p, const AttnPlan& pl, int D, cudaStream_t st);
 
-AttnPlan plan_attention(int dtype, int D, int M, int b, int B, int Hkv, int n1_max, int n2) {
+AttnPlan plan_attention(int dtype, int D, int M, int b, int B, int Hkv, int n1_max, int n2, bool prob_scores) {
   // bf16 goes to the tcgen05 kernels wherever they apply: heads with few query rows to the kernel that puts the keys on the
   // accumulator rows, the rest to the one that puts the queries there and has two softmax warpgroups (attn_pair.cu). fp32 and
   // the remaining bf16 shapes go to the cp.async kernels. Tuning::kernel forces a family.
+  // With the probability saliency (prob_scores) the attention pass stays on the query-row kernel of this file: that saliency ranks
+  // keys by differences as small as the rounding of exp2(S - log-sum-exp), so another order of the sums behind the log-sum-exp
+  // would keep other keys.
   const Tuning tn = tuning();
+  if (prob_scores && tn.kernel != 1 && umma_supported(dtype, D, M, b)) return plan_attention_umma(D, M, b, B, Hkv, n1_max, n2, tn);
   const bool kt_ok = kt_supported(dtype, D, M, b);
   if (kt_ok && (tn.kernel == 3 || (tn.kernel == 0 && kt_preferred(D, M, B, Hkv, n1_max, n2))))
     return plan_attention_kt(D, M, b, B, Hkv, n1_max, n2, tn);

@@ -98,7 +98,7 @@ struct CompactParams {
   int64_t kv_stride_bytes[3], c_stride_bytes[3];
 };
 
-AttnPlan plan_attention(int dtype, int D, int M, int b, int B, int Hkv, int n1_max, int n2);
+AttnPlan plan_attention(int dtype, int D, int M, int b, int B, int Hkv, int n1_max, int n2, bool prob_scores);
 cudaError_t launch_prob_saliency(const AttnParams& p, int D, cudaStream_t st);    // second pass of the probability saliency
 
 bool umma_tail_is_fused(const AttnPlan& pl, int D, int M, int n1_max, bool pool, bool merge);
