@@ -205,8 +205,8 @@ sdllm_status sdllm_plan_describe(const sdllm_desc* d, int op, char* buf, size_t 
     snprintf(buf, buf_bytes, "%s splits=%d cluster=%d stages=%d softmax_warpgroups=%d threads=%d smem=%zu", name, pl.cluster, pl.cluster,
              pl.stages, pl.c_warps * pl.warp_keys, pl.threads, pl.smem_bytes);
   else
-    snprintf(buf, buf_bytes, "%s splits=%d cluster=%d stages=%d key_tile=%d threads=%d smem=%zu", name, pl.splits, pl.cluster, pl.stages,
-             pl.key_tile, pl.threads, pl.smem_bytes);
+    snprintf(buf, buf_bytes, "%s splits=%d cluster=%d stages=%d key_tile=%d threads=%d%s", name, pl.splits, pl.cluster, pl.stages,
+             pl.key_tile, pl.threads, pl.kind == 4 ? " (attn_pair_kernel: two softmax warpgroups)" : "");
   return SDLLM_OK;
 }
 

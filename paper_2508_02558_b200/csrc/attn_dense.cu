@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(256) dense_fold_kernel(const DenseParams p) {
 // unit takes a whole SM, so without that 160 units on 148 SMs run in two waves (32 heads x 1280 rows: 46.2 us, 42.8 so; 28 heads
 // x 4096: 245 us, 200; 16 heads x 3000: 106, 81). Costs in us: a key tile 1.55, a CTA's set-up and way out 6.5, of which a cut unit overlaps 2 with the
 // wave in front, its partial rows and the launch that folds
-// them 9 (3 of it a margin).
+// them 7.25 (3 of it a margin) and 0.35 per share.
 // Batches of several sequences may be ragged, which the host cannot see: they are cut only where all units fit one wave.
 struct DensePlan {
   int whole, parts;
@@ -467,7 +467,7 @@ DensePlan plan_dense(int B, int Hq, int L) {
   if (rest == 0 || (B > 1 && rest != units)) return pl;
   double least = 6.5 + 1.55 * nt;
   for (int q = 2; q <= 16 && q <= nt && rest * q <= sms; ++q) {
-    const double cost = (rest == units ? 6.5 : 4.5) + 1.55 * ((nt + q - 1) / q) + 9.;
+    const double cost = (rest == units ? 6.5 : 4.5) + 1.55 * ((nt + q - 1) / q) + 7.25 + 0.35 * q;
     if (cost < least) { least = cost; pl.whole = (int)(units - rest); pl.parts = q; }
   }
   return pl;
