@@ -41,7 +41,8 @@ constexpr int KS_RAW = 6;                // tiles whose saliency is kept: five a
 __device__ __forceinline__ void pair_arrive(int id) { asm volatile("bar.arrive %0, 256;\n" ::"r"(id) : "memory"); }
 __device__ __forceinline__ void pair_sync(int id) { asm volatile("bar.sync %0, 256;\n" ::"r"(id) : "memory"); }
 
-template <int D>
+// SCORES: the refresh step's saliency and pooling (a template parameter, so that the reuse step does not carry their code).
+template <int D, bool SCORES>
 __global__ void __launch_bounds__(KS_THREADS, 1) attn_kt_stream_kernel(const __grid_constant__ KtMaps tm, const KtParams kp) {
   constexpr int NS = KS_NS;
   constexpr int H = D / 64;                  // 128-byte column halves of a K/V row
@@ -341,7 +342,7 @@ __global__ void __launch_bounds__(KS_THREADS, 1) attn_kt_stream_kernel(const __g
     const int row = q4 * 32 + lane;                    // key row of a tile; head dimension of O^T at the end of a unit
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q4 * 32) << 16);
     const float sl2 = p.scale_log2;
-    const bool scores = p.want_scores != 0;
+    constexpr bool scores = SCORES;
     const bool do_attn = p.out != nullptr;
     const int st = (tid - 64) & 127;                   // index inside the warpgroup
     const uint32_t o_col = O_COL + (uint32_t)w * NP;
@@ -655,9 +656,9 @@ __global__ void __launch_bounds__(KS_THREADS, 1) attn_kt_stream_kernel(const __g
   }
 }
 
-template <int D>
+template <int D, bool SCORES>
 cudaError_t launch_kt_stream_d(const KtMaps& tm, const KtParams& kp, size_t smem_bytes, bool pdl, cudaStream_t st) {
-  auto kern = attn_kt_stream_kernel<D>;
+  auto kern = attn_kt_stream_kernel<D, SCORES>;
   static SmemConfig configured;
   cudaError_t e = configure_smem(reinterpret_cast<const void*>(kern), smem_bytes, configured, true);
   if (e != cudaSuccess) return e;
@@ -689,7 +690,8 @@ size_t kt_stream_smem_bytes(int D) {
 }
 
 cudaError_t launch_kt_stream(const KtMaps& tm, const KtParams& kp, int D, size_t smem_bytes, bool pdl, cudaStream_t st) {
-  return D == 128 ? launch_kt_stream_d<128>(tm, kp, smem_bytes, pdl, st) : launch_kt_stream_d<64>(tm, kp, smem_bytes, pdl, st);
+  if (kp.a.want_scores) return D == 128 ? launch_kt_stream_d<128, true>(tm, kp, smem_bytes, pdl, st) : launch_kt_stream_d<64, true>(tm, kp, smem_bytes, pdl, st);
+  return D == 128 ? launch_kt_stream_d<128, false>(tm, kp, smem_bytes, pdl, st) : launch_kt_stream_d<64, false>(tm, kp, smem_bytes, pdl, st);
 }
 
 }  // namespace sdllm
