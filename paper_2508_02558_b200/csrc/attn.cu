@@ -554,13 +554,8 @@ __global__ void __launch_bounds__(256) merge_pool_kernel(const MergeParams p) {
     if (p.per_region) { if (c < o) hi = o; else lo = o; }
     const int w = (p.window - 1) / 2;
     const float* a = p.raw_scores + bh * p.Lmax;
-    float mx = -INFINITY, sum = 0.f;
-    for (int t = c - w; t <= c + w; ++t) {
-      if (t < lo || t >= hi) continue;
-      const float x = a[t < o ? t : t + b];
-      mx = fmaxf(mx, x);
-      sum += x;
-    }
+    float mx, sum;
+    pool_window(a, c, w, lo, hi, o, b, mx, sum);
     outv = p.pool_kind == SDLLM_POOL_MAX ? mx : sum / (float)p.window;
   }
   p.pooled[idx] = outv;

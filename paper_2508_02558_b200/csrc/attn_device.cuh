@@ -131,7 +131,34 @@ __device__ __forceinline__ float pool_at(const AttnParams& p, const float* a, in
   return p.pool_kind == SDLLM_POOL_MAX ? mx : sum / (float)p.window;
 }
 
-// Importance of one absolute position as pool_at, reading the raw saliency from global memory through L2 (other CTAs wrote it during this launch).
+// Maximum and sum of the raw saliency over the window [c - w, c + w] of candidates that lies inside [lo, hi), read through L2
+// (other CTAs wrote it). Windows of up to nine have all their loads in flight together: one L2 round trip instead of one each.
+__device__ __forceinline__ void pool_window(const float* a, int c, int w, int lo, int hi, int o, int b, float& mx, float& sum) {
+  mx = -INFINITY; sum = 0.f;
+  if (w <= 4) {
+    float v[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      const int t = c - 4 + i;
+      v[i] = 0.f;
+      if (t >= max(lo, c - w) && t < min(hi, c + w + 1)) v[i] = __ldcg(a + (t < o ? t : t + b));
+    }
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      const int t = c - 4 + i;
+      if (t >= max(lo, c - w) && t < min(hi, c + w + 1)) { mx = fmaxf(mx, v[i]); sum += v[i]; }
+    }
+    return;
+  }
+  for (int t = max(lo, c - w); t < min(hi, c + w + 1); ++t) {
+    const float x = __ldcg(a + (t < o ? t : t + b));
+    mx = fmaxf(mx, x);
+    sum += x;
+  }
+}
+
+// Importance of one absolute position as pool_at, reading the raw saliency from global memory through L2 (other CTAs wrote it
+// during this launch).
 __device__ __forceinline__ float pool_at_ldcg(const AttnParams& p, const float* a, int L, int o_in, int pos) {
   const int b = p.b;
   const int o = min(max(o_in, 0), max(L - b, 0));
@@ -140,13 +167,8 @@ __device__ __forceinline__ float pool_at_ldcg(const AttnParams& p, const float* 
   const int c = pos < o ? pos : pos - b;
   int lo = 0, hi = C;
   if (p.per_region) { if (c < o) hi = o; else lo = o; }
-  float mx = -INFINITY, sum = 0.f;
-  for (int t = c - w; t <= c + w; ++t) {
-    if (t < lo || t >= hi) continue;
-    const float x = __ldcg(a + (t < o ? t : t + b));
-    mx = fmaxf(mx, x);
-    sum += x;
-  }
+  float mx, sum;
+  pool_window(a, c, w, lo, hi, o, b, mx, sum);
   return p.pool_kind == SDLLM_POOL_MAX ? mx : sum / (float)p.window;
 }
 

@@ -854,6 +854,7 @@ bool kt_preferred(int D, int M, int B, int Hkv, int n1_max, int n2) {
   const long long units = (long long)B * Hkv;
   const int sms = sm_count(), tiles = (n1_max + 127) / 128 + (n2 > 0 ? (n2 + 127) / 128 : 0);
   if (n2 > 0) {
+    if (units > sms) return tiles <= 6;
     if (units * 2 > sms) return tiles <= 3;
     return tiles > 3 && !(units * 8 <= sms && tiles >= 24);
   }
