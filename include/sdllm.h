@@ -105,8 +105,9 @@ const char* sdllm_status_string(sdllm_status status);
 /* Bytes of device workspace a call of `op` needs for this description (host-only, no GPU needed).
  * Returns 0 for an invalid description or when the op needs none. The workspace needs 256-byte alignment and the
  * caller zeroes ALL of it once after allocating it: its first 4 bytes are a status word (see sdllm_read_status) and
- * it holds completion counters that every call leaves at zero again; the rest is unspecified after a call. One
- * workspace may serve any number of calls that run one after another on the GPU, never two that overlap.
+ * behind it lies a block of counters that every call leaves at zero again and that no call uses for anything else; the
+ * rest is unspecified after a call. One workspace may serve any number of calls, of different kinds and descriptions too
+ * as long as it is large enough for each, that run one after another on the GPU, never two that overlap.
  * After a call whose status word reads non-zero (SDLLM_ERR_TIMEOUT) zero the whole workspace again before reusing it:
  * the status word is sticky, and the call that gave up may have left its counters anywhere. */
 size_t sdllm_workspace_bytes(const sdllm_desc* desc, int op);
@@ -212,9 +213,10 @@ sdllm_status sdllm_dense_attn(const sdllm_desc* desc, const void* q, const int64
  * computes exactly what sdllm_sparse_block_attn computes, but takes no workspace. Some hosts of this library run under
  * a fixed memory plan - an inference server that sized every buffer at start-up, a plug-in whose host owns the
  * allocator - and must not call cudaMalloc (or any allocating library routine) once they are running; they have
- * nowhere to get the workspace from. For them the scratch (status word, completion counters, key-split partials) is a
- * 8 MiB array built into the library image; every GPU that loads the library holds one copy until the process exits.
- *   - Shapes whose workspace (sdllm_workspace_bytes(desc, SDLLM_OP_SPARSE_BLOCK_ATTN)) exceeds 8 MiB are refused with
+ * nowhere to get the workspace from. For them the scratch (status word, completion counters, key-split partials) is an
+ * array of 8 MiB plus 768 bytes built into the library image; every GPU that loads the library holds one copy until the
+ * process exits.
+ *   - Shapes whose workspace (sdllm_workspace_bytes(desc, SDLLM_OP_SPARSE_BLOCK_ATTN)) exceeds that are refused with
  *     SDLLM_ERR_WORKSPACE; use sdllm_sparse_block_attn with a caller-owned workspace for those.
  *   - The call allocates and frees nothing. The first call on each device looks the array's device address up
  *     (cudaGetSymbolAddress, with that device current); make that first call before any stream capture.

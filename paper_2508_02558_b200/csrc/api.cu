@@ -77,32 +77,6 @@ bool cuda_failed(cudaError_t e, const char* what) {
 
 float scale_of(const sdllm_desc* d) { return d->softmax_scale > 0.f ? d->softmax_scale : 1.0f / sqrtf((float)d->head_dim); }
 
-struct WsLayout {
-  size_t status, counters, part_o, part_ml, raw, lse, total;
-};
-
-WsLayout attn_ws(const sdllm_desc* d, const AttnPlan& pl, bool scores) {
-  WsLayout w{};
-  const int G = d->n_q_heads / d->n_kv_heads, M = G * d->block_len;
-  size_t off = 0;
-  w.status = off;
-  (void)M;
-  off += 256;                          // device status word (sdllm_read_status)
-  w.counters = off;                    // completion counters: zero between calls
-  off += align_up(pl.n_counters * 4, 256);
-  w.part_o = off;
-  off += align_up((size_t)d->batch * d->n_kv_heads * pl.part_rows * d->head_dim * 4, 256);
-  w.part_ml = off;
-  off += align_up((size_t)d->batch * d->n_kv_heads * pl.part_rows * 2 * 4, 256);
-  w.raw = off;
-  const bool prob = d->score == SDLLM_SCORE_PROB_MEAN;
-  if (scores) off += align_up((size_t)d->batch * d->n_kv_heads * d->seq_len_max * 4, 256);
-  w.lse = off;                         // probability saliency: the rows' log-sum-exp between its two passes
-  if (scores && prob) off += align_up((size_t)d->batch * d->n_q_heads * d->block_len * 4, 256);
-  w.total = off;
-  return w;
-}
-
 AttnPlan plan_for(const sdllm_desc* d, int op) {
   const int G = d->n_q_heads / d->n_kv_heads;
   const bool refresh = op == SDLLM_OP_REFRESH_SCORES;
@@ -123,13 +97,12 @@ void fill_common(AttnParams& p, const sdllm_desc* d, const AttnPlan& pl) {
 
 // Full-sequence attention runs on its own tcgen05 kernel: bf16, D in {64, 128}, one grid row per query head.
 // Of its workspace the status block is required; the partial rows behind it let the call share out its last units.
-constexpr size_t kDenseStatusBytes = 256;
 bool dense_supported(const sdllm_desc* d) {
   return umma_supported(d->dtype, d->head_dim, 128, 128) && d->n_q_heads <= 65535;
 }
 
 // Built-in scratch of sdllm_sparse_block_attn_static: lives in the library image, one copy per GPU that loads it.
-constexpr size_t kStaticScratchBytes = (size_t)8 << 20;
+constexpr size_t kStaticScratchBytes = ((size_t)8 << 20) + kWsDataOffset - kWsStatusBytes;     // 8 MiB, the counters beside them
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
 std::mutex g_static_mutex;
 void* g_static_scratch_ptr[kMaxDevices] = {};      // device address of g_static_scratch on each device, once looked up
@@ -150,6 +123,22 @@ sdllm_status static_scratch_address(void** out) {
 }
 
 }  // namespace
+
+AttnWorkspace sdllm::attn_workspace(const sdllm_desc* d, const AttnPlan& pl, bool scores) {
+  AttnWorkspace w{};
+  size_t off = kWsDataOffset;
+  w.part_o = off;
+  off += align_up((size_t)d->batch * d->n_kv_heads * pl.part_rows * d->head_dim * 4, 256);
+  w.part_ml = off;
+  off += align_up((size_t)d->batch * d->n_kv_heads * pl.part_rows * 2 * 4, 256);
+  w.raw = off;
+  const bool prob = d->score == SDLLM_SCORE_PROB_MEAN;
+  if (scores) off += align_up((size_t)d->batch * d->n_kv_heads * d->seq_len_max * 4, 256);
+  w.lse = off;                         // probability saliency: the rows' log-sum-exp between its two passes
+  if (scores && prob) off += align_up((size_t)d->batch * d->n_q_heads * d->block_len * 4, 256);
+  w.total = off;
+  return w;
+}
 
 extern "C" {
 
@@ -175,9 +164,9 @@ const char* sdllm_status_string(sdllm_status s) {
 
 size_t sdllm_workspace_bytes(const sdllm_desc* d, int op) {
   if (check_desc(d) != SDLLM_OK) return 0;
-  if (op == SDLLM_OP_REFRESH_SCORES) return attn_ws(d, plan_for(d, op), true).total;
-  if (op == SDLLM_OP_SPARSE_BLOCK_ATTN) return attn_ws(d, plan_for(d, op), false).total;
-  if (op == SDLLM_OP_DENSE_ATTN && dense_supported(d)) return dense_workspace_bytes(d->batch, d->n_q_heads, d->seq_len_max, d->head_dim);
+  if (op == SDLLM_OP_REFRESH_SCORES) return attn_workspace(d, plan_for(d, op), true).total;
+  if (op == SDLLM_OP_SPARSE_BLOCK_ATTN) return attn_workspace(d, plan_for(d, op), false).total;
+  if (op == SDLLM_OP_DENSE_ATTN && dense_supported(d)) return dense_workspace(d->batch, d->n_q_heads, d->seq_len_max, d->head_dim).total;
   return 0;
 }
 
@@ -255,7 +244,7 @@ sdllm_status sdllm_refresh_scores(const sdllm_desc* d, const void* q_blk, const 
     return SDLLM_ERR_INVALID_ARG;
   if (lse && !out) return SDLLM_ERR_INVALID_ARG;
   const AttnPlan pl = plan_for(d, SDLLM_OP_REFRESH_SCORES);
-  const WsLayout w = attn_ws(d, pl, true);
+  const AttnWorkspace w = attn_workspace(d, pl, true);
   if (w.total > 0 && (ws == nullptr || ws_bytes < w.total || (reinterpret_cast<uintptr_t>(ws) & 255u))) return SDLLM_ERR_WORKSPACE;
   if ((st = check_device()) != SDLLM_OK) return st;
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(cuda_stream);
@@ -266,13 +255,13 @@ sdllm_status sdllm_refresh_scores(const sdllm_desc* d, const void* q_blk, const 
   p.q = q_blk; p.k1 = k; p.v1 = v; p.k2 = nullptr; p.v2 = nullptr;
   p.n1_per_seq = seq_len; p.block_off = block_off;
   p.out = out; p.lse = lse;
-  p.status = reinterpret_cast<int32_t*>(wsb + w.status);
+  p.status = reinterpret_cast<int32_t*>(wsb);
   p.part_o = reinterpret_cast<float*>(wsb + w.part_o);
   p.part_ml = reinterpret_cast<float*>(wsb + w.part_ml);
   p.raw_scores = pooled_scores ? reinterpret_cast<float*>(wsb + w.raw) : nullptr;
   p.n1_max = d->seq_len_max; p.n2 = 0;
   p.want_scores = pooled_scores != nullptr;
-  p.counters = reinterpret_cast<int32_t*>(wsb + w.counters);
+  p.counters = reinterpret_cast<int32_t*>(wsb + kWsStatusBytes);
   p.pooled = pooled_scores; p.window = d->pool_window; p.pool_kind = d->pool;
   p.per_region = d->select != SDLLM_SELECT_JOINT_FLOOR;
   for (int i = 0; i < 3; ++i) { p.k1_stride[i] = d->kv_stride[i]; p.k2_stride[i] = 0; }
@@ -367,7 +356,7 @@ sdllm_status sdllm_sparse_block_attn(const sdllm_desc* d, const void* q_blk, con
   if (st != SDLLM_OK) return st;
   if ((st = check_sparse_args(d, q_blk, k_c, v_c, kept_cnt, k_blk, v_blk, out)) != SDLLM_OK) return st;
   const AttnPlan pl = plan_for(d, SDLLM_OP_SPARSE_BLOCK_ATTN);
-  const WsLayout w = attn_ws(d, pl, false);
+  const AttnWorkspace w = attn_workspace(d, pl, false);
   if (w.total > 0 && (ws == nullptr || ws_bytes < w.total || (reinterpret_cast<uintptr_t>(ws) & 255u))) return SDLLM_ERR_WORKSPACE;
   if ((st = check_device()) != SDLLM_OK) return st;
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(cuda_stream);
@@ -378,13 +367,13 @@ sdllm_status sdllm_sparse_block_attn(const sdllm_desc* d, const void* q_blk, con
   p.q = q_blk; p.k1 = k_c ? k_c : k_blk; p.v1 = v_c ? v_c : v_blk; p.k2 = k_blk; p.v2 = v_blk;
   p.n1_per_seq = kept_cnt; p.block_off = nullptr;
   p.out = out; p.lse = nullptr;
-  p.status = reinterpret_cast<int32_t*>(wsb + w.status);
+  p.status = reinterpret_cast<int32_t*>(wsb);
   p.part_o = reinterpret_cast<float*>(wsb + w.part_o);
   p.part_ml = reinterpret_cast<float*>(wsb + w.part_ml);
   p.raw_scores = nullptr;
   p.n1_max = d->n_keep_max; p.n2 = d->block_len;
   p.want_scores = 0;
-  p.counters = reinterpret_cast<int32_t*>(wsb + w.counters);
+  p.counters = reinterpret_cast<int32_t*>(wsb + kWsStatusBytes);
   p.pooled = nullptr;
   for (int i = 0; i < 3; ++i) { p.k1_stride[i] = d->c_stride[i]; p.k2_stride[i] = d->blk_stride[i]; }
   if (cuda_failed(launch_attn_partial(p, pl, d->dtype, d->head_dim, stream), "attention launch")) return SDLLM_ERR_CUDA;
@@ -407,7 +396,7 @@ sdllm_status sdllm_dense_attn(const sdllm_desc* d, const void* q, const int64_t*
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(out) || !aligned16(lse)) return SDLLM_ERR_INVALID_ARG;
   if (!strides_ok(q_stride, elem_size(d->dtype)) || !strides_ok(o_stride, elem_size(d->dtype))) return SDLLM_ERR_INVALID_ARG;
   if (!dense_supported(d)) return SDLLM_ERR_UNSUPPORTED;
-  if (ws == nullptr || ws_bytes < kDenseStatusBytes || (reinterpret_cast<uintptr_t>(ws) & 255u)) return SDLLM_ERR_WORKSPACE;
+  if (ws == nullptr || ws_bytes < kWsStatusBytes || (reinterpret_cast<uintptr_t>(ws) & 255u)) return SDLLM_ERR_WORKSPACE;
   if ((st = check_device()) != SDLLM_OK) return st;
   const DenseCall c{q, k, v, q_stride, d->kv_stride, o_stride, seq_len, out, lse, ws, ws_bytes,
                     d->batch, d->n_q_heads, d->n_kv_heads, d->seq_len_max, d->head_dim, scale_of(d)};
@@ -421,13 +410,13 @@ sdllm_status sdllm_sparse_block_attn_static(const sdllm_desc* d, const void* q_b
   sdllm_status st = check_desc(d);
   if (st != SDLLM_OK) return st;
   if ((st = check_sparse_args(d, q_blk, k_c, v_c, kept_cnt, k_blk, v_blk, out)) != SDLLM_OK) return st;
-  const WsLayout w = attn_ws(d, plan_for(d, SDLLM_OP_SPARSE_BLOCK_ATTN), false);
+  const AttnWorkspace w = attn_workspace(d, plan_for(d, SDLLM_OP_SPARSE_BLOCK_ATTN), false);
   if (w.total > kStaticScratchBytes) return SDLLM_ERR_WORKSPACE;       // this shape needs more than the built-in scratch
   if ((st = check_device()) != SDLLM_OK) return st;
   void* scratch = nullptr;
   if ((st = static_scratch_address(&scratch)) != SDLLM_OK) return st;
   // the status word and the completion counters must start at zero whatever the last call left behind
-  if (cuda_failed(cudaMemsetAsync(scratch, 0, w.part_o, reinterpret_cast<cudaStream_t>(cuda_stream)), "scratch clear")) return SDLLM_ERR_CUDA;
+  if (cuda_failed(cudaMemsetAsync(scratch, 0, kWsDataOffset, reinterpret_cast<cudaStream_t>(cuda_stream)), "scratch clear")) return SDLLM_ERR_CUDA;
   return sdllm_sparse_block_attn(d, q_blk, k_c, v_c, kept_cnt, k_blk, v_blk, out, scratch, kStaticScratchBytes, cuda_stream);
 }
 

@@ -472,8 +472,6 @@ DensePlan plan_dense(int B, int Hq, int L) {
   }
   return pl;
 }
-constexpr size_t DN_STATUS_BYTES = 256;
-size_t partial_bytes(long long cut, int parts, int D) { return (size_t)cut * parts * 256 * (D + 2) * 4; }
 
 cudaError_t launch_overlapped(const void* kern, void** args, dim3 grid, int threads, size_t smem, cudaStream_t st) {
   cudaLaunchConfig_t cfg{};
@@ -519,10 +517,15 @@ int dense_launches(int B, int Hq, int L) {
   return pl.parts == 1 ? 1 : (pl.whole > 0 ? 3 : 2);
 }
 
-size_t dense_workspace_bytes(int B, int Hq, int L, int D) {
+DenseWorkspace dense_workspace(int B, int Hq, int L, int D) {
   const DensePlan pl = plan_dense(B, Hq, L);
   const long long units = (long long)B * Hq * ((L + 255) / 256);
-  return DN_STATUS_BYTES + (pl.parts > 1 ? partial_bytes(units - pl.whole, pl.parts, D) : 0);
+  const size_t rows = pl.parts > 1 ? (size_t)(units - pl.whole) * pl.parts * 256 : 0;
+  DenseWorkspace w{};
+  w.part_o = kWsDataOffset;
+  w.part_ml = w.part_o + rows * D * 4;
+  w.total = rows > 0 ? w.part_ml + rows * 2 * 4 : kWsStatusBytes;
+  return w;
 }
 
 cudaError_t launch_dense(const DenseCall& c, cudaStream_t st) {
@@ -536,11 +539,12 @@ cudaError_t launch_dense(const DenseCall& c, cudaStream_t st) {
   ok = ok && umma_make_map(&tm.v, c.v, c.D, c.L, c.Hkv, c.B, c.kv_stride, 128, 1);
   if (!ok) return cudaErrorInvalidValue;
   DensePlan pl = plan_dense(c.B, c.Hq, c.L);
-  if (c.workspace_bytes < dense_workspace_bytes(c.B, c.Hq, c.L, c.D)) pl = {(int)units, 1};
+  const DenseWorkspace w = dense_workspace(c.B, c.Hq, c.L, c.D);
+  if (c.workspace_bytes < w.total) pl = {(int)units, 1};
   DenseParams p{};
   p.seq_len = c.seq_len; p.out = c.out; p.lse = c.lse; p.status = reinterpret_cast<int32_t*>(c.workspace);
-  p.part_o = reinterpret_cast<float*>(reinterpret_cast<char*>(c.workspace) + DN_STATUS_BYTES);
-  p.part_ml = p.part_o + (size_t)(units - pl.whole) * pl.parts * 256 * c.D;
+  p.part_o = reinterpret_cast<float*>(reinterpret_cast<char*>(c.workspace) + w.part_o);
+  p.part_ml = reinterpret_cast<float*>(reinterpret_cast<char*>(c.workspace) + w.part_ml);
   p.B = c.B; p.Hq = c.Hq; p.G = c.Hq / c.Hkv; p.L = c.L; p.pairs = pairs;
   p.scale_log2 = c.scale * kLog2e;
   p.wait_cycles = tuning().wait_cycles;

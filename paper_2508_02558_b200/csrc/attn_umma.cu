@@ -912,6 +912,8 @@ bool umma_tail_is_fused(const AttnPlan& pl, int D, int M, int n1_max, bool pool,
   bool fused = merge_bytes <= 32 * 1024 && (!pool || n1_max <= 8192);
   const int forced = tuning().fused_tail;
   if (forced >= 0) fused = forced == 1 && (!pool || n1_max <= 8192);
+  // the last CTA is found with a counter per unit (without an override of the splits there are never that many)
+  if (pl.splits > 1 && pl.n_counters > kWsCounters) fused = false;
   return fused;
 }
 
@@ -978,7 +980,7 @@ AttnPlan plan_attention_umma(int D, int M, int b, int B, int Hkv, int n1_max, in
   pl.parts = pl.splits;                 // replicas are merged inside the CTA
   pl.rows_rep = 128 / pl.rep;
   pl.part_rows = pl.splits > 1 ? (size_t)pl.row_tiles * pl.splits * (M < 128 ? M : 128) : 0;
-  pl.n_counters = (size_t)B * Hkv * pl.row_tiles;
+  pl.n_counters = pl.splits > 1 ? (size_t)B * Hkv * pl.row_tiles : 0;
   pl.smem_bytes = umma_smem_bytes(D, pl.key_tile, pl.dual);
   // Few key splits of a small problem: make them one thread-block cluster, so that they merge through distributed shared
   // memory instead of the workspace. Only where the whole grid is one wave (a cluster needs all its SMs at once).

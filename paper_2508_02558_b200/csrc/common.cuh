@@ -10,6 +10,13 @@ namespace sdllm {
 
 constexpr int kMaxRows = 256;         // b * G rows of one KV head handled by one CTA
 constexpr int kMaxSplits = 64;        // key-axis splits per (sequence, KV head)
+// Workspace of the attention calls: [status word][counters][everything else]. One workspace serves calls of every kind in turn,
+// and each call finds its counters at zero because the one before left them so; a call therefore keeps its data out of all of
+// the first kWsDataOffset bytes, also when its own plan uses no counter.
+constexpr size_t kWsStatusBytes = 256;
+constexpr size_t kWsCounters = 192;   // the query-row kernel counts per (sequence, KV head, row tile) and splits the keys of at most half
+                                      // as many of these as there are SMs (umma_tail_is_fused); the streaming kernel takes two
+constexpr size_t kWsDataOffset = kWsStatusBytes + kWsCounters * sizeof(int32_t);
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
@@ -37,7 +44,7 @@ struct AttnPlan {
   bool dual;        // tcgen05 kernel, small-footprint variant: two CTAs per SM
   bool persistent;  // key-row kernel, streaming variant: one resident CTA per SM walks the units
   size_t part_rows; // partial rows per (sequence, KV head) in the workspace (0: none)
-  size_t n_counters;// completion counters in the workspace
+  size_t n_counters;// counters that the kernel uses, of the workspace's kWsCounters
 };
 
 // Key sources of one attention launch. The virtual key axis is [src1 rows 0..n1) ++ [src2 rows 0..n2).
@@ -98,6 +105,10 @@ struct CompactParams {
   int64_t kv_stride_bytes[3], c_stride_bytes[3];
 };
 
+struct AttnWorkspace {         // offsets in bytes; what lies at an offset ends where the next one begins
+  size_t part_o, part_ml, raw, lse, total;
+};
+AttnWorkspace attn_workspace(const sdllm_desc* d, const AttnPlan& pl, bool scores);
 AttnPlan plan_attention(int dtype, int D, int M, int b, int B, int Hkv, int n1_max, int n2, bool prob_scores);
 cudaError_t launch_prob_saliency(const AttnParams& p, int D, cudaStream_t st);    // second pass of the probability saliency
 
@@ -115,7 +126,10 @@ struct DenseCall {
 };
 cudaError_t launch_dense(const DenseCall& c, cudaStream_t st);
 int dense_launches(int B, int Hq, int L);             // kernel launches of one call
-size_t dense_workspace_bytes(int B, int Hq, int L, int D);
+struct DenseWorkspace {
+  size_t part_o, part_ml, total;
+};
+DenseWorkspace dense_workspace(int B, int Hq, int L, int D);
 cudaError_t launch_attn_partial(const AttnParams& p, const AttnPlan& plan, int dtype, int D, cudaStream_t st);
 cudaError_t launch_merge_pool(const MergeParams& p, cudaStream_t st);
 cudaError_t launch_select_topk(const SelectParams& p, cudaStream_t st);
