@@ -615,7 +615,9 @@ bool pair_supported(int dtype, int D, int M, int b) {
 // The key splits of a unit, at most one wave of CTAs in all. Costs in us, fitted to sweeps over 1 to 16 units of 5 to 256 tiles:
 // a tile takes 1.0 (one Q tile) or 1.55 (two), the partial rows 0.43 per MB on their way to the fold and back, and a reuse step
 // without splits saves the second launch. (8 units x 17 tiles: 9 splits of two tiles 10.4, 17 of one 11.2; 4 units x 9 tiles of
-// two Q tiles: 9 splits 10.5, 6 splits 11.9; 8 units x 129 tiles: flat from 12 to 18, 22.4.)
+// two Q tiles: 9 splits 10.5, 6 splits 11.9; 8 units x 129 tiles: flat from 12 to 18, 22.4. Refresh calls of 1 to 37 units x 5 to
+// 256 tiles, every split count: the model's choice is 1.8 % behind the fastest on average; 21 % at worst, 16 units x 9 tiles of two Q
+// tiles, which nine splits take in 14.3 and its three in 17.3.)
 AttnPlan plan_attention_pair(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn) {
   (void)b;
   AttnPlan pl{};
@@ -635,8 +637,6 @@ AttnPlan plan_attention_pair(int D, int M, int b, int B, int Hkv, int n1_max, in
                         (s > 1 ? 0.43e-6 * (double)units * s * pl.row_tiles * 128 * D * 4 + (n2 > 0 ? 2.5 : 0.) : 0.);
     if (cost < least) { least = cost; pl.splits = s; }
   }
-  // refresh, 8 units: sixteen splits measured 2 % ahead of seventeen and eighteen (40.2 against 41.0 us at 256 tiles)
-  if (n2 == 0 && pl.splits > 16 && pl.splits < 24) pl.splits = 16;
   if (tn.splits > 0) pl.splits = tn.splits < tiles ? tn.splits : (tiles > 0 ? tiles : 1);
   pl.parts = pl.splits;
   pl.part_rows = pl.splits > 1 ? (size_t)pl.row_tiles * pl.splits * 128 : 0;

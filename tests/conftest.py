@@ -33,3 +33,18 @@ def tuning():
             B.tuning_set(name, value)
     yield apply
     B.tuning_reset()
+
+
+@pytest.fixture
+def host_program(tmp_path):
+    """Compile a program of tests/native/ against the library's headers and libsdllm.so (host code only); returns its path."""
+    def compile_program(source: str) -> str:
+        import subprocess
+        from paper_2508_02558_b200 import build as libbuild
+        lib = libbuild.build()
+        include = [os.path.join(ROOT, "include"), libbuild.CSRC, os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")]
+        exe = str(tmp_path / source.split(".")[0])
+        subprocess.run([os.environ.get("CXX", "g++"), "-O1", "-std=c++17", *(f"-I{d}" for d in include), "-o", exe,
+                        os.path.join(ROOT, "tests", "native", source), lib, f"-Wl,-rpath,{os.path.dirname(lib)}"], check=True)
+        return exe
+    return compile_program

@@ -1,5 +1,4 @@
 """One workspace serves every attention call of a layer: the counters that a call expects at zero lie where no call keeps data."""
-import os
 import subprocess
 
 import numpy as np
@@ -8,20 +7,13 @@ import torch
 
 import oracle
 from paper_2508_02558_b200 import binding as B
-from paper_2508_02558_b200 import build as libbuild
 from paper_2508_02558_b200 import workloads as W
 
-ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
-
-def test_no_plan_keeps_data_among_the_counters(tmp_path):
+def test_no_plan_keeps_data_among_the_counters(host_program):
     """Every planner of the library, the overrides of the key splits included, over batches, heads, blocks and lengths."""
-    lib = libbuild.build()
-    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
-    exe = tmp_path / "workspace_ranges"
-    subprocess.run(["g++", "-O1", "-std=c++17", "-I", os.path.join(ROOT, "include"), "-I", libbuild.CSRC, "-I", os.path.join(cuda, "include"),
-                    "-o", str(exe), os.path.join(ROOT, "tests", "native", "workspace_ranges.cpp"), lib, f"-Wl,-rpath,{os.path.dirname(lib)}"], check=True)
-    res = subprocess.run([str(exe)], capture_output=True, text=True)
+    exe = host_program("workspace_ranges.cpp")
+    res = subprocess.run([exe], capture_output=True, text=True)
     assert res.returncode == 0, res.stdout + res.stderr
     assert all(int(x) > 0 for x in res.stdout.split()), res.stdout        # the walk met every kind of user
 
