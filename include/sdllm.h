@@ -20,6 +20,8 @@
  *   - Arguments are validated on the host before anything is launched: a bad argument returns a
  *     status and launches nothing. Kernels never trap or assert.
  *   - Positions >= seq_len[i] of sequence i are padding and are ignored.
+ *   - A NaN among the scaled logits of an attention row, or a logit of +inf, makes the row's output NaN (and its
+ *     log-sum-exp); other rows are not affected.
  */
 #ifndef SDLLM_H_
 #define SDLLM_H_

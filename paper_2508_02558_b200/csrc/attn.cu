@@ -512,13 +512,13 @@ __global__ void __launch_bounds__(256) merge_pool_kernel(const MergeParams p) {
       float bm = mstar;
 #pragma unroll
       for (int u = 0; u < MB; ++u)
-        if (s0 + u < p.splits && x[u].y > 0.f) bm = fmaxf(bm, x[u].x);
+        if (s0 + u < p.splits && x[u].y != 0.f) bm = fmaxf(bm, x[u].x);
       const float a = bm == -INFINITY ? 1.f : exp2f(mstar - bm);       // 0 on the first batch with data
       acc.x *= a; acc.y *= a; acc.z *= a; acc.w *= a; l *= a;
       mstar = bm;
 #pragma unroll
       for (int u = 0; u < MB; ++u) {
-        if (s0 + u >= p.splits || !(x[u].y > 0.f)) continue;
+        if (s0 + u >= p.splits || x[u].y == 0.f) continue;
         const float w = exp2f(x[u].x - bm);
         l = fmaf(x[u].y, w, l);
         acc.x = fmaf(o[u].x, w, acc.x); acc.y = fmaf(o[u].y, w, acc.y); acc.z = fmaf(o[u].z, w, acc.z); acc.w = fmaf(o[u].w, w, acc.w);

@@ -275,8 +275,8 @@ __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __
         const bool grow = m_new > m_run + 8.f;          // also true on the first finite maximum
         if (__any_sync(0xffffffffu, grow)) {
           const float alpha = grow ? fast_exp2(m_run - m_new) : 1.f;      // 0 when m_run is -inf
-          if (grow) m_run = m_new;
-          l_run *= alpha;
+          if (grow) m_run = m_new == INFINITY ? NAN : m_new;       // a logit of +inf: the row is NaN from here on
+          l_run = l_run < kNanSum ? l_run * alpha : NAN;
           if (j > 0) {
             // every PV of this query tile issued so far must have landed before its rows are rewritten
             if (!wait_bar_warp(BAR(PV_DONE + t), (j - 1) & 1, abort_flag, p.status, 28, p.wait_cycles)) { ok = false; break; }
@@ -343,6 +343,8 @@ __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __
       if (ok) ok = (!CUT || nt > 0) && wait_bar_warp(BAR(PV_DONE + t), (nt - 1) & 1, abort_flag, p.status, 30, p.wait_cycles);
       tc_fence_after();
       const int r_glob = row00 + t * 128 + row;
+      // (written behind the wait: ahead of it, two selects on l_run cost the loop above 3 %)
+      const float l_fin = l_run >= kNanSum ? NAN : (m_run == -INFINITY && l_run < 1.f ? 0.f : l_run);   // 0: only logits of -inf, which poly_exp2 does not make 0
       if constexpr (CUT) {
         // A share of a unit: un-normalised rows and their (maximum, sum) go to the workspace, float4 columns apart so that the
         // lanes of a warp write in a row; dense_fold_kernel folds them.
@@ -360,9 +362,9 @@ __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __
                                                          __uint_as_float(ov[4 * i + 3])));
           }
         }
-        __stcg(reinterpret_cast<float2*>(p.part_ml) + slot * 256 + t * 128 + row, make_float2(m_run, ok ? l_run : 0.f));
+        __stcg(reinterpret_cast<float2*>(p.part_ml) + slot * 256 + t * 128 + row, make_float2(m_run, ok ? l_fin : 0.f));
       } else if (ok) {
-        const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
+        const float inv = l_fin != 0.f ? 1.f / l_fin : 0.f;
         __nv_bfloat16* orow = reinterpret_cast<__nv_bfloat16*>(p.out) + (int64_t)bi * p.o_stride[0] + (int64_t)h * p.o_stride[1] +
                               (int64_t)r_glob * p.o_stride[2];
 #pragma unroll 1
@@ -382,7 +384,7 @@ __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __
             }
           }
         }
-        if (r_glob < n && p.lse) p.lse[((int64_t)bi * p.Hq + h) * p.L + r_glob] = (m_run + log2f(l_run)) * kLn2;
+        if (r_glob < n && p.lse) p.lse[((int64_t)bi * p.Hq + h) * p.L + r_glob] = (m_run + log2f(l_fin)) * kLn2;
       }
     }
   }
@@ -432,19 +434,19 @@ __global__ void __launch_bounds__(256) dense_fold_kernel(const DenseParams p) {
     float bm = m;
 #pragma unroll
     for (int u = 0; u < MB; ++u)
-      if (s0 + u < p.parts && x[u].y > 0.f) bm = fmaxf(bm, x[u].x);
+      if (s0 + u < p.parts && x[u].y != 0.f) bm = fmaxf(bm, x[u].x);
     const float a = bm == -INFINITY ? 1.f : fast_exp2(m - bm);           // 0 on the first batch with data
     acc.x *= a; acc.y *= a; acc.z *= a; acc.w *= a; l *= a;
     m = bm;
 #pragma unroll
     for (int u = 0; u < MB; ++u) {
-      if (s0 + u >= p.parts || !(x[u].y > 0.f)) continue;
+      if (s0 + u >= p.parts || x[u].y == 0.f) continue;
       const float w = fast_exp2(x[u].x - bm);
       l = fmaf(x[u].y, w, l);
       acc.x = fmaf(v[u].x, w, acc.x); acc.y = fmaf(v[u].y, w, acc.y); acc.z = fmaf(v[u].z, w, acc.z); acc.w = fmaf(v[u].w, w, acc.w);
     }
   }
-  const float inv = l > 0.f ? 1.f / l : 0.f;
+  const float inv = l != 0.f ? 1.f / l : 0.f;
   __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(p.out) + (int64_t)bi * p.o_stride[0] + (int64_t)h * p.o_stride[1] + (int64_t)r * p.o_stride[2] + c4 * 4;
   *reinterpret_cast<uint2*>(out) = make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
   if (c4 == 0 && p.lse) p.lse[((int64_t)bi * p.Hq + h) * p.L + r] = (m + log2f(l)) * kLn2;

@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(64 + 128 * WG * CG, (WG == 1 && CG == 1) ? 2 :
       softmax_barrier_all<NG>();         // both warpgroups' references and sums are posted
       if (wg == 0 && st < NP) {
         const float mb = m_b[st], lb = l_b[st];
-        const bool ha = l_mine > 0.f, hb = lb > 0.f;
+        const bool ha = l_mine != 0.f, hb = lb != 0.f;
         const float ms = fmaxf(ha ? m_mine : -INFINITY, hb ? mb : -INFINITY);
         l_mine = (ha ? l_mine * fast_exp2(m_mine - ms) : 0.f) + (hb ? lb * fast_exp2(mb - ms) : 0.f);
         m_mine = ms;
@@ -569,7 +569,7 @@ __global__ void __launch_bounds__(64 + 128 * WG * CG, (WG == 1 && CG == 1) ? 2 :
         const float lav[4] = {la.x, la.y, la.z, la.w}, lbv[4] = {lb.x, lb.y, lb.z, lb.w};
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          const bool ha = lav[u] > 0.f, hb = lbv[u] > 0.f;
+          const bool ha = lav[u] != 0.f, hb = lbv[u] != 0.f;
           const float ms = fmaxf(ha ? mav[u] : -INFINITY, hb ? mbv[u] : -INFINITY);
           const float f = wg == 0 ? (ha ? fast_exp2(mav[u] - ms) : 0.f) : (hb ? fast_exp2(mbv[u] - ms) : 0.f);
           ov[4 * c4 + u] = __float_as_uint(__uint_as_float(ov[4 * c4 + u]) * f);
@@ -667,11 +667,11 @@ __global__ void __launch_bounds__(64 + 128 * WG * CG, (WG == 1 && CG == 1) ? 2 :
         float mstar = -INFINITY;
 #pragma unroll
         for (int s2 = 0; s2 < MS; ++s2)
-          if (s2 < S && x[s2].y > 0.f) mstar = fmaxf(mstar, x[s2].x);
+          if (s2 < S && x[s2].y != 0.f) mstar = fmaxf(mstar, x[s2].x);
         float w[MS], l = 0.f;
 #pragma unroll
         for (int s2 = 0; s2 < MS; ++s2) {
-          w[s2] = (s2 < S && x[s2].y > 0.f) ? fast_exp2(x[s2].x - mstar) : 0.f;
+          w[s2] = (s2 < S && x[s2].y != 0.f) ? fast_exp2(x[s2].x - mstar) : 0.f;
           l = fmaf(x[s2].y, w[s2], l);
         }
         const float inv = l > 0.f ? 1.f / l : 0.f;

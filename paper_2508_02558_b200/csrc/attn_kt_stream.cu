@@ -580,7 +580,7 @@ __global__ void __launch_bounds__(KS_THREADS, 1) attn_kt_stream_kernel(const __g
         pair_sync(7);                                  // warpgroup 1 has posted this unit's references and sums
         if (st < NP) {
           const float mb = post_other[(k & 1) * 64 + st], lb = post_other[(k & 1) * 64 + 32 + st];
-          const bool ha = l_mine > 0.f, hb = lb > 0.f;
+          const bool ha = l_mine != 0.f, hb = lb != 0.f;
           const float ms = fmaxf(ha ? m_mine : -INFINITY, hb ? mb : -INFINITY);
           const float fa = ha ? fast_exp2(m_mine - ms) : 0.f, fb = hb ? fast_exp2(mb - ms) : 0.f;
           const float l = l_mine * fa + lb * fb;

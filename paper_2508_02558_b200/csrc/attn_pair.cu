@@ -353,8 +353,8 @@ __global__ void __launch_bounds__(PR_THREADS, 1) attn_pair_kernel(const __grid_c
       const bool grow = m_new > m_run + 8.f;              // also true on the first finite maximum
       if (__any_sync(0xffffffffu, grow)) {
         const float alpha = grow ? fast_exp2(m_run - m_new) : 1.f;        // 0 when m_run is -inf
-        if (grow) m_run = m_new;
-        l_run *= alpha;
+        if (grow) m_run = m_new == INFINITY ? NAN : m_new;       // a logit of +inf: the row is NaN from here on
+        l_run = l_run < kNanSum ? l_run * alpha : NAN;
         if (k > 0) {
           // every P V of this warpgroup issued so far must have landed before its rows are rewritten
           if (!wait_bar_warp(BAR(PV_DONE + w), (k - 1) & 1, abort_flag, p.status, 50, p.wait_cycles)) { ok = false; break; }
@@ -426,7 +426,8 @@ __global__ void __launch_bounds__(PR_THREADS, 1) attn_pair_kernel(const __grid_c
     const int64_t part = ((int64_t)((bi * p.Hkv + g) * Sh::QT + (TWO ? w : 0)) * p.splits + split) * 128;     // rows of partials in front
     float4* part_o = reinterpret_cast<float4*>(p.part_o) + part * (D / 4) + row;
     float2* part_ml = reinterpret_cast<float2*>(p.part_ml) + part + row;
-    float m_row = m_run, l_row = have ? l_run : 0.f, w_own = 1.f, w_other = 0.f;
+    const float l_fin = l_run >= kNanSum ? NAN : (m_run == -INFINITY && l_run < 1.f ? 0.f : l_run);     // 0: only logits of -inf, which poly_exp2 does not make 0
+    float m_row = m_run, l_row = have ? l_fin : 0.f, w_own = 1.f, w_other = 0.f;
     int c_lo = 0, c_hi = D / 16;                          // columns, in chunks of 16, that this warpgroup carries out
     const float4* other = nullptr;                        // the other warpgroup's accumulator for them
     if constexpr (!TWO) {
@@ -452,16 +453,16 @@ __global__ void __launch_bounds__(PR_THREADS, 1) attn_pair_kernel(const __grid_c
       ml_s[w * 128 + row] = make_float2(m_row, l_row);
       asm volatile("bar.sync 1, 256;\n" ::: "memory");
       const float2 o2 = ml_s[(1 - w) * 128 + row];
-      const float mm = fmaxf(l_row > 0.f ? m_row : -INFINITY, o2.y > 0.f ? o2.x : -INFINITY);
-      w_own = l_row > 0.f ? fast_exp2(m_row - mm) : 0.f;
-      w_other = o2.y > 0.f ? fast_exp2(o2.x - mm) : 0.f;
-      l_row = l_row * w_own + (o2.y > 0.f ? o2.y * w_other : 0.f);
+      const float mm = fmaxf(l_row != 0.f ? m_row : -INFINITY, o2.y != 0.f ? o2.x : -INFINITY);
+      w_own = l_row != 0.f ? fast_exp2(m_row - mm) : 0.f;
+      w_other = o2.y != 0.f ? fast_exp2(o2.x - mm) : 0.f;
+      l_row = l_row * w_own + (o2.y != 0.f ? o2.y * w_other : 0.f);
       m_row = mm;
       c_lo = w * (D / 32); c_hi = c_lo + D / 32;
       other = box + (1 - w) * (D / 8) * 128 + row;
     }
     const bool first_half = TWO || w == 0;                // who writes the row's sum
-    const float inv = p.splits == 1 ? (l_row > 0.f ? 1.f / l_row : 0.f) : 1.f;
+    const float inv = p.splits == 1 ? (l_row != 0.f ? 1.f / l_row : 0.f) : 1.f;
     if (!*abort_flag) {
 #pragma unroll 1
       for (int c = c_lo; c < c_hi; ++c) {
@@ -479,7 +480,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) attn_pair_kernel(const __grid_c
           v[e] = make_float4(__uint_as_float(ov[4 * e]), __uint_as_float(ov[4 * e + 1]), __uint_as_float(ov[4 * e + 2]), __uint_as_float(ov[4 * e + 3]));
           if constexpr (!TWO) {
             v[e].x *= w_own; v[e].y *= w_own; v[e].z *= w_own; v[e].w *= w_own;
-            if (w_other > 0.f) {
+            if (w_other != 0.f) {
               const float4 y = other[((c - c_lo) * 4 + e) * 128];
               v[e].x = fmaf(y.x, w_other, v[e].x); v[e].y = fmaf(y.y, w_other, v[e].y);
               v[e].z = fmaf(y.z, w_other, v[e].z); v[e].w = fmaf(y.w, w_other, v[e].w);
@@ -548,19 +549,19 @@ __global__ void __launch_bounds__(128) pair_tail_kernel(const PairParams pp, con
       float bm = m_run;
 #pragma unroll
       for (int u = 0; u < MB; ++u)
-        if (ml[u].y > 0.f) bm = fmaxf(bm, ml[u].x);
+        if (ml[u].y != 0.f) bm = fmaxf(bm, ml[u].x);
       const float a = (bm == -INFINITY) ? 1.f : fast_exp2(m_run - bm);    // 0 on the first batch with data
       l *= a; acc.x *= a; acc.y *= a; acc.z *= a; acc.w *= a;
       m_run = bm;
 #pragma unroll
       for (int u = 0; u < MB; ++u) {
-        if (!(ml[u].y > 0.f)) continue;
+        if (ml[u].y == 0.f) continue;
         const float w = fast_exp2(ml[u].x - bm);
         l = fmaf(ml[u].y, w, l);
         acc.x = fmaf(v[u].x, w, acc.x); acc.y = fmaf(v[u].y, w, acc.y); acc.z = fmaf(v[u].z, w, acc.z); acc.w = fmaf(v[u].w, w, acc.w);
       }
     }
-    const float inv = l > 0.f ? 1.f / l : 0.f;
+    const float inv = l != 0.f ? 1.f / l : 0.f;
     __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(p.out) + (int64_t)bi * p.o_stride[0] + (int64_t)(g * p.G + hg) * p.o_stride[1] +
                          (int64_t)i * p.o_stride[2] + c4 * 4;
     *reinterpret_cast<uint2*>(out) = make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));

@@ -93,13 +93,13 @@ __device__ __forceinline__ void merge_slots(const AttnParams& p, int64_t unit, i
       float bm = m_run[s];
 #pragma unroll
       for (int u = 0; u < MB; ++u)
-        if (p0 + u < P && x[s][u].y > 0.f) bm = fmaxf(bm, x[s][u].x);
+        if (p0 + u < P && x[s][u].y != 0.f) bm = fmaxf(bm, x[s][u].x);
       const float a = (bm == -INFINITY) ? 1.f : fast_exp2(m_run[s] - bm);    // 0 on the first batch with data
       acc[s].x *= a; acc[s].y *= a; acc[s].z *= a; acc[s].w *= a; l[s] *= a;
       m_run[s] = bm;
 #pragma unroll
       for (int u = 0; u < MB; ++u) {
-        if (p0 + u >= P || !(x[s][u].y > 0.f)) continue;
+        if (p0 + u >= P || x[s][u].y == 0.f) continue;
         const float w = fast_exp2(x[s][u].x - bm);
         l[s] = fmaf(x[s][u].y, w, l[s]);
         acc[s].x = fmaf(o[s][u].x, w, acc[s].x); acc[s].y = fmaf(o[s][u].y, w, acc[s].y);
@@ -631,14 +631,14 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
     float mstar = -INFINITY;
     for (int r2 = 0; r2 < R; ++r2) {
       const float2 x = ml_s[r2 * rows_rep + m_local];
-      if (x.y > 0.f) mstar = fmaxf(mstar, x.x);
+      if (x.y != 0.f) mstar = fmaxf(mstar, x.x);
     }
     float lsum = 0.f;
     for (int r2 = 0; r2 < R; ++r2) {
       const float2 x = ml_s[r2 * rows_rep + m_local];
-      if (x.y > 0.f) lsum = fmaf(x.y, fast_exp2(x.x - mstar), lsum);
+      if (x.y != 0.f) lsum = fmaf(x.y, fast_exp2(x.x - mstar), lsum);
     }
-    const float w = l_run > 0.f ? fast_exp2(m_run - mstar) : 0.f;       // this replica's weight in the merged row
+    const float w = l_run != 0.f ? fast_exp2(m_run - mstar) : 0.f;       // this replica's weight in the merged row
     if (rep == 0) lm_s[m_local] = make_float2(mstar, lsum);
     // the finished accumulator row: TMEM -> weight -> shared memory, 32 columns at a time
     const bool have_o = sm_ok && sm_tiles > 0 &&
@@ -746,12 +746,12 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
         float mstar = -INFINITY;
 #pragma unroll
         for (int c = 0; c < 8; ++c)
-          if (c < S && x[c].y > 0.f) mstar = fmaxf(mstar, x[c].x);
+          if (c < S && x[c].y != 0.f) mstar = fmaxf(mstar, x[c].x);
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
         float l = 0.f;
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
-          if (c >= S || !(x[c].y > 0.f)) continue;
+          if (c >= S || x[c].y == 0.f) continue;
           const float w = fast_exp2(x[c].x - mstar);
           l = fmaf(x[c].y, w, l);
           acc.x = fmaf(o[c].x, w, acc.x); acc.y = fmaf(o[c].y, w, acc.y); acc.z = fmaf(o[c].z, w, acc.z); acc.w = fmaf(o[c].w, w, acc.w);

@@ -114,6 +114,12 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   asm("max.f32 %0, %1, %2, %3;\n" : "=f"(r) : "f"(a), "f"(b), "f"(c));
   return r;
 }
+// The larger of two, NaN when either is.
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;\n" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
 // Two fp32 operations per instruction (same rounding as the scalar forms).
 __device__ __forceinline__ uint64_t pack_f2(float lo, float hi) {
   uint64_t r;
@@ -134,9 +140,11 @@ __device__ __forceinline__ uint64_t add_f2(uint64_t a, uint64_t b) {
 // 2^x for two values on the FMA pipe, beside the exponential unit (16 results per clock and SM, the bottleneck of a softmax
 // that feeds tcgen05): x = n + f with n the nearest integer (round by adding 1.5 * 2^23), 2^f by the degree-5 polynomial of
 // least relative error on [-1/2, 1/2] (Remez exchange; 7.5e-8, 2.1e-7 evaluated in fp32 - ex2.approx is within 2.4e-7), n added
-// to the exponent. Values below 2^-126 come out as about 2^-126 instead of 0.
+// to the exponent. Values below 2^-126 come out as about 2^-126 instead of 0. NaN stays NaN up to the integer addition, which
+// makes the largest float of it: a row's sum of exponentials that reaches kNanSum has met one (ordinary sums stay below 2^8 a key).
+constexpr float kNanSum = 1e38f;
 __device__ __forceinline__ void poly_exp2(float x0, float x1, float& e0, float& e1) {
-  const uint64_t x = pack_f2(fmaxf(x0, -126.f), fmaxf(x1, -126.f));
+  const uint64_t x = pack_f2(max_nan(x0, -126.f), max_nan(x1, -126.f));
   const uint64_t magic = pack_f2(12582912.f, 12582912.f), minus_one = pack_f2(-1.f, -1.f);
   const uint64_t t = add_f2(x, magic);
   const uint64_t f = add_f2(x, fma_f2(t, minus_one, magic));

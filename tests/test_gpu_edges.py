@@ -128,3 +128,62 @@ def test_pooling_while_the_resident_walk_goes_on(lens, window, policy, ctas, tun
         g = U.gpu_refresh(q, k, v, bw.seq_len, bo, "bf16", 0.5, window, **policy)
         U.check_refresh_against_oracle(g, q, np.nan_to_num(k), np.nan_to_num(v), bw.seq_len, bo, "bf16", 0.5, window,
                                        select=policy.get("select", oracle.SELECT_JOINT_FLOOR), pool_kind=policy.get("pool", oracle.POOL_MAX))
+
+
+@pytest.mark.parametrize("op,Hkv,G,D,dtype,plan", [
+    ("dense", 8, 1, 128, "bf16", {}), ("dense", 8, 2, 64, "bf16", dict(ws=256)),          # units cut along the keys, and whole ones
+    ("refresh", 8, 4, 128, "bf16", dict(splits=1)), ("refresh", 8, 4, 64, "bf16", dict(splits=3)), ("refresh", 8, 7, 128, "bf16", {}),
+    ("reuse", 8, 4, 128, "bf16", {}), ("reuse", 8, 7, 128, "bf16", dict(splits=1)),
+    ("refresh", 8, 1, 128, "bf16", {}), ("refresh", 8, 1, 128, "bf16", dict(splits=1)), ("reuse", 8, 1, 128, "bf16", dict(splits=1, persist=1)),
+    ("prob", 8, 1, 128, "bf16", {}), ("prob", 8, 4, 128, "bf16", dict(splits=3)), ("refresh", 8, 2, 64, "f32", {}), ("reuse", 8, 1, 128, "f32", {}),
+    ("refresh", 8, 1, 128, "bf16", dict(kernel=1, splits=3)),
+])
+@pytest.mark.parametrize("bad", ["nan", "inf"])
+def test_a_logit_that_is_not_finite_makes_its_rows_nan(op, Hkv, G, D, dtype, plan, bad, tuning):
+    """One key of each head (and one query row) is NaN, or infinite in a dimension where the queries have either sign: NaN or +inf among a row's logits
+    makes its output (and log-sum-exp) NaN, -inf only takes the key out, and no other row changes - whichever unit computes the
+    key's exponential and however the keys are split."""
+    from parity_util import assert_close, to_dev, to_host_f32
+    plan = dict(plan)
+    ws_bytes = plan.pop("ws", None)
+    tuning(**plan)
+    b, L, n_kept = 32, 300, 268
+    rng = np.random.default_rng(Hkv * G + D)
+    n_rows = L if op == "dense" else b
+    q = (rng.standard_normal((1, Hkv * G, n_rows, D)) / np.sqrt(D)).astype(np.float32)
+    k, v = (rng.standard_normal((1, Hkv, L, D)).astype(np.float32) for _ in range(2))
+    at = [None, 0 if bad == "nan" else 1, 6, 7, 70, 135, 262, 299]        # (1: see the key-row kernel's references, lent by a first key)
+    for h, j in enumerate(at):
+        if j is not None:
+            k[0, h, j, :1 if bad == "inf" else D] = np.nan if bad == "nan" else np.inf
+    q[:, :, ::2, 0], q[:, :, 1::2, 0] = np.abs(q[:, :, ::2, 0]) + 0.1, -np.abs(q[:, :, 1::2, 0]) - 0.1
+    if bad == "nan":
+        q[0, 0, 5] = np.nan                                               # a row without a finite logit
+    qd, kd, vd = (to_dev(x, dtype) for x in (q, k, v))
+    d = B.make_desc(batch=1, n_q_heads=Hkv * G, n_kv_heads=Hkv, head_dim=D, seq_len_max=L, block_len=b, dtype=B.BF16 if dtype == "bf16" else B.F32,
+                    retention=0.5, n_keep_max=n_kept, score=B.SCORE_PROB_MEAN if op == "prob" else B.SCORE_LOGIT_MEAN)
+    code = {"dense": B.OP_DENSE_ATTN, "reuse": B.OP_SPARSE_BLOCK_ATTN}.get(op, B.OP_REFRESH_SCORES)
+    ws = torch.zeros((ws_bytes or B.workspace_bytes(d, code),), dtype=torch.uint8, device="cuda")
+    out, lse = torch.full_like(qd, 7.0), torch.full((1, Hkv * G, n_rows), 7.0, device="cuda")
+    if op == "dense":
+        B.dense_attn(d, qd, kd, vd, None, out, lse, ws)
+    elif op == "reuse":
+        kc, vc, kn, vn = kd[:, :, :n_kept].contiguous(), vd[:, :, :n_kept].contiguous(), kd[:, :, n_kept:].contiguous(), vd[:, :, n_kept:].contiguous()
+        B.sparse_block_attn(d, qd, kc, vc, torch.tensor([n_kept], dtype=torch.int32, device="cuda"), kn, vn, out, ws)
+    else:
+        pooled = torch.empty((1, Hkv, L), device="cuda")
+        B.refresh_scores(d, qd, kd, vd, None, torch.tensor([64], dtype=torch.int32, device="cuda"), out, lse, pooled, ws)
+    torch.cuda.synchronize()
+    assert B.read_status(ws) == 0
+    q64, k64, v64 = (x.cpu().double() for x in (qd, kd.repeat_interleave(G, 1), vd.repeat_interleave(G, 1)))
+    s = q64 @ k64.transpose(-1, -2) / np.sqrt(D)
+    ref, ref_lse = (torch.softmax(s, -1) @ v64).numpy(), torch.logsumexp(s, -1).numpy()
+    got = to_host_f32(out)
+    bad_rows = np.isnan(ref)
+    assert bad_rows.any() and not bad_rows.all()
+    np.testing.assert_array_equal(np.isnan(got), bad_rows)
+    assert_close(np.where(bad_rows, 0, got), np.where(bad_rows, 0, ref), dtype, op)
+    if op != "reuse":
+        rows = bad_rows[..., 0]
+        assert not np.isfinite(lse.cpu().numpy()[rows]).any()
+        np.testing.assert_allclose(lse.cpu().numpy()[~rows], ref_lse[~rows], rtol=0, atol=1e-4)
