@@ -97,6 +97,7 @@ __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __
   const int S_FULL = 1 + 4 * NS, P_FULL = S_FULL + 2, PV_DONE = S_FULL + 6, DRAIN = S_FULL + 8;   // P_FULL: two parts per query tile
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + 256);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + 260);
+  int* issued_s = reinterpret_cast<int*>(smem + 264);        // [2] tiles whose K / V loads are on their way (for an aborted CTA's way out)
   unsigned char* q_s = smem + 1024;
   unsigned char* stage0 = q_s + 2 * TILE;
 
@@ -115,6 +116,7 @@ __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __
     }
     mbar_init(BAR(DRAIN), 1);
     *abort_flag = 0;
+    issued_s[0] = issued_s[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   if (warp == 1) {                          // the MMA warp owns the tensor memory
@@ -139,30 +141,21 @@ __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __
         for (int t = 0; t < (act1 ? 2 : 1); ++t)
           for (int hh = 0; hh < H; ++hh)
             tma_load_4d(smem_u32(q_s + t * TILE + hh * HALF), &tm.q, BAR(Q_FULL), hh * 64, row00 + t * 128, h, bi);
-        int issued = 0;
-        bool ok = true;
-        for (int j = 0; j < nt && ok; ++j) {
+        int k_issued = 0, v_issued = 0;
+        for (int j = 0; j < nt; ++j) {
           const int s = j % NS;
           const uint32_t ph = ((j / NS) - 1) & 1;
           const uint32_t kdst = smem_u32(stage0 + (size_t)s * 2 * TILE), vdst = kdst + TILE;
-          if (j >= NS && !wait_bar(BAR(EMPTY_K + s), ph, abort_flag, p.status, 21, p.wait_cycles)) { ok = false; break; }
+          if (j >= NS && !wait_bar(BAR(EMPTY_K + s), ph, abort_flag, p.status, 21, p.wait_cycles)) break;
           mbar_expect_tx(BAR(FULL_K + s), (uint32_t)TILE);
           for (int hh = 0; hh < H; ++hh) tma_load_4d(kdst + hh * HALF, &tm.k, BAR(FULL_K + s), hh * 64, (t0 + j) * KT, g, bi);
-          if (j >= NS && !wait_bar(BAR(EMPTY_V + s), ph, abort_flag, p.status, 22, p.wait_cycles)) {
-            drain_bar(BAR(FULL_K + s), (j / NS) & 1);                 // the K half of this slot is already on its way
-            ok = false; break;
-          }
+          k_issued = j + 1;
+          if (j >= NS && !wait_bar(BAR(EMPTY_V + s), ph, abort_flag, p.status, 22, p.wait_cycles)) break;
           mbar_expect_tx(BAR(FULL_V + s), (uint32_t)TILE);
           for (int hh = 0; hh < H; ++hh) tma_load_4d(vdst + hh * HALF, &tm.v, BAR(FULL_V + s), hh * 64, (t0 + j) * KT, g, bi);
-          issued = j + 1;
+          v_issued = j + 1;
         }
-        if (*abort_flag) {                    // let the copies that were issued land before the CTA retires
-          for (int j = max(issued - NS, 0); j < issued; ++j) {
-            drain_bar(BAR(FULL_K + j % NS), (j / NS) & 1);
-            drain_bar(BAR(FULL_V + j % NS), (j / NS) & 1);
-          }
-          drain_bar(BAR(Q_FULL), 0);
-        }
+        issued_s[0] = k_issued; issued_s[1] = v_issued;
       }
     } else if (warp == 1) {
       // ======================================= MMA issuer =======================================
@@ -228,11 +221,6 @@ __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __
         if (!issue_pv(0, j, !act1)) { ok = false; break; }
       }
       if (ok && act1) ok = issue_pv(1, nt - 1, true);
-      if (*abort_flag && leader) {            // wait for the tensor pipe to finish what was issued before TMEM is freed
-        tc_commit(BAR(DRAIN));
-        drain_bar(BAR(DRAIN), 0);
-      }
-      __syncwarp();
     }
   } else {
     // ======================================= softmax warps =======================================
@@ -297,7 +285,7 @@ __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __
         const int n_mma = (nv + 15) & ~15;
         if (t == 0 && nv < n_mma) {
           const int s = j % NS;
-          if (!wait_bar_warp(BAR(FULL_V + s), (j / NS) & 1, abort_flag, p.status, 29, p.wait_cycles)) { ok = false; break; }
+          if (!wait_bar_warp(BAR(FULL_V + s), (j / NS) & 1, abort_flag, p.status, 29, p.wait_cycles)) { tc_wait_st(); ok = false; break; }   // (stores to tensor memory may be under way)
           unsigned char* vs = stage0 + (size_t)s * 2 * TILE + TILE;
           const int nz = (n_mma - nv) * H * 8;           // 16-byte chunks to clear
           for (int i = q4 * 32 + lane; i < nz; i += 128) {
@@ -393,7 +381,17 @@ __global__ void __launch_bounds__(DN_THREADS, 1) dense_attn_bf16_kernel(const __
   if (CUT && p.second) grid_dependency_wait();      // this launch must not be over before the one in front of it is
   tc_fence_before();
   __syncthreads();
+  if (warp == 0) {
+    if (__builtin_expect(*abort_flag, 0)) {
+      if (lane == 0) {
+        drain_loads(BAR(FULL_K), issued_s[0], NS);
+        drain_loads(BAR(FULL_V), issued_s[1], NS);
+        if (issued_s[0] > 0) drain_bar(BAR(Q_FULL), 0);
+      }
+    }
+  }
   if (warp == 1) {
+    if (__builtin_expect(*abort_flag, 0)) drain_mmas(BAR(DRAIN));
     __syncwarp();
     tc_fence_after();
     tmem_dealloc(tmem_base, 512);

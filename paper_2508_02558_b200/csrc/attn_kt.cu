@@ -117,6 +117,7 @@ __global__ void __launch_bounds__(64 + 128 * WG * CG, (WG == 1 && CG == 1) ? 2 :
   constexpr int S_FULL = 1 + 4 * KT_MAX_STAGES, P_FULL = S_FULL + 2, PV_DONE = S_FULL + 4, DRAIN = S_FULL + 6, MERGE = S_FULL + 7;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + 256);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + 260);
+  int* issued_s = reinterpret_cast<int*>(smem + 264);      // [2] tiles whose K / V loads are on their way (for an aborted CTA's way out)
   // per softmax warpgroup: its index, and which tiles / columns it takes
   const int grp = (NG > 1 && warp >= 2) ? (warp - 2) >> 2 : 0;
   const int wg = WG == 2 ? grp : 0;        // tile parity it works on
@@ -258,13 +259,10 @@ __global__ void __launch_bounds__(64 + 128 * WG * CG, (WG == 1 && CG == 1) ? 2 :
       mbar_expect_tx(BAR(Q_FULL), (uint32_t)(H * N * 128));
       for (int h = 0; h < H; ++h) tma_load_4d(smem_u32(q_s + h * NPT * 128), &tm.q, BAR(Q_FULL), h * 64, 0, g * p.G, bi);
       while (t_next < T && issue_tile(t_next)) ++t_next;
-      if (*abort_flag) {
-        // let the copies that were issued land before the CTA retires
-        for (int j = max(k_issued - NS, 0); j < k_issued; ++j) drain_bar(BAR(FULL_K + j % NS), (j / NS) & 1);
-        for (int j = max(v_issued - NS, 0); j < v_issued; ++j) drain_bar(BAR(FULL_V + j % NS), (j / NS) & 1);
-        drain_bar(BAR(Q_FULL), 0);
-      }
+      issued_s[0] = k_issued; issued_s[1] = v_issued;
     }
+    __syncwarp();
+    asm volatile("bar.arrive 6, %0;\n" ::"n"(64 + 128 * NG) : "memory");      // (see the MMA warp's end)
   } else if (warp == 1) {
     // ======================================= MMA issuer =======================================
     // The whole warp walks the tiles and one elected lane issues: with everything around the MMAs warp-uniform, their
@@ -326,11 +324,19 @@ __global__ void __launch_bounds__(64 + 128 * WG * CG, (WG == 1 && CG == 1) ? 2 :
         if (++s == NS) { s = 0; par ^= 1u; }
       }
       if (ok && T > 0) ok = issue_pv(T - 1, s_prev, par_prev);
-      if (*abort_flag && leader) {       // wait for the tensor pipe to finish what was issued before TMEM is freed
-        tc_commit(BAR(DRAIN));
-        drain_bar(BAR(DRAIN), 0);
-      }
+      // The tensor memory is given back as soon as the softmax warps have read their accumulators (or given up): behind that
+      // barrier every wait of this CTA but the one for its peers' rows is over, and so is what it has issued, unless a wait gave
+      // up - then what is under way has to land first (drain_mmas).
       __syncwarp();
+      asm volatile("bar.sync 6, %0;\n" ::"n"(64 + 128 * NG) : "memory");
+      if (*abort_flag) {
+        drain_mmas(BAR(DRAIN));
+        drain_loads(BAR(FULL_K), issued_s[0], NS);
+        drain_loads(BAR(FULL_V), issued_s[1], NS);
+        drain_bar(BAR(Q_FULL), 0);
+      }
+      tc_fence_after();
+      tmem_dealloc(tmem_base, TMEM_COLS);
     }
   } else {
     // ======================================= softmax warps =======================================
@@ -556,6 +562,8 @@ __global__ void __launch_bounds__(64 + 128 * WG * CG, (WG == 1 && CG == 1) ? 2 :
 #pragma unroll
       for (int c = 0; c < NP; ++c) ov[c] = 0u;
     }
+    tc_fence_before();
+    asm volatile("bar.arrive 6, %0;\n" ::"n"(64 + 128 * NG) : "memory");
     if (fold) {
       // The rows cross in the first ring slot, once both warpgroups have seen their last PV complete. Every thread scales
       // its own row to the common references; the factors are recomputed from the posted references and sums.
@@ -724,15 +732,6 @@ __global__ void __launch_bounds__(64 + 128 * WG * CG, (WG == 1 && CG == 1) ? 2 :
     const int p_lo = (int)(((long long)split * p.n1_max) / S), p_hi = (int)(((long long)(split + 1) * p.n1_max) / S);
     const int o = p.block_off[bi];
     kt_pool_span(p, a, p.pooled + (int64_t)(bi * p.Hkv + g) * p.n1_max, n1, o, p_lo, p_hi, tid, NTHREADS);
-  }
-
-  // ---- free the tensor memory ----
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 1) {
-    __syncwarp();
-    tc_fence_after();
-    tmem_dealloc(tmem_base, TMEM_COLS);
   }
 }
 

@@ -71,6 +71,7 @@ __global__ void __launch_bounds__(KS_THREADS, 1) attn_kt_stream_kernel(const __g
   constexpr int S_FULL = 2 + 4 * NS, P_FULL = S_FULL + 2, PV_DONE = S_FULL + 4, DRAIN = S_FULL + 6, RAW_DONE = S_FULL + 7;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + 256);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + 260);
+  int* issued_s = reinterpret_cast<int*>(smem + 264);      // [3] tiles whose K / V loads, and units whose Q load, are on their way (for an aborted CTA's way out)
   volatile int* unit_list = reinterpret_cast<volatile int*>(smem + 320);   // [16] the units this CTA took, in order (-1: no more)
   volatile int* n_pub = reinterpret_cast<volatile int*>(smem + 384);       // entries of the list published so far
   volatile int* n_done = reinterpret_cast<volatile int*>(smem + 388);      // units whose results have been stored
@@ -255,12 +256,7 @@ __global__ void __launch_bounds__(KS_THREADS, 1) attn_kt_stream_kernel(const __g
         __threadfence_block();
         *n_pub = n_listed + 1;
       }
-      if (*abort_flag) {
-        // let the copies that were issued land before the CTA retires
-        for (int j = max(k_issued - NS, 0); j < k_issued; ++j) drain_bar(BAR(FULL_K + j % NS), (uint32_t)(j / NS) & 1u);
-        for (int j = max(G - NS, 0); j < G; ++j) drain_bar(BAR(FULL_V + j % NS), (uint32_t)(j / NS) & 1u);
-        if (qn > 0) drain_bar(BAR(Q_FULL), (uint32_t)(qn - 1) & 1u);
-      }
+      issued_s[0] = k_issued; issued_s[1] = G; issued_s[2] = qn;
     }
   } else if (warp == 1) {
     // ======================================= MMA issuer =======================================
@@ -325,11 +321,6 @@ __global__ void __launch_bounds__(KS_THREADS, 1) attn_kt_stream_kernel(const __g
         }
       }
       if (ok && pv_G >= 0) ok = issue_pv();
-      if (*abort_flag && leader) {       // wait for the tensor pipe to finish what was issued before TMEM is freed
-        tc_commit(BAR(DRAIN));
-        drain_bar(BAR(DRAIN), 0);
-      }
-      __syncwarp();
     }
   } else {
     // ======================================= softmax warps =======================================
@@ -644,6 +635,12 @@ __global__ void __launch_bounds__(KS_THREADS, 1) attn_kt_stream_kernel(const __g
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
+    if (*abort_flag) {
+      drain_mmas(BAR(DRAIN));
+      drain_loads(BAR(FULL_K), issued_s[0], NS);
+      drain_loads(BAR(FULL_V), issued_s[1], NS);
+      drain_loads(BAR(Q_FULL), issued_s[2], 1);
+    }
     __syncwarp();
     tc_fence_after();
     tmem_dealloc(tmem_base, TMEM_COLS);

@@ -83,6 +83,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) attn_pair_kernel(const __grid_c
   const int S_FULL = 1 + 4 * NS, P_FULL = S_FULL + 2, PV_DONE = S_FULL + 6, DRAIN = S_FULL + 8;   // P_FULL: two parts per warpgroup
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + 256);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + 260);
+  int* issued_s = reinterpret_cast<int*>(smem + 264);     // [2] tiles whose K / V loads are on their way (for an aborted CTA's way out)
   float* qbar_s = reinterpret_cast<float*>(smem + 512);
   unsigned char* q_s = smem + 1024;
   unsigned char* stage0 = q_s + Sh::QT * TILE;
@@ -100,13 +101,12 @@ __global__ void __launch_bounds__(PR_THREADS, 1) attn_pair_kernel(const __grid_c
   auto tile_at = [&](int t) { return tile_of(t, tiles1, KT, pp.KT2, n1, n2); };
 
   int prod_it = 0;
-  bool prod_ok = true, v_missing = false, q_issued = false;
+  bool prod_ok = true, v_missing = false;
   auto issue_q = [&]() {
     mbar_expect_tx(BAR(Q_FULL), (uint32_t)(Sh::QT * H * p.b * pp.heads_rt * 128));
     for (int t = 0; t < Sh::QT; ++t)
       for (int h = 0; h < H; ++h)
         tma_load_4d(smem_u32(q_s + t * TILE + h * HALF), &tm.q, BAR(Q_FULL), h * 64, 0, g * p.G + t * pp.heads_rt, bi);
-    q_issued = true;
   };
   // loads of further tiles (producer lane only); first: only what fits the ring without waiting, source 1 only
   auto produce = [&](bool first) {
@@ -174,13 +174,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) attn_pair_kernel(const __grid_c
       // ======================================= TMA producer =======================================
       if (lane == 0) {
         produce(false);
-        if (*abort_flag) {                  // let the copies that were issued land before the CTA retires
-          for (int j = max(prod_it - NS, 0); j < prod_it; ++j) {
-            drain_bar(BAR(FULL_K + j % NS), (j / NS) & 1);
-            if (do_attn && !(v_missing && j == prod_it - 1)) drain_bar(BAR(FULL_V + j % NS), (j / NS) & 1);
-          }
-          drain_bar(BAR(Q_FULL), 0);
-        }
+        issued_s[0] = prod_it; issued_s[1] = do_attn ? prod_it - (v_missing ? 1 : 0) : 0;
       }
     } else if (warp == 1) {
       // ======================================= MMA issuer =======================================
@@ -248,11 +242,6 @@ __global__ void __launch_bounds__(PR_THREADS, 1) attn_pair_kernel(const __grid_c
           n_prev = n_mma;
         }
         if (ok && nt > 0) ok = TWO ? issue_pv(1, nt - 1, nt - 1, n_prev, true) : issue_pv((nt - 1) & 1, nt - 1, (nt - 1) >> 1, n_prev, true);
-        if (*abort_flag && leader) {        // wait for the tensor pipe to finish what was issued before TMEM is freed
-          tc_commit(BAR(DRAIN));
-          drain_bar(BAR(DRAIN), 0);
-        }
-        __syncwarp();
       }
     } else if (do_scores) {
       // ======================================= saliency warps (refresh) =======================================
@@ -374,7 +363,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) attn_pair_kernel(const __grid_c
       // V rows past the tile's end may hold anything: they are zeroed so that 0 * V stays 0
       if ((!TWO || w == 0) && nv < x.n_mma) {
         const int s = it % NS;
-        if (!wait_bar_warp(BAR(FULL_V + s), (it / NS) & 1, abort_flag, p.status, 51, p.wait_cycles)) { ok = false; break; }
+        if (!wait_bar_warp(BAR(FULL_V + s), (it / NS) & 1, abort_flag, p.status, 51, p.wait_cycles)) { tc_wait_st(); ok = false; break; }   // (stores to tensor memory may be under way)
         unsigned char* vs = stage0 + (size_t)s * 2 * TILE + TILE;
         const int nz = (x.n_mma - nv) * H * 8;            // 16-byte chunks to clear
         for (int e = row; e < nz; e += 128) {
@@ -511,6 +500,12 @@ __global__ void __launch_bounds__(PR_THREADS, 1) attn_pair_kernel(const __grid_c
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
+    if (*abort_flag) {
+      drain_mmas(BAR(DRAIN));
+      drain_loads(BAR(FULL_K), issued_s[0], NS);
+      drain_loads(BAR(FULL_V), issued_s[1], NS);
+      drain_bar(BAR(Q_FULL), 0);
+    }
     __syncwarp();
     tc_fence_after();
     tmem_dealloc(tmem_base, 512);

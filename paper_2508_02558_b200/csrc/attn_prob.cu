@@ -55,6 +55,7 @@ __global__ void __launch_bounds__(PB_THREADS) prob_saliency_kernel(const __grid_
   const int Q_FULL = 0, FULL_K = 1, EMPTY_K = 1 + NS, S_FULL = 1 + 2 * NS, S_FREE = 3 + 2 * NS, DRAIN = 5 + 2 * NS;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + 256);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + 260);
+  int* issued_s = reinterpret_cast<int*>(smem + 264);      // tiles whose loads are on their way (for an aborted CTA's way out)
   float* lse_s = reinterpret_cast<float*>(smem + 1024);    // [256] log-sum-exps in log2 units
   unsigned char* q_s = smem + 2048;
   unsigned char* ring = q_s + NP * D * 2;
@@ -66,6 +67,7 @@ __global__ void __launch_bounds__(PB_THREADS) prob_saliency_kernel(const __grid_
     for (int i = 0; i < 2; ++i) { mbar_init(BAR(S_FULL + i), 1); mbar_init(BAR(S_FREE + i), 4); }
     mbar_init(BAR(DRAIN), 1);
     *abort_flag = 0;
+    *issued_s = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   if (warp == 1) {
@@ -108,10 +110,7 @@ __global__ void __launch_bounds__(PB_THREADS) prob_saliency_kernel(const __grid_
         mbar_expect_tx(BAR(FULL_K + s), (uint32_t)TILE);
         for (int h = 0; h < H; ++h) tma_load_4d(smem_u32(ring + s * TILE + h * HALF), &tm.k, BAR(FULL_K + s), h * 64, (t0 + it) * 128, g, bi);
       }
-      if (*abort_flag) {                                   // let the copies that were issued land before the CTA retires
-        for (int j = max(it - NS, 0); j < it; ++j) drain_bar(BAR(FULL_K + j % NS), (j / NS) & 1);
-        drain_bar(BAR(Q_FULL), 0);
-      }
+      *issued_s = it;
     }
   } else if (warp == 1) {
     const bool leader = elect_one();
@@ -135,11 +134,6 @@ __global__ void __launch_bounds__(PB_THREADS) prob_saliency_kernel(const __grid_
       }
       __syncwarp();
     }
-    if (*abort_flag && leader) {                           // wait for the tensor pipe to finish what was issued before TMEM is freed
-      tc_commit(BAR(DRAIN));
-      drain_bar(BAR(DRAIN), 0);
-    }
-    __syncwarp();
   } else {
     const int q4 = warp & 3, row = q4 * 32 + lane;
     const float inv_rows = 1.f / (float)p.M;
@@ -193,6 +187,11 @@ __global__ void __launch_bounds__(PB_THREADS) prob_saliency_kernel(const __grid_
     for (int pos = lo + tid; pos < hi; pos += PB_THREADS) pooled[pos] = pool_at_ldcg(p, raw, n, o, pos);
   }
   if (warp == 1) {
+    if (*abort_flag) {
+      drain_mmas(BAR(DRAIN));
+      drain_loads(BAR(FULL_K), *issued_s, NS);
+      if (*issued_s > 0) drain_bar(BAR(Q_FULL), 0);
+    }
     __syncwarp();
     tc_fence_after();
     tmem_dealloc(tmem_base, (uint32_t)pp.tmem_cols);

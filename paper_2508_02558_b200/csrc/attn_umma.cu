@@ -213,6 +213,7 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + 256);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + 260);
   int* last_flag = reinterpret_cast<int*>(smem + 264);
+  int* issued_s = reinterpret_cast<int*>(smem + 268);  // [3] tiles whose K / V loads, and whether Q's, are on their way (for an aborted CTA's way out)
   float* qbar_s = reinterpret_cast<float*>(smem + 512);
   unsigned char* q_s = smem + CTRL;
   unsigned char* stage0 = q_s + H * 128 * 128;
@@ -235,7 +236,7 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
   // The producer lane sets the barriers up and, unless the Q tile has to be cleared first, starts the first loads
   // before the rest of the CTA is ready: the loads need nothing but the barriers.
   int prod_it = 0, prod_t = t_begin, prod_n1 = 0;
-  bool prod_ok = true;
+  bool prod_ok = true, v_missing = false;
   bool q_issued = false;
   auto issue_q = [&]() {              // the Q tile (replicated R times along the accumulator rows)
     q_issued = true;
@@ -260,14 +261,14 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
       const CUtensorMap* mv = x.src1 ? &tm.v1 : &tm.v2;
       const uint32_t tile_tx = (uint32_t)(H * (x.src1 ? KT : KT2) * 128);
       if (it >= NS && !wait_bar(BAR(EMPTY_K + s), ph, abort_flag, p.status, 1, p.wait_cycles)) { prod_ok = false; break; }
+      ++prod_it;
       mbar_expect_tx(BAR(FULL_K + s), tile_tx);
       for (int h = 0; h < H; ++h) tma_load_4d(kdst + h * half_bytes, mk, BAR(FULL_K + s), h * 64, x.row0, g, bi);
       if (do_attn) {
-        if (it >= NS && !wait_bar(BAR(EMPTY_V + s), ph, abort_flag, p.status, 2, p.wait_cycles)) { prod_ok = false; break; }
+        if (it >= NS && !wait_bar(BAR(EMPTY_V + s), ph, abort_flag, p.status, 2, p.wait_cycles)) { prod_ok = false; v_missing = true; break; }
         mbar_expect_tx(BAR(FULL_V + s), tile_tx);
         for (int h = 0; h < H; ++h) tma_load_4d(vdst + h * half_bytes, mv, BAR(FULL_V + s), h * 64, x.row0, g, bi);
       }
-      ++prod_it;
       --limit;
     }
   };
@@ -288,6 +289,7 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
     mbar_init(BAR(DRAIN), 1);
     *abort_flag = 0;
     *last_flag = 0;
+    issued_s[0] = issued_s[1] = issued_s[2] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     if (!zero_q && (do_attn || do_scores)) {
       if (up.early_src1) {
@@ -335,14 +337,7 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
       prod_n1 = n1;
       if (!q_issued) issue_q();
       produce(1 << 30, false);
-      if (*abort_flag) {
-        // let the copies that were issued land before the CTA retires
-        for (int j = max(prod_it - NS, 0); j < prod_it; ++j) {
-          drain_bar(BAR(FULL_K + j % NS), (j / NS) & 1);
-          if (do_attn) drain_bar(BAR(FULL_V + j % NS), (j / NS) & 1);
-        }
-        if (do_attn && q_issued) drain_bar(BAR(Q_FULL), 0);
-      }
+      issued_s[0] = prod_it; issued_s[1] = do_attn ? prod_it - (v_missing ? 1 : 0) : 0; issued_s[2] = do_attn ? 1 : 0;
     }
   } else if (warp == 1) {
     // ======================================= MMA issuer =======================================
@@ -399,11 +394,6 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
       if (do_attn && ok && prev_it >= 0) ok = issue_pv(prev, prev_it);
       // a CTA whose slice holds no valid key never used Q: its load must still have landed before the CTA retires
       if (ok && !have_q) ok = wait_bar_warp(BAR(Q_FULL), 0, abort_flag, p.status, 3, p.wait_cycles);
-      if (*abort_flag && leader) {     // wait for the tensor pipe to finish what was issued before TMEM is freed
-        tc_commit(BAR(DRAIN));
-        drain_bar(BAR(DRAIN), 0);
-      }
-      __syncwarp();
     }
   } else if (warp < 6) {
     // ======================================= softmax warps =======================================
@@ -517,7 +507,7 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
         l_run += psum;
         // ---- V rows past the source's count may hold anything: zero them so that 0 * V stays 0 ----
         if (x.nv < x.n_mma) {
-          if (!wait_bar_warp(BAR(FULL_V + s), (it / NS) & 1, abort_flag, p.status, 10, p.wait_cycles)) { ok = false; break; }
+          if (!wait_bar_warp(BAR(FULL_V + s), (it / NS) & 1, abort_flag, p.status, 10, p.wait_cycles)) { tc_wait_st(); ok = false; break; }   // (stores to tensor memory may be under way)
           unsigned char* vs = stage0 + (size_t)s * stage_bytes + kv_bytes;
           const int nz = (x.n_mma - x.nv) * H * 8;     // 16-byte chunks to clear
           for (int i = (warp - 2) * 32 + lane; i < nz; i += 128) {
@@ -815,6 +805,12 @@ __global__ void __launch_bounds__(UM_THREADS, DUAL ? 2 : 1) attn_umma_bf16_kerne
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
+    if (*abort_flag) {
+      drain_mmas(BAR(DRAIN));
+      drain_loads(BAR(FULL_K), issued_s[0], NS);
+      drain_loads(BAR(FULL_V), issued_s[1], NS);
+      drain_loads(BAR(Q_FULL), issued_s[2], 1);
+    }
     __syncwarp();
     tc_fence_after();
     tmem_dealloc(tmem_base, TMEM_COLS);
