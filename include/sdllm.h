@@ -243,7 +243,7 @@ sdllm_status sdllm_sparse_block_attn_static(const sdllm_desc* desc, const void* 
  *   "cluster", "fused_tail", "dual", "key_tile", "lpt", "stages", "trigger", "persist"   plan details of the tcgen05 kernels
  *   "select"      top-k kernel: 1 one CTA per head, 2 one cluster per head
  *   "wait_cycles" limit, in SM clock cycles, of every abortable device-side wait (default 400 000 000, ~0.2 s). A limit
- *                 of a few cycles makes the first wait that is not already satisfied give up: the call still returns,
+ *                 of zero makes the first wait that is not already satisfied give up: the call still returns,
  *                 its outputs are invalid and sdllm_read_status reports SDLLM_ERR_TIMEOUT (how the tests exercise
  *                 that path without hanging anything).
  *   "debug"       1: print the CUDA error behind an SDLLM_ERR_CUDA to stderr

@@ -452,7 +452,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) attn_pair_kernel(const __grid_c
     }
     const bool first_half = TWO || w == 0;                // who writes the row's sum
     const float inv = p.splits == 1 ? (l_row != 0.f ? 1.f / l_row : 0.f) : 1.f;
-    if (!*abort_flag) {
+    if (!__any_sync(0xffffffffu, *abort_flag)) {          // (tensor memory is read by whole warps)
 #pragma unroll 1
       for (int c = c_lo; c < c_hi; ++c) {
         uint32_t ov[16];

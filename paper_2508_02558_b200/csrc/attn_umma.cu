@@ -54,7 +54,6 @@ struct UmmaParams {
   int lpt;           // 1: grid z counts the sequences from the longest to the shortest (several waves of ragged work)
 };
 
-#define SDLLM_ZERO_LIMIT_NEVER_WAITS
 #include "umma_ptx.cuh"
 
 // Merge of the key-split partials of S (row, float4 column) slots of a unit and the final stores. slot[s] < 0 marks

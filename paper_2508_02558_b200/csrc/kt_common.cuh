@@ -5,8 +5,6 @@
 constexpr int KT_GRP = 3072;             // control block, per softmax warpgroup: references, raise scratch, sums, saliency partials
 constexpr int KT_CTRL0 = 1024;           // control block, common part: barriers and flags
 
-// (not in the kernels whose softmax loops are short of registers: the extra branch costs the dense step 1 to 2 %)
-#define SDLLM_ZERO_LIMIT_NEVER_WAITS
 #include "umma_ptx.cuh"
 
 __device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed;\n" ::: "memory"); }

@@ -187,3 +187,57 @@ def test_a_logit_that_is_not_finite_makes_its_rows_nan(op, Hkv, G, D, dtype, pla
         rows = bad_rows[..., 0]
         assert not np.isfinite(lse.cpu().numpy()[rows]).any()
         np.testing.assert_allclose(lse.cpu().numpy()[~rows], ref_lse[~rows], rtol=0, atol=1e-4)
+
+
+@pytest.mark.parametrize("op,Hkv,G,D,plan,codes", [
+    ("refresh", 4, 4, 128, {}, range(41, 53)), ("refresh", 4, 4, 64, dict(splits=1), range(41, 53)), ("refresh", 4, 7, 128, {}, range(41, 53)),
+    ("reuse", 4, 7, 128, {}, range(41, 53)), ("reuse", 4, 4, 128, dict(kernel=4, splits=1), range(41, 53)),
+    ("scores", 4, 7, 128, dict(splits=1), range(41, 53)), ("scores", 4, 4, 128, dict(splits=1), range(41, 53)),
+    ("prob", 8, 1, 128, {}, range(61, 66)), ("prob", 4, 7, 128, {}, range(61, 66)),
+    ("dense", 3, 2, 128, {}, range(21, 31)), ("dense", 3, 2, 64, dict(ws=256), range(21, 31)),
+    ("refresh", 8, 1, 128, {}, range(1, 16)), ("refresh", 8, 2, 128, dict(kernel=3), range(1, 16)),
+    ("refresh", 8, 1, 128, dict(splits=1, persist=2), range(1, 16)), ("reuse", 8, 1, 64, {}, range(1, 16)),
+])
+def test_every_kernel_reports_a_wait_that_runs_out_and_returns(op, Hkv, G, D, plan, codes, tuning):
+    """A limit of zero: the call returns, the status word holds one of the kernel's codes, and with the ordinary limit and the
+    workspace zeroed the next call gives what the first one gave."""
+    plan = dict(plan)
+    ws_bytes = plan.pop("ws", None)
+    tuning(**plan)
+    b, L, n_kept = 32, 700, 600
+    gen = torch.Generator(device="cuda").manual_seed(Hkv * G + D)
+
+    def draw(*shape):
+        return torch.randn(shape, generator=gen, device="cuda").mul_(D ** -0.5).bfloat16()
+
+    q, k, v = draw(1, Hkv * G, L if op == "dense" else b, D), draw(1, Hkv, L, D), draw(1, Hkv, L, D)
+    d = B.make_desc(batch=1, n_q_heads=Hkv * G, n_kv_heads=Hkv, head_dim=D, seq_len_max=L, block_len=b, dtype=B.BF16, retention=0.5,
+                    n_keep_max=n_kept, score=B.SCORE_PROB_MEAN if op == "prob" else B.SCORE_LOGIT_MEAN)
+    code = {"dense": B.OP_DENSE_ATTN, "reuse": B.OP_SPARSE_BLOCK_ATTN}.get(op, B.OP_REFRESH_SCORES)
+    ws = torch.zeros((ws_bytes or B.workspace_bytes(d, code),), dtype=torch.uint8, device="cuda")
+    count, bo = (torch.tensor([x], dtype=torch.int32, device="cuda") for x in (n_kept, 64))
+    kc, vc, kn, vn = draw(1, Hkv, n_kept, D), draw(1, Hkv, n_kept, D), draw(1, Hkv, b, D), draw(1, Hkv, b, D)
+
+    def call():
+        out, pooled = torch.full_like(q, 7.0), torch.full((1, Hkv, L), 7.0, device="cuda")
+        if op == "dense":
+            B.dense_attn(d, q, k, v, None, out, None, ws)
+        elif op == "reuse":
+            B.sparse_block_attn(d, q, kc, vc, count, kn, vn, out, ws)
+        else:
+            B.refresh_scores(d, q, k, v, None, bo, None if op == "scores" else out, None, pooled, ws)
+        torch.cuda.synchronize()
+        return out, pooled
+
+    want = call()
+    assert B.read_status(ws) == 0
+    tuning(wait_cycles=0)
+    for _ in range(20):
+        call()
+        assert B.read_status(ws) in codes
+        ws.zero_()
+    tuning(wait_cycles=400_000_000)
+    again = call()
+    assert B.read_status(ws) == 0
+    for x, y in zip(want, again):
+        torch.testing.assert_close(x, y, rtol=0, atol=0)
