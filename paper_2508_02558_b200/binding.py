@@ -9,11 +9,12 @@ from __future__ import annotations
 
 import ctypes
 import os
+import sysconfig
 from typing import Optional, Sequence
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libsdllm.so")
-MARSHAL_PATH = os.path.join(_PKG, "_marshal.so")
+MARSHAL_PATH = os.path.join(_PKG, "_marshal" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT = range(6)
 F32, BF16 = 0, 1
@@ -105,17 +106,25 @@ _DEVICE_CALLS = ("sdllm_refresh_scores", "sdllm_select_topk", "sdllm_compact_kv"
                  "sdllm_sparse_block_attn_static", "sdllm_dense_attn")
 
 
+def _stream_getters():
+    """(raw current stream of a device, current device). torch's private getters take 0.2 us where the public calls, which serve
+    where a torch does not have them, take 3."""
+    import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    device = getattr(torch._C, "_cuda_getDevice", None)
+    return raw or (lambda dev: torch.cuda.current_stream(dev).cuda_stream), device or torch.cuda.current_device
+
+
 def native():
     """The builtins that marshal the device calls (csrc/marshal.cpp), bound to the library; raises if they are missing."""
     global _native
     if _native is None:
-        import torch
         L = lib()
         if not os.path.exists(MARSHAL_PATH):
             raise RuntimeError(f"{MARSHAL_PATH} is missing: run `python -m paper_2508_02558_b200.build` "
                                "(there is no fallback path)")
         from . import _marshal
-        _marshal.bind(torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice, *(ctypes.cast(getattr(L, f), ctypes.c_void_p).value for f in _DEVICE_CALLS))
+        _marshal.bind(*_stream_getters(), *(ctypes.cast(getattr(L, f), ctypes.c_void_p).value for f in _DEVICE_CALLS))
         _native = _marshal
     return _native
 

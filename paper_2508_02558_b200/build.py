@@ -1,5 +1,5 @@
 """Builds libsdllm.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and beside it the native part of the
-Python binding (`_marshal.so`, host C++ only)."""
+Python binding (`_marshal`, host C++ only; its file name carries the ABI tag of the Python it is built for)."""
 from __future__ import annotations
 
 import os
@@ -14,7 +14,7 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OBJ_DIR = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libsdllm.so")
-MARSHAL = os.path.join(PKG, "_marshal.so")
+MARSHAL = os.path.join(PKG, "_marshal" + sysconfig.get_config_var("EXT_SUFFIX"))
 MARSHAL_SRC = os.path.join(CSRC, "marshal.cpp")
 
 NVCC_FLAGS = ["-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
@@ -42,7 +42,7 @@ def _build_marshal() -> None:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu under csrc/ and link libsdllm.so, and compile _marshal.so; a no-op when both are newer than their
+    """Compile every .cu under csrc/ and link libsdllm.so, and compile _marshal; a no-op when both are newer than their
     sources."""
     if force or not os.path.exists(MARSHAL) or os.path.getmtime(MARSHAL) < max(os.path.getmtime(MARSHAL_SRC), _deps_mtime()):
         _build_marshal()
