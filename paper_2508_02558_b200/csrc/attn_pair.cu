@@ -56,6 +56,7 @@ struct PairShape {
   static constexpr int QT = TWO ? 2 : 1;                  // Q tiles
   static constexpr int NS = D == 64 ? 4 : (TWO ? 2 : 3);  // ring slots: what fits beside Q
   static constexpr size_t SMEM = 1024 /*alignment slack*/ + 1024 /*barriers, qbar*/ + (size_t)QT * TILE + (size_t)NS * 2 * TILE;
+  static constexpr size_t LAUNCH_SMEM = SMEM > 120 * 1024 ? SMEM : 120 * 1024;    // more than half an SM's: a CTA takes all tensor memory
 };
 
 template <int D, bool TWO>
@@ -577,7 +578,7 @@ template <int D, bool TWO>
 cudaError_t launch_pair_shape(const PairMaps& tm, const PairParams& pp, bool pdl, cudaStream_t st) {
   auto kern = attn_pair_kernel<D, TWO>;
   static SmemConfig configured;
-  const size_t smem = PairShape<D, TWO>::SMEM > 120 * 1024 ? PairShape<D, TWO>::SMEM : 120 * 1024;    // one CTA per SM: it takes all TMEM
+  const size_t smem = PairShape<D, TWO>::LAUNCH_SMEM;
   cudaError_t e = configure_smem(reinterpret_cast<const void*>(kern), smem, configured, true);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
@@ -621,6 +622,8 @@ AttnPlan plan_attention_pair(int D, int M, int b, int B, int Hkv, int n1_max, in
   pl.threads = PR_THREADS; pl.key_tile = 128; pl.key_tile2 = n2 > 0 ? (n2 < 128 ? n2 : 128) : 128;
   pl.row_tiles = M > 128 ? 2 : 1; pl.rep = 1; pl.rows_rep = 128;
   pl.stages = D == 64 ? 4 : (M > 128 ? 2 : 3);
+  pl.smem_bytes = D == 64 ? (M > 128 ? PairShape<64, true>::LAUNCH_SMEM : PairShape<64, false>::LAUNCH_SMEM)
+                          : (M > 128 ? PairShape<128, true>::LAUNCH_SMEM : PairShape<128, false>::LAUNCH_SMEM);
   const long long units = (long long)B * Hkv;
   const int tiles = (n1_max + 127) / 128 + (n2 > 0 ? (n2 + pl.key_tile2 - 1) / pl.key_tile2 : 0);
   long long most = sm_count() / units;

@@ -484,10 +484,14 @@ def test_planner_picks_the_kernel_families_where_they_were_measured_to_win():
     assert name() == "attn_kt_kernel" and name(B.OP_REFRESH_SCORES) == "attn_kt_kernel"
     assert name(batch=16, seq_len_max=4352, n_keep_max=2160) == "attn_kt_stream_kernel"
     assert name(B.OP_REFRESH_SCORES, batch=16, seq_len_max=4352, n_keep_max=2160) == "attn_kt_stream_kernel"
-    assert name(n_q_heads=28, n_kv_heads=4, seq_len_max=4096, n_keep_max=1024) == "attn_umma_bf16_kernel"       # 224 query rows per KV head
-    assert name(n_kv_heads=8, seq_len_max=32768, n_keep_max=16368) == "attn_umma_bf16_kernel"                   # 8 units of 128 rows
+    assert name(n_q_heads=28, n_kv_heads=4, seq_len_max=4096, n_keep_max=1024) == "attn_pair_kernel"       # 224 query rows per KV head
+    assert name(n_kv_heads=8, seq_len_max=32768, n_keep_max=16368) == "attn_pair_kernel"                   # 8 units of 128 rows
     assert name(batch=8, n_q_heads=16, n_kv_heads=8, seq_len_max=4352, n_keep_max=2048) == "attn_kt_kernel"     # 64 units of 64 rows
     assert name(dtype=B.F32) == "attn_f32_kernel"
+    assert name(B.OP_REFRESH_SCORES, score=B.SCORE_PROB_MEAN) == "attn_umma_bf16_kernel"                        # the pass in front of the saliency
+    for heads in (8, 28):                                                                                       # every plan says what shared memory it takes
+        assert " smem=" in B.plan_describe(B.make_desc(batch=1, n_q_heads=heads, n_kv_heads=4, head_dim=128, seq_len_max=1280, block_len=32,
+                                                       dtype=B.BF16, retention=0.5, n_keep_max=496), B.OP_SPARSE_BLOCK_ATTN)
     # cluster sizes follow what the device keeps resident at once: 16 units of whole-SM CTAs get clusters of six, not eight
     plan = B.plan_describe(B.make_desc(batch=2, n_q_heads=16, n_kv_heads=8, head_dim=128, seq_len_max=2080, block_len=32, dtype=B.BF16,
                                        retention=0.5, n_keep_max=1024), B.OP_SPARSE_BLOCK_ATTN)
