@@ -139,8 +139,9 @@ __device__ __forceinline__ uint64_t add_f2(uint64_t a, uint64_t b) {
 }
 // 2^x for two values on the FMA pipe, beside the exponential unit (16 results per clock and SM, the bottleneck of a softmax
 // that feeds tcgen05): x = n + f with n the nearest integer (round by adding 1.5 * 2^23), 2^f by the degree-5 polynomial of
-// least relative error on [-1/2, 1/2] (Remez exchange; 7.5e-8, 2.1e-7 evaluated in fp32 - ex2.approx is within 2.4e-7), n added
-// to the exponent. Values below 2^-126 come out as about 2^-126 instead of 0. NaN stays NaN up to the integer addition, which
+// least relative error on [-1/2, 1/2] with 1 as its constant term, its coefficients rounded to fp32 one after the other and the rest
+// fitted again (9.4e-8, 1.5e-7 evaluated in fp32, as much as ex2.approx shows; with a free constant term, which rounds to 1 + 2^-23,
+// it was 2.1e-7), n added to the exponent. Values below 2^-126 come out as about 2^-126 instead of 0. NaN stays NaN up to the integer addition, which
 // makes the largest float of it: a row's sum of exponentials that reaches kNanSum has met one (ordinary sums stay below 2^8 a key).
 constexpr float kNanSum = 1e38f;
 __device__ __forceinline__ void poly_exp2(float x0, float x1, float& e0, float& e1) {
@@ -148,11 +149,11 @@ __device__ __forceinline__ void poly_exp2(float x0, float x1, float& e0, float& 
   const uint64_t magic = pack_f2(12582912.f, 12582912.f), minus_one = pack_f2(-1.f, -1.f);
   const uint64_t t = add_f2(x, magic);
   const uint64_t f = add_f2(x, fma_f2(t, minus_one, magic));
-  uint64_t y = fma_f2(pack_f2(1.3276472454890609e-3f, 1.3276472454890609e-3f), f, pack_f2(9.675540961325169e-3f, 9.675540961325169e-3f));
-  y = fma_f2(y, f, pack_f2(5.550713092088699e-2f, 5.550713092088699e-2f));
-  y = fma_f2(y, f, pack_f2(2.4022120237350464e-1f, 2.4022120237350464e-1f));
+  uint64_t y = fma_f2(pack_f2(1.3256072998046875e-3f, 1.3256072998046875e-3f), f, pack_f2(9.671226143836975e-3f, 9.671226143836975e-3f));
+  y = fma_f2(y, f, pack_f2(5.5507682263851166e-2f, 5.5507682263851166e-2f));
+  y = fma_f2(y, f, pack_f2(2.402224838733673e-1f, 2.402224838733673e-1f));
   y = fma_f2(y, f, pack_f2(6.931469440460205e-1f, 6.931469440460205e-1f));
-  y = fma_f2(y, f, pack_f2(1.0000001192092896f, 1.0000001192092896f));
+  y = fma_f2(y, f, pack_f2(1.f, 1.f));
   float y0, y1, t0, t1;
   unpack_f2(y, y0, y1);
   unpack_f2(t, t0, t1);
