@@ -236,11 +236,11 @@ sdllm_status sdllm_sparse_block_attn_static(const sdllm_desc* desc, const void* 
  * planner, so sdllm_workspace_bytes, sdllm_launch_count and the launches agree as long as no override changes between
  * them. Host-only, thread-safe; takes effect for calls made afterwards. `name` is a NUL-terminated host string:
  *   "splits"      > 0: key splits per (sequence, KV head) of the attention calls
- *   "kernel"      attention kernel family: 0 automatic, 1 cp.async, 2 tcgen05 with the queries on the accumulator rows,
- *                 (one softmax warpgroup), 3 tcgen05 with the keys on the accumulator rows, 4 as 2 with two softmax
- *                 warpgroups (each only where that kernel covers the shape)
+ *   "kernel"      attention kernel family: 0 automatic, 1 cp.async, 2 or 4 tcgen05 with the queries on the accumulator rows,
+ *                 3 tcgen05 with the keys on the accumulator rows (each only where that kernel covers the shape)
  *   "pdl"         0: no programmatic dependent launch     "early_loads" 0: no loads ahead of the grid dependency
- *   "cluster", "fused_tail", "dual", "key_tile", "lpt", "stages", "trigger", "persist"   plan details of the tcgen05 kernels
+ *   "fused_tail", "dual", "key_tile", "lpt", "stages", "trigger", "persist"   plan details of the tcgen05 kernels
+ *   "cluster"     accepted, no effect
  *   "select"      top-k kernel: 1 one CTA per head, 2 one cluster per head
  *   "wait_cycles" limit, in SM clock cycles, of every abortable device-side wait (default 400 000 000, ~0.2 s). A limit
  *                 of zero makes the first wait that is not already satisfied give up: the call still returns,

@@ -211,16 +211,10 @@ int32_t sdllm_launch_count(const sdllm_desc* d, int op) {
   if (op != SDLLM_OP_REFRESH_SCORES && op != SDLLM_OP_SPARSE_BLOCK_ATTN) return -1;
   const bool refresh = op == SDLLM_OP_REFRESH_SCORES;
   const AttnPlan pl = plan_for(d, op);
-  const int M = d->n_q_heads / d->n_kv_heads * d->block_len;
   if (refresh && d->score == SDLLM_SCORE_PROB_MEAN)         // attention pass (and its fold), saliency pass
-    return 2 + (pl.kind == 4 && pl.splits > 1 ? 1 : 0) + (pl.kind == 2 && pl.splits > 1 && !umma_tail_is_fused(pl, d->head_dim, M, d->seq_len_max, false, true) ? 1 : 0);
+    return 2 + (pl.splits > 1 && !umma_tail_is_fused(pl, d->head_dim, d->n_q_heads / d->n_kv_heads * d->block_len) ? 1 : 0);
   if (pl.kind == 3) return 1;       // the key splits merge, and the scores are pooled, inside the one launch
   if (pl.kind == 4) return pl.splits > 1 || refresh ? 2 : 1;       // the fold of the key splits and the pooling are one launch
-  if (pl.kind == 2) {
-    const int n1 = refresh ? d->seq_len_max : d->n_keep_max;
-    const bool tail_work = pl.splits > 1 || refresh;
-    return 1 + ((tail_work && !umma_tail_is_fused(pl, d->head_dim, M, n1, refresh, true)) ? 1 : 0);
-  }
   return 1 + ((refresh || pl.splits > 1) ? 1 : 0);
 }
 

@@ -626,7 +626,7 @@ size_t attn_legacy_smem_bytes(int dtype, int D, const AttnPlan& plan) {
 
 AttnPlan plan_attention_legacy(int dtype, int D, int M, int B, int Hkv, int n_keys_max, const Tuning& tn) {
   AttnPlan pl{};
-  pl.cluster = 1; pl.warp_keys = 32; pl.tma = false;
+  pl.cluster = 1; pl.warp_keys = 32;
   const long long base = (long long)B * Hkv;
   if (dtype == SDLLM_BF16) {
     pl.m_warps = (M + 15) / 16;

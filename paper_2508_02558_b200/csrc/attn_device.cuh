@@ -108,29 +108,6 @@ __device__ __forceinline__ void compute_qbar(const AttnParams& p, const CtaRange
   }
 }
 
-// Importance of one absolute position: Algorithm 1, MaxPool1D(A, kernel_size = s, padding = s/2) over the candidate
-// axis Concat(prefix, suffix) (AvgPool for the ablation); block positions and padding get -inf. `a` holds the raw
-// saliency by absolute position.
-__device__ __forceinline__ float pool_at(const AttnParams& p, const float* a, int L, int o_in, int pos, int n_arr = 1,
-                                         int64_t arr_stride = 0) {
-  const int b = p.b;
-  const int o = min(max(o_in, 0), max(L - b, 0));
-  if (pos >= L || (pos >= o && pos < o + b)) return -INFINITY;
-  const int C = max(L - b, 0), w = (p.window - 1) / 2;
-  const int c = pos < o ? pos : pos - b;
-  int lo = 0, hi = C;
-  if (p.per_region) { if (c < o) hi = o; else lo = o; }
-  float mx = -INFINITY, sum = 0.f;
-  for (int t = c - w; t <= c + w; ++t) {
-    if (t < lo || t >= hi) continue;
-    float x = a[t < o ? t : t + b];
-    for (int r2 = 1; r2 < n_arr; ++r2) x += a[r2 * arr_stride + (t < o ? t : t + b)];   // one array per row tile
-    mx = fmaxf(mx, x);
-    sum += x;
-  }
-  return p.pool_kind == SDLLM_POOL_MAX ? mx : sum / (float)p.window;
-}
-
 // Maximum and sum of the raw saliency over the window [c - w, c + w] of candidates that lies inside [lo, hi), read through L2
 // (other CTAs wrote it). Windows of up to nine have all their loads in flight together: one L2 round trip instead of one each.
 __device__ __forceinline__ void pool_window(const float* a, int c, int w, int lo, int hi, int o, int b, float& mx, float& sum) {
@@ -157,8 +134,9 @@ __device__ __forceinline__ void pool_window(const float* a, int c, int w, int lo
   }
 }
 
-// Importance of one absolute position as pool_at, reading the raw saliency from global memory through L2 (other CTAs wrote it
-// during this launch).
+// Importance of one absolute position: Algorithm 1, MaxPool1D(A, kernel_size = s, padding = s/2) over the candidate
+// axis Concat(prefix, suffix) (AvgPool for the ablation); block positions and padding get -inf. `a` holds the raw saliency by
+// absolute position and is read through L2 (other CTAs wrote it).
 __device__ __forceinline__ float pool_at_ldcg(const AttnParams& p, const float* a, int L, int o_in, int pos) {
   const int b = p.b;
   const int o = min(max(o_in, 0), max(L - b, 0));

@@ -863,9 +863,9 @@ bool kt_preferred(int D, int M, int B, int Hkv, int n1_max, int n2) {
 AttnPlan plan_attention_kt(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn) {
   (void)b;
   AttnPlan pl{};
-  pl.kind = 3; pl.tma = true; pl.fused_tail = true;
+  pl.kind = 3; pl.fused_tail = true;
   pl.key_tile = 128; pl.key_tile2 = n2 < 32 ? n2 : 32;
-  pl.rep = 1; pl.row_tiles = 1; pl.rows_rep = M;
+  pl.rep = 1; pl.row_tiles = 1;
   const int CG = (M + 31) / 32;          // column groups of 32 query columns: one softmax warpgroup each
   const int groups = (n1_max + 31) / 32 + (n2 + 31) / 32;
   const long long units = (long long)B * Hkv;
@@ -966,7 +966,6 @@ AttnPlan plan_attention_kt(int D, int M, int b, int B, int Hkv, int n1_max, int 
     while (NS > 1 && kt_smem_bytes(D, CG, WG, NS, PB, S) > 226 * 1024) --NS;
   }
   pl.splits = 1;                        // nothing is left in the workspace: the splits merge inside their cluster
-  pl.parts = 1;
   pl.cluster = S;
   pl.stages = NS;
   pl.m_warps = PB;                      // (field reused: P^T buffers)

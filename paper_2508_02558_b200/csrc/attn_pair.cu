@@ -618,9 +618,9 @@ bool pair_supported(int dtype, int D, int M, int b) {
 AttnPlan plan_attention_pair(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn) {
   (void)b;
   AttnPlan pl{};
-  pl.kind = 4; pl.tma = true; pl.cluster = 1; pl.fused_tail = true;
+  pl.kind = 4; pl.cluster = 1; pl.fused_tail = true;
   pl.threads = PR_THREADS; pl.key_tile = 128; pl.key_tile2 = n2 > 0 ? (n2 < 128 ? n2 : 128) : 128;
-  pl.row_tiles = M > 128 ? 2 : 1; pl.rep = 1; pl.rows_rep = 128;
+  pl.row_tiles = M > 128 ? 2 : 1; pl.rep = 1;
   pl.stages = D == 64 ? 4 : (M > 128 ? 2 : 3);
   pl.smem_bytes = D == 64 ? (M > 128 ? PairShape<64, true>::LAUNCH_SMEM : PairShape<64, false>::LAUNCH_SMEM)
                           : (M > 128 ? PairShape<128, true>::LAUNCH_SMEM : PairShape<128, false>::LAUNCH_SMEM);
@@ -637,7 +637,6 @@ AttnPlan plan_attention_pair(int D, int M, int b, int B, int Hkv, int n1_max, in
     if (cost < least) { least = cost; pl.splits = s; }
   }
   if (tn.splits > 0) pl.splits = tn.splits < tiles ? tn.splits : (tiles > 0 ? tiles : 1);
-  pl.parts = pl.splits;
   pl.part_rows = pl.splits > 1 ? (size_t)pl.row_tiles * pl.splits * 128 : 0;
   pl.n_counters = 0;
   return pl;

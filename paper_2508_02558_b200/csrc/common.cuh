@@ -31,17 +31,14 @@ struct AttnPlan {
   int cluster;      // > 1: the key splits of a unit form a thread-block cluster and merge through distributed shared memory
   int splits;       // partials per (sequence, KV head) left in the workspace (1 = final output written directly)
   int threads;
-  bool tma;         // the kernel is fed by TMA (tcgen05 kernel), else by cp.async
   size_t smem_bytes;
-  int kind;         // 0: cp.async kernels (fp32 FMA / bf16 mma.sync), 2: tcgen05 kernel, queries on the accumulator rows,
-                    // 3: tcgen05 kernel, keys on the accumulator rows (its key splits merge inside their cluster)
+  int kind;         // 0: cp.async kernels (fp32 FMA / bf16 mma.sync); tcgen05 kernels - 2: attention pass of the probability saliency
+                    // (attn_umma.cu), 3: keys on the accumulator rows (key splits merge inside their cluster), 4: queries on the
+                    // accumulator rows, two softmax warpgroups (attn_pair.cu)
   int key_tile2;    // tcgen05 kernel: keys per tile of source 2
   int rep;          // tcgen05 kernel: replicas of the query rows along the 128 accumulator rows
   int row_tiles;    // tcgen05 kernel: 128-row tiles of the b*G rows
-  int parts;        // partials per (sequence, KV head, row tile) = splits * rep
-  int rows_rep;     // rows of one partial
-  bool fused_tail;  // the attention kernel merges the partials and pools the scores itself
-  bool dual;        // tcgen05 kernel, small-footprint variant: two CTAs per SM
+  bool fused_tail;  // nothing is left to launch_merge_pool: the attention launch merges the partials and pools the scores itself
   bool persistent;  // key-row kernel, streaming variant: one resident CTA per SM walks the units
   size_t part_rows; // partial rows per (sequence, KV head) in the workspace (0: none)
   size_t n_counters;// counters that the kernel uses, of the workspace's kWsCounters
@@ -112,7 +109,7 @@ AttnWorkspace attn_workspace(const sdllm_desc* d, const AttnPlan& pl, bool score
 AttnPlan plan_attention(int dtype, int D, int M, int b, int B, int Hkv, int n1_max, int n2, bool prob_scores);
 cudaError_t launch_prob_saliency(const AttnParams& p, int D, cudaStream_t st);    // second pass of the probability saliency
 
-bool umma_tail_is_fused(const AttnPlan& pl, int D, int M, int n1_max, bool pool, bool merge);
+bool umma_tail_is_fused(const AttnPlan& pl, int D, int M);
 bool umma_supported(int dtype, int D, int M, int b);
 // Full-sequence attention (attn_dense.cu).
 struct DenseCall {

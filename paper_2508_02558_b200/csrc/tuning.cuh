@@ -13,15 +13,14 @@ constexpr int kMaxDevices = 64;
 // override changes between them.
 struct Tuning {
   int splits = 0;            // > 0: key splits per (sequence, KV head)
-  int kernel = 0;            // 0: automatic; 1: cp.async kernels; 2: tcgen05 kernel with the queries on the accumulator
-                             // rows, one softmax warpgroup; 3: tcgen05 kernel with the keys on the accumulator rows; 4: as 2,
-                             // two softmax warpgroups
+  int kernel = 0;            // 0: automatic; 1: cp.async kernels; 2, 4: tcgen05 kernel with the queries on the accumulator rows; 3: tcgen05
+                             // kernel with the keys on the accumulator rows
   int pdl = 1;               // 0: no programmatic dependent launch
   int early_loads = 1;       // 0: no loads ahead of the grid dependency
-  int cluster = 1;           // query-row kernel: 2 merges few key splits through a cluster where the shape allows (off otherwise)
-  int fused_tail = -1;       // query-row kernel: 0 / 1 forces the tail into the second launch / into the last CTA
-  int dual = -1;             // query-row kernel: 0 / 1 forces the two-CTAs-per-SM variant off / on
-  int key_tile = 0;          // query-row kernel: 64 or 128
+  int cluster = 1;           // no effect (what it chose is gone; the name is still accepted)
+  int fused_tail = -1;       // attention pass of the probability saliency: 0 / 1 forces the merge into the second launch / into the last CTA
+  int dual = -1;             // key-row kernel: 0 / 1 forces the two-CTAs-per-SM footprint off / on
+  int key_tile = 0;          // attention pass of the probability saliency: 64 or 128
   int lpt = -1;              // 0 / 1 forces the longest-first order of ragged batches off / on
   int select = 0;            // top-k: 1 one CTA per head, 2 a cluster per head
   int stages = 0;            // key-row kernel: ring slots (1..3)

@@ -9,7 +9,7 @@
 namespace sdllm {
 AttnPlan plan_attention_kt(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn);
 AttnPlan plan_attention_pair(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn);
-AttnPlan plan_attention_umma(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn);
+AttnPlan plan_attention_umma(int D, int M, int b, int B, int Hkv, int n1_max, const Tuning& tn);
 }  // namespace sdllm
 using namespace sdllm;
 
@@ -30,13 +30,13 @@ int main() {
       const int n1 = refresh ? L : d.n_keep_max, n2 = refresh ? 0 : b;
       for (int kind = 0; kind < 4; ++kind) {
         if (kind == 1 && (M > 128 || M % 4 != 0)) continue;
-        if (kind == 3 && (b % 16 != 0 || (M > 128 && 128 % b != 0))) continue;
+        if (kind == 3 && (!prob || b % 16 != 0 || (M > 128 && 128 % b != 0))) continue;
         const AttnPlan pl = kind == 0   ? plan_attention(SDLLM_F32, D, M, b, B, Hkv, n1, n2, false)
                             : kind == 1 ? plan_attention_kt(D, M, b, B, Hkv, n1, n2, tn)
                             : kind == 2 ? plan_attention_pair(D, M, b, B, Hkv, n1, n2, tn)
-                                        : plan_attention_umma(D, M, b, B, Hkv, n1, n2, tn);
+                                        : plan_attention_umma(D, M, b, B, Hkv, n1, tn);
         const AttnWorkspace w = attn_workspace(&d, pl, refresh);
-        const bool counts = pl.persistent || (pl.kind == 2 && pl.splits > 1 && umma_tail_is_fused(pl, D, M, n1, refresh && !prob, true));
+        const bool counts = pl.persistent || (pl.kind == 2 && pl.splits > 1 && umma_tail_is_fused(pl, D, M));
         const size_t rows = (size_t)B * Hkv * pl.part_rows;
         if (w.part_o < counters_end || w.part_ml < w.part_o + rows * D * 4 || w.raw < w.part_ml + rows * 8 ||
             w.lse < w.raw + (refresh ? (size_t)B * Hkv * L * 4 : 0) || w.total < w.lse + (prob ? (size_t)B * Hkv * M * 4 : 0) ||

@@ -193,7 +193,7 @@ def test_a_logit_that_is_not_finite_makes_its_rows_nan(op, Hkv, G, D, dtype, pla
     ("refresh", 4, 4, 128, {}, range(41, 53)), ("refresh", 4, 4, 64, dict(splits=1), range(41, 53)), ("refresh", 4, 7, 128, {}, range(41, 53)),
     ("reuse", 4, 7, 128, {}, range(41, 53)), ("reuse", 4, 4, 128, dict(kernel=4, splits=1), range(41, 53)),
     ("scores", 4, 7, 128, dict(splits=1), range(41, 53)), ("scores", 4, 4, 128, dict(splits=1), range(41, 53)),
-    ("prob", 8, 1, 128, {}, range(61, 66)), ("prob", 4, 7, 128, {}, range(61, 66)),
+    ("prob", 8, 1, 128, {}, range(61, 66)), ("prob", 4, 7, 128, {}, range(61, 66)), ("prob", 4, 4, 128, dict(splits=3, fused_tail=1), range(61, 66)),
     ("dense", 3, 2, 128, {}, range(21, 31)), ("dense", 3, 2, 64, dict(ws=256), range(21, 31)),
     ("refresh", 8, 1, 128, {}, range(1, 16)), ("refresh", 8, 2, 128, dict(kernel=3), range(1, 16)),
     ("refresh", 8, 1, 128, dict(splits=1, persist=2), range(1, 16)), ("reuse", 8, 1, 64, {}, range(1, 16)),
@@ -241,3 +241,12 @@ def test_every_kernel_reports_a_wait_that_runs_out_and_returns(op, Hkv, G, D, pl
     assert B.read_status(ws) == 0
     for x, y in zip(want, again):
         torch.testing.assert_close(x, y, rtol=0, atol=0)
+
+
+@pytest.mark.parametrize("cfg,block", [(_wide("prob_m32", 4, 4, 128, 333, 64), 1), (_wide("prob_m64", 4, 2, 64, 500, 64), 0), (_wide("prob_m224", 14, 2, 128, 300, 64), 1)])
+@pytest.mark.parametrize("plan", [dict(key_tile=64), dict(splits=4, fused_tail=1), dict(splits=9, fused_tail=0), dict(splits=2, key_tile=64)])
+def test_attention_pass_of_the_probability_saliency(cfg, block, plan, tuning):
+    """Replicated query rows, both key tile heights, the key splits merged by the last CTA and by the second launch."""
+    from test_gpu_parity import _run_sequence_case
+    tuning(**plan)
+    _run_sequence_case(cfg, seed=29, block=block, n_sparse=0, score=B.SCORE_PROB_MEAN)

@@ -178,14 +178,14 @@ def test_pool_windows(window):
     dict(kernel=3, splits=1, persist=1), dict(kernel=3, splits=1, persist=2),   # streaming variant (where one column group suffices)
     dict(kernel=2),                                      # the tcgen05 kernel with the queries on the accumulator rows
     dict(kernel=2, splits=7), dict(kernel=2, splits=1),
-    dict(kernel=2, splits=5, fused_tail=0),              # split merge and pooling in the second launch
+    dict(kernel=2, splits=5, fused_tail=0),
     dict(kernel=2, early_loads=0),
-    dict(kernel=2, cluster=0, splits=4),                 # key splits merged by the last CTA instead of a cluster
-    dict(kernel=2, cluster=2, splits=4),                 # ... and by a cluster of four
+    dict(kernel=2, cluster=0, splits=4),                 # (from here on with overrides that mean nothing to this kernel: they are accepted)
+    dict(kernel=2, cluster=2, splits=4),
     dict(kernel=2, cluster=2), dict(kernel=2, cluster=2, splits=7),
-    dict(kernel=2, dual=1, splits=1),                    # small-footprint variant (two CTAs per SM)
+    dict(kernel=2, dual=1, splits=1),
     dict(kernel=2, dual=1, splits=3),
-    dict(kernel=2, key_tile=64, splits=2),               # 64-key tiles
+    dict(kernel=2, key_tile=64, splits=2),
     dict(select=2),                                      # top-k by a cluster of CTAs per head
 ])
 def test_alternative_launch_plans_agree_with_oracle(plan, tuning):
@@ -407,8 +407,8 @@ def test_dense_step_strided_tensors_and_argument_checks():
     {},                                  # key-row kernel: its splits still meet in the cluster merge while they give up
     dict(splits=1),                      # ... one CTA per head
     dict(splits=1, persist=2),           # ... streaming variant: two resident CTAs walk the heads
-    dict(kernel=2, cluster=0, splits=3), # query-row kernel, partials and completion counters in the workspace
-    dict(kernel=2, cluster=2),           # ... cluster tail
+    dict(kernel=2, cluster=0, splits=3), # query-row kernel, partials in the workspace
+    dict(kernel=2, cluster=2),           # ... with the splits that the planner takes
 ])
 def test_a_bounded_wait_that_runs_out_is_reported_and_leaves_a_usable_library(plan, tuning):
     """With the limit of the abortable device-side waits set to zero, the first wait that is not already satisfied gives

@@ -6,7 +6,7 @@ may not allocate device memory once they run, so they cannot provide the workspa
 static variant keeps that scratch inside the library image. This file checks, through the C ABI and on two calls
 in a row (the second one finds whatever the first left in the shared scratch), that both calls give the same
 output and that this output is the oracle's. One of the shapes is planned so that its key splits leave partials in
-the scratch and meet through the completion counters, the part of the scratch that has to start at zero.
+the scratch.
 It is collected last on purpose: a run that stops at the first failure has then run everything else."""
 import numpy as np
 import pytest
@@ -38,7 +38,7 @@ def _dev(x):
 @pytest.mark.parametrize("Hq,Hkv,n_keep,cnt,plan", [
     (8, 8, 700, 700, {}),                         # few query rows per head: the splits merge inside their cluster, scratch = status word
     (8, 2, 300, 211, dict(kernel=3)),             # grouped heads on the key-row kernel: four softmax warpgroups share every tile
-    (8, 2, 1500, 1333, dict(kernel=2, cluster=0)),          # key splits leave partials in the scratch; the last CTA of a head merges them (counters)
+    (8, 2, 1500, 1333, dict(kernel=2, cluster=0)),          # key splits leave partials in the scratch; a second launch folds them
 ])
 def test_static_scratch_variant_matches_the_workspace_variant_and_the_oracle_twice(Hq, Hkv, n_keep, cnt, plan, tuning):
     import parity_util as U
