@@ -714,11 +714,20 @@ __global__ void __launch_bounds__(64 + 128 * WG * CG, (WG == 1 && CG == 1) ? 2 :
               acc.z = fmaf(r4[s2].z, w4[s2].z, acc.z); acc.w = fmaf(r4[s2].w, w4[s2].w, acc.w);
             }
           const float a[4] = {acc.x, acc.y, acc.z, acc.w};
-          const int hg = c0 / p.b, i0 = c0 - hg * p.b;    // b is a multiple of 16: the four columns are rows of one head
+          const int hg = c0 / p.b;
+          int i = c0 - hg * p.b;
           __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(p.out) + (int64_t)bi * p.o_stride[0] +
-                             (int64_t)(g * p.G + hg) * p.o_stride[1] + (int64_t)i0 * p.o_stride[2] + d_lo + dl;
+                             (int64_t)(g * p.G + hg) * p.o_stride[1] + (int64_t)i * p.o_stride[2] + d_lo + dl;
+          if ((p.b & 3) == 0) {                           // the four columns are rows of one head
 #pragma unroll
-          for (int i4 = 0; i4 < 4; ++i4) o[(int64_t)i4 * p.o_stride[2]] = __float2bfloat16_rn(a[i4]);
+            for (int i4 = 0; i4 < 4; ++i4) o[(int64_t)i4 * p.o_stride[2]] = __float2bfloat16_rn(a[i4]);
+          } else {                                        // ... or of several
+#pragma unroll
+            for (int i4 = 0; i4 < 4; ++i4) {
+              *o = __float2bfloat16_rn(a[i4]);
+              if (++i == p.b) { i = 0; o += p.o_stride[1] - (int64_t)(p.b - 1) * p.o_stride[2]; } else o += p.o_stride[2];
+            }
+          }
         }
       }
     }

@@ -250,3 +250,37 @@ def test_attention_pass_of_the_probability_saliency(cfg, block, plan, tuning):
     from test_gpu_parity import _run_sequence_case
     tuning(**plan)
     _run_sequence_case(cfg, seed=29, block=block, n_sparse=0, score=B.SCORE_PROB_MEAN)
+
+
+@pytest.mark.parametrize("b,G,D,plan", [
+    (2, 2, 128, {}), (6, 2, 128, {}), (6, 2, 64, dict(kernel=3, splits=3)), (10, 2, 128, dict(splits=1)), (14, 6, 128, dict(kernel=3)),
+    (6, 4, 128, dict(splits=1, persist=2)), (6, 10, 128, dict(kernel=4)), (3, 4, 128, dict(kernel=4, splits=1)), (5, 1, 128, {}),
+])
+def test_output_rows_behind_one_another_in_heads_first_order(b, G, D, plan, tuning):
+    """The output as [batch, row, head, D], the way a projection reads it, with a guard row behind every block: block lengths that 4
+    does not divide put rows of two heads into one group of four columns."""
+    from parity_util import assert_close, to_dev, to_host_f32
+    tuning(**plan)
+    Hkv, L, n_kept = 3, 500, 420
+    rng = np.random.default_rng(b * G)
+    q = (rng.standard_normal((1, Hkv * G, b, D)) / np.sqrt(D)).astype(np.float32)
+    k, v = (rng.standard_normal((1, Hkv, L, D)).astype(np.float32) for _ in range(2))
+    qd, kd, vd = (to_dev(x, "bf16") for x in (q, k, v))
+    d = B.make_desc(batch=1, n_q_heads=Hkv * G, n_kv_heads=Hkv, head_dim=D, seq_len_max=L, block_len=b, dtype=B.BF16, retention=0.5,
+                    n_keep_max=n_kept, o_stride=((b + 1) * Hkv * G * D, D, Hkv * G * D))
+    q64, k64, v64 = (x.cpu().double() for x in (qd, kd.repeat_interleave(G, 1), vd.repeat_interleave(G, 1)))
+    kc, vc, kn, vn = (x.contiguous() for x in (kd[:, :, :n_kept], vd[:, :, :n_kept], kd[:, :, n_kept:n_kept + b], vd[:, :, n_kept:n_kept + b]))
+    for keys in (L, n_kept + b):
+        out = torch.full((1, b + 1, Hkv * G, D), 7.0, dtype=torch.bfloat16, device="cuda")
+        code = B.OP_REFRESH_SCORES if keys == L else B.OP_SPARSE_BLOCK_ATTN
+        ws = torch.zeros((B.workspace_bytes(d, code),), dtype=torch.uint8, device="cuda")
+        if keys == L:
+            B.refresh_scores(d, qd, kd, vd, None, torch.tensor([64], dtype=torch.int32, device="cuda"), out, None, torch.empty((1, Hkv, L), device="cuda"), ws)
+        else:
+            B.sparse_block_attn(d, qd, kc, vc, torch.tensor([n_kept], dtype=torch.int32, device="cuda"), kn, vn, out, ws)
+        torch.cuda.synchronize()
+        assert B.read_status(ws) == 0
+        ref = (torch.softmax(q64 @ k64[:, :, :keys].transpose(-1, -2) / np.sqrt(D), -1) @ v64[:, :, :keys]).numpy()
+        got = to_host_f32(out)
+        assert (got[:, b] == 7.0).all(), "a row behind the block was written"
+        assert_close(got[:, :b].transpose(0, 2, 1, 3), ref, "bf16", f"{keys} keys")
