@@ -16,7 +16,7 @@
 //   - P is handed over in two parts (96 keys, then 32), so that the first MMAs of P V run under the last exponentials;
 //   - three-operand maxima, two-lane fp32 arithmetic, a quarter of the exponentials on the FMA pipe (poly_exp2), one
 //     warp-uniform branch for the rare rescale, registers moved to the softmax warps (208 instead of 168).
-// 32 heads x 1280 rows: 56.3 -> 46.2 us; 32 (8 KV) heads x 32768 rows: 17.1 -> 14.6 ms, 1206 TFLOP/s. The long case is
+// 32 heads x 1280 rows: 56.3 -> 46.2 us (40.3 with the last wave cut, see plan_dense); 32 (8 KV) heads x 32768 rows: 17.1 -> 14.6 ms, 1204 TFLOP/s. The long case is
 // bound by power (1.6 GHz under the 1000 W cap, where a library GEMM sustains 1408); a burst at full clock runs at 1368.
 // The finished rows go from TMEM through registers straight to global memory (bf16), normalised by the row sum.
 // Every wait on an mbarrier is bounded; on expiry the CTA sets an abort flag, records a code in the status word and
@@ -452,8 +452,8 @@ __global__ void __launch_bounds__(256) dense_fold_kernel(const DenseParams p) {
 
 // How the units (a sequence's head and pair of query tiles) of a call are launched: the first `whole` of them one CTA each, the
 // rest - what the last full wave leaves over, or all of less than a wave - with their key tiles shared out to `parts` CTAs. A
-// unit takes a whole SM, so without that 160 units on 148 SMs run in two waves (32 heads x 1280 rows: 46.2 us, 42.8 so; 28 heads
-// x 4096: 245 us, 200; 16 heads x 3000: 106, 81). Costs in us: a key tile 1.55, a CTA's set-up and way out 6.5, of which a cut unit overlaps 2 with the
+// unit takes a whole SM, so without that 160 units on 148 SMs run in two waves (32 heads x 1280 rows: 46.2 us, 40.3 so; 28 heads
+// x 4096: 245 us, 199; 16 heads x 3000: 102, 82). Costs in us: a key tile 1.55, a CTA's set-up and way out 6.5, of which a cut unit overlaps 2 with the
 // wave in front, its partial rows and the launch that folds
 // them 7.25 (3 of it a margin) and 0.35 per share.
 // Batches of several sequences may be ragged, which the host cannot see: they are cut only where all units fit one wave.
