@@ -11,11 +11,12 @@
 //   * the mean-query saliency of Algorithm 1 ("qbar <- Mean(Q_b)", "A <- MatMul(qbar, K_f^T)") is, by linearity, the
 //     mean of the key's N logits: the thread that owns the key already holds them, no separate pass over K;
 //   * the finished O^T has one head dimension per thread and N columns: key splits are merged column by column.
-// The softmax needs one reference value per query (column) that all keys share. It is taken once, from the column
-// maxima of the CTA's first tile (warp reductions and a shared-memory max), and afterwards only checked: a tile
-// whose logits exceed a reference by more than 2^8 makes the softmax threads raise the references and rescale O^T and
-// the partial sums (rare). P is bf16, whose exponent range is that of fp32, so a reference within 2^8 of the true
-// maximum loses nothing.
+// The softmax needs one reference value per query (column) that all keys share: the logit of the first key of the CTA's first
+// tile, and afterwards only checked: a tile whose logits exceed a reference by more than 2^64 makes the softmax threads raise
+// the references to its column maxima and rescale O^T and the partial sums (rare). P is bf16, whose exponent range is that of
+// fp32, so a reference within 2^64 of the true maximum loses nothing. The raised references come from the logits themselves, which
+// tensor memory still holds: the distance to a reference far below them (a first key that is taken out, or nearly) has lost their
+// last digits, or all of them.
 //
 // The key axis is  [source 1 rows 0..n1) ++ [source 2 rows 0..n2)  cut into groups of 32 rows; a CTA takes a contiguous
 // range of groups and walks it in tiles of up to four groups (128 keys), so a tile may mix the two sources.
@@ -397,54 +398,53 @@ __global__ void __launch_bounds__(64 + 128 * WG * CG, (WG == 1 && CG == 1) ? 2 :
       }
       // ---- the references. The first key of the CTA's first tile lends its logits: it is part of the softmax, so sums
       //      never vanish, and exp2 of anything up to 2^64 above it is still an ordinary bf16 / fp32 number. Every tile is
-      //      only checked against the references; one that exceeds them by more than 64 raises them (rare). ----
+      //      only checked against the references; one that exceeds them by more than 64 raises them (rare, and where the
+      //      first key is taken out). ----
       if (t < WG) {
         if (row == 0 && work) {
 #pragma unroll
           for (int c = 0; c < NP; c += 4)
             *reinterpret_cast<float4*>(m_ref + c) = make_float4(sv[c] * sl2, sv[c + 1] * sl2, sv[c + 2] * sl2, sv[c + 3] * sl2);
-          if constexpr (SHARE) {                       // a key that is taken out (-inf) cannot lend: zero stands in
-#pragma unroll
-            for (int c = 0; c < NP; ++c)
-              if (sv[c] == -INFINITY) m_ref[c] = 0.f;
-          }
         }
         softmax_barrier(bar_id);
       }
-      float far0 = -INFINITY, far1 = -INFINITY;        // the largest distance above a reference
+      float far0 = -INFINITY, far1 = -INFINITY;        // the largest distance above a reference, NaN where one is unusable
 #pragma unroll
       for (int c = 0; c < NP; c += 4) {
         const float4 m4 = *reinterpret_cast<const float4*>(m_ref + c);
         sv[c] = fmaf(sv[c], sl2, -m4.x); sv[c + 1] = fmaf(sv[c + 1], sl2, -m4.y);
         sv[c + 2] = fmaf(sv[c + 2], sl2, -m4.z); sv[c + 3] = fmaf(sv[c + 3], sl2, -m4.w);
-        far0 = fmaxf(far0, fmaxf(sv[c], sv[c + 1])); far1 = fmaxf(far1, fmaxf(sv[c + 2], sv[c + 3]));
+        far0 = max3_nan(far0, sv[c], sv[c + 1]); far1 = max3_nan(far1, sv[c + 2], sv[c + 3]);
       }
-      const bool over = fmaxf(far0, far1) > 64.f;
+      const bool over = !(max_nan(far0, far1) <= 64.f);
       if (softmax_barrier_or(bar_id, over && work && valid)) {
-        // ---- raise the references by the tile's column maxima (where positive) and rescale what has been accumulated.
+        // ---- raise the references to the tile's column maxima (where higher) and rescale what has been accumulated.
         //      Every PV issued so far must have landed before O^T is rewritten; the PV of this tile waits for our arrive. ----
         if (t >= WG && !dead && !wait_bar_warp(BAR(PV_DONE + ((t - WG) & 1)), ((t - WG) >> 1) & 1, abort_flag, p.status, 8, wlim)) dead = true;
         tc_fence_after();
-        if (st < NP) enc[st] = f2ord(0.f);
+        if (st < NP) enc[st] = f2ord(usable_reference(m_ref[st]));
         softmax_barrier(bar_id);
         if (work) {
-          float mine = 0.f;
+          tmem_ld32(lane_addr + (uint32_t)sb * NPT + (uint32_t)cg * 32, *reinterpret_cast<uint32_t(*)[32]>(&sv[0]));
+          tc_wait_ld();
+          float mine = -INFINITY;
 #pragma unroll
           for (int c = 0; c < NP; ++c) {
-            const float r = warp_max_f32(valid ? sv[c] : -INFINITY);
+            const float r = warp_max_f32(valid ? sv[c] * sl2 : -INFINITY);
             if (c == lane) mine = r;
           }
           atomicMax(enc + lane, f2ord(mine));
         }
         softmax_barrier(bar_id);
         if (st < NP) {
-          const float dlt = ord2f(enc[st]);            // >= 0
-          delta_s[st] = dlt;
-          m_ref[st] += dlt;
+          const float up = ord2f(enc[st]);
+          delta_s[st] = up - usable_reference(m_ref[st]);      // >= 0
+          m_ref[st] = up;
         }
         softmax_barrier(bar_id);
+        // (at most zero but for the rounding of the reference, which for logits beyond 10^9 would be more than exp2 can take)
 #pragma unroll
-        for (int c = 0; c < NP; ++c) sv[c] -= delta_s[c];
+        for (int c = 0; c < NP; ++c) sv[c] = min_nan(fmaf(sv[c], sl2, -m_ref[c]), 0.f);
         l_lane *= fast_exp2(-delta_s[lane]);
         if (t >= WG && !dead) {
           // this thread's TMEM lane is a head dimension of O^T here, not a key: all four warps rescale their lanes

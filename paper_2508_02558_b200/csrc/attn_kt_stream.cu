@@ -419,40 +419,43 @@ __global__ void __launch_bounds__(KS_THREADS, 1) attn_kt_stream_kernel(const __g
           }
           softmax_barrier(bar_id);
         }
-        float far0 = -INFINITY, far1 = -INFINITY;      // the largest distance above a reference
+        float far0 = -INFINITY, far1 = -INFINITY;      // the largest distance above a reference, NaN where one is unusable
 #pragma unroll
         for (int c = 0; c < NP; c += 4) {
           const float4 m4 = *reinterpret_cast<const float4*>(m_ref + c);
           sv[c] = fmaf(sv[c], sl2, -m4.x); sv[c + 1] = fmaf(sv[c + 1], sl2, -m4.y);
           sv[c + 2] = fmaf(sv[c + 2], sl2, -m4.z); sv[c + 3] = fmaf(sv[c + 3], sl2, -m4.w);
-          far0 = fmaxf(far0, fmaxf(sv[c], sv[c + 1])); far1 = fmaxf(far1, fmaxf(sv[c + 2], sv[c + 3]));
+          far0 = max3_nan(far0, sv[c], sv[c + 1]); far1 = max3_nan(far1, sv[c + 2], sv[c + 3]);
         }
-        const bool over = fmaxf(far0, far1) > 64.f;
+        const bool over = !(max_nan(far0, far1) <= 64.f);
         if (softmax_barrier_or(bar_id, over && work && valid)) {
-          // ---- raise the references by the tile's column maxima (where positive) and rescale what has been accumulated:
+          // ---- raise the references to the tile's column maxima (where higher) and rescale what has been accumulated:
           //      the warpgroup's previous PV of this unit must have landed before O^T_w is rewritten ----
           if (t > t0 && !dead && !wait_bar_warp(BAR(PV_DONE + w), (uint32_t)((G - 2) >> 1) & 1u, abort_flag, p.status, 8, wlim)) dead = true;
           tc_fence_after();
-          if (st < NP) enc[st] = f2ord(0.f);
+          if (st < NP) enc[st] = f2ord(usable_reference(m_ref[st]));
           softmax_barrier(bar_id);
           if (work) {
-            float mine = 0.f;
+            tmem_ld32(lane_addr + (uint32_t)w * NP, *reinterpret_cast<uint32_t(*)[32]>(&sv[0]));
+            tc_wait_ld();
+            float mine = -INFINITY;
 #pragma unroll
             for (int c = 0; c < NP; ++c) {
-              const float r = warp_max_f32(valid ? sv[c] : -INFINITY);
+              const float r = warp_max_f32(valid ? sv[c] * sl2 : -INFINITY);
               if (c == lane) mine = r;
             }
             atomicMax(enc + lane, f2ord(mine));
           }
           softmax_barrier(bar_id);
           if (st < NP) {
-            const float dlt = ord2f(enc[st]);          // >= 0
-            delta_s[st] = dlt;
-            m_ref[st] += dlt;
+            const float up = ord2f(enc[st]);
+            delta_s[st] = up - usable_reference(m_ref[st]);      // >= 0
+            m_ref[st] = up;
           }
           softmax_barrier(bar_id);
+          // (at most zero but for the rounding of the reference, which for logits beyond 10^9 would be more than exp2 can take)
 #pragma unroll
-          for (int c = 0; c < NP; ++c) sv[c] -= delta_s[c];
+          for (int c = 0; c < NP; ++c) sv[c] = min_nan(fmaf(sv[c], sl2, -m_ref[c]), 0.f);
           l_lane *= fast_exp2(-delta_s[lane]);
           if (t > t0 && !dead) {
             // this thread's TMEM lane is a head dimension of O^T here, not a key: all four warps rescale their lanes

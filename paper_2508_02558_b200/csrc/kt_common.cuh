@@ -74,6 +74,10 @@ __device__ __forceinline__ uint32_t f2ord(float x) {
 }
 __device__ __forceinline__ float ord2f(uint32_t k) { return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k); }
 
+// A softmax reference that the first key of a walk lent: the lowest finite number where that key is taken out (-inf) or NaN, which no
+// distance can be taken to. Every ordinary logit lies far above it and raises it.
+__device__ __forceinline__ float usable_reference(float m) { return fmaxf(m, -3.402823466e38f); }
+
 // Shared-memory matrix descriptor with the 64-byte swizzle (mode 4 in bits 61-63): rows of 64 bytes, 8 rows per atom.
 __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
   return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo_bytes >> 4) << 16) | ((uint64_t)(sbo_bytes >> 4) << 32) |
