@@ -54,7 +54,7 @@ constexpr int KT_MAX_STAGES = 3;
 
 // WG = 2: two softmax warpgroups take the tiles in turn, each with its own accumulator and references (32 query columns).
 // CG > 1: CG softmax warpgroups share every tile, each owning 32 of the 32 * CG query columns (one accumulator).
-// SHARE: a unit holds part of a KV head's query rows (reuse step, see kt_units_per_head; a variant of its own, the few
+// SHARE: a unit holds part of a KV head's query rows (reuse step, see plan_attention_units; a variant of its own, the few
 // instructions more at the start cost 0.7 % of the ordinary reuse step).
 template <int D, int WG, int CG, bool SHARE>
 __global__ void __launch_bounds__(64 + 128 * WG * CG, (WG == 1 && CG == 1) ? 2 : 1) attn_kt_kernel(const __grid_constant__ KtMaps tm, const KtParams kp) {
@@ -884,42 +884,6 @@ bool kt_preferred(int D, int M, int B, int Hkv, int n1_max, int n2) {
   return !(units * 8 <= sms && tiles > (D == 64 ? 20 : 40));
 }
 
-// Reuse step: how many units the query rows of a KV head are shared out to (1: it is one unit). Each unit walks the KV head's keys
-// for itself, so K and V come from L2 once per unit; in exchange a unit has the 32 columns of a softmax warpgroup (or 64, two),
-// two CTAs share an SM, its splits merge in their cluster, and there is no second launch. Ahead of the kernels that take a KV
-// head's rows together (600 random shapes of 33 to 256 rows, 1 to 16 sequences, 40 to 20000 cached keys: the rule below 6 %
-// faster on average) while the walks are short - at most five tiles of 128 keys per SM in all (at 5.6, 8 KV heads of 4 x 32 rows and
-// 3273 keys, 12.4 us against 11.3), and 36 a unit, since a cluster has no more than eight CTAs:
-//   - 65 to 128 rows: 8 KV heads of 4 x 32 rows, 400 / 1000 / 2000 keys: 8.3 / 9.3 / 10.0 us, now 6.6 / 8.0 / 8.6; 8000 keys 16.6
-//     against 20.6;
-//   - more rows, two Q tiles in the query-row kernel: up to four tiles (100 / 400 keys, 4 KV heads of 7 x 32 rows: 9.4 / 9.2 us,
-//     now 5.3 / 6.5); where half the lead is gone, at 1000 keys (9.8 and 7.6), the query-row kernel stays. Heads of 4 x 64 rows
-//     make full units of 64, which pay further (4 sequences x 8 KV heads x 760 keys: 19.8 us, now 13.7);
-//   - 33 to 64 rows: up to four tiles (8 KV heads of 4 x 16 rows, 150 keys: 7.3 us, now 5.4; at 400 keys 7.3 and 6.5);
-//   - head dimension 64 with at most 64 rows: nearly always (5 to 15 %), since a tile is half the bytes.
-// Units that fill a quarter of their columns (heads of 8 rows) count as four times as long; half-filled ones (7 x 16 rows) lose 2 to 4 %
-// from nine tiles on and are for four tiles only.
-int kt_units_per_head(int dtype, int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn) {
-  const int sms = sm_count(), G = M / b;
-  // the fewest units of at most `rows` rows each: whole heads, or equal parts of one
-  auto units_of = [&](int rows) {
-    int s = 1;
-    if (b > rows) s = b % rows == 0 ? M / rows : 0;
-    else while (s < G && (G % s != 0 || M / s > rows)) ++s;
-    return s > 1 && kt_supported(dtype, D, M / s, b) ? s : 0;
-  };
-  if (M <= 32 || M > 256 || tn.persist > 0 || tn.splits > 0) return 1;
-  if (tn.unit_rows > 0) { const int s = tn.unit_rows <= 64 ? units_of(tn.unit_rows) : 0; return s > 0 ? s : 1; }
-  const double tiles = 0.25 * ((n1_max + 31) / 32 + (n2 + 31) / 32);
-  const long long heads = (long long)B * Hkv;
-  const int s32 = units_of(32), s64 = units_of(64);
-  if (M <= 64 && D == 64) return s32 > 0 && heads * s32 <= sms && tiles <= 100 ? s32 : 1;
-  if (tiles > 36) return 1;
-  if (s32 > 0 && (tiles <= 4.5 || (M > 64 && M <= 128 && 16 * s32 < M)) && heads * s32 <= (M > 128 ? 2 : 1) * sms && heads * s32 * tiles * (32 * s32) <= 5. * sms * M) return s32;
-  if (s64 > 0 && D == 128 && 64 * s64 == M && heads * s64 <= sms && heads * s64 * tiles <= 5. * sms) return s64;
-  return 1;
-}
-
 AttnPlan plan_attention_kt(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn) {
   (void)b;
   AttnPlan pl{};
@@ -1052,6 +1016,68 @@ AttnPlan plan_attention_kt(int D, int M, int b, int B, int Hkv, int n1_max, int 
     pl.n_counters = 2;                  // the next unit to hand out, and the CTAs that have finished
   }
   return pl;
+}
+
+// Reuse step: whether the query rows of a KV head are shared out to several units, and their plan. Each unit walks the KV head's keys
+// for itself, so K and V come from L2 once per unit; in exchange a unit has the 32 columns of a softmax warpgroup (or 64, two),
+// two CTAs share an SM, its splits merge in their cluster, and there is no second launch. Ahead of the kernels that take a KV
+// head's rows together while the walks are short: what counts is how many tiles the CTA with the most walks, since a cluster has no
+// more than eight. From 2628 calls (head dimension 64 and 128, 33 to 256 rows, 1 to 64 heads, 50 to 12500 cached keys; units and whole
+// heads timed one after the other): the rule takes units for 2010 of them, 18 % faster on average there; 29 lose more than 2 %, at most 10.
+//   - 65 to 128 rows: two tiles a CTA, three where whole heads have few splits or are few themselves (8 KV heads of 4 x 32 rows, 400 / 1000 /
+//     2000 keys: 8.6 / 9.4 / 10.1 us, now 7.0 / 8.4 / 9.0; at 3273 keys, four tiles, 13.5 against 11.3). Units of 64 rows, which walk twice as many
+//     tiles, only from 25 heads on (32 heads x 1000 keys 15.3, now 14.1; 8 x 3000, where there were such units, 11.8 and 12.4);
+//   - more rows, two Q tiles in the query-row kernel: units of 32 rows up to four and a half tiles in all (100 / 400 keys, 4 KV heads of
+//     7 x 32 rows: 9.4 / 9.2 us, now 5.3 / 6.5), full units of 64 up to four a CTA, further with more units (8 KV heads of 4 x 64 rows, 1000
+//     keys: 13.0 us, now 11.2; 4 x 4000, five tiles, 13.0 and 14.4);
+//   - 33 to 64 rows, head dimension 128: four and a half tiles in all (8 KV heads of 4 x 16 rows, 150 keys: 7.3 us, now 5.4);
+//   - head dimension 64, whose tile is half the bytes: four tiles a CTA while the units are few (2 heads of 4 x 16 rows, 3000 keys: 8.6 us, now
+//     6.9; 8500 keys, nine tiles, 10.0 and 12.7), beyond one per four SMs only full units. Half-filled ones (7 x 8 rows) walk the
+//     keys once per unit for little: 12 heads x 12500 keys 18.1 against 63 us.
+// Nine to twelve groups are few for so many units: four splits that walk less than a tile each cost more than they save.
+bool plan_attention_units(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn, AttnPlan* pl) {
+  const int sms = sm_count(), G = M / b, groups = (n1_max + 31) / 32 + (n2 + 31) / 32, T = (groups + 3) / 4;
+  const double tiles = 0.25 * groups;
+  const long long heads = (long long)B * Hkv;
+  // the fewest units of at most `rows` rows each: whole heads, or equal parts of one
+  auto units_of = [&](int rows) {
+    int s = 1;
+    if (b > rows) s = b % rows == 0 ? M / rows : 0;
+    else while (s < G && (G % s != 0 || M / s > rows)) ++s;
+    return s > 1 && M / s % 4 == 0 && M / s <= 128 ? s : 0;
+  };
+  if (M <= 32 || M > 256 || b > 128 || tn.persist > 0 || tn.splits > 0) return false;
+  int s = 0;
+  if (tn.unit_rows > 0) {
+    s = tn.unit_rows <= 64 ? units_of(tn.unit_rows) : 0;
+  } else {
+    // Units that fill a quarter of their columns (heads of 8 rows) count as four times as long.
+    const int s32 = units_of(32), s64 = units_of(64);
+    if (M <= 64 && D == 64) s = heads * s32 <= sms && tiles <= 100 ? s32 : 0;
+    else if (tiles > 36) return false;
+    else if (s32 > 0 && (tiles <= 4.5 || (M > 64 && M <= 128 && 16 * s32 < M)) && heads * s32 <= (M > 128 ? 2 : 1) * sms && heads * s32 * tiles * (32 * s32) <= 5. * sms * M) s = s32;
+    else if (s64 > 0 && D == 128 && 64 * s64 == M && heads * s64 <= sms && heads * s64 * tiles <= 5. * sms) s = s64;
+  }
+  if (s == 0) return false;
+  Tuning one_unit = tn;                      // (the streaming variant's units are KV heads)
+  one_unit.persist = 0;
+  *pl = plan_attention_kt(D, M / s, b, B, Hkv * s, n1_max, n2, one_unit);
+  pl->kv_share = s;
+  if (tn.unit_rows > 0 || groups <= 6) return true;
+  const int rows = M / s, walk = ((groups + pl->cluster - 1) / pl->cluster + 3) / 4;      // tiles of the longest walk
+  const long long units = heads * s;
+  if (M > 128) return rows <= 32 || walk <= 4 || (units > 16 && walk <= 6) || units > 64;
+  if (D == 128) {
+    if (rows > 32) return units > 48 && T != 3;
+    if (M <= 64) return units <= 32 || (T > 3 && rows >= 24);
+    return rows <= 16 || walk <= 2 || units > 64 || (walk == 3 && (units <= 8 || units > 16));
+  }
+  if (M <= 64) {
+    if (T <= 4 && units <= 28) return true;
+    return units <= rows ? walk <= 4 && (units <= 24 || walk != 2 || T > 12) : rows >= 24 && units <= 64 && T > 3 && tiles <= 48.;
+  }
+  if (rows <= 16) return units <= 32;
+  return units <= 16 ? walk <= 4 : walk <= 2 && (units <= 32 || T != 3);
 }
 
 // The attention of a refresh whose saliency and selection run beside it (refresh_select.cu): CTAs of the small footprint on about

@@ -752,7 +752,7 @@ AttnPlan plan_attention_kt(int D, int M, int b, int B, int Hkv, int n1_max, int 
 cudaError_t launch_attn_kt(const AttnParams& p, const AttnPlan& pl, int D, cudaStream_t st);
 
 bool pair_supported(int dtype, int D, int M, int b);
-int kt_units_per_head(int dtype, int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn);
+bool plan_attention_units(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn, AttnPlan* pl);
 AttnPlan plan_attention_pair(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn);
 cudaError_t launch_attn_pair(const AttnParams& p, const AttnPlan& pl, int D, cudaStream_t st);
 
@@ -763,14 +763,8 @@ AttnPlan plan_attention(int dtype, int D, int M, int b, int B, int Hkv, int n1_m
   // With the probability saliency (prob_scores) the attention pass is the kernel of this file, whatever the family.
   const Tuning tn = tuning();
   if (prob_scores && tn.kernel != 1 && umma_supported(dtype, D, M, b)) return plan_attention_umma(D, M, b, B, Hkv, n1_max, tn);
-  const int share = n2 > 0 && tn.kernel == 0 ? kt_units_per_head(dtype, D, M, b, B, Hkv, n1_max, n2, tn) : 1;
-  if (share > 1) {
-    Tuning one_unit = tn;                // (the streaming variant's units are KV heads)
-    one_unit.persist = 0;
-    AttnPlan pl = plan_attention_kt(D, M / share, b, B, Hkv * share, n1_max, n2, one_unit);
-    pl.kv_share = share;
-    return pl;
-  }
+  AttnPlan units;
+  if (n2 > 0 && tn.kernel == 0 && umma_supported(dtype, D, 16, 16) && plan_attention_units(D, M, b, B, Hkv, n1_max, n2, tn, &units)) return units;
   const bool kt_ok = kt_supported(dtype, D, M, b);
   if (kt_ok && (tn.kernel == 3 || (tn.kernel == 0 && kt_preferred(D, M, B, Hkv, n1_max, n2))))
     return plan_attention_kt(D, M, b, B, Hkv, n1_max, n2, tn);
