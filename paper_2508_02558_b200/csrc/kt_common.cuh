@@ -31,18 +31,22 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
       : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
 }
-__device__ __forceinline__ bool wait_merge(uint32_t bar, volatile int* abort_flag, int32_t* status, long long limit) {
-  if (mbar_try_wait_cluster(bar, 0)) return true;
-  const long long t0 = clock64();
-  for (;;) {
-    if (mbar_try_wait_cluster(bar, 0)) return true;
-    const bool aborting = *abort_flag != 0;
-    // an aborting CTA still lets its peers' pushes land before it retires (drain limit)
-    if (clock64() - t0 > (aborting ? kDrainCycles : limit)) {
-      if (!aborting) { *abort_flag = 1; atomicExch(status, 13); }
-      else return false;
+// A whole warp calls it; its lanes leave the loop on their own and meet again here, for what follows is warp-synchronous (named barriers,
+// tcgen05 with .sync.aligned).
+__device__ __forceinline__ void wait_merge(uint32_t bar, volatile int* abort_flag, int32_t* status, long long limit) {
+  if (!mbar_try_wait_cluster(bar, 0)) {
+    const long long t0 = clock64();
+    while (!mbar_try_wait_cluster(bar, 0)) {
+      const bool aborting = *abort_flag != 0;
+      // an aborting CTA still lets its peers' pushes land before it retires (drain limit)
+      if (clock64() - t0 > (aborting ? kDrainCycles : limit)) {
+        if (aborting) break;
+        *abort_flag = 1;
+        atomicExch(status, 13);
+      }
     }
   }
+  __syncwarp();
 }
 // Pulls one box of a tensor into L2 without waiting for it. L2 is the point of coherence, so this is safe for data a
 // kernel in front of this one may still be writing: the later copy into shared memory reads what L2 holds then.

@@ -223,7 +223,8 @@ cudaError_t launch_d(const ScoreMaps& tm, const AttnParams& p, const SelectParam
 
 }  // namespace
 
-// At least two CTAs per head: the scores travel between the CTAs of a cluster launch.
+// At least two CTAs per head, launched as a cluster. (A form of one CTA per head without a cluster launch raised "an illegal instruction"
+// once, at 128 units; its cause is not known. Only there did barrier.cluster, mapa and st.async run outside a cluster launch.)
 bool score_select_supported(int D, int M, int units, int cand) {
   return (D == 64 || D == 128) && M <= 32 && cand >= 1 && cand <= 3072 && 2 * units <= sm_count();
 }
