@@ -14,8 +14,9 @@
 // here; this kernel ends only behind that one's end.
 // Twelve warps of at most 56 registers and less than 120 KB leave room for a CTA of attn_kt.cu on the same SM (registers are
 // allotted per SM quarter: its six warps take up to 10752 of 16384 there; with sixteen warps of 64 nothing ran beside anything).
-// Every mbarrier wait is bounded; on expiry the CTA sets an abort flag, records a code in the status word, meets its peers at
-// the cluster barriers all the same and runs to its end.
+// Every mbarrier wait is bounded; on expiry the CTA sets an abort flag, records a code in the status word, sends its peers the scores they
+// count on all the same, waits at a second cluster barrier until theirs are on their way and for the bytes themselves (a CTA must not
+// leave while a peer still writes to it), and runs to its end.
 #include <cuda.h>
 #include <string.h>
 
@@ -104,7 +105,7 @@ __global__ void __launch_bounds__(RS_THREADS, 3) score_select_kernel(const __gri
   const int L = min(max(len, 0), p.n1_max);
   const HeadPlace h = place_head(sp, L, off);
   const RawAxis axis(sp, h);
-  if (tid == 0 && h.C > 0) mbar_expect_tx(BAR(SCORES), (uint32_t)h.C * 4u);      // the scores that come from all CTAs of the cluster, this one included
+  if (tid == 0) mbar_expect_tx(BAR(SCORES), (uint32_t)h.C * 4u);      // the scores that come from all CTAs of the cluster, this one included
   axis.clear_ends(raw_s, h.C, tid, NT);
 
   // ======================================= scores =======================================
@@ -158,8 +159,9 @@ __global__ void __launch_bounds__(RS_THREADS, 3) score_select_kernel(const __gri
     }
   }
   if (warp >= 4 || nt == 0) cluster_wait_acquire();    // (every thread passes the barrier once)
+  cluster_arrive_relaxed();                            // "this CTA's scores are on their way"
   tc_fence_before();
-  if (h.C > 0) wait_merge(BAR(SCORES), abort_flag, p.status, p.wait_cycles);      // the head's scores are here
+  wait_merge(BAR(SCORES), abort_flag, p.status, p.wait_cycles);      // the head's scores are here
   __syncthreads();
   if (*abort_flag) {                                   // a wait gave up, in whichever warp: what is under way lands first
     if (warp == 4 && nt > 0) {
@@ -168,6 +170,8 @@ __global__ void __launch_bounds__(RS_THREADS, 3) score_select_kernel(const __gri
       drain_bar(BAR(Q_FULL), 0);
       __syncwarp();
     }
+    cluster_wait_acquire();                            // a slower peer may still be sending: this CTA goes on, and leaves, when all is here
+    drain_bar(BAR(SCORES), 0);
     __syncthreads();
   }
   tc_fence_after();
@@ -195,6 +199,7 @@ __global__ void __launch_bounds__(RS_THREADS, 3) score_select_kernel(const __gri
   __syncthreads();
   for (int i = i_lo + tid; i < i_hi; i += NT) out[i] = kept_s[i - i_lo];
   gather_rows<NT, Sh::STAGES>(cp, gh, ring, kept_s, i_lo, i_hi);
+  if (!*abort_flag) cluster_wait_acquire();            // (every thread passes the second barrier once)
   grid_dependency_wait();                              // this launch must not be over before the one in front of it is
 }
 
