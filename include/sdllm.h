@@ -131,8 +131,9 @@ int32_t sdllm_cache_state(int32_t step_in_block, int32_t delay);
 int32_t sdllm_launch_count(const sdllm_desc* desc, int op);
 
 /* Host-only; the paper has no counterpart. Writes a short NUL-terminated description of the launch plan of an attention
- * call (`op` = SDLLM_OP_REFRESH_SCORES or SDLLM_OP_SPARSE_BLOCK_ATTN) into buf[0..buf_bytes): the kernel's name first,
- * then its grid in words, e.g. "attn_kt_kernel splits=6 cluster=6 stages=1 threads=192". For logs and for naming the
+ * call (`op` = SDLLM_OP_REFRESH_SCORES, SDLLM_OP_SPARSE_BLOCK_ATTN or SDLLM_OP_REFRESH, which names the launch that selects
+ * behind its attention) into buf[0..buf_bytes): the kernel's name first, then its grid in words, e.g.
+ * "attn_kt_kernel splits=6 cluster=6 stages=1 threads=192". For logs and for naming the
  * kernel a measurement belongs to; the text is not a stable format. The plan depends on the current device's SM
  * count and on sdllm_tuning_set. Returns SDLLM_ERR_INVALID_ARG for a bad description, op, or a NULL / empty buffer. */
 sdllm_status sdllm_plan_describe(const sdllm_desc* desc, int op, char* buf, size_t buf_bytes);

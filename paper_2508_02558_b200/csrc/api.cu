@@ -330,18 +330,27 @@ sdllm_status sdllm_keep_count(const sdllm_desc* d, int32_t seq_len, int32_t bloc
 sdllm_status sdllm_plan_describe(const sdllm_desc* d, int op, char* buf, size_t buf_bytes) {
   if (buf == nullptr || buf_bytes == 0) return SDLLM_ERR_INVALID_ARG;
   buf[0] = 0;
-  if (check_desc(d) != SDLLM_OK || (op != SDLLM_OP_REFRESH_SCORES && op != SDLLM_OP_SPARSE_BLOCK_ATTN)) return SDLLM_ERR_INVALID_ARG;
-  const AttnPlan pl = plan_for(d, op);
+  if (check_desc(d) != SDLLM_OK || (op != SDLLM_OP_REFRESH_SCORES && op != SDLLM_OP_SPARSE_BLOCK_ATTN && op != SDLLM_OP_REFRESH)) return SDLLM_ERR_INVALID_ARG;
+  const bool whole = op == SDLLM_OP_REFRESH;
+  AttnPlan pl = plan_for(d, whole ? SDLLM_OP_REFRESH_SCORES : op);
+  const bool fused = whole && refresh_is_fused(d, pl), beside = fused && refresh_is_beside(d, pl) && d->score != SDLLM_SCORE_PROB_MEAN;
+  if (beside) pl = plan_attention_kt_beside(d->head_dim, d->n_q_heads / d->n_kv_heads * d->block_len, d->batch, d->n_kv_heads, d->seq_len_max);
   const char* name = pl.kind == 3   ? (pl.persistent ? "attn_kt_stream_kernel" : "attn_kt_kernel")
                      : pl.kind == 4 ? "attn_pair_kernel"
                      : pl.kind == 2 ? "attn_umma_bf16_kernel"
                                     : (d->dtype == SDLLM_BF16 ? "attn_bf16_kernel" : "attn_f32_kernel");
+  const char* rest = "";
+  if (whole) {
+    const bool one = select_compact_is_fused(d->batch, d->n_kv_heads, d->seq_len_max, d->block_len, d->n_keep_max);
+    rest = beside ? "; beside it score_select_kernel" : fused ? (one ? "; pooled and folded in select_gather_kernel" : "; pooled and folded in select_topk_kernel")
+                                                              : (one ? "; then select_gather_kernel" : "; then selection and gather");
+  }
   if (pl.kind == 3)
-    snprintf(buf, buf_bytes, "%s splits=%d cluster=%d stages=%d softmax_warpgroups=%d threads=%d smem=%zu", name, pl.cluster, pl.cluster,
-             pl.stages, pl.c_warps * pl.warp_keys, pl.threads, pl.smem_bytes);
+    snprintf(buf, buf_bytes, "%s splits=%d cluster=%d stages=%d softmax_warpgroups=%d threads=%d smem=%zu%s", name, pl.cluster, pl.cluster,
+             pl.stages, pl.c_warps * pl.warp_keys, pl.threads, pl.smem_bytes, rest);
   else
-    snprintf(buf, buf_bytes, "%s splits=%d cluster=%d stages=%d key_tile=%d threads=%d smem=%zu", name, pl.splits, pl.cluster, pl.stages,
-             pl.key_tile, pl.threads, pl.smem_bytes);
+    snprintf(buf, buf_bytes, "%s splits=%d cluster=%d stages=%d key_tile=%d threads=%d smem=%zu%s", name, pl.splits, pl.cluster, pl.stages,
+             pl.key_tile, pl.threads, pl.smem_bytes, rest);
   return SDLLM_OK;
 }
 
