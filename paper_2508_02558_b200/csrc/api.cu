@@ -148,15 +148,35 @@ bool refresh_is_beside(const sdllm_desc* d, const AttnPlan& pl) {
   return pl.kind == 3 && tuning().fused_refresh == 1 &&
          score_select_supported(d->head_dim, d->n_q_heads / d->n_kv_heads * d->block_len, d->batch * d->n_kv_heads, d->seq_len_max - d->block_len);
 }
+// CTAs per (sequence, KV head) of the launch behind that fold the key splits: each folds 1024 float4 columns at a time, and they take at
+// most half of the SMs. 0: there are none to fold.
+int fold_ctas(const sdllm_desc* d, const AttnPlan& pl) {
+  const int M = d->n_q_heads / d->n_kv_heads * d->block_len;
+  if (pl.splits <= 1 || (d->score == SDLLM_SCORE_PROB_MEAN && umma_tail_is_fused(pl, d->head_dim, M))) return 0;
+  const int items = (pl.kind == 4 ? pl.row_tiles * 128 : M) * (d->head_dim / 4), room = sm_count() / (2 * d->batch * d->n_kv_heads);
+  return (items + 1023) / 1024 < room ? (items + 1023) / 1024 : (room > 1 ? room : 1);
+}
+// Whether the CTAs that fold take more from the gather than the launch that they spare costs. A CTA copies some 85 GB/s (read and written),
+// and each of them is one less to copy the head's rows, where a head has more than one: 4 us (7.5 with the probability saliency, where fold and
+// pooling leave a longer chain) is where both ways are even over 428 refreshes of 8 to 148 heads. (50 KV heads of 96 rows, retention
+// 0.9, 700 / 2300 / 4500 keys: 27.8 / 62.4 / 116.6 us folding beside the gather, 29.1 / 54.8 / 95.0 in a launch of its own.)
+bool fold_delays_gather(const sdllm_desc* d, const AttnPlan& pl) {
+  const int folds = fold_ctas(d, pl);
+  if (folds == 0) return false;
+  const double us = (double)d->n_keep_max * d->head_dim * elem_size(d->dtype) * 4 / 85e3;         // one CTA alone
+  return us / gather_ctas(d->batch, d->n_kv_heads, d->n_keep_max, folds) - us / gather_ctas(d->batch, d->n_kv_heads, d->n_keep_max, 0) >
+         (d->score == SDLLM_SCORE_PROB_MEAN ? 7.5 : 4.);
+}
+
 // Whether its second launch does more than select and gather: that, or, behind the kernels that pool and fold in a launch of their
 // own, their pooling and fold. (The key-row kernel pools behind its merge, which costs it less than the other launch: 16 x 600 keys
 // 14.1 against 14.5 us, 74 x 800 25.7 against 26.4, 64 x 3000 48.3 against 46.9. The probability saliency with one row tile: its second
 // pass folds the rows' sums itself, so the fold is off the chain.)
 bool refresh_is_fused(const sdllm_desc* d, const AttnPlan& pl) {
   const bool kind = d->score == SDLLM_SCORE_PROB_MEAN ? pl.kind == 2 && pl.row_tiles == 1 : pl.kind != 3 || refresh_is_beside(d, pl);
-  return kind && d->pool_window <= kMaxFusedWindow && d->n_keep_max <= d->seq_len_max - d->block_len && tuning().fused_refresh != 0 &&
-         (select_compact_is_fused(d->batch, d->n_kv_heads, d->seq_len_max, d->block_len, d->n_keep_max) ||
-          (pl.kind != 3 && select_is_clustered(d->batch, d->n_kv_heads, d->seq_len_max, d->block_len, d->n_keep_max)));
+  if (!kind || d->pool_window > kMaxFusedWindow || d->n_keep_max > d->seq_len_max - d->block_len || tuning().fused_refresh == 0) return false;
+  if (select_compact_is_fused(d->batch, d->n_kv_heads, d->seq_len_max, d->block_len, d->n_keep_max)) return pl.kind == 3 || !fold_delays_gather(d, pl);
+  return pl.kind != 3 && select_is_clustered(d->batch, d->n_kv_heads, d->seq_len_max, d->block_len, d->n_keep_max);
 }
 
 // What is left of a refresh to the launch that pools, selects and gathers.
@@ -167,10 +187,7 @@ void describe_rest(const sdllm_desc* d, const AttnPlan& pl, const AttnParams& p,
   fold->Hq = p.Hq; fold->G = p.G; fold->b = p.b; fold->M = p.M; fold->D = d->head_dim; fold->splits = pl.splits; fold->dtype = d->dtype;
   fold->row_tiles = pl.kind == 4 ? pl.row_tiles : 0;
   for (int i = 0; i < 3; ++i) fold->o_stride[i] = d->o_stride[i];
-  // a CTA of the launch behind folds 1024 float4 columns at a time
-  const int items = (fold->row_tiles > 0 ? fold->row_tiles * 128 : p.M) * (d->head_dim / 4);
-  const int room = sm_count() / (2 * d->batch * d->n_kv_heads);          // (at most half of the SMs)
-  fold->ctas = !folds ? 0 : ((items + 1023) / 1024 < room ? (items + 1023) / 1024 : (room > 1 ? room : 1));
+  fold->ctas = folds ? fold_ctas(d, pl) : 0;
 }
 
 // Part 1 of the refresh step. With `fold` the saliency is left unpooled in the workspace and the key splits unfolded; both are

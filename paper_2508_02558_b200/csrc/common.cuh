@@ -159,6 +159,7 @@ bool score_select_supported(int D, int M, int units, int cand);
 AttnPlan plan_attention_kt_beside(int D, int M, int B, int Hkv, int n1_max);       // the attention beside it
 cudaError_t launch_score_select(const AttnParams& p, const SelectParams& sp, const CompactParams& cp, int D, cudaStream_t st);
 bool select_compact_is_fused(int B, int Hkv, int Lmax, int b, int n_keep_max);
+int gather_ctas(int B, int Hkv, int n_keep_max, int folds);       // CTAs per head that copy rows there, beside `folds` that fold
 
 __host__ __device__ inline int keep_count_total(int pre, int suf, double r, int mode, int* n_pre, int* n_suf) {
   // Algorithm 1: n = floor(|I| * r) in double; the other policies are described in sdllm.h.

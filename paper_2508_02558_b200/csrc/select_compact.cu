@@ -368,12 +368,7 @@ template <bool RAW>
 cudaError_t launch_fused(const SelectParams& p, const CompactParams& cp, const FoldOf<RAW>& fold, cudaStream_t st) {
   int folds = 0;
   if constexpr (RAW) folds = fold.ctas;
-  // CTAs per head: fill the SMs, but leave every CTA at least 64 rows to copy
-  long long R = sm_count() / ((long long)p.B * p.Hkv) - folds;
-  if (R > p.n_keep_max / 64) R = p.n_keep_max / 64;
-  if (tuning().splits > 0) R = tuning().splits;
-  if (R > 16) R = 16;
-  if (R < 1) R = 1;
+  const int R = gather_ctas(p.B, p.Hkv, p.n_keep_max, folds);
   LaunchConfig lc(dim3((unsigned)R + folds, p.Hkv, p.B), 1024, (size_t)((p.n_keep_max + R - 1) / R + 1 + (RAW ? raw_axis_floats(p.Lmax, p.b, p.window) : 0)) * 4, st);
   if (tuning().pdl != 0) lc.after_start_of_previous();       // never releases its own dependents early
   const int cand = p.Lmax - p.b;
@@ -395,6 +390,14 @@ cudaError_t launch_compact(const CompactParams& p, cudaStream_t st) { return lau
 bool select_compact_is_fused(int B, int Hkv, int Lmax, int b, int n_keep_max) {
   const int cand = Lmax - b;
   return cand >= 1 && cand <= 8192 && n_keep_max >= 1 && (long long)B * Hkv <= sm_count() && tuning().select == 0;
+}
+
+// CTAs per head: fill the SMs, but leave every CTA at least 64 rows to copy.
+int gather_ctas(int B, int Hkv, int n_keep_max, int folds) {
+  long long R = sm_count() / ((long long)B * Hkv) - folds;
+  if (R > n_keep_max / 64) R = n_keep_max / 64;
+  if (tuning().splits > 0) R = tuning().splits;
+  return R > 16 ? 16 : (R < 1 ? 1 : (int)R);
 }
 
 cudaError_t launch_select_compact(const SelectParams& p, const CompactParams& cp, cudaStream_t st) {
