@@ -1083,8 +1083,14 @@ bool plan_attention_units(int D, int M, int b, int B, int Hkv, int n1_max, int n
 // The attention of a refresh whose saliency and selection run beside it (refresh_select.cu): CTAs of the small footprint on about
 // two thirds of the SMs, three tiles each or more. (32 heads x 1280 keys, the whole refresh with 2 / 3 / 4 / 6 splits: 18.6 / 18.2 /
 // 19.0 / 23.9 us; 64 units x 1280: 22.8 with two, 27.2 with one; 8 x 1280: 12.0 with four, 12.8 with three, 12.2 with six.)
+// From 66 units on that would be one split, which walks alone longer than all the rest takes (74 x 3100 keys, retention 0.25: 63.5 us, 43.1 with two; in
+// two parts 51.4): two, but for walks of up to six tiles of head dimension 64 (74 x 700: 14.8 with one, 15.7 with two). And three while they find an SM each
+// where the walks are long (43 x 2900: 34.1 with two, 29.6 with three).
 AttnPlan plan_attention_kt_beside(int D, int M, int B, int Hkv, int n1_max) {
-  const int units = B * Hkv, tiles = (n1_max + 127) / 128, fill = (2 * sm_count() / 3 + units / 2) / units, most = (tiles + 2) / 3;
+  const int sms = sm_count(), units = B * Hkv, tiles = (n1_max + 127) / 128, most = (tiles + 2) / 3;
+  int fill = (2 * sms / 3 + units / 2) / units;
+  if (fill < 2 && (D == 128 || tiles > 6)) fill = 2;
+  if (fill == 2 && D == 128 && tiles >= 14 && 3 * units <= sms) fill = 3;
   Tuning tn = tuning();
   if (tn.splits <= 0) tn.splits = fill < most ? (fill < 4 ? fill : 4) : (most < 4 ? most : 4);
   if (tn.splits < 1) tn.splits = 1;
