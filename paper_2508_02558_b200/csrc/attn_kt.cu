@@ -424,13 +424,18 @@ __global__ void __launch_bounds__(64 + 128 * WG * CG, (WG == 1 && CG == 1) ? 2 :
         tc_fence_after();
         if (st < NP) enc[st] = f2ord(usable_reference(m_ref[st]));
         softmax_barrier(bar_id);
+        // The logits again. With several column groups into registers of their own, and once more behind the barriers: over the distances
+        // it made the loop around this rare branch 2 to 3 % slower there (50 heads of 64 rows x 14387 keys 100.6 -> 103.0 us, so 99.2);
+        // with one column group it is the other way round (32 heads x 656 keys 6.85 and 6.94).
+        uint32_t again[NP];
+        uint32_t(&raw)[NP] = CG == 1 ? *reinterpret_cast<uint32_t(*)[NP]>(&sv[0]) : again;
         if (work) {
-          tmem_ld32(lane_addr + (uint32_t)sb * NPT + (uint32_t)cg * 32, *reinterpret_cast<uint32_t(*)[32]>(&sv[0]));
+          tmem_ld32(lane_addr + (uint32_t)sb * NPT + (uint32_t)cg * 32, raw);
           tc_wait_ld();
           float mine = -INFINITY;
 #pragma unroll
           for (int c = 0; c < NP; ++c) {
-            const float r = warp_max_f32(valid ? sv[c] * sl2 : -INFINITY);
+            const float r = warp_max_f32(valid ? __uint_as_float(raw[c]) * sl2 : -INFINITY);
             if (c == lane) mine = r;
           }
           atomicMax(enc + lane, f2ord(mine));
@@ -443,8 +448,14 @@ __global__ void __launch_bounds__(64 + 128 * WG * CG, (WG == 1 && CG == 1) ? 2 :
         }
         softmax_barrier(bar_id);
         // (at most zero but for the rounding of the reference, which for logits beyond 10^9 would be more than exp2 can take)
+        if (CG > 1 && work) {
+          tmem_ld32(lane_addr + (uint32_t)sb * NPT + (uint32_t)cg * 32, raw);
+          tc_wait_ld();
+        }
+        if (CG == 1 || work) {
 #pragma unroll
-        for (int c = 0; c < NP; ++c) sv[c] = min_nan(fmaf(sv[c], sl2, -m_ref[c]), 0.f);
+          for (int c = 0; c < NP; ++c) sv[c] = min_nan(fmaf(__uint_as_float(raw[c]), sl2, -m_ref[c]), 0.f);
+        }
         l_lane *= fast_exp2(-delta_s[lane]);
         if (t >= WG && !dead) {
           // this thread's TMEM lane is a head dimension of O^T here, not a key: all four warps rescale their lanes
