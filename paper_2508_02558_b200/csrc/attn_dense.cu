@@ -459,8 +459,10 @@ __global__ void __launch_bounds__(256) dense_fold_kernel(const DenseParams p) {
 // Costs in us beyond the full waves: a key tile 1.55, a CTA's set-up and way out 6.5.
 //   front   the cut units' launch first; the whole ones take the SMs as they come free and two idle warps of each fold the partial
 //           rows: 2 more for the partial rows and 0.25 per share (32 heads x 1280: 34.3 us; 8 x 5000: 91). A task of the fold, 64 rows
-//           of one float4 column, takes those warps 1.1 per six shares, so this is for few cut units: up to 0.6 of a CTA's time. The
-//           whole units' variant is 2 % slower per wave (32 / 8 heads x 5000, four waves: 334, and 332 with the cut units behind).
+//           of one float4 column, takes those warps 1.1 per six shares, up to 0.6 of a CTA's time. Per wave the whole units' variant is 2 %
+//           slower and the fold costs a tenth of its time there (head dimension 64, whose softmax is short of issue slots: 7 % from the second wave
+//           on, and three tenths), so this is for few cut units and few waves. 110 calls of one wave to six, behind / in front wherever the fold fits / by this rule: 16 heads x 5402, 56 cut
+//           units, 207.6 / 231.5 / 207.4; 32 x 2618 of head dimension 64, 56 cut units, 104.6 / 117.2 / 102.7; 64 x 1240, 24 cut, 65.0 / 60.8 / 60.8.
 //   behind  the cut units' launch overlaps the last wave and 2 of its set-up, a launch of its own folds: 7.25 (3 of it a margin)
 //           and 0.35 per share (39.3 and 94.4 us; 32 heads x 2600, 56 cut units: 116, and 124 with them in front).
 // Batches of several sequences may be ragged, which the host cannot see: they are cut only where all units fit one wave.
@@ -477,8 +479,10 @@ DensePlan plan_dense(int B, int Hq, int L, int D) {
   double least = whole;
   for (int q = 2; q <= 16 && q <= nt && rest * q <= sms; ++q) {
     const double tiles = 1.55 * ((nt + q - 1) / q), behind = (rest == units ? 6.5 : 4.5) + tiles + 7.25 + 0.35 * q;
-    const bool front = rest != units && 1.1 * ((q + 5) / 6) * (double)(rest * D) / (double)(units - rest) <= 0.6 * whole;
-    const double cost = front ? 8.5 + tiles + 0.25 * q + 0.02 * whole * (double)((units - rest) / sms) : behind;
+    const double fold = 1.1 * ((q + 5) / 6) * (double)(rest * D) / (double)(units - rest), waves = (double)((units - rest) / sms);
+    const double in_front = 8.5 + tiles + 0.25 * q + (D == 64 ? 0.07 * whole * (waves - 1) + 0.3 * fold * waves : (0.02 * whole + 0.1 * fold) * waves);
+    const bool front = rest != units && fold <= 0.6 * whole && in_front < behind;
+    const double cost = front ? in_front : behind;
     if (cost < least) { least = cost; pl.whole = (int)(units - rest); pl.parts = q; pl.front = front; }
   }
   return pl;

@@ -45,3 +45,21 @@ def test_query_rows_are_shared_out_to_units_where_that_is_faster(host_program):
     assert len(got) == len(UNITS)
     for (shape, (units, whole)), s in zip(UNITS.items(), got):
         assert (int(s) > 1) == (units < whole), (shape, s)
+
+
+# dense step, (head dimension, query heads, length): us with the cut units behind the whole ones, us with them in front, on a B200; the faster one is
+# to be taken
+CUT_UNITS = {
+    (128, 32, 1280): (40.4, 34.7), (128, 64, 1240): (65.0, 60.8), (128, 16, 2439): (59.1, 54.3), (128, 8, 4993): (94.4, 89.7), (128, 40, 1848): (81.0, 77.7),
+    (128, 16, 5402): (207.6, 231.5), (128, 24, 5212): (278.6, 297.5), (128, 28, 2937): (116.9, 121.6), (128, 32, 3915): (220.9, 226.8), (128, 12, 3516): (73.2, 77.9),
+    (64, 28, 1458): (39.6, 33.6), (64, 16, 2456): (52.9, 45.6), (64, 12, 3281): (59.3, 54.6), (64, 8, 5096): (85.5, 79.7), (64, 32, 1268): (35.1, 29.7),
+    (64, 32, 2618): (104.6, 117.2), (64, 24, 5139): (242.4, 268.6), (64, 12, 3757): (75.4, 80.7), (64, 28, 2901): (102.6, 110.6), (64, 64, 1548): (79.7, 83.2),
+}
+
+
+def test_cut_units_of_the_dense_step_go_in_front_where_that_is_faster(host_program):
+    exe = host_program("dense_plans.cpp")
+    got = subprocess.run([exe, *(str(x) for shape in CUT_UNITS for x in shape)], capture_output=True, text=True, check=True).stdout.split()
+    assert len(got) == len(CUT_UNITS)
+    for (shape, (behind, front)), n in zip(CUT_UNITS.items(), got):
+        assert int(n) == (2 if front < behind else 3), (shape, n)
