@@ -36,14 +36,16 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
 __device__ __forceinline__ void wait_merge(uint32_t bar, volatile int* abort_flag, int32_t* status, long long limit) {
   if (!mbar_try_wait_cluster(bar, 0)) {
     long long t0 = clock64();
-    bool draining = false;               // this CTA is aborting: its peers' pushes may still land before it retires, up to the drain limit
     while (!mbar_try_wait_cluster(bar, 0)) {
-      const long long waited = clock64() - t0;
-      if (!draining && *abort_flag != 0) { draining = true; t0 += waited; continue; }
-      if (waited <= (draining ? kDrainCycles : limit)) continue;
-      if (draining) break;
-      *abort_flag = 1;
-      atomicExch(status, 13);
+      const bool aborting = *abort_flag != 0;
+      // an aborting CTA still lets its peers' pushes land before it retires: a wait that gives up here begins again with the drain
+      // limit, and a warp whose wait gave up before comes here later
+      if (clock64() - t0 > (aborting ? kDrainCycles : limit)) {
+        if (aborting) break;
+        *abort_flag = 1;
+        atomicExch(status, 13);
+        t0 = clock64();
+      }
     }
   }
   __syncwarp();
