@@ -194,7 +194,10 @@ __global__ void __launch_bounds__(RS_THREADS, 3) score_select_kernel(const __gri
       if (w >= i_lo && w < i_hi) kept_s[w - i_lo] = c < h.o ? c : c + h.b;
     });
   } else {
-    others_of_share(sp, cp, gh, raw_s, h, out, head, r, R, z_lo, z_hi, tid - 32 * SW, NT - 32 * SW, g == 0);
+    const int t = tid - 32 * SW, nt = NT - 32 * SW;    // what does not wait for the selection
+    if (g == 0 && r == 0 && t == 0) sp.kept_cnt[bi] = h.kept;
+    write_pooled(sp, raw_s, h, head, r, R, t, nt);
+    write_empty_entries(cp, gh, out, z_lo, z_hi, t, nt);
   }
   __syncthreads();
   for (int i = i_lo + tid; i < i_hi; i += NT) out[i] = kept_s[i - i_lo];

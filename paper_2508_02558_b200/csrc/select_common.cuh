@@ -2,6 +2,8 @@
 // select (select_compact.cu, refresh_select.cu). Included inside namespace sdllm { namespace { ... } } of each of them.
 #pragma once
 
+#include "umma_ptx.cuh"
+
 // Order-preserving map fp32 -> u32 (larger float <=> larger key). -0 is folded onto +0 and NaN sorts lowest so the
 // order agrees with a numeric comparison of the values. No value maps to 0, which stands for "no candidate".
 __device__ __forceinline__ uint32_t score_key(float x) {
@@ -312,19 +314,8 @@ __device__ __forceinline__ void pool_keys(uint32_t (&key)[KPT], const RawAxis& a
   else pool_keys<0>(key, axis, raw, C, kpt, c0);
 }
 
-// What the warps that do not select write meanwhile, thread t of nt: CTA r's share of the head's pooled scores, its empty entries
-// [z_lo, z_hi) and their zero rows, and the count (once per sequence).
-__device__ __forceinline__ void others_of_share(const SelectParams& p, const CompactParams& cp, const GatherHead& gh, const float* raw, const HeadPlace& h,
-                                                int32_t* out, int64_t head, int r, int R, int z_lo, int z_hi, int t, int nt, bool first_head) {
-  if (first_head && r == 0 && t == 0) p.kept_cnt[head / p.Hkv] = h.kept;
-  if (raw != nullptr) {
-    const RawAxis axis(p, h);
-    const int p_hi = (int)((int64_t)(r + 1) * p.Lmax / R);
-    for (int pos = (int)((int64_t)r * p.Lmax / R) + t; pos < p_hi; pos += nt) {
-      const bool candidate = pos < h.o || (pos >= h.o + h.b && pos < h.C + h.b);
-      p.pooled_out[head * p.Lmax + pos] = candidate ? axis.pool<0>(raw, pos < h.o ? pos : pos - h.b) : -INFINITY;
-    }
-  }
+// The empty entries [z_lo, z_hi) of a head's list and their zero rows, by thread t of nt.
+__device__ __forceinline__ void write_empty_entries(const CompactParams& cp, const GatherHead& gh, int32_t* out, int z_lo, int z_hi, int t, int nt) {
   for (int i = z_lo + t; i < z_hi; i += nt) out[i] = -1;
   const int lg = 31 - __clz(cp.row_bytes / 16);        // log2 of the threads per row
   const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
@@ -334,11 +325,16 @@ __device__ __forceinline__ void others_of_share(const SelectParams& p, const Com
   }
 }
 
-__device__ __forceinline__ float ex2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;\n" : "=f"(y) : "f"(x));
-  return y;
+// CTA r's share of the head's pooled scores, pooled from the raw ones in shared memory, by thread t of nt.
+__device__ __forceinline__ void write_pooled(const SelectParams& p, const float* raw, const HeadPlace& h, int64_t head, int r, int R, int t, int nt) {
+  const RawAxis axis(p, h);
+  const int p_hi = (int)((int64_t)(r + 1) * p.Lmax / R);
+  for (int pos = (int)((int64_t)r * p.Lmax / R) + t; pos < p_hi; pos += nt) {
+    const bool candidate = pos < h.o || (pos >= h.o + h.b && pos < h.C + h.b);
+    p.pooled_out[head * p.Lmax + pos] = candidate ? axis.pool<0>(raw, pos < h.o ? pos : pos - h.b) : -INFINITY;
+  }
 }
+
 // CTA `part` of f.ctas folds its share of the rows of one (sequence, KV head).
 template <int NT>
 __device__ __forceinline__ void fold_head(const FoldParams& f, int bg, int bi, int g, int part) {
@@ -353,7 +349,7 @@ __device__ __forceinline__ void fold_head(const FoldParams& f, int bg, int bi, i
       const int64_t first = ((int64_t)bg * f.row_tiles + (m >> 7)) * f.splits;
       const float4* po = reinterpret_cast<const float4*>(f.part_o) + (first * c4n + c4) * 128 + (m & 127);
       const float2* pm = reinterpret_cast<const float2*>(f.part_ml) + first * 128 + (m & 127);
-      x = dev::fold_splits<6>(f.splits, [&](int s) { return __ldcg(pm + s * 128); }, [&](int s) { return __ldcg(po + (int64_t)s * c4n * 128); }, ex2_approx);
+      x = dev::fold_splits<6>(f.splits, [&](int s) { return __ldcg(pm + s * 128); }, [&](int s) { return __ldcg(po + (int64_t)s * c4n * 128); }, fast_exp2);
     } else {
       const float4* po = reinterpret_cast<const float4*>(f.part_o) + ((int64_t)bg * f.splits * f.M + m) * c4n + c4;
       const float2* pm = reinterpret_cast<const float2*>(f.part_ml) + (int64_t)bg * f.splits * f.M + m;

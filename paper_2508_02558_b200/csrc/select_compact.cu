@@ -1,5 +1,7 @@
 // Top-k selection over the pooled importance scores and the K/V gather-compaction
 // (Algorithm 1: "n <- floor(|I| r)", "TopKIndices(I, n)", "Select(K_f, I)", "Select(V_f, I)").
+#include <cuda.h>
+
 #include <type_traits>
 
 #include "common.cuh"
@@ -264,17 +266,9 @@ __global__ void __launch_bounds__(1024) select_gather_kernel(const SelectParams 
     });
   } else {
     const int t = tid - 32 * SW, nt = NT - 32 * SW;
-    if constexpr (RAW) {
-      others_of_share(p, cp, gh, raw_s, h, out, bi * p.Hkv + g, r, R, z_lo, z_hi, t, nt, g == 0);
-    } else {
-      if (g == 0 && r == 0 && t == 0) p.kept_cnt[bi] = h.kept;
-      for (int i = z_lo + t; i < z_hi; i += nt) out[i] = -1;
-      const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-      for (int i = z_lo + (t >> lg); i < z_hi; i += nt >> lg) {
-        reinterpret_cast<uint4*>(gh.k_c + (int64_t)i * cp.c_stride_bytes[2])[t & ((1 << lg) - 1)] = zero;
-        reinterpret_cast<uint4*>(gh.v_c + (int64_t)i * cp.c_stride_bytes[2])[t & ((1 << lg) - 1)] = zero;
-      }
-    }
+    if (g == 0 && r == 0 && t == 0) p.kept_cnt[bi] = h.kept;
+    if constexpr (RAW) write_pooled(p, raw_s, h, bi * p.Hkv + g, r, R, t, nt);
+    write_empty_entries(cp, gh, out, z_lo, z_hi, t, nt);
   }
   __syncthreads();
 
