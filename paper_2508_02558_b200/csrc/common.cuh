@@ -68,8 +68,8 @@ struct AttnParams {
   int32_t* counters;           // completion counters (tcgen05 kernel), zero between calls
   float* pooled;               // refresh with a fused tail: pooled scores [B][Hkv][n1_max], else null
   int window, pool_kind, per_region;
-  const float* lse_in;         // probability saliency, second pass: log-sum-exp of every block row [B][Hq][b]
   int releases_late;           // key-row kernel: the next launch may start once this one has seen everything before it complete, not earlier
+  const float* lse_in;         // probability saliency, second pass: log-sum-exp of every block row [B][Hq][b]
   int unfolded;                // the key splits are folded, and the saliency is pooled, by the launch behind
   int want_scores;             // compute mean-query logit scores for src1 keys
   float scale;                 // softmax scale
