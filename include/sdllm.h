@@ -185,8 +185,8 @@ sdllm_status sdllm_select_compact(const sdllm_desc* desc, const float* pooled_sc
                                   int32_t* kept_cnt, void* k_c, void* v_c, void* cuda_stream);
 
 /* The whole refresh step in one call: the results of sdllm_refresh_scores followed by sdllm_select_compact (pooled_scores is an
- * output here, not NULL). Where sdllm_select_compact is one launch, that launch also pools the saliency and folds the attention's
- * key splits, or computes the saliency itself beside the attention; sdllm_launch_count tells how many launches that leaves. out and
+ * output here, not NULL). Where it is faster, the launch that selects also pools the saliency and folds the attention's key splits,
+ * or computes the saliency itself beside the attention; sdllm_plan_describe tells which, sdllm_launch_count how many launches. out and
  * lse may then differ from sdllm_refresh_scores' in the rounding of other key splits; pooled_scores, kept_idx, k_c and v_c do not.
  * seq_len and block_off are read early, as by sdllm_select_compact, and the compacted cache may be read early behind it. Workspace:
  * sdllm_workspace_bytes(desc, SDLLM_OP_REFRESH). */

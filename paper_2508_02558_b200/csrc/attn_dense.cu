@@ -16,7 +16,7 @@
 //   - P is handed over in two parts (96 keys, then 32), so that the first MMAs of P V run under the last exponentials;
 //   - three-operand maxima, two-lane fp32 arithmetic, a quarter of the exponentials on the FMA pipe (poly_exp2), one
 //     warp-uniform branch for the rare rescale, registers moved to the softmax warps (208 instead of 168).
-// 32 heads x 1280 rows: 56.3 -> 44.0 us (34.3 with the last wave's units cut, see plan_dense); 32 (8 KV) heads x 32768 rows: 17.1 -> 14.6 ms, 1204 TFLOP/s. The long case is
+// 32 heads x 1280 rows: 56.3 -> 44.0 us (34.7 with the last wave's units cut, see plan_dense); 32 (8 KV) heads x 32768 rows: 17.1 -> 14.6 ms, 1204 TFLOP/s. The long case is
 // bound by power (1.6 GHz under the 1000 W cap, where a library GEMM sustains 1408); a burst at full clock runs at 1368.
 // The finished rows go from TMEM through registers straight to global memory (bf16), normalised by the row sum.
 // Every wait on an mbarrier is bounded; on expiry the CTA sets an abort flag, records a code in the status word and
@@ -458,13 +458,13 @@ __global__ void __launch_bounds__(256) dense_fold_kernel(const DenseParams p) {
 // unit takes a whole SM, so without that 160 units on 148 SMs run in two waves (32 heads x 1280 rows: 44.0 us).
 // Costs in us beyond the full waves: a key tile 1.55, a CTA's set-up and way out 6.5.
 //   front   the cut units' launch first; the whole ones take the SMs as they come free and two idle warps of each fold the partial
-//           rows: 2 more for the partial rows and 0.25 per share (32 heads x 1280: 34.3 us; 8 x 5000: 91). A task of the fold, 64 rows
+//           rows: 2 more for the partial rows and 0.25 per share (32 heads x 1280: 34.7 us; 8 x 5000: 90). A task of the fold, 64 rows
 //           of one float4 column, takes those warps 1.1 per six shares, up to 0.6 of a CTA's time. Per wave the whole units' variant is 2 %
 //           slower and the fold costs a tenth of its time there (head dimension 64, whose softmax is short of issue slots: 7 % from the second wave
 //           on, and three tenths), so this is for few cut units and few waves. 110 calls of one wave to six, behind / in front wherever the fold fits / by this rule: 16 heads x 5402, 56 cut
 //           units, 207.6 / 231.5 / 207.4; 32 x 2618 of head dimension 64, 56 cut units, 104.6 / 117.2 / 102.7; 64 x 1240, 24 cut, 65.0 / 60.8 / 60.8.
 //   behind  the cut units' launch overlaps the last wave and 2 of its set-up, a launch of its own folds: 7.25 (3 of it a margin)
-//           and 0.35 per share (39.3 and 94.4 us; 32 heads x 2600, 56 cut units: 116, and 124 with them in front).
+//           and 0.35 per share (40.4 and 94.4 us; 32 heads x 2600, 56 cut units: 116, and 124 with them in front).
 // Batches of several sequences may be ragged, which the host cannot see: they are cut only where all units fit one wave.
 struct DensePlan {
   int whole, parts;

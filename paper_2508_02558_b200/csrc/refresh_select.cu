@@ -4,7 +4,7 @@
 // The kept entries depend on the logits' means alone, not on the softmax, so nothing here has to wait for the attention; in a chain
 // of the two a refresh of 32 heads x 1280 keys took 10 us of attention and 10 of selection and gather. For 10 MB of keys a second
 // product K Q^T is cheap: K comes from L2 the second time. Whole refreshes, one after the other and beside: 32 heads x 300 / 1280 /
-// 3100 keys 13.1 / 20.6 / 33.5 us and 11.0 / 17.4 / 30.4; 8 x 1280 15.6 and 12.3; 64 x 1280 28.7 and 22.7; 16 x 2048 alike. What is
+// 3100 keys 13.0 / 21.6 / 33.2 us and 11.0 / 17.6 / 30.0; 8 x 1280 15.0 and 12.0; 64 x 1280 28.6 and 21.9; 74 x 1280 31.1 and 23.6. What is
 // left is a chain: 2 us to start behind the attention's first CTAs, 4 for the scores, 5 for the selection, 2.5 for the gather.
 //   scores   the CTAs of the cluster share the head's tiles of 128 keys: TMA, S^T [128 keys x N queries] = K_tile Q^T (tcgen05), and
 //            the thread that owns a key adds its logits up in the order of attn_kt.cu, so that the scores are that kernel's bit for
