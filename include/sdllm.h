@@ -230,7 +230,8 @@ sdllm_status sdllm_dense_attn(const sdllm_desc* desc, const void* q, const int64
  * nowhere to get the workspace from. For them the scratch (status word, completion counters, key-split partials) is an
  * array of 8 MiB plus 768 bytes built into the library image; every GPU that loads the library holds one copy until the
  * process exits.
- *   - Shapes whose workspace (sdllm_workspace_bytes(desc, SDLLM_OP_SPARSE_BLOCK_ATTN)) exceeds that are refused with
+ *   - Shapes whose workspace (sdllm_workspace_bytes(desc, SDLLM_OP_SPARSE_BLOCK_ATTN)) exceeds that run with a plan that needs
+ *     less where there is one (grouped heads with short caches; the rounding may then differ), or are refused with
  *     SDLLM_ERR_WORKSPACE; use sdllm_sparse_block_attn with a caller-owned workspace for those.
  *   - The call allocates and frees nothing. The first call on each device looks the array's device address up
  *     (cudaGetSymbolAddress, with that device current); make that first call before any stream capture.

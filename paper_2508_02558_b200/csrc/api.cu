@@ -77,12 +77,12 @@ bool cuda_failed(cudaError_t e, const char* what) {
 
 float scale_of(const sdllm_desc* d) { return d->softmax_scale > 0.f ? d->softmax_scale : 1.0f / sqrtf((float)d->head_dim); }
 
-AttnPlan plan_for(const sdllm_desc* d, int op) {
+AttnPlan plan_for(const sdllm_desc* d, int op, bool small = false) {
   const int G = d->n_q_heads / d->n_kv_heads;
   const bool refresh = op == SDLLM_OP_REFRESH_SCORES;
   return plan_attention(d->dtype, d->head_dim, G * d->block_len, d->block_len, d->batch, d->n_kv_heads,
                         refresh ? d->seq_len_max : d->n_keep_max, refresh ? 0 : d->block_len,
-                        refresh && d->score == SDLLM_SCORE_PROB_MEAN);
+                        refresh && d->score == SDLLM_SCORE_PROB_MEAN, small);
 }
 
 void fill_common(AttnParams& p, const sdllm_desc* d, const AttnPlan& pl) {
@@ -299,6 +299,41 @@ sdllm_status check_select_compact_args(const sdllm_desc* d, const float* pooled_
   return SDLLM_OK;
 }
 
+// The reuse step with plan `pl`.
+sdllm_status sparse_block_attn(const sdllm_desc* d, const AttnPlan& pl, const void* q_blk, const void* k_c, const void* v_c, const int32_t* kept_cnt,
+                               const void* k_blk, const void* v_blk, void* out, void* ws, size_t ws_bytes, void* cuda_stream) {
+  sdllm_status st = SDLLM_OK;
+  const AttnWorkspace w = attn_workspace(d, pl, false);
+  if (w.total > 0 && (ws == nullptr || ws_bytes < w.total || (reinterpret_cast<uintptr_t>(ws) & 255u))) return SDLLM_ERR_WORKSPACE;
+  if ((st = check_device()) != SDLLM_OK) return st;
+  cudaStream_t stream = reinterpret_cast<cudaStream_t>(cuda_stream);
+  char* wsb = reinterpret_cast<char*>(ws);
+
+  AttnParams p{};
+  fill_common(p, d, pl);
+  p.q = q_blk; p.k1 = k_c ? k_c : k_blk; p.v1 = v_c ? v_c : v_blk; p.k2 = k_blk; p.v2 = v_blk;
+  p.n1_per_seq = kept_cnt; p.block_off = nullptr;
+  p.out = out; p.lse = nullptr;
+  p.status = reinterpret_cast<int32_t*>(wsb);
+  p.part_o = reinterpret_cast<float*>(wsb + w.part_o);
+  p.part_ml = reinterpret_cast<float*>(wsb + w.part_ml);
+  p.raw_scores = nullptr;
+  p.n1_max = d->n_keep_max; p.n2 = d->block_len;
+  p.want_scores = 0;
+  p.counters = reinterpret_cast<int32_t*>(wsb + kWsStatusBytes);
+  p.pooled = nullptr;
+  for (int i = 0; i < 3; ++i) { p.k1_stride[i] = d->c_stride[i]; p.k2_stride[i] = d->blk_stride[i]; }
+  if (cuda_failed(launch_attn_partial(p, pl, d->dtype, d->head_dim, stream), "attention launch")) return SDLLM_ERR_CUDA;
+  if (pl.splits > 1 && !pl.fused_tail) {
+    MergeParams m{};
+    m.part_o = p.part_o; m.part_ml = p.part_ml; m.out = out; m.lse = nullptr;
+    m.B = p.B; m.Hq = p.Hq; m.Hkv = p.Hkv; m.G = p.G; m.b = p.b; m.M = p.M; m.D = d->head_dim; m.splits = pl.splits; m.dtype = d->dtype;
+    for (int i = 0; i < 3; ++i) m.o_stride[i] = d->o_stride[i];
+    if (cuda_failed(launch_merge_pool(m, stream), "merge/pool launch")) return SDLLM_ERR_CUDA;
+  }
+  return SDLLM_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -478,36 +513,7 @@ sdllm_status sdllm_sparse_block_attn(const sdllm_desc* d, const void* q_blk, con
   sdllm_status st = check_desc(d);
   if (st != SDLLM_OK) return st;
   if ((st = check_sparse_args(d, q_blk, k_c, v_c, kept_cnt, k_blk, v_blk, out)) != SDLLM_OK) return st;
-  const AttnPlan pl = plan_for(d, SDLLM_OP_SPARSE_BLOCK_ATTN);
-  const AttnWorkspace w = attn_workspace(d, pl, false);
-  if (w.total > 0 && (ws == nullptr || ws_bytes < w.total || (reinterpret_cast<uintptr_t>(ws) & 255u))) return SDLLM_ERR_WORKSPACE;
-  if ((st = check_device()) != SDLLM_OK) return st;
-  cudaStream_t stream = reinterpret_cast<cudaStream_t>(cuda_stream);
-  char* wsb = reinterpret_cast<char*>(ws);
-
-  AttnParams p{};
-  fill_common(p, d, pl);
-  p.q = q_blk; p.k1 = k_c ? k_c : k_blk; p.v1 = v_c ? v_c : v_blk; p.k2 = k_blk; p.v2 = v_blk;
-  p.n1_per_seq = kept_cnt; p.block_off = nullptr;
-  p.out = out; p.lse = nullptr;
-  p.status = reinterpret_cast<int32_t*>(wsb);
-  p.part_o = reinterpret_cast<float*>(wsb + w.part_o);
-  p.part_ml = reinterpret_cast<float*>(wsb + w.part_ml);
-  p.raw_scores = nullptr;
-  p.n1_max = d->n_keep_max; p.n2 = d->block_len;
-  p.want_scores = 0;
-  p.counters = reinterpret_cast<int32_t*>(wsb + kWsStatusBytes);
-  p.pooled = nullptr;
-  for (int i = 0; i < 3; ++i) { p.k1_stride[i] = d->c_stride[i]; p.k2_stride[i] = d->blk_stride[i]; }
-  if (cuda_failed(launch_attn_partial(p, pl, d->dtype, d->head_dim, stream), "attention launch")) return SDLLM_ERR_CUDA;
-  if (pl.splits > 1 && !pl.fused_tail) {
-    MergeParams m{};
-    m.part_o = p.part_o; m.part_ml = p.part_ml; m.out = out; m.lse = nullptr;
-    m.B = p.B; m.Hq = p.Hq; m.Hkv = p.Hkv; m.G = p.G; m.b = p.b; m.M = p.M; m.D = d->head_dim; m.splits = pl.splits; m.dtype = d->dtype;
-    for (int i = 0; i < 3; ++i) m.o_stride[i] = d->o_stride[i];
-    if (cuda_failed(launch_merge_pool(m, stream), "merge/pool launch")) return SDLLM_ERR_CUDA;
-  }
-  return SDLLM_OK;
+  return sparse_block_attn(d, plan_for(d, SDLLM_OP_SPARSE_BLOCK_ATTN), q_blk, k_c, v_c, kept_cnt, k_blk, v_blk, out, ws, ws_bytes, cuda_stream);
 }
 
 sdllm_status sdllm_dense_attn(const sdllm_desc* d, const void* q, const int64_t* q_stride, const void* k, const void* v,
@@ -533,14 +539,15 @@ sdllm_status sdllm_sparse_block_attn_static(const sdllm_desc* d, const void* q_b
   sdllm_status st = check_desc(d);
   if (st != SDLLM_OK) return st;
   if ((st = check_sparse_args(d, q_blk, k_c, v_c, kept_cnt, k_blk, v_blk, out)) != SDLLM_OK) return st;
-  const AttnWorkspace w = attn_workspace(d, plan_for(d, SDLLM_OP_SPARSE_BLOCK_ATTN), false);
-  if (w.total > kStaticScratchBytes) return SDLLM_ERR_WORKSPACE;       // this shape needs more than the built-in scratch
+  AttnPlan pl = plan_for(d, SDLLM_OP_SPARSE_BLOCK_ATTN);
+  if (attn_workspace(d, pl, false).total > kStaticScratchBytes) pl = plan_for(d, SDLLM_OP_SPARSE_BLOCK_ATTN, true);
+  if (attn_workspace(d, pl, false).total > kStaticScratchBytes) return SDLLM_ERR_WORKSPACE;       // this shape needs more than the built-in scratch
   if ((st = check_device()) != SDLLM_OK) return st;
   void* scratch = nullptr;
   if ((st = static_scratch_address(&scratch)) != SDLLM_OK) return st;
   // the status word and the completion counters must start at zero whatever the last call left behind
   if (cuda_failed(cudaMemsetAsync(scratch, 0, kWsDataOffset, reinterpret_cast<cudaStream_t>(cuda_stream)), "scratch clear")) return SDLLM_ERR_CUDA;
-  return sdllm_sparse_block_attn(d, q_blk, k_c, v_c, kept_cnt, k_blk, v_blk, out, scratch, kStaticScratchBytes, cuda_stream);
+  return sparse_block_attn(d, pl, q_blk, k_c, v_c, kept_cnt, k_blk, v_blk, out, scratch, kStaticScratchBytes, cuda_stream);
 }
 
 }  // extern "C"

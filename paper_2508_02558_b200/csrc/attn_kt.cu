@@ -1046,7 +1046,8 @@ AttnPlan plan_attention_kt(int D, int M, int b, int B, int Hkv, int n1_max, int 
 //     6.9; 8500 keys, nine tiles, 10.0 and 12.7), beyond one per four SMs only full units. Half-filled ones (7 x 8 rows) walk the
 //     keys once per unit for little: 12 heads x 12500 keys 18.1 against 63 us.
 // Nine to twelve groups are few for so many units: four splits that walk less than a tile each cost more than they save.
-bool plan_attention_units(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn, AttnPlan* pl) {
+// With `small`, wherever there are units for it at all: their splits merge in their cluster, so they leave nothing in the workspace.
+bool plan_attention_units(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn, bool small, AttnPlan* pl) {
   const int sms = sm_count(), G = M / b, groups = (n1_max + 31) / 32 + (n2 + 31) / 32, T = (groups + 3) / 4;
   const double tiles = 0.25 * groups;
   const long long heads = (long long)B * Hkv;
@@ -1074,7 +1075,7 @@ bool plan_attention_units(int D, int M, int b, int B, int Hkv, int n1_max, int n
   one_unit.persist = 0;
   *pl = plan_attention_kt(D, M / s, b, B, Hkv * s, n1_max, n2, one_unit);
   pl->kv_share = s;
-  if (tn.unit_rows > 0 || groups <= 6) return true;
+  if (small || tn.unit_rows > 0 || groups <= 6) return true;
   const int rows = M / s, walk = ((groups + pl->cluster - 1) / pl->cluster + 3) / 4;      // tiles of the longest walk
   const long long units = heads * s;
   if (M > 128) return rows <= 32 || walk <= 4 || (units > 16 && walk <= 6) || units > 64;

@@ -752,11 +752,11 @@ AttnPlan plan_attention_kt(int D, int M, int b, int B, int Hkv, int n1_max, int 
 cudaError_t launch_attn_kt(const AttnParams& p, const AttnPlan& pl, int D, cudaStream_t st);
 
 bool pair_supported(int dtype, int D, int M, int b);
-bool plan_attention_units(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn, AttnPlan* pl);
+bool plan_attention_units(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn, bool small, AttnPlan* pl);
 AttnPlan plan_attention_pair(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn);
 cudaError_t launch_attn_pair(const AttnParams& p, const AttnPlan& pl, int D, cudaStream_t st);
 
-AttnPlan plan_attention(int dtype, int D, int M, int b, int B, int Hkv, int n1_max, int n2, bool prob_scores) {
+AttnPlan plan_attention(int dtype, int D, int M, int b, int B, int Hkv, int n1_max, int n2, bool prob_scores, bool small) {
   // bf16 goes to the tcgen05 kernels wherever they apply: heads with few query rows to the kernel that puts the keys on the
   // accumulator rows, the rest to the one that puts the queries there and has two softmax warpgroups (attn_pair.cu). fp32 and
   // the remaining bf16 shapes go to the cp.async kernels. Tuning::kernel forces a family.
@@ -764,7 +764,7 @@ AttnPlan plan_attention(int dtype, int D, int M, int b, int B, int Hkv, int n1_m
   const Tuning tn = tuning();
   if (prob_scores && tn.kernel != 1 && umma_supported(dtype, D, M, b)) return plan_attention_umma(D, M, b, B, Hkv, n1_max, tn);
   AttnPlan units;
-  if (n2 > 0 && tn.kernel == 0 && umma_supported(dtype, D, 16, 16) && plan_attention_units(D, M, b, B, Hkv, n1_max, n2, tn, &units)) return units;
+  if (n2 > 0 && tn.kernel == 0 && umma_supported(dtype, D, 16, 16) && plan_attention_units(D, M, b, B, Hkv, n1_max, n2, tn, small, &units)) return units;
   const bool kt_ok = kt_supported(dtype, D, M, b);
   if (kt_ok && (tn.kernel == 3 || (tn.kernel == 0 && kt_preferred(D, M, B, Hkv, n1_max, n2))))
     return plan_attention_kt(D, M, b, B, Hkv, n1_max, n2, tn);

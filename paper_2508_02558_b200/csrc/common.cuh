@@ -123,7 +123,8 @@ struct AttnWorkspace {         // offsets in bytes; what lies at an offset ends 
   size_t part_o, part_ml, raw, lse, total;
 };
 AttnWorkspace attn_workspace(const sdllm_desc* d, const AttnPlan& pl, bool scores);
-AttnPlan plan_attention(int dtype, int D, int M, int b, int B, int Hkv, int n1_max, int n2, bool prob_scores);
+// small: a reuse step of grouped heads takes the plan with the smaller workspace where there are two.
+AttnPlan plan_attention(int dtype, int D, int M, int b, int B, int Hkv, int n1_max, int n2, bool prob_scores, bool small = false);
 cudaError_t launch_prob_saliency(const AttnParams& p, int D, cudaStream_t st);    // second pass of the probability saliency
 
 bool umma_tail_is_fused(const AttnPlan& pl, int D, int M);

@@ -8,7 +8,7 @@
 #include "tuning.cuh"
 
 namespace sdllm {
-bool plan_attention_units(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn, AttnPlan* pl);
+bool plan_attention_units(int D, int M, int b, int B, int Hkv, int n1_max, int n2, const Tuning& tn, bool small, AttnPlan* pl);
 }
 
 int main(int argc, char** argv) {
@@ -16,7 +16,7 @@ int main(int argc, char** argv) {
     int a[5];
     for (int j = 0; j < 5; ++j) a[j] = atoi(argv[i + j]);
     sdllm::AttnPlan pl{};
-    printf("%d\n", sdllm::plan_attention_units(a[0], a[1] * a[2], a[2], 1, a[3], a[4], a[2], sdllm::Tuning{}, &pl) ? pl.kv_share : 0);
+    printf("%d\n", sdllm::plan_attention_units(a[0], a[1] * a[2], a[2], 1, a[3], a[4], a[2], sdllm::Tuning{}, false, &pl) ? pl.kv_share : 0);
   }
   return 0;
 }
