@@ -1036,14 +1036,14 @@ AttnPlan plan_attention_kt(int D, int M, int b, int B, int Hkv, int n1_max, int 
 // more than eight. From 2628 calls (head dimension 64 and 128, 33 to 256 rows, 1 to 64 heads, 50 to 12500 cached keys; units and whole
 // heads timed one after the other): the rule takes units for 2010 of them, 18 % faster on average there; 29 lose more than 2 %, at most 10.
 //   - 65 to 128 rows: two tiles a CTA, three where whole heads have few splits or are few themselves (8 KV heads of 4 x 32 rows, 400 / 1000 /
-//     2000 keys: 8.6 / 9.4 / 10.1 us, now 7.0 / 8.4 / 9.0; at 3273 keys, four tiles, 13.5 against 11.3). Units of 64 rows, which walk twice as many
+//     2000 keys: 8.6 / 9.4 / 10.1 us, now 7.0 / 8.4 / 9.0; at 3273 keys, four tiles, 13.5 against 11.5). Units of 64 rows, which walk twice as many
 //     tiles, only from 25 heads on (32 heads x 1000 keys 15.3, now 14.1; 8 x 3000, where there were such units, 11.8 and 12.4);
 //   - more rows, two Q tiles in the query-row kernel: units of 32 rows up to four and a half tiles in all (100 / 400 keys, 4 KV heads of
 //     7 x 32 rows: 9.4 / 9.2 us, now 5.3 / 6.5), full units of 64 up to four a CTA, further with more units (8 KV heads of 4 x 64 rows, 1000
 //     keys: 13.0 us, now 11.2; 4 x 4000, five tiles, 13.0 and 14.4);
 //   - 33 to 64 rows, head dimension 128: four and a half tiles in all (8 KV heads of 4 x 16 rows, 150 keys: 7.3 us, now 5.4);
 //   - head dimension 64, whose tile is half the bytes: four tiles a CTA while the units are few (2 heads of 4 x 16 rows, 3000 keys: 8.6 us, now
-//     6.9; 8500 keys, nine tiles, 10.0 and 12.7), beyond one per four SMs only full units. Half-filled ones (7 x 8 rows) walk the
+//     6.9; 8500 keys, nine tiles, 10.0 and 12.7), beyond one per four SMs only full units. Those that fill a quarter (7 x 8 rows) walk the
 //     keys once per unit for little: 12 heads x 12500 keys 18.1 against 63 us.
 // Nine to twelve groups are few for so many units: four splits that walk less than a tile each cost more than they save.
 // With `small`, wherever there are units for it at all: their splits merge in their cluster, so they leave nothing in the workspace.
